@@ -1,59 +1,84 @@
 // efim_decode_attn: split-KV paged decode attention with a log-sum-exp merge
-// (decode of the generated middle, EFIM Sec. 2.2 / Fig. 4).  Bandwidth-bound:
-// every K/V byte of the visible context is read once with 128-bit loads, the dot
-// products run on fp32 FMAs, the reductions on warp shuffles; no tensor cores.
+// (decode of the generated middle, EFIM Sec. 2.2 / Fig. 4).  Bandwidth-bound: every K/V
+// byte of the visible context is read once, whatever the number of query heads that share it.
 //
-// One CTA = (query row, kv head [x group tile], key chunk).  Each of its 4 warps
-// walks whole pages (16 tokens) round-robin, staged into shared memory by bulk
-// copies (one per K page and V page).  Inside a warp D/8 lanes share one token
-// row (16 bytes each), so 32/(D/8) tokens are read per 128-bit shared-memory load.
+// One CTA = (query row, kv head [x tile of at most 16 query heads], key chunk).  Each of its 4
+// warps walks whole pages (16 tokens) round-robin, staged into shared memory by one bulk-tensor
+// copy per K page and V page.  A page is one 16-row tile of the warp's matrix instructions
+// (mma.sync m16n8k16, bf16 in, fp32 accumulation), with the query heads along n:
+//   S^T [16 tokens][heads]  = K [16][D] Q^T [D][heads]
+//   O^T [D][heads]         += V^T [D][16] P^T [16][heads]
+// The softmax runs on the S^T fragments (a lane holds 2 tokens x 2 heads, so 4 exponentials a
+// page); P^T is the same fragments transposed by movmatrix.  P keeps its fp32 precision: it enters
+// the second product as three bf16 terms (hi + mid + lo, 24 significant bits in all).
+//
+// Bound: HBM.  A page's 16 tokens are exactly one m-tile and there is nothing to share between
+// pages, so warp-level instructions fit where a 128-row tcgen05 tile would be mostly padding; one
+// page costs a warp about 160 instructions for any group of up to 8 heads, against some 600 for
+// 4 heads on fp32 FMAs (which bound groups of 5 and more, and through the power limit long steps
+// of 4).  Split kernel, before -> after: 64 rows x 1-16k keys at 28/4 heads 233 -> 113 us (3.1 ->
+// 6.5 TB/s), 256 rows x 4-32k at 32/8 3.2-3.4 -> 2.58 ms (7.1 TB/s), 16 rows x 2-8k at 32/32 179 ->
+// 173 us, 16 rows x 2-2.9k at 32/8 41 -> 28 us.
 #include "decode_attn.cuh"
 #include "mbar.cuh"
+#include "prefill_tc.cuh"
 #include <algorithm>
+#include <atomic>
 
 namespace efim {
 
-// Sum x[0..N) across the `LPT` lanes of a token group, leaving N/LPT sums per lane.
-// Round with lane-bit `off`: lanes with the bit clear keep the lower half of the
-// values and receive the partner's lower half; the others the upper half.  After
-// all rounds lane j holds the values whose index has, from the top bit down, the
-// bits of j; the remaining low index bits enumerate the values it keeps.
-template <int N, int LPT>
-__device__ __forceinline__ void transposed_reduce(float* x, int j) {
-  int n = N;
-#pragma unroll
-  for (int off = LPT / 2; off >= 1; off >>= 1) {
-    const int half = n / 2;
-    const bool up = (j & off) != 0;
-#pragma unroll
-    for (int i = 0; i < N / 2; ++i) {
-      if (i < half) {
-        const float send = up ? x[i] : x[i + half];
-        const float keep = up ? x[i + half] : x[i];
-        x[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-      }
-    }
-    n = half;
-  }
-}
-
 // ---- shared-memory staging of whole pages -------------------------------------------
-// One (page, kv head) tile is 16*D*2 contiguous bytes in a pool, so a single bulk copy
-// brings it into shared memory.  Every warp owns a ring of DEC_STAGES stages (K page +
-// V page), keeps DEC_STAGES pages in flight without holding them in registers, and
-// consumes them in order; an mbarrier per stage counts the copied bytes.  Two stages make
-// the ring 64 KB per CTA at D = 128, so three CTAs (12 warps) share an SM: the kernel is
-// short of warps to issue from, not of bytes in flight (with three stages and two CTAs
-// per SM it ran at 84 % of the measured copy bandwidth, with two and three at 99 %).
-// Group tiles of more than 4 query heads need the registers of a third CTA for their q and o
-// rows: they run two CTAs to an SM and take a third stage instead.
-__host__ __device__ constexpr int dec_stages(int group_tile) { return group_tile > 4 ? 3 : 2; }
-__host__ __device__ constexpr int dec_ctas_per_sm(int group_tile) { return group_tile > 4 ? 2 : 3; }
+// Every warp owns a ring of dec_stages pages (K + V), keeps them in flight without holding them
+// in registers and consumes them in order; an mbarrier per stage counts the copied bytes.  64 KB
+// of ring per CTA, three CTAs (12 warps, 192 KB in flight) per SM.
+constexpr int DEC_WARPS = 4;
+constexpr int DEC_THREADS = 32 * DEC_WARPS;
+constexpr int DEC_CTAS_PER_SM = 3;
+__host__ __device__ constexpr int dec_stages(int D) { return D == 128 ? 2 : 4; }
+__host__ __device__ constexpr int dec_ring_bytes(int D) { return DEC_WARPS * dec_stages(D) * 2 * 16 * D * 2; }
 
-__device__ __forceinline__ void dec_bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
+// One (page, kv head) of a pool into shared memory as [slot / 8][dim / 64][slot % 8][64 dims],
+// 16-byte chunk c of a 128-byte row at chunk position c ^ (slot & 7): ldmatrix reads it without
+// bank conflicts, plain or transposed.
+__device__ __forceinline__ void dec_load_page(uint32_t dst, const CUtensorMap* map, uint32_t bar, int page_head) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %3, %3, %3, %4}], "
+      "[%2];" ::"r"(dst),
+      "l"(map), "r"(bar), "r"(0), "r"(page_head)
+      : "memory");
+}
+// byte offset of 16-byte chunk `c` (0 .. D/8-1) of slot `t` in a staged page
+template <int D>
+__device__ __forceinline__ uint32_t dec_page_off(int t, int c) {
+  return (uint32_t)((t >> 3) * (D * 16) + (c >> 3) * 1024 + (t & 7) * 128 + (((c & 7) ^ (t & 7)) << 4));
+}
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t* r) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
                : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t addr, uint32_t* r) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t movm_t(uint32_t v) {
+  uint32_t r;
+  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
+}
+// c += a b, a 16 x 16 (row), b 16 x 8 (col), bf16 in, fp32 accumulation
+__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ float dec_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // Rotation of one 16-byte vector (8 bf16) of a head row, exactly as efim_kv_append does it
@@ -89,43 +114,40 @@ __device__ __forceinline__ uint4 dec_rotate_vec(uint4 mine, uint4 other, const f
   return mine;
 }
 
-// GT query heads of one kv head per CTA.  Up to 4 heads are scored in one pass over a staged
-// page; 5 to 7 in two passes of 4 (the second padded with zero queries) over the same page in
-// shared memory - the K/V bytes come from HBM once.
-template <int D, int GT, bool FUSED>
-__global__ void __launch_bounds__(128, dec_ctas_per_sm(GT)) decode_splitkv_kernel(const DecodeParams p) {
-  constexpr int DEC_STAGES = dec_stages(GT);
-  constexpr int LPT = D / 8;            // lanes sharing one token row
-  constexpr int TPS = 32 / LPT;         // tokens per warp-wide 16-byte read
-  constexpr int STEPS = 16 / TPS;       // reads per page
-  constexpr int PH = GT > 4 ? 2 : 1;    // passes over a page's keys
-  constexpr int HPP = GT > 4 ? 4 : ((GT + 1) & ~1);   // heads per pass (padded to even)
-  constexpr int GP = PH * HPP;          // heads with padding
-  constexpr int NV = STEPS * HPP;       // partial dot products per lane per pass
-  constexpr int NF = HPP / 2;           // finished scores per lane per pass
+// NT tiles of 8 query heads per CTA (heads beyond the group's are zero queries, dropped at the end).
+template <int D, int NT, bool FUSED>
+__global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM)
+decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map_k,
+                      const __grid_constant__ CUtensorMap map_v) {
+  constexpr int ST = dec_stages(D);
+  constexpr int VEC = D / 8;            // 16-byte vectors per head row
+  constexpr int KS = D / 16;            // k-steps of S^T, m-tiles of O^T
+  constexpr int GP = 8 * NT;            // heads with padding
   constexpr int PAGE_BYTES = 16 * D * 2;
-  static_assert(NV / LPT == NF, "reduction leaves HPP/2 values per lane");
+  constexpr int XD = D + 4;             // floats per row of the warps' exchange buffer (padded: no bank conflicts)
+  static_assert(DEC_WARPS * GP * XD * 4 <= dec_ring_bytes(D), "the exchange buffer re-uses the ring");
 
-  extern __shared__ __align__(128) uint8_t dec_ring[];   // [4 warps][DEC_STAGES][K page | V page]
-  __shared__ __align__(8) uint64_t s_bar[4][DEC_STAGES];
-  __shared__ float s_p[4][16][GP];      // per warp: probabilities of the current page
-  __shared__ float s_m[4][GP], s_l[4][GP];
-  __shared__ float s_o[4][GT][D];
+  extern __shared__ uint8_t dec_smem[];                  // ring, 1024-byte aligned below
+  __shared__ __align__(8) uint64_t s_bar[DEC_WARPS][ST];
+  __shared__ __align__(16) uint16_t s_q[GP][D + 8];      // query rows (rotated in a fused step)
+  __shared__ float s_m[DEC_WARPS][GP], s_l[DEC_WARPS][GP];
 
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r = blockIdx.x;
   const int G = p.Hq / p.Hkv;
-  const int gsplit = (G + GT - 1) / GT;
+  const int gsplit = (G + p.group_tile - 1) / p.group_tile;
   const int kvh = blockIdx.y / gsplit;
-  const int g0 = (blockIdx.y % gsplit) * GT;
-  const int ng = min(GT, G - g0);
+  const int g0 = (blockIdx.y % gsplit) * p.group_tile;
+  const int ng = min(p.group_tile, G - g0);
   const int c = blockIdx.z;
+  const uint32_t ring0 = (smem_u32(dec_smem) + 1023u) & ~1023u;
+  uint8_t* ring_gen = dec_smem + (ring0 - smem_u32(dec_smem));
   // The first block-table entries of every warp are fetched before the row's length is known
   // (any entry of the row may be read; those past the length are dropped below), so that the
   // two loads share one round trip: a short step's time is mostly this ramp.
-  const int seq = p.row_seq ? __ldg(p.row_seq + r) : r;
-  const int32_t* bt = p.block_table + (size_t)seq * p.max_pages_per_seq;
-  const int first_pg = ((c * p.chunk_tokens) >> 4) + (threadIdx.x >> 5);
-  const int my_pg = first_pg + 4 * (threadIdx.x & 31);
+  const int32_t* bt = p.block_table + (size_t)r * p.max_pages_per_seq;
+  const int first_pg = ((c * p.chunk_tokens) >> 4) + warp;
+  const int my_pg = first_pg + DEC_WARPS * lane;
   const int pid_early = my_pg < p.max_pages_per_seq ? __ldg(bt + my_pg) : -1;
   int len = __ldg(p.row_len + r);
   // longer than the launch was planned for (max_ctx_len) or than the block table can address:
@@ -135,11 +157,10 @@ __global__ void __launch_bounds__(128, dec_ctas_per_sm(GT)) decode_splitkv_kerne
   if (len > p.key_cap) {
     len = p.key_cap;
     append = false;
-    if (threadIdx.x == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_POSITION);
+    if (tid == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_POSITION);
   }
   const int begin = c * p.chunk_tokens;
   const int head0 = kvh * G + g0;
-  const int tid = threadIdx.x;
   // fused step: the new token sits at position len - 1; its rotation needs a table row
   const float* cs_row = nullptr;
   bool skip_row = false;
@@ -158,11 +179,11 @@ __global__ void __launch_bounds__(128, dec_ctas_per_sm(GT)) decode_splitkv_kerne
     // defined result: directly, or as an empty partial for every chunk the merge will read.
     if (p.n_chunks == 1) {
       if (len <= 0 || skip_row) {
-        for (int i = tid; i < ng * D; i += 128) p.out[((size_t)r * p.Hq + head0) * D + i] = 0;
+        for (int i = tid; i < ng * D; i += DEC_THREADS) p.out[((size_t)r * p.Hq + head0) * D + i] = 0;
         if (p.lse && tid < ng) p.lse[(size_t)r * p.Hq + head0 + tid] = -INFINITY;
       }
     } else if (skip_row && begin < len) {
-      for (int i = tid; i < ng * D; i += 128) {
+      for (int i = tid; i < ng * D; i += DEC_THREADS) {
         const size_t row_head = (size_t)r * p.Hq + head0 + i / D;
         p.part_o[(row_head * p.n_chunks + c) * D + i % D] = 0.f;
         if (i % D == 0) p.part_lse[row_head * p.n_chunks + c] = -INFINITY;
@@ -171,34 +192,30 @@ __global__ void __launch_bounds__(128, dec_ctas_per_sm(GT)) decode_splitkv_kerne
     return;
   }
   const int end = min(len, begin + p.chunk_tokens);
-  const int lane = tid & 31, warp = tid >> 5;
-  const int j = lane % LPT, tg = lane / LPT;
 
   // ---- this warp's pages: first_pg, first_pg + 4, ... ; start their copies before anything else
   const int last_pg = (end - 1) >> 4;
-  const int n_pages = first_pg <= last_pg ? (last_pg - first_pg) / 4 + 1 : 0;
-  uint8_t* ring = dec_ring + warp * (DEC_STAGES * 2 * PAGE_BYTES);
+  const int n_pages = first_pg <= last_pg ? (last_pg - first_pg) / DEC_WARPS + 1 : 0;
+  const uint32_t ring = ring0 + warp * (ST * 2 * PAGE_BYTES);
   if (lane == 0) {
-    for (int sg = 0; sg < DEC_STAGES; ++sg)
-      mbar_init(smem_u32(&s_bar[warp][sg]), 1);
+    for (int sg = 0; sg < ST; ++sg) mbar_init(smem_u32(&s_bar[warp][sg]), 1);
     mbar_fence_init();
   }
   __syncwarp();
   // page ids of the next 32 pages of this warp, one per lane (refilled every 32 pages)
   int pid_cache = (lane < n_pages) ? pid_early : -1;
-  auto issue = [&](int i) {             // start the copies of this warp's i-th page into stage i % DEC_STAGES
+  auto issue = [&](int i) {             // start the copies of this warp's i-th page into stage i % ST
     const int pid = __shfl_sync(0xffffffffu, pid_cache, i & 31);
     const bool ok = pid >= 0 && pid < p.num_pages;
     if (lane == 0) {
-      const uint32_t bar = smem_u32(&s_bar[warp][i % DEC_STAGES]);
+      const uint32_t bar = smem_u32(&s_bar[warp][i % ST]);
       if (ok) {
-        const uint32_t dst = smem_u32(ring + (i % DEC_STAGES) * 2 * PAGE_BYTES);
-        const size_t off = ((size_t)pid * p.Hkv + kvh) * 16 * D;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * PAGE_BYTES) : "memory");
-        dec_bulk_load(dst, p.k_pool + off, PAGE_BYTES, bar);
-        dec_bulk_load(dst + PAGE_BYTES, p.v_pool + off, PAGE_BYTES, bar);
+        const uint32_t dst = ring + (i % ST) * 2 * PAGE_BYTES;
+        mbar_expect_tx(bar, 2 * PAGE_BYTES);
+        dec_load_page(dst, &map_k, bar, pid * p.Hkv + kvh);
+        dec_load_page(dst + PAGE_BYTES, &map_v, bar, pid * p.Hkv + kvh);
       } else {
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");   // nothing to copy
+        mbar_arrive(bar);                                                // nothing to copy
         if (p.status) atomicOr(p.status, EFIM_DEV_BAD_PAGE);
       }
     }
@@ -206,175 +223,181 @@ __global__ void __launch_bounds__(128, dec_ctas_per_sm(GT)) decode_splitkv_kerne
   };
   uint32_t ok_bits = 0;                 // which of the in-flight pages are valid (bit = stage)
 #pragma unroll
-  for (int i = 0; i < DEC_STAGES; ++i)
+  for (int i = 0; i < ST; ++i)
     if (i < n_pages && issue(i)) ok_bits |= 1u << i;
 
-  // q and o as packed fp32 pairs (dims 2e, 2e+1): the inner products and the P V
-  // update run on two-wide FMAs
-  uint64_t q2[GP][4];
-#pragma unroll
-  for (int g = 0; g < GP; ++g) {
+  // ---- query rows: through shared memory (rotated there) into B fragments, dims 2q, 2q+1 (+8) of
+  // head lane / 4 for every k-step, kept in registers
+  for (int i = tid; i < GP * VEC; i += DEC_THREADS) {
+    const int g = i / VEC, j = i % VEC;
+    uint4 w = make_uint4(0, 0, 0, 0);
     if (g < ng) {
       const uint4* qrow = reinterpret_cast<const uint4*>(p.q + ((size_t)r * p.Hq + head0 + g) * D);
-      uint4 w = __ldg(qrow + j);
-      if (FUSED && cs_row) w = dec_rotate_vec(w, __ldg(qrow + (j ^ (LPT / 2))), cs_row, D, j, p.interleaved);
-      const uint32_t* u = reinterpret_cast<const uint32_t*>(&w);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) q2[g][e] = pack2(bf16lo(u[e]) * p.scale_log2, bf16hi(u[e]) * p.scale_log2);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) q2[g][e] = 0ull;
+      w = __ldg(qrow + j);
+      if (FUSED && cs_row) w = dec_rotate_vec(w, __ldg(qrow + (j ^ (VEC / 2))), cs_row, D, j, p.interleaved);
     }
+    *reinterpret_cast<uint4*>(&s_q[g][j * 8]) = w;
   }
-  uint64_t o2[GT][4];
+  __syncthreads();
+  const int hq = lane >> 2, tq = lane & 3;
+  uint32_t qf[NT][KS][2];
 #pragma unroll
-  for (int g = 0; g < GT; ++g)
+  for (int n = 0; n < NT; ++n)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) o2[g][e] = 0ull;
-  float m_run[GP], l_part[PH][NF];
+    for (int k = 0; k < KS; ++k) {
+      qf[n][k][0] = *reinterpret_cast<const uint32_t*>(&s_q[n * 8 + hq][k * 16 + 2 * tq]);
+      qf[n][k][1] = *reinterpret_cast<const uint32_t*>(&s_q[n * 8 + hq][k * 16 + 8 + 2 * tq]);
+    }
+  float o[NT][KS][4];                   // O^T fragments: dims 16 k + hq (+8), heads 8 n + 2 tq + {0, 1}
 #pragma unroll
-  for (int g = 0; g < GP; ++g) m_run[g] = -INFINITY;
+  for (int n = 0; n < NT; ++n)
 #pragma unroll
-  for (int ph = 0; ph < PH; ++ph)
+    for (int k = 0; k < KS; ++k)
 #pragma unroll
-    for (int i = 0; i < NF; ++i) l_part[ph][i] = 0.f;
+      for (int e = 0; e < 4; ++e) o[n][k][e] = 0.f;
+  float m_ref[NT][2], l_part[NT][2];    // of heads 8 n + 2 tq + {0, 1}; the sum over this lane's tokens
+#pragma unroll
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) { m_ref[n][e] = -INFINITY; l_part[n][e] = 0.f; }
 
-  const int odd = j & 1;
-  const int st_mine = j >> 1;                   // step whose scores this lane ends up with
-  int gave_up_at = -1;                          // page index at which a stage wait expired
+  // ldmatrix row addresses of this lane inside a staged page: K (tokens along m), V (dims along m)
+  const uint32_t k_lane = (uint32_t)(((lane >> 3) & 1) * (D * 16) + (lane & 7) * 128 + (((lane >> 4) ^ (lane & 7)) << 4));
+  const uint32_t v_lane = (uint32_t)((lane >> 4) * (D * 16) + (lane & 7) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4));
+  int gave_up_at = -1;                  // page index at which a stage wait expired
 
   for (int i = 0; i < n_pages; ++i) {
-    const int pg = first_pg + 4 * i;
-    const int sg = i % DEC_STAGES;
+    const int pg = first_pg + DEC_WARPS * i;
+    const int sg = i % ST;
     const bool page_ok = (ok_bits >> sg) & 1u;
     // ---- wait for the stage (bounded; on expiry flag and stop walking)
     {
-      const bool ok = mbar_wait_bounded(smem_u32(&s_bar[warp][sg]), (i / DEC_STAGES) & 1, p.wait_ns, nullptr,
+      const bool ok = mbar_wait_bounded(smem_u32(&s_bar[warp][sg]), (i / ST) & 1, p.wait_ns, nullptr,
                                         lane == 0 ? p.status : nullptr);
       if (__any_sync(0xffffffffu, !ok)) {
         gave_up_at = i;
         break;
       }
     }
-    if (FUSED && append && page_ok && pg == ((len - 1) >> 4)) {
-      // The page of the new token: whatever the copy brought for its slot is replaced, in
-      // shared memory, by the token's rotated k and its v; the CTA of the kv head's first
-      // group tile also puts them into the pools.  (Other CTAs that read this page patch
-      // their own copy the same way, so nobody depends on when the pool is written.)
-      if (tg == 0) {
-        const int slot = (len - 1) & 15;
-        const uint4* krow = reinterpret_cast<const uint4*>(p.k_new + ((size_t)r * p.Hkv + kvh) * D);
-        const uint4* vrow = reinterpret_cast<const uint4*>(p.v_new + ((size_t)r * p.Hkv + kvh) * D);
-        uint4 kv = __ldg(krow + j);
-        if (cs_row) kv = dec_rotate_vec(kv, __ldg(krow + (j ^ (LPT / 2))), cs_row, D, j, p.interleaved);
-        const uint4 vv = __ldg(vrow + j);
-        uint8_t* kpage = ring + sg * 2 * PAGE_BYTES;
-        *reinterpret_cast<uint4*>(kpage + (slot * D + j * 8) * 2) = kv;
-        *reinterpret_cast<uint4*>(kpage + PAGE_BYTES + (slot * D + j * 8) * 2) = vv;
-        if (g0 == 0) {
-          const int pid = __ldg(bt + pg);
-          const size_t off = (((size_t)pid * p.Hkv + kvh) * 16 + slot) * D + j * 8;
-          *reinterpret_cast<uint4*>(p.k_pool_w + off) = kv;
-          *reinterpret_cast<uint4*>(p.v_pool_w + off) = vv;
-        }
-      }
-      __syncwarp();
-    }
+    const uint32_t k_page = ring + sg * 2 * PAGE_BYTES, v_page = k_page + PAGE_BYTES;
     if (page_ok) {
-      const uint8_t* kst = ring + sg * 2 * PAGE_BYTES + (tg * D + j * 8) * 2;
-      const uint8_t* vst = kst + PAGE_BYTES;
-      // ---- scores: partial dot products over this lane's 8 dims, then the cross-lane sum;
-      // HPP heads per pass
-      const int tok_in_page = st_mine * TPS + tg;       // the token whose scores this lane ends up with
-      const bool visible = (pg << 4) + tok_in_page < end;
-      float alpha[GP];
-#pragma unroll
-      for (int ph = 0; ph < PH; ++ph) {
-        float x[NV];
-#pragma unroll
-        for (int st = 0; st < STEPS; ++st) {
-          const uint4 kv = *reinterpret_cast<const uint4*>(kst + st * TPS * D * 2);
-          const uint32_t* u = reinterpret_cast<const uint32_t*>(&kv);
-          uint64_t k2[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) k2[e] = pack2(bf16lo(u[e]), bf16hi(u[e]));
-#pragma unroll
-          for (int g = 0; g < HPP; ++g) {
-            float acc = 0.f;
-            if (ph * HPP + g < GT) {
-              uint64_t a2 = 0ull;
-#pragma unroll
-              for (int e = 0; e < 4; ++e) a2 = ffma2(q2[ph * HPP + g][e], k2[e], a2);
-              float lo, hi;
-              unpack2(a2, lo, hi);
-              acc = lo + hi;
-            }
-            x[st * HPP + g] = acc;
+      const int left = end - (pg << 4);                     // keys of this page the chunk may see
+      if (FUSED && append && pg == ((len - 1) >> 4)) {
+        // The page of the new token: whatever the copy brought for its slot is replaced, in
+        // shared memory, by the token's rotated k and its v; the CTA of the kv head's first
+        // group tile also puts them into the pools.  (Other CTAs that read this page patch
+        // their own copy the same way, so nobody depends on when the pool is written.)
+        if (lane < VEC) {
+          const int j = lane, slot = (len - 1) & 15;
+          const uint4* krow = reinterpret_cast<const uint4*>(p.k_new + ((size_t)r * p.Hkv + kvh) * D);
+          const uint4* vrow = reinterpret_cast<const uint4*>(p.v_new + ((size_t)r * p.Hkv + kvh) * D);
+          uint4 kv = __ldg(krow + j);
+          if (cs_row) kv = dec_rotate_vec(kv, __ldg(krow + (j ^ (VEC / 2))), cs_row, D, j, p.interleaved);
+          const uint4 vv = __ldg(vrow + j);
+          uint8_t* kpage = ring_gen + (k_page - ring0);
+          *reinterpret_cast<uint4*>(kpage + dec_page_off<D>(slot, j)) = kv;
+          *reinterpret_cast<uint4*>(kpage + PAGE_BYTES + dec_page_off<D>(slot, j)) = vv;
+          if (g0 == 0) {
+            const int pid = __ldg(bt + pg);
+            const size_t off = (((size_t)pid * p.Hkv + kvh) * 16 + slot) * D + j * 8;
+            *reinterpret_cast<uint4*>(p.k_pool_w + off) = kv;
+            *reinterpret_cast<uint4*>(p.v_pool_w + off) = vv;
           }
         }
-        transposed_reduce<NV, LPT>(x, j);
-        // lane j now holds, for token (st_mine*TPS + tg) of the page, heads ph*HPP + odd*NF + i
-        float sc[NF], mx[NF];
+        __syncwarp();
+      }
+      if (left < 16) {
+        // values of slots past the context are anything (NaN included): P is 0 there, 0 * NaN is not
+        uint8_t* vpage = ring_gen + (v_page - ring0);
+        for (int idx = left * VEC + lane; idx < 16 * VEC; idx += 32)
+          *reinterpret_cast<uint4*>(vpage + dec_page_off<D>(idx / VEC, idx % VEC)) = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+      }
+      // ---- S^T: lane's tokens hq and hq + 8, heads 8 n + 2 tq + {0, 1}; two chains of k-steps
+      float s[NT][4], s2[NT][4];
 #pragma unroll
-        for (int a = 0; a < NF; ++a) { sc[a] = visible ? x[a] : -INFINITY; mx[a] = sc[a]; }
+      for (int n = 0; n < NT; ++n)
 #pragma unroll
-        for (int off = 2; off < 32; off <<= 1)
+        for (int e = 0; e < 4; ++e) { s[n][e] = 0.f; s2[n][e] = 0.f; }
 #pragma unroll
-          for (int a = 0; a < NF; ++a) mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], off));
-        float mine[NF], alpha_mine[NF];
+      for (int k = 0; k < KS; k += 2) {
+        uint32_t a[4], b[4];
+        ldsm4((k_page + k_lane + (k >> 2) * 1024) ^ ((k & 3) << 5), a);
+        ldsm4((k_page + k_lane + (k >> 2) * 1024) ^ (((k & 3) + 1) << 5), b);
 #pragma unroll
-        for (int a = 0; a < NF; ++a) {
-          const int h_lo = ph * HPP + a, h_hi = ph * HPP + NF + a;
-          const float other = __shfl_xor_sync(0xffffffffu, mx[a], 1);
-          const float m_lo = odd ? other : mx[a];       // head h_lo
-          const float m_hi = odd ? mx[a] : other;       // head h_hi
-          const float n_lo = fmaxf(m_run[h_lo], m_lo), n_hi = fmaxf(m_run[h_hi], m_hi);
-          alpha[h_lo] = exp2f(m_run[h_lo] - n_lo);
-          alpha[h_hi] = exp2f(m_run[h_hi] - n_hi);
-          m_run[h_lo] = n_lo;
-          m_run[h_hi] = n_hi;
-          mine[a] = odd ? n_hi : n_lo;
-          alpha_mine[a] = odd ? alpha[h_hi] : alpha[h_lo];
-        }
-#pragma unroll
-        for (int a = 0; a < NF; ++a) {
-          const float pr = exp2f(sc[a] - mine[a]);      // masked: exp2(-inf) = 0
-          l_part[ph][a] = fmaf(l_part[ph][a], alpha_mine[a], pr);
-          s_p[warp][tok_in_page][ph * HPP + odd * NF + a] = pr;
+        for (int n = 0; n < NT; ++n) {
+          mma16816(s[n], a, qf[n][k][0], qf[n][k][1]);
+          mma16816(s2[n], b, qf[n][k + 1][0], qf[n][k + 1][1]);
         }
       }
-      __syncwarp();
-      // ---- values
+      float mx[NT][2];
+      bool grow = false;
 #pragma unroll
-      for (int g = 0; g < GT; ++g) {
-        const uint64_t al2 = pack2(alpha[g], alpha[g]);
+      for (int n = 0; n < NT; ++n) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) o2[g][e] = fmul2(o2[g][e], al2);
+        for (int e = 0; e < 4; ++e) s[n][e] = (s[n][e] + s2[n][e]) * p.scale_log2;
+        if (left < 16) {
+          if (hq >= left) s[n][0] = s[n][1] = -INFINITY;
+          if (hq + 8 >= left) s[n][2] = s[n][3] = -INFINITY;
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          mx[n][e] = fmaxf(s[n][e], s[n][e + 2]);
+          grow |= mx[n][e] > m_ref[n][e] + 8.f;
+        }
       }
+      // Lazy rescale: the reference maximum of a head only moves when a score exceeds it by more
+      // than 2^8 (always on the first page), so the lanes need not agree on every page's maximum.
+      if (__any_sync(0xffffffffu, grow)) {
 #pragma unroll
-      for (int st = 0; st < STEPS; ++st) {
-        const int tp = st * TPS + tg;
-        if ((pg << 4) + tp < end) {                   // never touch slots past the context
-          const uint4 vv = *reinterpret_cast<const uint4*>(vst + st * TPS * D * 2);
-          const uint32_t* u = reinterpret_cast<const uint32_t*>(&vv);
-          uint64_t v2[4];
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) v2[e] = pack2(bf16lo(u[e]), bf16hi(u[e]));
+          for (int e = 0; e < 2; ++e) {
+            float x = mx[n][e];
 #pragma unroll
-          for (int g = 0; g < GT; ++g) {
-            const float pr = s_p[warp][tp][g];
-            const uint64_t pr2 = pack2(pr, pr);
+            for (int off = 4; off < 32; off <<= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, off));
+            const float m_new = fmaxf(m_ref[n][e], x);
+            const float alpha = m_new == -INFINITY ? 1.f : dec_ex2(m_ref[n][e] - m_new);
+            m_ref[n][e] = m_new;
+            l_part[n][e] *= alpha;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) o2[g][e] = ffma2(pr2, v2[e], o2[g][e]);
+            for (int k = 0; k < KS; ++k) { o[n][k][e] *= alpha; o[n][k][e + 2] *= alpha; }
+          }
+      }
+      // ---- P^T: exponentials, split into three bf16 terms, transposed into B fragments
+      uint32_t pb[NT][3][2];
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float x0 = dec_ex2(s[n][2 * h] - m_ref[n][0]), x1 = dec_ex2(s[n][2 * h + 1] - m_ref[n][1]);
+          l_part[n][0] += x0;
+          l_part[n][1] += x1;
+#pragma unroll
+          for (int t = 0; t < 3; ++t) {
+            const uint32_t w = pack_bf16x2(x0, x1);
+            pb[n][t][h] = movm_t(w);
+            x0 -= bf16lo(w);
+            x1 -= bf16hi(w);
           }
         }
+      }
+      // ---- O^T
+#pragma unroll
+      for (int k = 0; k < KS; ++k) {
+        uint32_t a[4];
+        ldsm4_t((v_page + v_lane + (k >> 2) * 1024) ^ ((k & 3) << 5), a);
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int t = 0; t < 3; ++t) mma16816(o[n][k], a, pb[n][t][0], pb[n][t][1]);
       }
     }
-    __syncwarp();                                     // everyone is done with the stage and with s_p
-    // ---- refill the stage with the page DEC_STAGES ahead
-    const int nxt = i + DEC_STAGES;
+    __syncwarp();                                     // everyone is done with the stage
+    // ---- refill the stage with the page ST ahead
+    const int nxt = i + ST;
     if (nxt < n_pages) {
-      if ((nxt & 31) == 0) pid_cache = (nxt + lane < n_pages) ? __ldg(bt + first_pg + 4 * (nxt + lane)) : -1;
+      if ((nxt & 31) == 0) pid_cache = (nxt + lane < n_pages) ? __ldg(bt + first_pg + DEC_WARPS * (nxt + lane)) : -1;
       ok_bits &= ~(1u << sg);
       if (issue(nxt)) ok_bits |= 1u << sg;
     }
@@ -382,63 +405,62 @@ __global__ void __launch_bounds__(128, dec_ctas_per_sm(GT)) decode_splitkv_kerne
 
   if (gave_up_at >= 0) {
     // copies issued for the stages still in flight must land before the CTA's shared memory
-    // can be handed to another CTA
-    for (int k = gave_up_at; k < min(gave_up_at + DEC_STAGES, n_pages); ++k)
-      mbar_drain(smem_u32(&s_bar[warp][k % DEC_STAGES]), (k / DEC_STAGES) & 1);
+    // is used for anything else or handed to another CTA
+    for (int k = gave_up_at; k < min(gave_up_at + ST, n_pages); ++k)
+      mbar_drain(smem_u32(&s_bar[warp][k % ST]), (k / ST) & 1);
   }
-  float o[GT][8];
+  // ---- fold the lanes' sums, then the 4 warps (their rings are quiet: the exchange buffer takes their place)
 #pragma unroll
-  for (int g = 0; g < GT; ++g)
+  for (int n = 0; n < NT; ++n)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) unpack2(o2[g][e], o[g][2 * e], o[g][2 * e + 1]);
-  // ---- fold the token groups of the warp, then the 4 warps
+    for (int e = 0; e < 2; ++e) {
 #pragma unroll
-  for (int off = LPT; off < 32; off <<= 1)
-#pragma unroll
-    for (int g = 0; g < GT; ++g)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) o[g][e] += __shfl_xor_sync(0xffffffffu, o[g][e], off);
-#pragma unroll
-  for (int off = 2; off < 32; off <<= 1)
-#pragma unroll
-    for (int ph = 0; ph < PH; ++ph)
-#pragma unroll
-      for (int i = 0; i < NF; ++i) l_part[ph][i] += __shfl_xor_sync(0xffffffffu, l_part[ph][i], off);
-  if (lane < 2) {
-#pragma unroll
-    for (int ph = 0; ph < PH; ++ph)
-#pragma unroll
-      for (int i = 0; i < NF; ++i) s_l[warp][ph * HPP + lane * NF + i] = l_part[ph][i];
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int g = 0; g < GP; ++g) s_m[warp][g] = m_run[g];
-  }
-  if (tg == 0) {
-#pragma unroll
-    for (int g = 0; g < GT; ++g)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s_o[warp][g][j * 8 + e] = o[g][e];
-  }
-  __syncthreads();
-  for (int idx = tid; idx < ng * D; idx += 128) {
-    const int g = idx / D, d = idx % D;
-    float M = fmaxf(fmaxf(s_m[0][g], s_m[1][g]), fmaxf(s_m[2][g], s_m[3][g]));   // warp 0 always has a page
-    float L = 0.f, O = 0.f;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const float sc = exp2f(s_m[w][g] - M);
-      L = fmaf(s_l[w][g], sc, L);
-      O = fmaf(s_o[w][g][d], sc, O);
+      for (int off = 4; off < 32; off <<= 1) l_part[n][e] += __shfl_xor_sync(0xffffffffu, l_part[n][e], off);
+      if (lane < 4) {
+        s_l[warp][n * 8 + 2 * lane + e] = l_part[n][e];
+        s_m[warp][n * 8 + 2 * lane + e] = m_ref[n][e];
+      }
     }
-    const float val = (L > 0.f) ? O / L : 0.f;    // all pages of the chunk rejected: defined output
+  __syncthreads();
+  float* xo = reinterpret_cast<float*>(ring_gen);           // [warp][head][XD]
+#pragma unroll
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int k = 0; k < KS; ++k)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        xo[(warp * GP + n * 8 + 2 * tq + (e & 1)) * XD + k * 16 + hq + (e >> 1) * 8] = o[n][k][e];
+  __syncthreads();
+  for (int idx = tid; idx < ng * (D / 4); idx += DEC_THREADS) {
+    const int g = idx / (D / 4), d = (idx % (D / 4)) * 4;
+    float M = s_m[0][g];
+#pragma unroll
+    for (int w = 1; w < DEC_WARPS; ++w) M = fmaxf(M, s_m[w][g]);
+    float L = 0.f;
+    float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (M > -INFINITY) {                                    // else every page of the chunk was rejected: 0, -inf
+#pragma unroll
+      for (int w = 0; w < DEC_WARPS; ++w) {
+        const float sc = exp2f(s_m[w][g] - M);
+        const float4 x = *reinterpret_cast<const float4*>(xo + (w * GP + g) * XD + d);
+        L = fmaf(s_l[w][g], sc, L);
+        O.x = fmaf(x.x, sc, O.x);
+        O.y = fmaf(x.y, sc, O.y);
+        O.z = fmaf(x.z, sc, O.z);
+        O.w = fmaf(x.w, sc, O.w);
+      }
+    }
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+    const float lse2 = L > 0.f ? M + log2f(L) : -INFINITY;
     const size_t row_head = (size_t)r * p.Hq + head0 + g;
     if (p.n_chunks == 1) {
-      p.out[row_head * D + d] = __bfloat16_as_ushort(__float2bfloat16_rn(val));
-      if (p.lse && d == 0) p.lse[row_head] = (M + log2f(L)) * 0.6931471805599453f;
+      *reinterpret_cast<uint2*>(p.out + row_head * D + d) =
+          make_uint2(pack_bf16x2(O.x * inv, O.y * inv), pack_bf16x2(O.z * inv, O.w * inv));
+      if (p.lse && d == 0) p.lse[row_head] = lse2 * 0.6931471805599453f;
     } else {
-      p.part_o[(row_head * p.n_chunks + c) * D + d] = val;
-      if (d == 0) p.part_lse[row_head * p.n_chunks + c] = M + log2f(L);
+      *reinterpret_cast<float4*>(p.part_o + (row_head * p.n_chunks + c) * D + d) =
+          make_float4(O.x * inv, O.y * inv, O.z * inv, O.w * inv);
+      if (d == 0) p.part_lse[row_head * p.n_chunks + c] = lse2;
     }
   }
 }
@@ -513,34 +535,28 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p)
 DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len) {
   DecodePlan pl;
   const int G = Hq / Hkv;
-  // Groups of up to 7 query heads share one CTA's walk over the K/V pages (5 to 7 in two
-  // passes over the page in shared memory: 3.1-3.7 TB/s of K/V against 3.0 when the pages
-  // were fetched twice).  From 8 heads on the fp32 FMAs, not the bytes, are the bound (8 heads
-  // in one CTA measured 1.9 TB/s against 3.2 as two CTAs of 4), so larger groups are cut into
-  // tiles of 4, or of 3 where that divides the group and 4 does not.
-  if (G <= 7) {
-    pl.group_tile = G;
-  } else {
-    pl.group_tile = (G % 4 != 0 && G % 3 == 0) ? 3 : 4;
-  }
+  // Up to 16 query heads share one CTA's walk over the K/V pages; larger groups are cut evenly.
+  pl.gsplit = (G + 15) / 16;
+  pl.group_tile = (G + pl.gsplit - 1) / pl.gsplit;
   pl.gsplit = (G + pl.group_tile - 1) / pl.group_tile;
   if (max_len < 1) max_len = 1;
-  // Aim for ~32 CTAs per SM over the launch so that ragged lengths even out, but keep a
-  // chunk between 768 and 2048 tokens (384 KB .. 1 MB of K+V at head_dim 128): a CTA pays
-  // a few microseconds before its pages stream, and shorter chunks were measured slower
-  // (16 rows x 8 kv heads x 2.5k keys: 48.9 us per step with 256-key chunks, 43 with 768).
-  // Only when that leaves fewer than two CTAs per SM do the chunks shrink, down to 256.
-  const long long n_sm = sm_count();
-  const long long ctas_per_chunkless = (long long)rows * Hkv * pl.gsplit;
-  long long want_chunks = (n_sm * 32 + ctas_per_chunkless - 1) / ctas_per_chunkless;
-  if (want_chunks < 1) want_chunks = 1;
-  long long chunk = (max_len + want_chunks - 1) / want_chunks;
-  if (chunk < 768) chunk = 768;
-  if (chunk > 2048) chunk = 2048;
-  if (ctas_per_chunkless * ((max_len + chunk - 1) / chunk) < n_sm * 2) {
-    const long long need_chunks = (n_sm * 2 + ctas_per_chunkless - 1) / ctas_per_chunkless;
-    chunk = std::max<long long>(256, (max_len + need_chunks - 1) / need_chunks);
-    if (chunk > 2048) chunk = 2048;
+  // A CTA pays a few microseconds before its pages stream, and CTAs beyond the ones that are
+  // resident together (slots) wait for a whole CTA to end: chunks of 2048 keys when even those
+  // make several waves, else as many chunks as one wave holds, but neither shorter than 256 keys
+  // (the merge then costs more than the split gains) nor longer than 1024 (ragged rows).  Steps of
+  // 32/8 heads in microseconds at 256 / 384 / 768 / 1024 / 2048 keys: 1 row x 2.3k keys 9.0 / 10.1 /
+  // 13.1 / 15.4 / 25; 4 rows x 2-2.9k 15.8 / 15.6 / 16.5 / 17.5 / 27; 16 rows 35.3 / 35.2 / 33.7 /
+  // 31.4 / 34.4; 64 rows x 4-32k - / 636 / 611 / 603 / 596.
+  const long long slots = (long long)sm_count() * DEC_CTAS_PER_SM;
+  const long long units = (long long)rows * Hkv * pl.gsplit;
+  long long chunk = 2048;
+  if (units * ((max_len + 2047) / 2048) < 4 * slots) {
+    const long long n = std::max<long long>(1, slots / units);
+    chunk = std::min<long long>(1024, std::max<long long>(256, (max_len + n - 1) / n));
+    // partials that the fixed array of efim_decode_attn_static holds, where longer chunks allow it
+    const long long per_chunk = (long long)rows * Hq * (D + 1) * (long long)sizeof(float);
+    const long long n_fit = std::max<long long>(1, ((8 << 20) - 512) / per_chunk);
+    if ((max_len + chunk - 1) / chunk > n_fit) chunk = std::min<long long>(2048, (max_len + n_fit - 1) / n_fit);
   }
   chunk = (chunk + 63) / 64 * 64;
   pl.chunk_tokens = (int)chunk;
@@ -550,32 +566,42 @@ DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len) {
   return pl;
 }
 
-template <int D, int GT, bool FUSED>
-static efim_status launch_split_f(const DecodeParams& p, dim3 grid, cudaStream_t s) {
-  constexpr int ring_bytes = 4 * dec_stages(GT) * 2 * 16 * D * 2;  // 4 warps x stages x (K page + V page)
-  EFIM_CUDA_TRY(cudaFuncSetAttribute(decode_splitkv_kernel<D, GT, FUSED>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, ring_bytes));
-  decode_splitkv_kernel<D, GT, FUSED><<<grid, 128, ring_bytes, s>>>(p);
+// The kernel's shared-memory size has to be raised once per device.
+template <int D, int NT, bool FUSED>
+static efim_status dec_raise_smem_limit() {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<bool> done[kMaxDevices];
+  int dev = 0;
+  EFIM_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return EFIM_OK;
+  EFIM_CUDA_TRY(cudaFuncSetAttribute(decode_splitkv_kernel<D, NT, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     dec_ring_bytes(D) + 1024));
+  if (dev >= 0 && dev < kMaxDevices) done[dev].store(true, std::memory_order_release);
   return EFIM_OK;
 }
-template <int D, int GT>
-static efim_status launch_split(const DecodeParams& p, dim3 grid, cudaStream_t s) {
-  return p.fused ? launch_split_f<D, GT, true>(p, grid, s) : launch_split_f<D, GT, false>(p, grid, s);
+
+template <int D, int NT, bool FUSED>
+static efim_status launch_split(const efim_cache_desc* cache, const DecodeParams& p, dim3 grid, cudaStream_t s) {
+  const CUtensorMap* pk = pf::pool_map(cache->d_k_pool, cache->num_pages, cache->num_kv_heads, D);
+  if (!pk) return EFIM_ERR_CUDA;
+  const CUtensorMap mk = *pk;
+  const CUtensorMap* pv = pf::pool_map(cache->d_v_pool, cache->num_pages, cache->num_kv_heads, D);
+  if (!pv) return EFIM_ERR_CUDA;
+  const efim_status st = dec_raise_smem_limit<D, NT, FUSED>();
+  if (st != EFIM_OK) return st;
+  decode_splitkv_kernel<D, NT, FUSED><<<grid, DEC_THREADS, dec_ring_bytes(D) + 1024, s>>>(p, mk, *pv);
+  return EFIM_OK;
 }
 
 template <int D>
-static efim_status launch_decode_d(const DecodeParams& p, const DecodePlan& pl, cudaStream_t s) {
+static efim_status launch_decode_d(const efim_cache_desc* cache, const DecodeParams& p, const DecodePlan& pl,
+                                   cudaStream_t s) {
   dim3 grid(p.R, p.Hkv * pl.gsplit, pl.n_chunks);
   efim_status st;
-  switch (pl.group_tile) {
-    case 1: st = launch_split<D, 1>(p, grid, s); break;
-    case 2: st = launch_split<D, 2>(p, grid, s); break;
-    case 3: st = launch_split<D, 3>(p, grid, s); break;
-    case 4: st = launch_split<D, 4>(p, grid, s); break;
-    case 5: st = launch_split<D, 5>(p, grid, s); break;
-    case 6: st = launch_split<D, 6>(p, grid, s); break;
-    default: st = launch_split<D, 7>(p, grid, s); break;
-  }
+  if (pl.group_tile <= 8)
+    st = p.fused ? launch_split<D, 1, true>(cache, p, grid, s) : launch_split<D, 1, false>(cache, p, grid, s);
+  else
+    st = p.fused ? launch_split<D, 2, true>(cache, p, grid, s) : launch_split<D, 2, false>(cache, p, grid, s);
   if (st != EFIM_OK) return st;
   EFIM_CUDA_TRY(cudaGetLastError());
   if (pl.n_chunks > 1) {
@@ -586,10 +612,11 @@ static efim_status launch_decode_d(const DecodeParams& p, const DecodePlan& pl, 
   return EFIM_OK;
 }
 
-efim_status launch_decode(const DecodeParams& p, const DecodePlan& pl, int D, cudaStream_t s) {
+static efim_status launch_decode(const efim_cache_desc* cache, const DecodeParams& p, const DecodePlan& pl,
+                                 cudaStream_t s) {
   if (p.R == 0) return EFIM_OK;
   if (p.R > 2147483647 / 4 || p.Hkv * pl.gsplit > 65535 || pl.n_chunks > 65535) return EFIM_ERR_UNSUPPORTED;
-  return D == 128 ? launch_decode_d<128>(p, pl, s) : launch_decode_d<64>(p, pl, s);
+  return cache->head_dim == 128 ? launch_decode_d<128>(cache, p, pl, s) : launch_decode_d<64>(cache, p, pl, s);
 }
 
 }  // namespace efim
@@ -635,10 +662,7 @@ efim_status efim::decode_run(const efim_cache_desc* cache, int32_t batch, const 
   }
   efim::DecodeParams p{};
   p.q = static_cast<const uint16_t*>(d_q);
-  p.k_pool = static_cast<const uint16_t*>(cache->d_k_pool);
-  p.v_pool = static_cast<const uint16_t*>(cache->d_v_pool);
   p.row_len = d_ctx_len;
-  p.row_seq = nullptr;
   p.block_table = d_block_table;
   p.out = static_cast<uint16_t*>(d_out);
   p.lse = d_lse;
@@ -650,6 +674,7 @@ efim_status efim::decode_run(const efim_cache_desc* cache, int32_t batch, const 
   p.Hkv = cache->num_kv_heads;
   p.max_pages_per_seq = max_pages_per_seq;
   p.num_pages = cache->num_pages;
+  p.group_tile = pl.group_tile;
   p.chunk_tokens = pl.chunk_tokens;
   p.n_chunks = pl.n_chunks;
   p.key_cap = (int)std::min<long long>((long long)pl.n_chunks * pl.chunk_tokens, cap);
@@ -671,7 +696,7 @@ efim_status efim::decode_run(const efim_cache_desc* cache, int32_t batch, const 
       p.interleaved = rope->interleaved;
     }
   }
-  return efim::launch_decode(p, pl, cache->head_dim, static_cast<cudaStream_t>(stream));
+  return efim::launch_decode(cache, p, pl, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" efim_status efim_decode_attn(const efim_cache_desc* cache, int32_t batch, const int32_t* d_ctx_len,

@@ -1,5 +1,4 @@
-// Internal interface of the split-KV row-attention kernels (shared by the
-// decode entry point and the small-row path of append-prefill).
+// Internal interface of the split-KV decode kernels.
 #pragma once
 #include "common.cuh"
 
@@ -7,17 +6,14 @@ namespace efim {
 
 struct DecodeParams {
   const uint16_t* q;          // [R][Hq][D] bf16
-  const uint16_t* k_pool;     // [pages][Hkv][16][D]
-  const uint16_t* v_pool;
   const int32_t* row_len;     // [R] keys visible to row r: [0, row_len[r])
-  const int32_t* row_seq;     // [R] block-table row of r, or null for identity
-  const int32_t* block_table; // [*][max_pages_per_seq]
+  const int32_t* block_table; // [R][max_pages_per_seq]
   uint16_t* out;              // [R][Hq][D] bf16
   float* lse;                 // [R][Hq] natural log, or null
   float* part_o;              // [R][Hq][n_chunks][D]   (n_chunks > 1)
   float* part_lse;            // [R][Hq][n_chunks]      base-2 log
   int32_t* status;
-  int R, Hq, Hkv, max_pages_per_seq, num_pages, chunk_tokens, n_chunks;
+  int R, Hq, Hkv, group_tile, max_pages_per_seq, num_pages, chunk_tokens, n_chunks;
   int key_cap;                // keys the launch can cover: min(n_chunks * chunk_tokens, table capacity);
                               // a longer device length is clamped to it and reported
   unsigned long long wait_ns; // limit of every device-side wait
@@ -27,14 +23,14 @@ struct DecodeParams {
   // kernel; q comes in unrotated.  All null / 0 for a plain decode.
   const uint16_t* k_new;      // [R][Hkv][D]
   const uint16_t* v_new;
-  uint16_t* k_pool_w;         // the pools again, writable
+  uint16_t* k_pool_w;         // the pools, [pages][Hkv][16][D]
   uint16_t* v_pool_w;
   const float* cos_sin;       // [max_position][D] or null (no rotation)
   int fused, interleaved, max_position;
 };
 
 struct DecodePlan {
-  int group_tile;             // q heads of one kv head handled per CTA (<= 7)
+  int group_tile;             // q heads of one kv head handled per CTA (<= 16)
   int gsplit;                 // CTAs per kv head
   int chunk_tokens;           // keys per chunk (multiple of 64)
   int n_chunks;
@@ -42,7 +38,6 @@ struct DecodePlan {
 };
 
 DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len);
-efim_status launch_decode(const DecodeParams& p, const DecodePlan& pl, int D, cudaStream_t s);
 
 // Validation, planning and launch behind efim_decode_attn, efim_decode_step (fused = true:
 // rope / d_k_new / d_v_new are used) and efim_decode_attn_static.  The latter passes a

@@ -1120,7 +1120,7 @@ struct PoolMapEntry {
   int pages, Hkv, D;
   CUtensorMap map;
 };
-static const CUtensorMap* pool_map(void* pool, int pages, int Hkv, int D) {
+const CUtensorMap* pool_map(void* pool, int pages, int Hkv, int D) {
   constexpr int kEntries = 16;
   thread_local PoolMapEntry cache[kEntries] = {};
   thread_local int next = 0;

@@ -68,5 +68,9 @@ Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b, WorkItem* ite
 
 efim_status launch(const efim_cache_desc* c, const Params& p, const Plan& pl, cudaStream_t s);
 
+// Tensor map of a page pool (one box = the 16 slots x head_dim of one (page, kv head)), kept per
+// host thread; null if it cannot be encoded.  Valid until the thread's next call: copy it.
+const CUtensorMap* pool_map(void* pool, int pages, int Hkv, int D);
+
 }  // namespace pf
 }  // namespace efim

@@ -200,6 +200,41 @@ def test_decode_group_sizes_against_oracle(Hq, Hkv, D):
     H.assert_rope_close(dw.pages_from_device("k", used), kp, "k pages after the loop")
 
 
+@pytest.mark.parametrize("Hq,Hkv,D", [(1, 1, 128), (9, 1, 128), (15, 1, 64), (34, 2, 128), (40, 1, 64)])
+def test_decode_head_tiles_and_page_edges(Hq, Hkv, D):
+    """The edges of the decode kernel's tiles: 1, 8 + 1, 15 heads in one CTA, groups of 17 and 40
+    cut over two and three CTAs; rows that end on, just before and just past a page, the 64 keys
+    the four warps take per round, and a chunk.  Fused steps against the oracle (the probabilities
+    keep fp32 precision, so the error is the output's rounding to bf16 and what a rotated q or k
+    that rounds to the neighbouring bf16 value moves a score)."""
+    H = _harness()
+    import paper_2505_21889_b200 as efim
+    from efim_synth import bf16_bits_to_f32
+    ctx0 = [0, 14, 15, 16, 62, 63, 64, 254, 255, 256, 600]
+    w = _custom(Hq, Hkv, D, np.maximum(ctx0, 1), [0] * len(ctx0), seed=Hq + D, extra=1)
+    dw = H.DeviceWorkload(w)
+    kp, vp, bt, seqs = w.compact_host_pool()
+    ctx = np.array(ctx0, np.int32)
+    B, max_ctx = w.batch, int(ctx.max()) + 1
+    one = np.ones(B, np.int32)
+    q, k, v = w.decode_qkv(0)
+    q_rot = orc.kv_append(kp, vp, bt, ctx, one, q, k, v, w.rope_base)
+    o, lse = orc.decode_attention(q_rot, kp, vp, bt, ctx + 1, Hq)
+    ws = torch.empty(max(efim.efim_decode_workspace_bytes(dw.cache, B, max_ctx), 256), dtype=torch.uint8, device="cuda")
+    out = torch.empty((B, Hq, D), dtype=torch.bfloat16, device="cuda")
+    lse_d = torch.empty((B, Hq), dtype=torch.float32, device="cuda")
+    efim.efim_decode_step(dw.cache, B, torch.from_numpy(ctx + 1).cuda(), max_ctx, dw.batch.d_block_table, dw.rope,
+                          H.bits_to_torch(q), H.bits_to_torch(k), H.bits_to_torch(v), out, lse_d, 0.0, ws, dw.status)
+    torch.cuda.synchronize()
+    assert int(dw.status.item()) == 0
+    H.assert_attn_close(H.torch_to_bits(out), o, f"heads {Hq}/{Hkv} D={D}")
+    H.assert_lse_close(lse_d.cpu().numpy(), lse, f"heads {Hq}/{Hkv} D={D}")
+    # mean: rounding to nearest bf16 is off by at most 2^-9 |o|, by half of it on average; probabilities
+    # of bf16 precision would add as much again
+    err = np.abs(bf16_bits_to_f32(H.torch_to_bits(out)).astype(np.float64) - o)
+    assert err.mean() <= np.abs(o).mean() * 2.0 ** -9
+
+
 def test_decode_one_long_row_many_chunks():
     """A lone long row is cut into more than 32 chunks (so that every SM gets work); the merge
     then takes more than one pass over the lanes for the chunks' lse values."""
