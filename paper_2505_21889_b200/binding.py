@@ -7,6 +7,8 @@ from ctypes import c_int32, c_void_p, c_float, c_double, c_size_t, c_char_p, POI
 
 import numpy as np
 
+from torch import _C as _torch_c
+
 _LIB = None
 _HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -152,8 +154,8 @@ def _ptr(t):
 
 def _stream_ptr(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the raw handle of torch's current stream (building a Stream object costs 3 us more)
+        return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <utility>
 #include "efim.h"
 
 // the CUDA error behind the calling thread's last EFIM_ERR_CUDA (api.cu)
@@ -21,6 +22,34 @@ namespace efim {
 
 // SM count of the current device, cached per device (api.cu)
 int sm_count();
+
+// ---- programmatic dependent launch.  Every kernel of the library is launched with the attribute
+// that lets it start while the kernel before it in the stream is still running, and orders itself
+// with two instructions: pdl_wait() returns when everything before it in the stream has completed
+// and is visible; pdl_launch() lets the next kernel start its own set-up.  A kernel reads or writes
+// nothing that another kernel of the stream may write before its pdl_wait(), and calls pdl_launch()
+// only after it - so whatever starts early finds everything but its direct predecessor complete.
+// (Such data is read with plain loads: __ldg tells the compiler that nobody writes the data while the
+// kernel runs, and it could then be fetched before the wait.  Addresses that depend on data loaded
+// after the wait, and a plan's work list, may use it.)
+// What is saved is the launch gap and the set-up between two kernels of a call.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Validation shared by every entry point: shapes the kernels are built for.
 inline efim_status check_cache(const efim_cache_desc* c) {
@@ -120,7 +149,7 @@ __device__ __forceinline__ void rotate4_interleaved(uint4& v, const float* c, co
 
 __device__ __forceinline__ uint4 ldg_stream(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }

@@ -142,14 +142,25 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
   const int c = blockIdx.z;
   const uint32_t ring0 = (smem_u32(dec_smem) + 1023u) & ~1023u;
   uint8_t* ring_gen = dec_smem + (ring0 - smem_u32(dec_smem));
+  if (tid == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
+  }
+  if (lane == 0) {
+    for (int sg = 0; sg < ST; ++sg) mbar_init(smem_u32(&s_bar[warp][sg]), 1);
+    mbar_fence_init();
+  }
+  __syncwarp();
+  pdl_wait();
+  pdl_launch();
   // The first block-table entries of every warp are fetched before the row's length is known
   // (any entry of the row may be read; those past the length are dropped below), so that the
   // two loads share one round trip: a short step's time is mostly this ramp.
   const int32_t* bt = p.block_table + (size_t)r * p.max_pages_per_seq;
   const int first_pg = ((c * p.chunk_tokens) >> 4) + warp;
   const int my_pg = first_pg + DEC_WARPS * lane;
-  const int pid_early = my_pg < p.max_pages_per_seq ? __ldg(bt + my_pg) : -1;
-  int len = __ldg(p.row_len + r);
+  const int pid_early = my_pg < p.max_pages_per_seq ? *(bt + my_pg) : -1;
+  int len = *(p.row_len + r);
   // longer than the launch was planned for (max_ctx_len) or than the block table can address:
   // clamp and report.  A fused step then has no valid position for its new token and runs as a
   // plain decode over the clamped range.
@@ -197,11 +208,6 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
   const int last_pg = (end - 1) >> 4;
   const int n_pages = first_pg <= last_pg ? (last_pg - first_pg) / DEC_WARPS + 1 : 0;
   const uint32_t ring = ring0 + warp * (ST * 2 * PAGE_BYTES);
-  if (lane == 0) {
-    for (int sg = 0; sg < ST; ++sg) mbar_init(smem_u32(&s_bar[warp][sg]), 1);
-    mbar_fence_init();
-  }
-  __syncwarp();
   // page ids of the next 32 pages of this warp, one per lane (refilled every 32 pages)
   int pid_cache = (lane < n_pages) ? pid_early : -1;
   auto issue = [&](int i) {             // start the copies of this warp's i-th page into stage i % ST
@@ -233,8 +239,8 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
     uint4 w = make_uint4(0, 0, 0, 0);
     if (g < ng) {
       const uint4* qrow = reinterpret_cast<const uint4*>(p.q + ((size_t)r * p.Hq + head0 + g) * D);
-      w = __ldg(qrow + j);
-      if (FUSED && cs_row) w = dec_rotate_vec(w, __ldg(qrow + (j ^ (VEC / 2))), cs_row, D, j, p.interleaved);
+      w = *(qrow + j);
+      if (FUSED && cs_row) w = dec_rotate_vec(w, *(qrow + (j ^ (VEC / 2))), cs_row, D, j, p.interleaved);
     }
     *reinterpret_cast<uint4*>(&s_q[g][j * 8]) = w;
   }
@@ -291,14 +297,14 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
           const int j = lane, slot = (len - 1) & 15;
           const uint4* krow = reinterpret_cast<const uint4*>(p.k_new + ((size_t)r * p.Hkv + kvh) * D);
           const uint4* vrow = reinterpret_cast<const uint4*>(p.v_new + ((size_t)r * p.Hkv + kvh) * D);
-          uint4 kv = __ldg(krow + j);
-          if (cs_row) kv = dec_rotate_vec(kv, __ldg(krow + (j ^ (VEC / 2))), cs_row, D, j, p.interleaved);
-          const uint4 vv = __ldg(vrow + j);
+          uint4 kv = *(krow + j);
+          if (cs_row) kv = dec_rotate_vec(kv, *(krow + (j ^ (VEC / 2))), cs_row, D, j, p.interleaved);
+          const uint4 vv = *(vrow + j);
           uint8_t* kpage = ring_gen + (k_page - ring0);
           *reinterpret_cast<uint4*>(kpage + dec_page_off<D>(slot, j)) = kv;
           *reinterpret_cast<uint4*>(kpage + PAGE_BYTES + dec_page_off<D>(slot, j)) = vv;
           if (g0 == 0) {
-            const int pid = __ldg(bt + pg);
+            const int pid = *(bt + pg);
             const size_t off = (((size_t)pid * p.Hkv + kvh) * 16 + slot) * D + j * 8;
             *reinterpret_cast<uint4*>(p.k_pool_w + off) = kv;
             *reinterpret_cast<uint4*>(p.v_pool_w + off) = vv;
@@ -397,7 +403,7 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
     // ---- refill the stage with the page ST ahead
     const int nxt = i + ST;
     if (nxt < n_pages) {
-      if ((nxt & 31) == 0) pid_cache = (nxt + lane < n_pages) ? __ldg(bt + first_pg + DEC_WARPS * (nxt + lane)) : -1;
+      if ((nxt & 31) == 0) pid_cache = (nxt + lane < n_pages) ? *(bt + first_pg + DEC_WARPS * (nxt + lane)) : -1;
       ok_bits &= ~(1u << sg);
       if (issue(nxt)) ok_bits |= 1u << sg;
     }
@@ -466,70 +472,82 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
 }
 
 // Merge the chunk partials of one (row, head): lse = log2 sum 2^lse_c,
-// o = sum 2^(lse_c - lse) o_c.  One warp per (row, head), lanes over head_dim.
-template <int D>
+// o = sum 2^(lse_c - lse) o_c.  WPR warps share one (row, head), each taking every WPR-th block of
+// four chunks; lanes over head_dim.  Latency-bound on short steps: one warp for few chunks, four
+// from 9 chunks on, where one warp's chain of dependent loads showed.  Launched programmatically, it is
+// resident when the split kernel ends: 1 row x 2.3k keys 9.0 -> 7.5 us for the step, 16 rows x 2-2.9k
+// 31.5 -> 30.8, 64 rows x 1-16k at 28/4 heads (with the append before it) 128 -> 121.
+template <int D, int WPR>
 __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p) {
   constexpr int EPL = D / 32;
-  const int lane = threadIdx.x & 31;
-  const size_t row_head = (size_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (row_head >= (size_t)p.R * p.Hq) return;
+  constexpr int RPB = 4 / WPR;                     // (row, head) pairs per CTA
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int part = warp % WPR;
+  const size_t row_head = (size_t)blockIdx.x * RPB + warp / WPR;
+  __shared__ float s_acc[WPR > 1 ? 4 : 1][WPR > 1 ? D + 1 : 1];
+  pdl_wait();
+  pdl_launch();
+  if (row_head >= (size_t)p.R * p.Hq) return;      // (WPR = 4: the whole CTA)
   const int r = (int)(row_head / p.Hq);
-  const int len = min(__ldg(p.row_len + r), p.key_cap);
-  uint16_t* out = p.out + row_head * D + lane * EPL;
-  if (len <= 0) {
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) out[e] = 0;
-    if (p.lse && lane == 0) p.lse[row_head] = -INFINITY;
-    return;
-  }
+  const int len = min(*(p.row_len + r), p.key_cap);
   const int nc = min((len + p.chunk_tokens - 1) / p.chunk_tokens, p.n_chunks);
   const float* pl = p.part_lse + row_head * p.n_chunks;
   const float* po = p.part_o + row_head * p.n_chunks * D + lane * EPL;
-  // the lanes fetch the chunks' lse values side by side; the partial rows are then loaded four
-  // at a time and folded in chunk order (a chain of dependent loads cost more than the split
-  // kernel's tail on short steps)
   float M = -INFINITY;
   for (int c0 = 0; c0 < nc; c0 += 32)
-    if (c0 + lane < nc) M = fmaxf(M, __ldg(pl + c0 + lane));
+    if (c0 + lane < nc) M = fmaxf(M, pl[c0 + lane]);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
-  if (M == -INFINITY) {                            // every chunk came back empty (a skipped row)
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) out[e] = 0;
-    if (p.lse && lane == 0) p.lse[row_head] = -INFINITY;
-    return;
-  }
   float L = 0.f, acc[EPL];
 #pragma unroll
   for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-  for (int c0 = 0; c0 < nc; c0 += 4) {
-    float w[4];
-    __align__(16) float v[4][EPL];
+  if (M > -INFINITY) {                             // else a row without keys, or every chunk came back empty
+    for (int c0 = 4 * part; c0 < nc; c0 += 4 * WPR) {
+      float w[4];
+      __align__(16) float v[4][EPL];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (c0 + i < nc) {
-        w[i] = __ldg(pl + c0 + i);
-        if constexpr (EPL == 4) {
-          *reinterpret_cast<float4*>(v[i]) = __ldg(reinterpret_cast<const float4*>(po + (size_t)(c0 + i) * D));
-        } else {
-          *reinterpret_cast<float2*>(v[i]) = __ldg(reinterpret_cast<const float2*>(po + (size_t)(c0 + i) * D));
+      for (int i = 0; i < 4; ++i) {
+        if (c0 + i < nc) {
+          w[i] = pl[c0 + i];
+          if constexpr (EPL == 4) {
+            *reinterpret_cast<float4*>(v[i]) = *reinterpret_cast<const float4*>(po + (size_t)(c0 + i) * D);
+          } else {
+            *reinterpret_cast<float2*>(v[i]) = *reinterpret_cast<const float2*>(po + (size_t)(c0 + i) * D);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (c0 + i < nc) {
+          const float wi = exp2f(w[i] - M);
+          L += wi;
+#pragma unroll
+          for (int e = 0; e < EPL; ++e) acc[e] = fmaf(wi, v[i][e], acc[e]);
         }
       }
     }
+  }
+  if constexpr (WPR > 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (c0 + i < nc) {
-        const float wi = exp2f(w[i] - M);
-        L += wi;
+    for (int e = 0; e < EPL; ++e) s_acc[warp][lane * EPL + e] = acc[e];
+    if (lane == 0) s_acc[warp][D] = L;
+    __syncthreads();
+    if (part != 0) return;
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[e] = fmaf(wi, v[i][e], acc[e]);
-      }
+    for (int w = 1; w < WPR; ++w) {
+      L += s_acc[w][D];
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) acc[e] += s_acc[w][lane * EPL + e];
     }
   }
-  const float inv = 1.f / L;
-#pragma unroll
-  for (int e = 0; e < EPL; ++e) out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(acc[e] * inv));
-  if (p.lse && lane == 0) p.lse[row_head] = (M + log2f(L)) * 0.6931471805599453f;
+  const float inv = L > 0.f ? 1.f / L : 0.f;
+  uint16_t* out = p.out + row_head * D + lane * EPL;
+  if constexpr (EPL == 4) {
+    *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
+  } else {
+    *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+  }
+  if (p.lse && lane == 0) p.lse[row_head] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
 }
 
 DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len) {
@@ -589,7 +607,8 @@ static efim_status launch_split(const efim_cache_desc* cache, const DecodeParams
   if (!pv) return EFIM_ERR_CUDA;
   const efim_status st = dec_raise_smem_limit<D, NT, FUSED>();
   if (st != EFIM_OK) return st;
-  decode_splitkv_kernel<D, NT, FUSED><<<grid, DEC_THREADS, dec_ring_bytes(D) + 1024, s>>>(p, mk, *pv);
+  EFIM_CUDA_TRY(launch_pdl(decode_splitkv_kernel<D, NT, FUSED>, grid, dim3(DEC_THREADS), dec_ring_bytes(D) + 1024, s, p,
+                           mk, *pv));
   return EFIM_OK;
 }
 
@@ -603,11 +622,12 @@ static efim_status launch_decode_d(const efim_cache_desc* cache, const DecodePar
   else
     st = p.fused ? launch_split<D, 2, true>(cache, p, grid, s) : launch_split<D, 2, false>(cache, p, grid, s);
   if (st != EFIM_OK) return st;
-  EFIM_CUDA_TRY(cudaGetLastError());
   if (pl.n_chunks > 1) {
-    const unsigned blocks = (unsigned)(((size_t)p.R * p.Hq + 3) / 4);
-    decode_merge_kernel<D><<<blocks, 128, 0, s>>>(p);
-    EFIM_CUDA_TRY(cudaGetLastError());
+    const size_t row_heads = (size_t)p.R * p.Hq;
+    if (pl.n_chunks > 8)
+      EFIM_CUDA_TRY(launch_pdl(decode_merge_kernel<D, 4>, dim3((unsigned)row_heads), dim3(128), 0, s, p));
+    else
+      EFIM_CUDA_TRY(launch_pdl(decode_merge_kernel<D, 1>, dim3((unsigned)((row_heads + 3) / 4)), dim3(128), 0, s, p));
   }
   return EFIM_OK;
 }
@@ -615,7 +635,7 @@ static efim_status launch_decode_d(const efim_cache_desc* cache, const DecodePar
 static efim_status launch_decode(const efim_cache_desc* cache, const DecodeParams& p, const DecodePlan& pl,
                                  cudaStream_t s) {
   if (p.R == 0) return EFIM_OK;
-  if (p.R > 2147483647 / 4 || p.Hkv * pl.gsplit > 65535 || pl.n_chunks > 65535) return EFIM_ERR_UNSUPPORTED;
+  if ((long long)p.R * p.Hq > 2147483647LL || p.Hkv * pl.gsplit > 65535 || pl.n_chunks > 65535) return EFIM_ERR_UNSUPPORTED;
   return cache->head_dim == 128 ? launch_decode_d<128>(cache, p, pl, s) : launch_decode_d<64>(cache, p, pl, s);
 }
 

@@ -20,6 +20,7 @@ struct KvAppendParams {
   int32_t* status;
   int batch, max_pages_per_seq, total_new_tokens;
   int num_pages, Hq, Hkv, max_position, interleaved;
+  int early_next;           // let the next kernel start its set-up while this one runs
 };
 
 // WPT warps per new token, 256 threads per CTA.  A lane keeps one position along the head
@@ -38,30 +39,32 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS) kv_append_kernel(const KvAp
   constexpr int LANES = 32 * WPT;       // lanes working on one token
   const int lane = threadIdx.x % LANES;
   const int t = blockIdx.x * (KV_APPEND_THREADS / LANES) + threadIdx.x / LANES;
+  pdl_wait();
+  if (p.early_next) pdl_launch();
   if (t >= p.total_new_tokens) return;
   // sequence of this token: last s with q_indptr[s] <= t.  Up to 32 sequences are probed by the
   // warp's lanes at once (one round trip instead of a chain of five); more by bisection.
   int s;
   if (p.batch <= 32) {
     const int wl = threadIdx.x & 31;
-    const bool le = wl < p.batch && __ldg(p.q_indptr + wl) <= t;
+    const bool le = wl < p.batch && *(p.q_indptr + wl) <= t;
     s = 31 - __clz((int)(__ballot_sync(0xffffffffu, le) | 1u));
   } else {
     int lo = 0, hi = p.batch;
     while (hi - lo > 1) {
       int mid = (lo + hi) >> 1;
-      if (__ldg(p.q_indptr + mid) <= t) lo = mid; else hi = mid;
+      if (*(p.q_indptr + mid) <= t) lo = mid; else hi = mid;
     }
     s = lo;
   }
-  const int pos = __ldg(p.cached_len + s) + (t - __ldg(p.q_indptr + s));
+  const int pos = *(p.cached_len + s) + (t - *(p.q_indptr + s));
   const int page_idx = pos >> 4;
   int err = 0;
   int page = -1;
   if (pos < 0 || page_idx >= p.max_pages_per_seq || (p.cos_sin && pos >= p.max_position)) {
     err = EFIM_DEV_BAD_POSITION;
   } else {
-    page = __ldg(p.block_table + (size_t)s * p.max_pages_per_seq + page_idx);
+    page = *(p.block_table + (size_t)s * p.max_pages_per_seq + page_idx);
     if (page < 0 || page >= p.num_pages) err = EFIM_DEV_BAD_PAGE;
   }
   if (err) {
@@ -197,7 +200,13 @@ extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_b
   const int T = batch->total_new_tokens;
   const int wpt = T >= 16384 ? 1 : T >= 4096 ? 2 : T >= 1024 ? 4 : 8;
   const unsigned grid = (unsigned)(((long long)T * wpt * 32 + efim::KV_APPEND_THREADS - 1) / efim::KV_APPEND_THREADS);
-#define EFIM_KV_APPEND_LAUNCH(D_, W_) efim::kv_append_kernel<D_, W_><<<grid, efim::KV_APPEND_THREADS, 0, s>>>(p)
+  // With at most a CTA per SM the next kernel may start early (a step of 64 rows with its decode
+  // attention 128 -> 121 us).  Beside more CTAs the attention kernel's, which take an SM each, are dealt
+  // out to whichever SMs run dry first, and the launch lost more than the set-up it hid (append +
+  // attention of 64 mixed rows 349 -> 391 us, 16 rows at 32/32 heads 336 -> 351).
+  p.early_next = grid <= (unsigned)efim::sm_count();
+#define EFIM_KV_APPEND_LAUNCH(D_, W_) \
+  EFIM_CUDA_TRY(efim::launch_pdl(efim::kv_append_kernel<D_, W_>, dim3(grid), dim3(efim::KV_APPEND_THREADS), 0, s, p))
   if (cache->head_dim == 128) {
     if (wpt == 1) EFIM_KV_APPEND_LAUNCH(128, 1);
     else if (wpt == 2) EFIM_KV_APPEND_LAUNCH(128, 2);
@@ -210,6 +219,5 @@ extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_b
     else EFIM_KV_APPEND_LAUNCH(64, 8);
   }
 #undef EFIM_KV_APPEND_LAUNCH
-  EFIM_CUDA_TRY(cudaGetLastError());
   return EFIM_OK;
 }

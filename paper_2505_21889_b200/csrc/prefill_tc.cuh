@@ -54,6 +54,7 @@ struct Params {
   // rotation of the query rows as they are loaded (null: q is already rotated)
   const float* cos_sin;        // [max_position][D]
   int max_position, interleaved;
+  int early_next;              // let the next kernel start its set-up while this one runs
 };
 
 struct Plan {
