@@ -7,10 +7,14 @@ namespace efim {
 namespace pf {
 
 constexpr int BM = 128;        // query rows per tile (one TMEM lane each)
-constexpr int BN = 128;        // keys per KV tile (8 pages)
+constexpr int PT = 128;        // keys per tile of the work list (8 pages)
 constexpr int NQ = 2;          // query tiles per CTA sharing one K/V stream
-constexpr int NSTAGE = 5;      // K/V ring entries (one K or V tile of 128 keys each)
-constexpr int NSTAGE_MAX = 6;  // ring entries when there is a single query tile (the other tile's space is used)
+// Keys per step of the kernel's inner loop.  A stream keeps its scores S (fp32, BN columns), its
+// probabilities P (bf16, BN / 2 columns) and its O (fp32, D columns) in tensor memory side by side;
+// two streams share the 512 columns, so 2 * (1.5 * BN + D) <= 512 and BN is a whole number of pages:
+// 80 keys at head_dim 128, 128 at head_dim 64.  With P in columns of its own the scores of the next
+// step can be computed while this step's are being exponentiated.
+constexpr int bn_of(int D) { return D == 128 ? 80 : 128; }
 constexpr int THREADS = 384;   // 2 softmax warpgroups + 1 service warpgroup (2 TMA warps, 2 MMA warps)
 // Register split (setmaxnreg): the block launches with 168 registers per thread
 // (65536 / 384, rounded to 8) = 64512 in total; 2 x 128 x 216 + 128 x 72 = 64512 uses them all
@@ -19,8 +23,8 @@ constexpr int THREADS = 384;   // 2 softmax warpgroups + 1 service warpgroup (2 
 constexpr int REGS_SOFTMAX = 216;
 constexpr int REGS_SERVICE = 72;
 
-// One CTA's work: packed rows [row0, row0 + 256) of (seq, kv head) against KV tiles
-// [tile_begin, tile_end).  Packed row R = token * G + head-in-group.  The sequence's
+// One CTA's work: packed rows [row0, row0 + 256) of (seq, kv head) against the keys of the
+// 128-key tiles [tile_begin, tile_end).  Packed row R = token * G + head-in-group.  The sequence's
 // lengths and first query row ride along (the planner has them from the host mirrors),
 // so that a CTA's first dependent chain is "item -> block table / query rows" instead of
 // "item -> lengths -> block table / query rows".

@@ -311,6 +311,46 @@ def test_decode_rows_of_very_different_lengths_in_a_few_chunks(Hq, Hkv, D):
     H.assert_lse_close(lse_d.cpu().numpy()[keep], lse[keep], "decode, ragged rows")
 
 
+@pytest.mark.parametrize("Hq,Hkv,D,new", [(8, 2, 128, 70), (8, 2, 128, 20), (28, 4, 128, 3), (8, 2, 64, 70)])
+def test_scores_far_above_the_first_keys(Hq, Hkv, D, new):
+    """A row's reference maximum comes from its first key step and moves only when a later step's sum
+    leaves the range: keys whose scores lie hundreds of powers of two above (and below) the first ones,
+    far enough for the exponentials to overflow against the old reference, at step edges (80 and 128
+    keys) and in the last step; all three CTA shapes."""
+    efim, H, _custom, _check_turn = _mods()
+    cached = [1000, 79, 300]
+    w = _custom(Hq, Hkv, D, cached, [new, 2, 5], seed=61, extra=0)
+    dw = H.DeviceWorkload(w, use_rope=False)
+    big = {0: [79, 80, 160, 333, 640, 999], 1: [78], 2: [0, 127, 128, 255]}
+    real_page_bits = w.page_bits
+    scale = {}
+    for s, poss in big.items():
+        for j, pos in enumerate(poss):
+            scale[int(w.block_table[s, pos // 16]), pos % 16] = np.float32(2.0 ** (3 + j) * (-1) ** (j == 3))
+
+    def page_bits(which, page_ids):
+        out = real_page_bits(which, page_ids)
+        if which == "k":
+            from efim_synth import bf16_bits_to_f32, f32_to_bf16_bits
+            for n, pg in enumerate(page_ids):
+                for (p, slot), f in scale.items():
+                    if p == int(pg):
+                        out[n, :, slot] = f32_to_bf16_bits(bf16_bits_to_f32(out[n, :, slot]) * f)
+        return out
+    w.page_bits = page_bits
+    for (pg, slot), f in scale.items():
+        dw.k_pool[pg, :, slot] = dw.k_pool[pg, :, slot] * float(f)          # a power of two: exact
+    dw.gpu_kv_append()
+    dw.gpu_prefill()
+    torch.cuda.synchronize()
+    assert int(dw.status.item()) == 0
+    ref = dw.oracle_turn()
+    H.assert_attn_close(H.torch_to_bits(dw.out), ref["o"], "keys far above the first")
+    # scores of up to ~2^8 x 30: the tensor core's sums of D products carry about 2^-21 of that
+    lse = dw.lse.cpu().numpy().astype(np.float64)
+    assert (np.abs(lse - ref["lse"]) <= 1e-3 + np.abs(ref["lse"]) * 2.0 ** -18).all()
+
+
 def test_garbage_beyond_the_context_and_odd_cached_values():
     """What a real cache holds: the slots of a sequence's last page beyond its context are
     uninitialised (here NaN and Inf patterns, in K and in V), and cached values include
