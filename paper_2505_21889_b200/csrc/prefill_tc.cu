@@ -44,6 +44,14 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// One lane of a converged warp.  (Asked for this way the compiler keeps an MMA's descriptors in uniform
+// registers: an issuing thread then needs 48 cycles or less per tcgen05.mma, against 60 behind `lane == 0`;
+// 16 rows x 2-8k keys at 32/32 heads 331 -> 318 us for append and attention.)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -312,54 +320,75 @@ __device__ __forceinline__ float row_exp(const uint32_t* s, float scale, float n
   return lo + hi;
 }
 
-// One query row -> its row of a shared-memory query tile (swizzled), zero for a row past the
-// sequence; with a rotary table the row is rotated by its position on the way (the
-// arithmetic of efim_kv_append).  `qrow` = tile base + 128 * tile row, `r` = tile row.
+// 32 query rows (lane i knows row i: its index `th` in the packed [token * Hq + head] rows, or -1 for
+// a row past the sequence, and its position) into rows row0 .. row0+31 of a shared-memory query tile
+// (swizzled), zeros for absent rows; with a rotary table every row is rotated by its position on the
+// way (the arithmetic of efim_kv_append).  The warp reads whole rows, 32 * 16 bytes of them per
+// instruction: with a row per lane every instruction touched 32 lines (16 prompts of 1-3.5k tokens,
+// whose CTAs have some 16 steps, 1053 -> 1040 us for the append and this).
 template <int D>
-__device__ __forceinline__ void q_row_to_smem(const Params& p, uint8_t* qrow, int r, bool valid, int pos,
-                                              size_t row_off) {
+__device__ __noinline__ void q_rows_rotated_to_smem(const uint4* q, const float* cos_sin, int max_position, int interleaved,
+                                                    int32_t* status, uint8_t* tile, int row0, int lane, int th, int pos) {
   using L = Smem<D>;
-  const uint4* src = reinterpret_cast<const uint4*>(p.q + row_off);
-  auto put = [&](int c, uint4 v) {
-    *reinterpret_cast<uint4*>(qrow + (c >> 3) * L::HALF_BYTES + (((c & 7) ^ (r & 7)) << 4)) = v;
-  };
-  if (p.cos_sin == nullptr || !valid) {
-#pragma unroll
-    for (int c = 0; c < D / 8; ++c) {
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (valid) v = *(src + c);
-      put(c, v);
-    }
-  } else if (pos >= p.max_position) {
-    if (p.status) atomicOr(p.status, EFIM_DEV_BAD_POSITION);
-#pragma unroll
-    for (int c = 0; c < D / 8; ++c) put(c, make_uint4(0, 0, 0, 0));
-  } else {
-    const float* cs = p.cos_sin + (size_t)pos * D;
-    if (!p.interleaved) {
-#pragma unroll
-      for (int c = 0; c < D / 16; ++c) {
-        uint4 a = *(src + c), b = *(src + c + D / 16);
+  constexpr int VEC = D / 8, RPI = 32 / VEC;                 // 16-byte vectors per row, rows per instruction
+  const int c = lane % VEC, sub = lane / VEC;
+  if (th >= 0 && pos >= max_position) {                      // no table row: reported, attends with a zero query (finite)
+    if (status) atomicOr(status, EFIM_DEV_BAD_POSITION);
+    th = -1;
+  }
+#pragma unroll 4
+  for (int i = 0; i < VEC; ++i) {
+    const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub), ps = __shfl_sync(0xffffffffu, pos, i * RPI + sub);
+    const int r = row0 + i * RPI + sub;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (t >= 0) {
+      const uint4* src = q + (size_t)t * VEC;
+      const float* cs = cos_sin + (size_t)ps * D;
+      v = src[c];
+      if (!interleaved) {
+        uint4 o = src[c ^ (VEC / 2)];
+        const float* cp = cs + (c % (VEC / 2)) * 8;
         float cf[8], sf[8];
-        *reinterpret_cast<float4*>(cf) = *(reinterpret_cast<const float4*>(cs + c * 8));
-        *reinterpret_cast<float4*>(cf + 4) = *(reinterpret_cast<const float4*>(cs + c * 8 + 4));
-        *reinterpret_cast<float4*>(sf) = *(reinterpret_cast<const float4*>(cs + D / 2 + c * 8));
-        *reinterpret_cast<float4*>(sf + 4) = *(reinterpret_cast<const float4*>(cs + D / 2 + c * 8 + 4));
-        rotate8(a, b, cf, sf);
-        put(c, a);
-        put(c + D / 16, b);
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < D / 8; ++c) {
-        uint4 a = *(src + c);
+        *reinterpret_cast<float4*>(cf) = *reinterpret_cast<const float4*>(cp);
+        *reinterpret_cast<float4*>(cf + 4) = *reinterpret_cast<const float4*>(cp + 4);
+        *reinterpret_cast<float4*>(sf) = *reinterpret_cast<const float4*>(cp + D / 2);
+        *reinterpret_cast<float4*>(sf + 4) = *reinterpret_cast<const float4*>(cp + D / 2 + 4);
+        if (c < VEC / 2) {
+          rotate8(v, o, cf, sf);
+        } else {
+          rotate8(o, v, cf, sf);
+        }
+      } else {
         float cf[4], sf[4];
-        *reinterpret_cast<float4*>(cf) = *(reinterpret_cast<const float4*>(cs + c * 4));
-        *reinterpret_cast<float4*>(sf) = *(reinterpret_cast<const float4*>(cs + D / 2 + c * 4));
-        rotate4_interleaved(a, cf, sf);
-        put(c, a);
+        *reinterpret_cast<float4*>(cf) = *reinterpret_cast<const float4*>(cs + c * 4);
+        *reinterpret_cast<float4*>(sf) = *reinterpret_cast<const float4*>(cs + D / 2 + c * 4);
+        rotate4_interleaved(v, cf, sf);
       }
     }
+    *reinterpret_cast<uint4*>(tile + (c >> 3) * L::HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
+  }
+}
+template <int D>
+__device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* tile, int row0, int lane, int th, int pos) {
+  using L = Smem<D>;
+  constexpr int VEC = D / 8, RPI = 32 / VEC;
+  if (p.cos_sin != nullptr) {
+    q_rows_rotated_to_smem<D>(reinterpret_cast<const uint4*>(p.q), p.cos_sin, p.max_position, p.interleaved, p.status,
+                              tile, row0, lane, th, pos);
+    return;
+  }
+  const int c = lane % VEC, sub = lane / VEC;
+  uint4 v[VEC];
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) {
+    const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
+    v[i] = make_uint4(0, 0, 0, 0);
+    if (t >= 0) v[i] = reinterpret_cast<const uint4*>(p.q)[(size_t)t * VEC + c];
+  }
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) {
+    const int r = row0 + i * RPI + sub;
+    *reinterpret_cast<uint4*>(tile + (c >> 3) * L::HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v[i];
   }
 }
 
@@ -465,7 +494,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     const int vis = valid ? min(C + i_tok + 1, kv_cap) : kv_cap;
     const size_t row_off = ((size_t)(tok0 + i_tok) * p.Hq + (size_t)it.kvh * G + g) * D;
     if (st == 0) {
-      q_row_to_smem<D>(p, smem_gen + L::Q_OFF + r * 128, r, valid, C + i_tok, row_off);
+      q_rows_to_smem<D>(p, smem_gen + L::Q_OFF, w * 32, lane, valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1, C + i_tok);
       fence_async_smem();
       warp_arrive(bar(BAR_Q + 0), lane);
     }
@@ -563,7 +592,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     const int vis = valid ? min(C + i_tok + 1, kv_cap) : kv_cap;
     const size_t row_off = ((size_t)(tok0 + i_tok) * p.Hq + (size_t)it.kvh * G + g) * D;
     if (dual || st == 0) {
-      q_row_to_smem<D>(p, smem_gen + L::Q_OFF + qt * L::Q_BYTES + r * 128, r, valid, C + i_tok, row_off);
+      q_rows_to_smem<D>(p, smem_gen + L::Q_OFF + qt * L::Q_BYTES, (warp & 3) * 32, lane, valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1, C + i_tok);
       fence_async_smem();
       warp_arrive(bar(BAR_Q + qt), lane);
     }
@@ -646,13 +675,20 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
       const float lse2 = l_sum > 0.f ? m_ref + log2f(l_sum) : -INFINITY;
       const float a0 = w0 * inv, a1 = w1 * inv;
-      const size_t th = (size_t)(tok0 + i_tok) * p.Hq + (size_t)it.kvh * G + g;
-#pragma unroll
-      for (int c0 = 0; c0 < D; c0 += 32) {
+      const int th = valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1;
+      // The rows leave through the query tile's space (its MMAs are done; a warp uses its own 32 rows
+      // only): a lane writes its row, then the warp stores whole rows, two or four per instruction
+      // (with a row per lane every store touched 32 lines: 16 prompts of 1-3.5k tokens 1094 -> 1053 us).
+      constexpr int VEC = D / 8, RPI = 32 / VEC;
+      uint8_t* tile = smem_gen + L::Q_OFF + qt * L::Q_BYTES;
+      auto slot_of = [&](int row, int c) {
+        return reinterpret_cast<uint4*>(tile + (c >> 3) * L::HALF_BYTES + row * 128 + (((c & 7) ^ (row & 7)) << 4));
+      };
+      const int cc = lane % VEC, sub = lane / VEC;
+      auto load_o = [&](int c0, float* f) {                 // 32 columns of this row, both streams' states merged
         uint32_t o[32];
         tmem_ld<32>(o_addr + c0, o);
         tmem_wait_ld();
-        float f[32];
 #pragma unroll
         for (int c = 0; c < 32; ++c) f[c] = __uint_as_float(o[c]) * a0;
         if (merge) {
@@ -665,25 +701,54 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
             f[c + 3] = fmaf(x.w, a1, f[c + 3]);
           }
         }
-        if (valid) {
-          if (it.chunk < 0) {
-            uint4* dst = reinterpret_cast<uint4*>(p.out + row_off + c0);
+      };
+      if (it.chunk < 0) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              dst[c] = make_uint4(pack_bf16x2(f[c * 8], f[c * 8 + 1]), pack_bf16x2(f[c * 8 + 2], f[c * 8 + 3]),
-                                  pack_bf16x2(f[c * 8 + 4], f[c * 8 + 5]), pack_bf16x2(f[c * 8 + 6], f[c * 8 + 7]));
-          } else {
-            float4* dst = reinterpret_cast<float4*>(p.part_o + (th * p.s_max + it.chunk) * D + c0);
+        for (int c0 = 0; c0 < D; c0 += 32) {
+          float f[32];
+          load_o(c0, f);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) dst[c] = make_float4(f[4 * c], f[4 * c + 1], f[4 * c + 2], f[4 * c + 3]);
+          for (int c = 0; c < 4; ++c)
+            *slot_of(r, c0 / 8 + c) =
+                make_uint4(pack_bf16x2(f[c * 8], f[c * 8 + 1]), pack_bf16x2(f[c * 8 + 2], f[c * 8 + 3]),
+                           pack_bf16x2(f[c * 8 + 4], f[c * 8 + 5]), pack_bf16x2(f[c * 8 + 6], f[c * 8 + 7]));
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+          const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
+          const uint4 x = *slot_of((warp & 3) * 32 + i * RPI + sub, cc);
+          if (t >= 0) reinterpret_cast<uint4*>(p.out)[(size_t)t * VEC + cc] = x;
+        }
+      } else {
+        // a partial is fp32: half a row at a time fills the same space
+#pragma unroll
+        for (int hb = 0; hb < 2; ++hb) {
+#pragma unroll
+          for (int c0 = 0; c0 < D / 2; c0 += 32) {
+            float f[32];
+            load_o(hb * (D / 2) + c0, f);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+              *slot_of(r, c0 / 4 + c) = make_uint4(__float_as_uint(f[4 * c]), __float_as_uint(f[4 * c + 1]),
+                                                   __float_as_uint(f[4 * c + 2]), __float_as_uint(f[4 * c + 3]));
           }
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < VEC; ++i) {
+            const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
+            const uint4 x = *slot_of((warp & 3) * 32 + i * RPI + sub, cc);
+            if (t >= 0)
+              *reinterpret_cast<uint4*>(p.part_o + ((size_t)t * p.s_max + it.chunk) * D + hb * (D / 2) + cc * 4) = x;
+          }
+          __syncwarp();
         }
       }
       if (valid) {
         if (it.chunk < 0) {
           if (p.lse) p.lse[th] = lse2 * 0.6931471805599453f;
         } else {
-          p.part_lse[th * p.s_max + it.chunk] = lse2;
+          p.part_lse[(size_t)th * p.s_max + it.chunk] = lse2;
         }
       }
     }
@@ -751,7 +816,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     else produce(std::false_type{});
   } else if (warp == 9 || warp == 10) {
     // ============================================================ MMA issuers
-    // Issuing an MMA costs its thread about as long as the tensor core needs to run it,
+    // Issuing an MMA costs its thread nearly as long as the tensor core needs to run it,
     // so the work is split: warp 9 issues the PV MMAs of both streams, warp 10 the QK
     // MMAs.  QK(k+1) of a stream needs S(k) read (barrier SFREE), PV(k) needs P(k) written:
     // neither waits for the other, so the tensor core has a stream's next scores ready when
@@ -811,7 +876,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
           }
           mbar_wait(bar(BAR_P + st), k & 1, abort_flag, p.status, p.wait_ns);
           tc_fence_after();
-          if (lane == 0) {
+          if (elect_one()) {
             issue_pv(st, k == 0);
             if (last_user) tc_commit(bar(BAR_VEMPTY + slot));
             tc_commit(bar(k + 1 == my_cnt ? BAR_O + st : BAR_PV + st));
@@ -848,7 +913,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
           // phase meanwhile: stream 0's next scores are issued by this warp.)
           if (k == 0 && st == 1) mbar_wait(bar(BAR_P + 0), 0, abort_flag, p.status, p.wait_ns);
           tc_fence_after();
-          if (lane == 0) {
+          if (elect_one()) {
             issue_qk(st);
             tc_commit(bar(BAR_S + st));
             if (last_user) tc_commit(bar(BAR_KEMPTY + slot));
