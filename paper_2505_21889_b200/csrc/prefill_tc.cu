@@ -938,11 +938,16 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
   }
 }
 
-template <int D>
+// The work list: in the workspace (List = NoList), or, a short one planned inside the call, in the launch
+// parameters (List = InlineList) - which saves the copy between the append and this kernel.
+template <int D, typename List>
 __global__ void __launch_bounds__(THREADS, 1)
-prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
+prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                  const __grid_constant__ List list) {
   WorkItem it;                                                // 32 bytes: two vector loads, no dependent load after them
-  {
+  if constexpr (std::is_same<List, InlineList>::value) {
+    it = list.items[blockIdx.x];
+  } else {
     const uint4* src = reinterpret_cast<const uint4*>(p.items + blockIdx.x);
     uint4* dst = reinterpret_cast<uint4*>(&it);
     dst[0] = __ldg(src);
@@ -957,6 +962,11 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
     prefill_tc_body<D, 2>(p, map_k, map_v, it);
   else
     prefill_tc_body<D, 0>(p, map_k, map_v, it);
+  // A work list that came in the launch parameters is left in the workspace like any other: a call that
+  // plans for itself may be followed by planned calls with resident lists.
+  if constexpr (std::is_same<List, InlineList>::value) {
+    if (threadIdx.x == 0) p.items_out[blockIdx.x] = list.items[blockIdx.x];
+  }
 }
 
 // Merge the KV-chunk partials of split sequences: one warp per (token, head).
@@ -1007,139 +1017,163 @@ namespace {
 constexpr long long COST_TILE_DUAL = 21, COST_TILE_SINGLE = 15, COST_CTA = 100, COST_PARTIAL = 8, COST_MERGE = 80;
 constexpr long long COST_TILE_SINGLE_TAIL = 9;     // a one-tile CTA's tile when the GPU is no longer full
 
-// Finish time of the launch if the K/V range of every sequence is cut into chunks of
-// `chunk_tiles` tiles: the hardware hands CTAs, longest first, to whichever SM is free.
-long long estimate_makespan(const efim_cache_desc* c, const efim_batch_desc* b, long long chunk_tiles, int n_sm) {
-  const int G = c->num_q_heads / c->num_kv_heads;
-  std::vector<long long> cost;
-  bool split = false;
+// A run of consecutive work items that differ in the kv head only.
+struct Block {
+  int32_t seq, row0, tile_begin, tile_end;
+  int16_t chunk;
+  int32_t cost;                // place in the launch order
+};
+
+// Walks the blocks of a batch whose sequences' K/V ranges are cut into chunks of about `chunk_tiles`
+// tiles (at most 16 per sequence): f(seq, row0, rows of the block, tile_begin, tile_end, chunk or -1);
+// returns the largest number of chunks, writes keys per chunk of every cut sequence to `split`.
+template <typename F>
+int walk_blocks(const efim_cache_desc* c, const efim_batch_desc* b, long long chunk_tiles, int32_t* split, F&& f) {
+  const long long G = c->num_q_heads / c->num_kv_heads;
+  int s_max = 1;
   for (int s = 0; s < b->batch; ++s) {
     const long long N = b->h_new_len[s], C = b->h_cached_len[s];
+    if (split) split[s] = 0;
     if (N <= 0) continue;
     const long long rows = N * G;
     const long long kt_max = (C + N + PT - 1) / PT;
-    long long S = std::max<long long>(1, std::min<long long>(16, (kt_max + chunk_tiles - 1) / chunk_tiles));
-    const long long ct = (kt_max + S - 1) / S;
-    S = (kt_max + ct - 1) / ct;
-    split |= S > 1;
+    long long S = 1, ct = kt_max;
+    if (chunk_tiles < kt_max) {
+      S = std::min<long long>(16, (kt_max + chunk_tiles - 1) / chunk_tiles);
+      ct = (kt_max + S - 1) / S;                             // tiles per chunk
+      S = (kt_max + ct - 1) / ct;
+      if (S > 1 && split) split[s] = (int32_t)(ct * PT);
+      s_max = std::max<int>(s_max, (int)S);
+    }
     for (long long row0 = 0; row0 < rows; row0 += NQ * BM) {
       const long long rows_here = std::min<long long>(rows - row0, NQ * BM);
       const long long kt = (C + (row0 + rows_here - 1) / G + 1 + PT - 1) / PT;
-      const long long tc = rows_here > BM ? COST_TILE_DUAL : COST_TILE_SINGLE;
-      for (long long tb = 0; tb < kt; tb += ct)
-        cost.insert(cost.end(), (size_t)c->num_kv_heads,
-                    COST_CTA + std::min(ct, kt - tb) * tc + (S > 1 ? COST_PARTIAL : 0));
+      for (long long tb = 0, ch = 0; tb < kt; tb += ct, ++ch)
+        f(s, (int32_t)row0, (int)rows_here, (int32_t)tb, (int32_t)std::min(kt, tb + ct), (int)(S > 1 ? ch : -1));
     }
   }
-  std::sort(cost.begin(), cost.end(), std::greater<long long>());
-  std::vector<long long> sm((size_t)n_sm, 0);                // min-heap of SM finish times
-  auto later = std::greater<long long>();
-  for (long long x : cost) {
-    std::pop_heap(sm.begin(), sm.end(), later);
-    sm.back() += x;
-    std::push_heap(sm.begin(), sm.end(), later);
-  }
-  return *std::max_element(sm.begin(), sm.end()) + (split ? COST_MERGE : 0);
+  return s_max;
+}
+
+// Finish time of the launch with that cut: the hardware hands CTAs, longest first, to whichever SM is
+// free.  `best`: the earliest finish known; a cut whose lower bound is no better is not simulated.
+long long estimate_makespan(const efim_cache_desc* c, const efim_batch_desc* b, long long chunk_tiles, int n_sm,
+                            long long best, std::vector<int32_t>& cost, std::vector<int32_t>& sm) {
+  cost.clear();
+  long long total = 0, longest = 0;
+  const int s_max = walk_blocks(c, b, chunk_tiles, nullptr, [&](int, int32_t, int rows, int32_t tb, int32_t te, int ch) {
+    const long long x = COST_CTA + (te - tb) * (rows > BM ? COST_TILE_DUAL : COST_TILE_SINGLE) + (ch >= 0 ? COST_PARTIAL : 0);
+    cost.push_back((int32_t)std::min<long long>(x, 1 << 30));
+    total += x;
+    longest = std::max(longest, x);
+  });
+  const long long Hkv = c->num_kv_heads;
+  const long long merge = s_max > 1 ? COST_MERGE : 0;
+  const long long bound = std::max(longest, (total * Hkv + n_sm - 1) / n_sm) + merge;
+  if (bound >= best || (long long)cost.size() * Hkv <= n_sm) return bound;
+  std::sort(cost.begin(), cost.end(), std::greater<int32_t>());
+  sm.assign((size_t)n_sm, 0);                                // min-heap of SM finish times
+  long long end = 0;
+  for (int32_t x : cost)
+    for (long long h = 0; h < Hkv; ++h) {
+      const int32_t v = sm[0] + x;                           // the earliest SM takes the item: sift it down
+      end = std::max<long long>(end, v);
+      size_t i = 0;
+      for (size_t k = 1; k < sm.size(); k = 2 * i + 1) {
+        if (k + 1 < sm.size() && sm[k + 1] < sm[k]) ++k;
+        if (sm[k] >= v) break;
+        sm[i] = sm[k];
+        i = k;
+      }
+      sm[i] = v;
+    }
+  return end + merge;
 }
 }  // namespace
 
-Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b, WorkItem* items, int32_t* split_tokens) {
-  const int G = c->num_q_heads / c->num_kv_heads;
+Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b) {
   const int Hkv = c->num_kv_heads;
-  // pass 1: count unsplit items and KV tiles
-  long long n_unsplit = 0, tiles_total = 0;
-  for (int s = 0; s < b->batch; ++s) {
-    const long long N = b->h_new_len[s], C = b->h_cached_len[s];
-    if (N <= 0) continue;
-    const long long rows = N * G;
-    for (long long row0 = 0; row0 < rows; row0 += NQ * BM) {
-      const long long i_last = (std::min(rows, row0 + NQ * BM) - 1) / G;
-      const long long kt = (C + i_last + 1 + PT - 1) / PT;
-      n_unsplit += Hkv;
-      tiles_total += kt * Hkv;
-    }
-  }
+  long long n_blocks = 0, tiles_total = 0;
+  constexpr long long NO_CUT = 1LL << 40;
+  walk_blocks(c, b, NO_CUT, nullptr, [&](int, int32_t, int, int32_t tb, int32_t te, int) {
+    ++n_blocks;
+    tiles_total += (long long)(te - tb) * Hkv;
+  });
   // Few long items cannot fill the SMs, or leave a ragged last wave: try cutting the K/V
   // range of every sequence into chunks that give about 1, 2, 3 or 4 CTAs per SM (each at
   // least 4 tiles long) and keep the cut, or none, with the earliest estimated finish.
   const int n_sm = sm_count();
-  long long chunk_tiles = 1LL << 40;
-  if (n_unsplit < 4LL * n_sm && tiles_total > 0) {
-    long long best = estimate_makespan(c, b, chunk_tiles, n_sm);
+  Plan pl{};
+  pl.chunk_tiles = NO_CUT;
+  pl.s_max = 1;
+  if (n_blocks * Hkv < 4LL * n_sm && tiles_total > 0) {
+    std::vector<int32_t> cost, sm;
+    cost.reserve((size_t)n_blocks * 2);
+    long long best = estimate_makespan(c, b, NO_CUT, n_sm, 1LL << 60, cost, sm);
     for (int k = 1; k <= 4; ++k) {
       const long long ct = std::max<long long>(4, (tiles_total + (long long)n_sm * k - 1) / ((long long)n_sm * k));
-      const long long t = estimate_makespan(c, b, ct, n_sm);
-      if (t < best) { best = t; chunk_tiles = ct; }
+      const long long t = estimate_makespan(c, b, ct, n_sm, best, cost, sm);
+      if (t < best) { best = t; pl.chunk_tiles = ct; }
+    }
+    if (pl.chunk_tiles != NO_CUT) {
+      n_blocks = 0;
+      pl.s_max = walk_blocks(c, b, pl.chunk_tiles, nullptr, [&](int, int32_t, int, int32_t, int32_t, int) { ++n_blocks; });
     }
   }
-  Plan pl{};
-  int s_max = 1;
-  long long n_items = 0, tok0 = 0;
-  for (int s = 0; s < b->batch; tok0 += b->h_new_len[s], ++s) {
-    const long long N = b->h_new_len[s], C = b->h_cached_len[s];
-    if (split_tokens) split_tokens[s] = 0;
-    if (N <= 0) continue;
-    const long long rows = N * G;
-    const long long kt_max = (C + N + PT - 1) / PT;
-    long long S = std::min<long long>(16, (kt_max + chunk_tiles - 1) / chunk_tiles);
-    if (S < 1) S = 1;
-    const long long ct = (kt_max + S - 1) / S;               // tiles per chunk
-    S = (kt_max + ct - 1) / ct;
-    if (S > 1 && split_tokens) split_tokens[s] = (int32_t)(ct * PT);
-    s_max = std::max<int>(s_max, (int)S);
-    for (long long row0 = 0; row0 < rows; row0 += NQ * BM) {
-      const long long i_last = (std::min(rows, row0 + NQ * BM) - 1) / G;
-      const long long kt = (C + i_last + 1 + PT - 1) / PT;
-      for (long long ch = 0; ch < S; ++ch) {
-        const long long tb = ch * ct, te = std::min(kt, (ch + 1) * ct);
-        if (tb >= te) continue;
-        for (int h = 0; h < Hkv; ++h) {
-          if (items) {
-            WorkItem w{};
-            w.seq = s; w.kvh = (int16_t)h; w.row0 = (int)row0; w.tile_begin = (int)tb; w.tile_end = (int)te;
-            w.chunk = (int16_t)(S > 1 ? (int)ch : -1);
-            w.cached = (int32_t)C; w.new_len = (int32_t)N; w.tok0 = (int32_t)tok0;
-            items[n_items] = w;
-          }
-          ++n_items;
-        }
-      }
-    }
-  }
-  if (items) {
-    if (n_items > 8LL * n_sm) {
-      // Many waves: CTAs that run together should read the same K/V.  Keep the row tiles
-      // of one (sequence, kv head) adjacent (longest first inside the group), so the
-      // concurrent working set is a few heads' K/V and stays in L2.
-      std::stable_sort(items, items + n_items, [](const WorkItem& a, const WorkItem& b2) {
-        if (a.seq != b2.seq) return a.seq < b2.seq;
-        if (a.kvh != b2.kvh) return a.kvh < b2.kvh;
-        return a.row0 > b2.row0;
-      });
-    } else {
-      // Few waves: costliest first, so the tail of the launch is made of cheap items.  A tile
-      // costs a two-tile CTA (bound by its softmax) 2.1 us wherever it runs; a one-tile CTA is
-      // bound by its K/V bytes and speeds up once SMs fall idle at the end of the launch (measured:
-      // 0.89 us per tile with 8 to 32 such CTAs on the GPU, 1.5 us with 148), so it is weighted
-      // 0.9 us here (cfg2: 0.305 ms ordered by tile count, 0.290 by cost at 2.1 : 1.5, 0.281 at
-      // 2.1 : 1.2; 2.1 : 0.9 is 3-5 % faster still on three of four other draws of cfg2).
-      auto cost = [G](const WorkItem& w) {
-        const long long rows_here = std::min<long long>((long long)w.new_len * G - w.row0, NQ * BM);
-        return (long long)(w.tile_end - w.tile_begin) * (rows_here > BM ? COST_TILE_DUAL : COST_TILE_SINGLE_TAIL);
-      };
-      std::stable_sort(items, items + n_items,
-                       [&](const WorkItem& a, const WorkItem& b2) { return cost(a) > cost(b2); });
-    }
-  }
-  pl.n_items = (int)n_items;
-  pl.s_max = s_max;
+  pl.n_items = (int)(n_blocks * Hkv);
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
-  pl.items_bytes = up((size_t)n_items * sizeof(WorkItem));
+  pl.items_bytes = up((size_t)pl.n_items * sizeof(WorkItem));
   pl.split_bytes = up((size_t)b->batch * sizeof(int32_t));
   const size_t th = (size_t)b->total_new_tokens * c->num_q_heads;
-  pl.part_lse_bytes = s_max > 1 ? up(th * s_max * sizeof(float)) : 0;
-  pl.part_o_bytes = s_max > 1 ? up(th * s_max * c->head_dim * sizeof(float)) : 0;
+  pl.part_lse_bytes = pl.s_max > 1 ? up(th * pl.s_max * sizeof(float)) : 0;
+  pl.part_o_bytes = pl.s_max > 1 ? up(th * pl.s_max * c->head_dim * sizeof(float)) : 0;
   return pl;
+}
+
+void fill_lists(const efim_cache_desc* c, const efim_batch_desc* b, const Plan& pl, WorkItem* items, int32_t* split_tokens) {
+  const int Hkv = c->num_kv_heads;
+  std::vector<Block> blocks;
+  blocks.reserve((size_t)pl.n_items / Hkv);
+  // A tile costs a two-tile CTA (bound by its softmax) 2.1 us wherever it runs; a one-tile CTA is
+  // bound by its K/V bytes and speeds up once SMs fall idle at the end of a launch (measured:
+  // 0.89 us per tile with 8 to 32 such CTAs on the GPU, 1.5 us with 148), so it is weighted
+  // 0.9 us here (cfg2: 0.305 ms ordered by tile count, 0.290 by cost at 2.1 : 1.5, 0.281 at
+  // 2.1 : 1.2; 2.1 : 0.9 is 3-5 % faster still on three of four other draws of cfg2).
+  walk_blocks(c, b, pl.chunk_tiles, split_tokens, [&](int s, int32_t row0, int rows, int32_t tb, int32_t te, int ch) {
+    blocks.push_back(Block{s, row0, tb, te, (int16_t)ch,
+                           (int32_t)((te - tb) * (rows > BM ? COST_TILE_DUAL : COST_TILE_SINGLE_TAIL))});
+  });
+  std::vector<int32_t> tok0((size_t)b->batch);
+  for (int s = 0, t = 0; s < b->batch; t += b->h_new_len[s], ++s) tok0[s] = t;
+  auto put = [&](WorkItem*& w, const Block& k, int h) {
+    *w = WorkItem{};
+    w->seq = k.seq;
+    w->kvh = (int16_t)h;
+    w->chunk = k.chunk;
+    w->row0 = k.row0;
+    w->tile_begin = k.tile_begin;
+    w->tile_end = k.tile_end;
+    w->cached = b->h_cached_len[k.seq];
+    w->new_len = b->h_new_len[k.seq];
+    w->tok0 = tok0[k.seq];
+    ++w;
+  };
+  WorkItem* w = items;
+  if (pl.n_items > 8LL * sm_count()) {
+    // Many waves: CTAs that run together should read the same K/V.  Keep the row tiles
+    // of one (sequence, kv head) adjacent (longest first inside the group), so the
+    // concurrent working set is a few heads' K/V and stays in L2.
+    for (size_t i = 0, j = 0; i < blocks.size(); i = j) {
+      while (j < blocks.size() && blocks[j].seq == blocks[i].seq) ++j;
+      for (int h = 0; h < Hkv; ++h)
+        for (size_t k = j; k-- > i;) put(w, blocks[k], h);
+    }
+  } else {
+    // Few waves: costliest first, so the tail of the launch is made of cheap items.
+    std::stable_sort(blocks.begin(), blocks.end(), [](const Block& x, const Block& y) { return x.cost > y.cost; });
+    for (const Block& k : blocks)
+      for (int h = 0; h < Hkv; ++h) put(w, k, h);
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1200,32 +1234,34 @@ const CUtensorMap* pool_map(void* pool, int pages, int Hkv, int D) {
 }
 
 // The kernel's shared-memory size has to be raised once per device.
-template <int D>
+template <int D, typename List>
 static efim_status raise_smem_limit() {
   constexpr int kMaxDevices = 64;
   static std::atomic<bool> done[kMaxDevices];
   int dev = 0;
   EFIM_CUDA_TRY(cudaGetDevice(&dev));
   if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return EFIM_OK;
-  EFIM_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  EFIM_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<D, List>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      Smem<D>::TOTAL));
   if (dev >= 0 && dev < kMaxDevices) done[dev].store(true, std::memory_order_release);
   return EFIM_OK;
 }
 
-template <int D>
-static efim_status launch_d(const efim_cache_desc* c, const Params& args, const Plan& pl, cudaStream_t s) {
+template <int D, typename List>
+static efim_status launch_d(const efim_cache_desc* c, const Params& args, const Plan& pl, const List& list, cudaStream_t s) {
   Params p = args;
   // Few waves: the next kernel's set-up hides in the tail (8 x 128 tokens over 8k: 171 -> 169 us).  Many
   // waves: nothing to hide it in, 1 % lost (16 prompts of 1-3.5k tokens 1172 -> 1183 us).
   p.early_next = pl.n_items <= 4 * sm_count();
+  p.items_out = std::is_same<List, InlineList>::value ? const_cast<WorkItem*>(p.items) : nullptr;
   const CUtensorMap* pk = pool_map(c->d_k_pool, c->num_pages, c->num_kv_heads, D);
+  if (!pk) return EFIM_ERR_CUDA;
+  const CUtensorMap mk = *pk;
   const CUtensorMap* pv = pool_map(c->d_v_pool, c->num_pages, c->num_kv_heads, D);
-  if (!pk || !pv) return EFIM_ERR_CUDA;
-  const CUtensorMap mk = *pk, mv = *pv;
-  const efim_status st = raise_smem_limit<D>();
+  if (!pv) return EFIM_ERR_CUDA;
+  const efim_status st = raise_smem_limit<D, List>();
   if (st != EFIM_OK) return st;
-  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, mv));
+  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, List>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv, list));
   if (pl.s_max > 1) {
     const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + 3) / 4);
     EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D>, dim3(blocks), dim3(128), 0, s, p));
@@ -1233,9 +1269,10 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   return EFIM_OK;
 }
 
-efim_status launch(const efim_cache_desc* c, const Params& p, const Plan& pl, cudaStream_t s) {
+efim_status launch(const efim_cache_desc* c, const Params& p, const Plan& pl, const InlineList* list, cudaStream_t s) {
   if (pl.n_items == 0) return EFIM_OK;
-  return c->head_dim == 128 ? launch_d<128>(c, p, pl, s) : launch_d<64>(c, p, pl, s);
+  if (list) return c->head_dim == 128 ? launch_d<128>(c, p, pl, *list, s) : launch_d<64>(c, p, pl, *list, s);
+  return c->head_dim == 128 ? launch_d<128>(c, p, pl, NoList{}, s) : launch_d<64>(c, p, pl, NoList{}, s);
 }
 
 }  // namespace pf

@@ -48,6 +48,7 @@ struct Params {
   const int32_t* q_indptr;
   const int32_t* block_table;
   const WorkItem* items;
+  WorkItem* items_out;         // where to leave a work list that came in the launch parameters, or null
   const int32_t* split_tokens; // [batch] keys per KV chunk of a split sequence, 0 = not split
   float* part_o;               // [T][Hq][s_max][D]
   float* part_lse;             // [T][Hq][s_max]  base-2
@@ -65,14 +66,24 @@ struct Params {
 struct Plan {
   int n_items;
   int s_max;                   // largest KV split count (1 = no partials, no merge)
+  long long chunk_tiles;       // key tiles per KV chunk aimed at
   size_t items_bytes, split_bytes, part_lse_bytes, part_o_bytes;
   size_t total() const { return items_bytes + split_bytes + part_lse_bytes + part_o_bytes; }
 };
 
-// Host: size the plan (items == nullptr) or fill `items`/`split_tokens` too.
-Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b, WorkItem* items, int32_t* split_tokens);
+// A work list that travels in the launch parameters.
+struct NoList {};
+struct InlineList {
+  static constexpr int MAX_ITEMS = 256;
+  WorkItem items[MAX_ITEMS];
+};
 
-efim_status launch(const efim_cache_desc* c, const Params& p, const Plan& pl, cudaStream_t s);
+// Host: choose the cut and size the lists; then write them.
+Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b);
+void fill_lists(const efim_cache_desc* c, const efim_batch_desc* b, const Plan& pl, WorkItem* items, int32_t* split_tokens);
+
+// `list`: the work list if it is to travel in the launch parameters, else null (it is in the workspace).
+efim_status launch(const efim_cache_desc* c, const Params& p, const Plan& pl, const InlineList* list, cudaStream_t s);
 
 // Tensor map of a page pool (one box = the 16 slots x head_dim of one (page, kv head)), kept per
 // host thread; null if it cannot be encoded.  Valid until the thread's next call: copy it.

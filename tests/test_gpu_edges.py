@@ -432,6 +432,34 @@ def test_planned_prefill_with_resident_lists_can_be_captured_in_a_graph():
         assert torch.equal(dw.out.view(torch.int16), want_out.view(torch.int16)) and torch.equal(dw.lse, want_lse)
 
 
+@pytest.mark.parametrize("batch,new", [(8, 32), (33, 32)])
+def test_resident_lists_after_a_call_that_planned_for_itself(batch, new):
+    """A call without a plan leaves its work list in the workspace whether it was copied there (264 items)
+    or travelled in the launch parameters (64, up to 256): a planned call with resident lists behind it
+    gives the same bits, from a workspace that held something else before."""
+    efim, H, _custom, _check_turn = _mods()
+    w = _custom(8, 8, 64, [200 + 16 * i for i in range(batch)], [new] * batch, seed=71)
+    dw = H.DeviceWorkload(w)
+    dw.gpu_kv_append()
+    assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 1
+    plan = efim.efim_prefill_plan(dw.cache, dw.batch)
+    ws = torch.full((efim.efim_prefill_workspace_bytes(dw.cache, dw.batch),), 0, dtype=torch.uint8, device="cuda")
+    efim.efim_append_prefill_attn(dw.cache, dw.batch, dw.q, dw.out, dw.lse, 0.0, ws, dw.status)
+    torch.cuda.synchronize()
+    n = int(np.frombuffer(plan.tobytes()[:64], np.int32)[6]) * 32
+    assert n == batch * 8 * 32
+    assert np.array_equal(ws[:n].cpu().numpy(), plan[256:256 + n])       # checked before a kernel trusts them
+    want, want_lse = dw.out.clone(), dw.lse.clone()
+    dw.out.zero_()
+    efim.efim_append_prefill_attn(dw.cache, dw.batch, dw.q, dw.out, dw.lse, 0.0, ws, dw.status, plan=plan,
+                                  lists_resident=True)
+    torch.cuda.synchronize()
+    assert int(dw.status.item()) == 0
+    assert torch.equal(dw.out.view(torch.int16), want.view(torch.int16)) and torch.equal(dw.lse, want_lse)
+    ref = dw.oracle_turn([0, batch - 1])
+    H.assert_attn_close(H.torch_to_bits(dw.out)[ref["rows"]], ref["o"], "planned inside the call")
+
+
 def test_bounded_wait_expires_and_reports():
     """One warp waits on a barrier nothing completes, with nothing in flight: after the
     limit the kernel sets EFIM_DEV_TIMEOUT and ends normally; the context stays usable."""
