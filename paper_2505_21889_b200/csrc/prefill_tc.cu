@@ -139,6 +139,14 @@ __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t* r) {
 #undef EFIM_S16
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for this thread's tcgen05.ld; the registers they fill are named so that no use of them can be
+// moved before the wait (it costs no instruction).
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
+  tmem_wait_ld();
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -277,7 +285,7 @@ __device__ __noinline__ void rescale_o_row(uint32_t o_addr, float alpha) {
   for (int c0 = 0; c0 < D; c0 += 32) {
     uint32_t o[32];
     tmem_ld<32>(o_addr + c0, o);
-    tmem_wait_ld();
+    tmem_wait_ld<32>(o);
 #pragma unroll
     for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
     tmem_st<32>(o_addr + c0, o);
@@ -517,7 +525,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       tc_fence_after();
       uint32_t s[KQ];
       tmem_ld<KQ>(s_addr + KQ * w, s);
-      tmem_wait_ld();
+      tmem_wait_ld<KQ>(s);
       tc_fence_before();
       warp_arrive(bar(BAR_SFREE + st), lane);
       const int kv0 = key0 + (2 * k + st) * BN + KQ * w;
@@ -565,7 +573,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       uint32_t o[32];
       if (my_cnt > 0) {                                                 // warp-uniform: the load is warp-wide
         tmem_ld<32>(o_addr + c0, o);
-        tmem_wait_ld();
+        tmem_wait_ld<32>(o);
       }
 #pragma unroll
       for (int c = 0; c < 32; c += 4)
@@ -611,12 +619,12 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       // mixed rows 312 -> 306; first parts of 32 and 64 keys: 156 and 145 us, 2.71 and 2.56 ms).
       constexpr int LA = 48;
       tmem_ld<LA>(s_addr, s);
-      tmem_wait_ld();
+      tmem_wait_ld<LA>(s);
       tmem_ld<BN - LA>(s_addr + LA, s + LA);
       const int kv0 = key0 + (dual ? k : 2 * k + st) * BN;
       const bool edge = __any_sync(0xffffffffu, kv0 + BN > vis);
       if (edge) {
-        tmem_wait_ld();
+        tmem_wait_ld<BN - LA>(s + LA);
 #pragma unroll
         for (int c = 0; c < BN; ++c)
           if (kv0 + c >= vis) s[c] = 0xff800000u;           // -inf
@@ -624,7 +632,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       // The first step's exact maximum is the row's reference; later steps only check that their sum
       // stays in range (SUM_LIMIT), so a step has no row maximum to take before its first exponential.
       auto freed = [&]() {
-        tmem_wait_ld();
+        tmem_wait_ld<BN - LA>(s + LA);
         tc_fence_before();
         warp_arrive(bar(BAR_SFREE + st), lane);             // the next step's scores may be computed
       };
@@ -671,7 +679,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       for (int c0 = 0; c0 < D; c0 += 32) {
         uint32_t o[32];
         tmem_ld<32>(o_addr + c0, o);
-        tmem_wait_ld();
+        tmem_wait_ld<32>(o);
 #pragma unroll
         for (int c = 0; c < 32; c += 4)
           *reinterpret_cast<uint4*>(xbuf + c0 + c) = make_uint4(o[c], o[c + 1], o[c + 2], o[c + 3]);
@@ -704,7 +712,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       auto load_o = [&](int c0, float* f) {                 // 32 columns of this row, both streams' states merged
         uint32_t o[32];
         tmem_ld<32>(o_addr + c0, o);
-        tmem_wait_ld();
+        tmem_wait_ld<32>(o);
 #pragma unroll
         for (int c = 0; c < 32; ++c) f[c] = __uint_as_float(o[c]) * a0;
         if (merge) {
