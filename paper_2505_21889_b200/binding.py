@@ -1,7 +1,10 @@
-"""ctypes binding of include/efim.h.  Argument marshalling only: every step of the
-path runs inside libefim.so.  There is no fallback: if the library is missing or
-cannot be loaded, load_library() raises."""
+"""Binding of include/efim.h.  Argument marshalling only (the per-step calls through the
+extension csrc/calls.c, everything else through ctypes): every step of the path runs inside
+libefim.so.  There is no fallback: if the library is missing or cannot be loaded,
+load_library() raises."""
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from ctypes import c_int32, c_void_p, c_float, c_double, c_size_t, c_char_p, POINTER, Structure
 
@@ -127,6 +130,26 @@ def load_library():
     return lib
 
 
+class _Calls:
+    """The extension module with the per-step calls, loaded (with the library) on first use."""
+
+    def __getattr__(self, name):
+        load_library()
+        path = os.path.join(_HERE, "_calls.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} not found: build it first (python -m paper_2505_21889_b200.build)")
+        loader = importlib.machinery.ExtensionFileLoader("_calls", path)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
+        loader.exec_module(module)
+        for m in ("kv_append", "append_prefill_attn", "append_prefill_step", "decode_attn", "decode_step"):
+            setattr(self, m, getattr(module, m))          # found directly from now on
+        return self.__dict__[name]
+
+
+_calls = _Calls()
+_addr = ctypes.addressof
+
+
 def exported_symbols():
     """Names declared in include/efim.h that the loaded library exports."""
     lib = load_library()
@@ -214,9 +237,8 @@ def efim_rope_table_build(base, head_dim, max_position) -> np.ndarray:
 
 
 def efim_kv_append(cache: Cache, batch: Batch, rope, q, k_new, v_new, status=None, stream=None):
-    st = load_library().efim_kv_append(ctypes.byref(cache.desc), ctypes.byref(batch.desc),
-                                       ctypes.byref(rope.desc) if rope is not None else None,
-                                       _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(status), _stream_ptr(stream))
+    st = _calls.kv_append(_addr(cache.desc), _addr(batch.desc), _addr(rope.desc) if rope is not None else None,
+                          q, k_new, v_new, status, _stream_ptr(stream))
     if st != 0:
         raise EfimError(st, "efim_kv_append")
 
@@ -241,18 +263,8 @@ def efim_prefill_plan(cache: Cache, batch: Batch) -> np.ndarray:
 
 def efim_append_prefill_attn(cache: Cache, batch: Batch, q, out, lse=None, sm_scale=0.0,
                              workspace=None, status=None, stream=None, plan=None, lists_resident=False):
-    nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    lib = load_library()
-    if plan is None:
-        st = lib.efim_append_prefill_attn(ctypes.byref(cache.desc), ctypes.byref(batch.desc),
-                                          _ptr(q), _ptr(out), _ptr(lse), float(sm_scale),
-                                          _ptr(workspace), nbytes, _ptr(status), _stream_ptr(stream))
-    else:
-        st = lib.efim_append_prefill_attn_planned(ctypes.byref(cache.desc), ctypes.byref(batch.desc),
-                                                  plan.ctypes.data, plan.nbytes, 1 if lists_resident else 0,
-                                                  _ptr(q), _ptr(out), _ptr(lse),
-                                                  float(sm_scale), _ptr(workspace), nbytes, _ptr(status),
-                                                  _stream_ptr(stream))
+    st = _calls.append_prefill_attn(_addr(cache.desc), _addr(batch.desc), q, out, lse, sm_scale, workspace, status,
+                                    _stream_ptr(stream), plan, 1 if lists_resident else 0)
     if st != 0:
         raise EfimError(st, "efim_append_prefill_attn")
 
@@ -261,12 +273,9 @@ def efim_append_prefill_step(cache: Cache, batch: Batch, rope, q, k_new, v_new, 
                              workspace=None, status=None, stream=None, plan=None, lists_resident=False):
     """kv_append of the new tokens' k/v and append-prefill attention with q rotated on load
     (q is not modified)."""
-    nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    st = load_library().efim_append_prefill_step(
-        ctypes.byref(cache.desc), ctypes.byref(batch.desc), ctypes.byref(rope.desc) if rope is not None else None,
-        _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out), _ptr(lse), float(sm_scale),
-        plan.ctypes.data if plan is not None else None, plan.nbytes if plan is not None else 0,
-        1 if lists_resident else 0, _ptr(workspace), nbytes, _ptr(status), _stream_ptr(stream))
+    st = _calls.append_prefill_step(_addr(cache.desc), _addr(batch.desc), _addr(rope.desc) if rope is not None else None,
+                                    q, k_new, v_new, out, lse, sm_scale, plan, 1 if lists_resident else 0, workspace,
+                                    status, _stream_ptr(stream))
     if st != 0:
         raise EfimError(st, "efim_append_prefill_step")
 
@@ -283,11 +292,8 @@ def efim_decode_workspace_bytes(cache: Cache, batch: int, max_ctx_len: int) -> i
 
 def efim_decode_attn(cache: Cache, batch: int, d_ctx_len, max_ctx_len, d_block_table, q, out, lse=None,
                      sm_scale=0.0, workspace=None, status=None, stream=None):
-    nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    st = load_library().efim_decode_attn(ctypes.byref(cache.desc), batch, _ptr(d_ctx_len), int(max_ctx_len),
-                                         _ptr(d_block_table), int(d_block_table.shape[1]), _ptr(q), _ptr(out),
-                                         _ptr(lse), float(sm_scale), _ptr(workspace), nbytes,
-                                         _ptr(status), _stream_ptr(stream))
+    st = _calls.decode_attn(_addr(cache.desc), batch, d_ctx_len, int(max_ctx_len), d_block_table, d_block_table.shape[1],
+                            q, out, lse, sm_scale, workspace, status, _stream_ptr(stream))
     if st != 0:
         raise EfimError(st, "efim_decode_attn")
 
@@ -376,11 +382,8 @@ class Frontend:
 def efim_decode_step(cache: Cache, batch: int, d_ctx_len, max_ctx_len, d_block_table, rope, q, k_new, v_new, out,
                      lse=None, sm_scale=0.0, workspace=None, status=None, stream=None):
     """kv_append of one token per row and decode attention in one launch (q is not modified)."""
-    nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    st = load_library().efim_decode_step(ctypes.byref(cache.desc), batch, _ptr(d_ctx_len), int(max_ctx_len),
-                                         _ptr(d_block_table), int(d_block_table.shape[1]),
-                                         ctypes.byref(rope.desc) if rope is not None else None,
-                                         _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out), _ptr(lse), float(sm_scale),
-                                         _ptr(workspace), nbytes, _ptr(status), _stream_ptr(stream))
+    st = _calls.decode_step(_addr(cache.desc), batch, d_ctx_len, int(max_ctx_len), d_block_table, d_block_table.shape[1],
+                            _addr(rope.desc) if rope is not None else None, q, k_new, v_new, out, lse, sm_scale,
+                            workspace, status, _stream_ptr(stream))
     if st != 0:
         raise EfimError(st, "efim_decode_step")
