@@ -4,10 +4,10 @@
 //
 // One CTA owns up to 256 packed query rows (row = token * G + head-in-group) of one
 // (sequence, kv head) as two 128-row tiles, and streams the visible K/V range in
-// steps of 80 keys (5 pages; 128 keys at head_dim 64):
+// steps of 80 keys (5 pages):
 //   warps 8,11 TMA producers (K tiles / V tiles): walk the block table, one tiled bulk-tensor
 //             copy per page (16 slots x all dims of the kv head) into rings of 4 entries each
-//             (128B swizzle; 5 K entries with one query tile)
+//             (8 at head_dim 64; 128B swizzle; one K entry more with one query tile)
 //   warp 10   issues the tcgen05.mma for S_t = Q_t K^T into TMEM
 //   warp 9    issues the tcgen05.mma for O_t += P_t V (P read from TMEM)
 //   warps 0-7 two softmax groups ("streams"), one TMEM lane (row) per thread: S from TMEM, mask,
@@ -190,29 +190,28 @@ __host__ __device__ constexpr uint32_t instr_desc(int n, int b_mn_major) {
 // phase.  With a single query tile the second tile's space holds one more K entry (NK + 1).
 template <int D>
 struct Smem {
-  static constexpr int BN = bn_of(D);
   static constexpr int HALVES = D / 64;
   static constexpr int HALF_BYTES = 128 * 128;                  // 16 KB
   static constexpr int Q_BYTES = HALVES * HALF_BYTES;
   static constexpr int GROUP_BYTES = HALVES * 1024;             // 8 keys of a K/V tile, all dims
   static constexpr int PAGE_BYTES = 2 * GROUP_BYTES;            // one page = one copy
-  static constexpr int KV_BYTES = BN / 16 * PAGE_BYTES;         // 20 KB at head_dim 128, 16 KB at 64
-  static constexpr int NK = 4, NV = 4;                          // ring entries
+  static constexpr int KV_BYTES = BN / 16 * PAGE_BYTES;         // 20 KB at head_dim 128, 10 KB at 64
+  static constexpr int NK = D == 128 ? 4 : 8, NV = NK;            // ring entries
   static constexpr int NK_MAX = NK + 1;
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = Q_OFF + NQ * Q_BYTES;
   static constexpr int BAR_OFF = KV_OFF + (NK + NV) * KV_BYTES;
-  static constexpr int TOTAL = BAR_OFF + 256 + 1024;            // + alignment slack
+  static constexpr int TOTAL = BAR_OFF + 512 + 1024;            // + alignment slack
   static_assert(KV_BYTES <= Q_BYTES, "the extra K entry takes the second query tile's place");
   // epilogue exchange between the two softmax groups (re-uses the K/V rings)
   static constexpr int XROW = D + 4;                            // floats per row, padded
   static_assert(BM * XROW * 4 <= (NK + NV) * KV_BYTES, "exchange buffer must fit in the rings");
   static_assert(8 * 32 * XROW * 4 <= (NK + NV) * KV_BYTES, "the eight states must fit in the rings");
   // tensor memory: [S | P] of each stream, then O of each
-  static constexpr int SP_COLS = D == 128 ? 128 : 192;
+  static constexpr int SP_COLS = 128;
   static_assert(BN + BN / 2 <= SP_COLS && NQ * (SP_COLS + D) <= 512, "tensor memory has 512 columns");
 };
-// barrier slots (8 bytes each) inside the BAR_OFF block, per stream or per ring entry
+// barrier slots (8 bytes each) inside the BAR_OFF block, per stream or per ring entry (at most 9 K, 8 V)
 enum {
   BAR_Q = 0,         // query tile is in shared memory
   BAR_S = 2,         // scores of a step are in tensor memory
@@ -220,7 +219,7 @@ enum {
   BAR_P = 6,         // probabilities of a step are in tensor memory (and O has been rescaled if need be)
   BAR_PV = 8,        // PV of a step has finished (the last step's is BAR_O)
   BAR_O = 10,        // all of a stream's MMAs have finished
-  BAR_KFULL = 12, BAR_KEMPTY = 17, BAR_VFULL = 22, BAR_VEMPTY = 26, BAR_COUNT = 30
+  BAR_KFULL = 12, BAR_KEMPTY = 21, BAR_VFULL = 30, BAR_VEMPTY = 38, BAR_COUNT = 46
 };
 // A step's probabilities are taken relative to the reference maximum of the steps before; a row whose
 // sum of one step leaves this range (2^40) takes its exact maximum as the new reference and redoes the
@@ -416,7 +415,7 @@ template <int D, int MODE>
 __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                                 const WorkItem& it) {
   using L = Smem<D>;
-  constexpr int BN = L::BN, HALVES = L::HALVES;
+  constexpr int HALVES = L::HALVES;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));

@@ -315,8 +315,8 @@ def test_decode_rows_of_very_different_lengths_in_a_few_chunks(Hq, Hkv, D):
 def test_scores_far_above_the_first_keys(Hq, Hkv, D, new):
     """A row's reference maximum comes from its first key step and moves only when a later step's sum
     leaves the range: keys whose scores lie hundreds of powers of two above (and below) the first ones,
-    far enough for the exponentials to overflow against the old reference, at step edges (80 and 128
-    keys) and in the last step; all three CTA shapes."""
+    far enough for the exponentials to overflow against the old reference, at step edges (80 keys) and
+    in the last step; all three CTA shapes."""
     efim, H, _custom, _check_turn = _mods()
     cached = [1000, 79, 300]
     w = _custom(Hq, Hkv, D, cached, [new, 2, 5], seed=61, extra=0)
