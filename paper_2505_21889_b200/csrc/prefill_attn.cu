@@ -176,7 +176,7 @@ efim_status run_planned(const efim_cache_desc* cache, const efim_batch_desc* bat
                   nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
 }
 
-// Plans, then runs.  Up to InlineList::MAX_ITEMS items without a cut travel in the launch parameters: no
+// Plans, then runs.  Lists of up to InlineItems::MAX items travel in the launch parameters: no
 // copy stands between the append and the attention kernel (append and attention of 16 tokens over 240 in
 // one call 15.2 -> 10.7 us; the kernel leaves the list in the workspace all the same).
 efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
@@ -190,9 +190,9 @@ efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* ba
   if (!batch_has_work(batch)) return EFIM_OK;
   const pf::Plan pl = pf::make_plan(cache, batch);
   if (pl.n_items == 0) return EFIM_OK;
-  if (pl.s_max == 1 && pl.n_items <= pf::InlineList::MAX_ITEMS) {
+  if (pl.n_items <= pf::InlineItems::MAX && batch->batch <= pf::InlineSplit::MAX_BATCH) {
     pf::InlineList list;
-    pf::fill_lists(cache, batch, pl, list.items, nullptr);
+    pf::fill_lists(cache, batch, pl, list.items.items, list.split.keys);
     return run_plan(cache, batch, rope, pl, nullptr, &list, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
                     d_status, stream);
   }

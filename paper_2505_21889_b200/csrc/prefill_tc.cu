@@ -962,13 +962,13 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
 }
 
 // The work list: in the workspace (List = NoList), or, a short one planned inside the call, in the launch
-// parameters (List = InlineList) - which saves the copy between the append and this kernel.
+// parameters (List = InlineItems) - which saves the copy between the append and this kernel.
 template <int D, typename List>
 __global__ void __launch_bounds__(THREADS, 1)
 prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                   const __grid_constant__ List list) {
   WorkItem it;                                                // 32 bytes: two vector loads, no dependent load after them
-  if constexpr (std::is_same<List, InlineList>::value) {
+  if constexpr (std::is_same<List, InlineItems>::value) {
     it = list.items[blockIdx.x];
   } else {
     const uint4* src = reinterpret_cast<const uint4*>(p.items + blockIdx.x);
@@ -987,58 +987,91 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
     prefill_tc_body<D, 0>(p, map_k, map_v, it);
   // A work list that came in the launch parameters is left in the workspace like any other: a call that
   // plans for itself may be followed by planned calls with resident lists.
-  if constexpr (std::is_same<List, InlineList>::value) {
+  if constexpr (std::is_same<List, InlineItems>::value) {
     if (threadIdx.x == 0) p.items_out[blockIdx.x] = list.items[blockIdx.x];
   }
 }
 
-// Merge the KV-chunk partials of split sequences: one warp per (token, head).
-template <int D>
-__global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p) {
+// Merge the KV-chunk partials of split sequences: one warp per (token, head), four partial rows in flight.
+// `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the launch
+// parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
+template <int D, typename Split>
+__global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p, const __grid_constant__ Split split) {
   constexpr int EPL = D / 32;
+  constexpr bool inl = std::is_same<Split, InlineSplit>::value;
   const int lane = threadIdx.x & 31;
   const size_t th = (size_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  // (everything before the attention kernel has completed, and that kernel writes partials only: the
+  // look-ups need not wait for it)
+  int st = 0, nc = 0;
+  if (th < (size_t)p.total_new_tokens * p.Hq) {
+    const int t = (int)(th / p.Hq);
+    int lo = 0, hi = p.batch;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (p.q_indptr[mid] <= t) lo = mid; else hi = mid;
+    }
+    if constexpr (inl) st = split.keys[lo];
+    else st = p.split_tokens[lo];
+    if (st > 0) nc = min(p.s_max, (p.cached_len[lo] + (t - p.q_indptr[lo]) + 1 + st - 1) / st);
+  }
   pdl_wait();
   pdl_launch();
-  if (th >= (size_t)p.total_new_tokens * p.Hq) return;
-  const int t = (int)(th / p.Hq);
-  int lo = 0, hi = p.batch;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (*(p.q_indptr + mid) <= t) lo = mid; else hi = mid;
+  if constexpr (inl) {
+    if (blockIdx.x == 0)
+      for (int i = threadIdx.x; i < p.batch; i += 128) p.split_out[i] = split.keys[i];
   }
-  const int st = *(p.split_tokens + lo);
-  if (st == 0) return;                                      // written directly by the main kernel
-  const int vis = *(p.cached_len + lo) + (t - *(p.q_indptr + lo)) + 1;
-  const int nc = min(p.s_max, (vis + st - 1) / st);
+  if (nc == 0) return;                                      // written directly by the main kernel
   const float* pl = p.part_lse + th * p.s_max;
   const float* po = p.part_o + th * p.s_max * D + lane * EPL;
-  float M = -INFINITY;
-  for (int c = 0; c < nc; ++c) M = fmaxf(M, pl[c]);
+  const float mine = lane < nc ? pl[lane] : -INFINITY;      // at most 16 chunks
+  float M = mine;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
   float Lsum = 0.f, acc[EPL];
 #pragma unroll
   for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-  for (int c = 0; c < nc; ++c) {
-    const float w = exp2f(pl[c] - M);
-    Lsum += w;
+  if (M > -INFINITY) {
+    const float w_mine = exp2f(mine - M);                   // 0 beyond the last chunk
+    for (int c0 = 0; c0 < nc; c0 += 4) {
+      __align__(16) float v[4][EPL];
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) acc[e] = fmaf(w, po[(size_t)c * D + e], acc[e]);
+      for (int i = 0; i < 4; ++i) {
+        const float* src = po + (size_t)min(c0 + i, nc - 1) * D;
+        if constexpr (EPL == 4) {
+          *reinterpret_cast<float4*>(v[i]) = *reinterpret_cast<const float4*>(src);
+        } else {
+          *reinterpret_cast<float2*>(v[i]) = *reinterpret_cast<const float2*>(src);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float w = __shfl_sync(0xffffffffu, w_mine, c0 + i);
+        Lsum += w;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[e] = fmaf(w, v[i][e], acc[e]);
+      }
+    }
   }
   const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
   uint16_t* out = p.out + th * D + lane * EPL;
-#pragma unroll
-  for (int e = 0; e < EPL; ++e) out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(acc[e] * inv));
-  if (p.lse && lane == 0) p.lse[th] = (M + log2f(Lsum)) * 0.6931471805599453f;
+  if constexpr (EPL == 4) {
+    *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
+  } else {
+    *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+  }
+  if (p.lse && lane == 0) p.lse[th] = Lsum > 0.f ? (M + log2f(Lsum)) * 0.6931471805599453f : -INFINITY;
 }
 
 // ------------------------------------------------------------------ host side
 namespace {
-// Relative cost of a CTA in tenths of a microsecond, as measured on B200: a 128-key tile
-// with two query tiles is bound by the softmax / tensor pipeline, with one by its K/V
-// bytes; every CTA pays for its set-up, query load, pipeline fill and epilogue; a split
-// adds the partials' round trip and the merge launch.
-constexpr long long COST_TILE_DUAL = 21, COST_TILE_SINGLE = 15, COST_CTA = 100, COST_PARTIAL = 8, COST_MERGE = 80;
-constexpr long long COST_TILE_SINGLE_TAIL = 9;     // a one-tile CTA's tile when the GPU is no longer full
+// Cost of a CTA in tenths of a microsecond, as measured on B200 with a wave or less of them: a 128-key
+// tile with two query tiles is bound by the softmax / tensor pipeline, with one by its K/V bytes; every
+// CTA pays for its set-up, query load, pipeline fill and epilogue; a split adds the partials' round
+// trip and the merge.
+constexpr long long COST_TILE_DUAL = 18, COST_TILE_SINGLE = 12, COST_CTA = 95, COST_PARTIAL = 8, COST_MERGE = 40;
+// Weights of a tile in the launch order of a few waves (see fill_lists).
+constexpr long long ORDER_TILE_DUAL = 21, ORDER_TILE_SINGLE = 9;
 
 // A run of consecutive work items that differ in the kv head only.
 struct Block {
@@ -1122,9 +1155,12 @@ Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b) {
     ++n_blocks;
     tiles_total += (long long)(te - tb) * Hkv;
   });
-  // Few long items cannot fill the SMs, or leave a ragged last wave: try cutting the K/V
-  // range of every sequence into chunks that give about 1, 2, 3 or 4 CTAs per SM (each at
-  // least 4 tiles long) and keep the cut, or none, with the earliest estimated finish.
+  // Few long items cannot fill the SMs, or leave a ragged last wave: try cutting the K/V range of every
+  // sequence into chunks that would give between half a CTA and 4 CTAs per SM if they came out even
+  // (each at least 3 tiles long) and keep the cut, or none, with the earliest estimated finish.  (Cuts for
+  // less than one CTA per SM matter: ragged sequences round up, and a few CTAs too many are a second
+  // wave: 4 x 8-112 tokens over 1-3k keys at 32/8 heads, planned in the call, 62 -> 35 us; 1 x 40 over 4k 22 ->
+  // 19; 2 x 32-256 over 2-8k at 32/32 90 -> 80.)
   const int n_sm = sm_count();
   Plan pl{};
   pl.chunk_tiles = NO_CUT;
@@ -1133,8 +1169,11 @@ Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b) {
     std::vector<int32_t> cost, sm;
     cost.reserve((size_t)n_blocks * 2);
     long long best = estimate_makespan(c, b, NO_CUT, n_sm, 1LL << 60, cost, sm);
-    for (int k = 1; k <= 4; ++k) {
-      const long long ct = std::max<long long>(4, (tiles_total + (long long)n_sm * k - 1) / ((long long)n_sm * k));
+    long long last = 0;
+    for (const int k : {4, 5, 6, 7, 8, 10, 12, 16, 24, 32}) {    // CTAs per SM aimed at, in eighths
+      const long long ct = std::max<long long>(3, (tiles_total * 8 + (long long)n_sm * k - 1) / ((long long)n_sm * k));
+      if (ct == last) continue;
+      last = ct;
       const long long t = estimate_makespan(c, b, ct, n_sm, best, cost, sm);
       if (t < best) { best = t; pl.chunk_tiles = ct; }
     }
@@ -1164,7 +1203,7 @@ void fill_lists(const efim_cache_desc* c, const efim_batch_desc* b, const Plan& 
   // 2.1 : 1.2; 2.1 : 0.9 is 3-5 % faster still on three of four other draws of cfg2).
   walk_blocks(c, b, pl.chunk_tiles, split_tokens, [&](int s, int32_t row0, int rows, int32_t tb, int32_t te, int ch) {
     blocks.push_back(Block{s, row0, tb, te, (int16_t)ch,
-                           (int32_t)((te - tb) * (rows > BM ? COST_TILE_DUAL : COST_TILE_SINGLE_TAIL))});
+                           (int32_t)((te - tb) * (rows > BM ? ORDER_TILE_DUAL : ORDER_TILE_SINGLE))});
   });
   std::vector<int32_t> tok0((size_t)b->batch);
   for (int s = 0, t = 0; s < b->batch; t += b->h_new_len[s], ++s) tok0[s] = t;
@@ -1276,18 +1315,24 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   // Few waves: the next kernel's set-up hides in the tail (8 x 128 tokens over 8k: 171 -> 169 us).  Many
   // waves: nothing to hide it in, 1 % lost (16 prompts of 1-3.5k tokens 1172 -> 1183 us).
   p.early_next = pl.n_items <= 4 * sm_count();
-  p.items_out = std::is_same<List, InlineList>::value ? const_cast<WorkItem*>(p.items) : nullptr;
+  constexpr bool inl = std::is_same<List, InlineList>::value;
+  p.items_out = inl ? const_cast<WorkItem*>(p.items) : nullptr;
+  p.split_out = inl ? const_cast<int32_t*>(p.split_tokens) : nullptr;
   const CUtensorMap* pk = pool_map(c->d_k_pool, c->num_pages, c->num_kv_heads, D);
   if (!pk) return EFIM_ERR_CUDA;
   const CUtensorMap mk = *pk;
   const CUtensorMap* pv = pool_map(c->d_v_pool, c->num_pages, c->num_kv_heads, D);
   if (!pv) return EFIM_ERR_CUDA;
-  const efim_status st = raise_smem_limit<D, List>();
+  using Items = std::decay_t<decltype(items_of(list))>;
+  const efim_status st = raise_smem_limit<D, Items>();
   if (st != EFIM_OK) return st;
-  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, List>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv, list));
+  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, Items>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv, items_of(list)));
   if (pl.s_max > 1) {
     const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + 3) / 4);
-    EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D>, dim3(blocks), dim3(128), 0, s, p));
+    if constexpr (inl)
+      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, InlineSplit>, dim3(blocks), dim3(128), 0, s, p, list.split));
+    else
+      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, NoList>, dim3(blocks), dim3(128), 0, s, p, NoList{}));
   }
   return EFIM_OK;
 }

@@ -49,7 +49,8 @@ struct Params {
   const int32_t* q_indptr;
   const int32_t* block_table;
   const WorkItem* items;
-  WorkItem* items_out;         // where to leave a work list that came in the launch parameters, or null
+  WorkItem* items_out;         // where to leave lists that came in the launch parameters, or null
+  int32_t* split_out;
   const int32_t* split_tokens; // [batch] keys per KV chunk of a split sequence, 0 = not split
   float* part_o;               // [T][Hq][s_max][D]
   float* part_lse;             // [T][Hq][s_max]  base-2
@@ -72,12 +73,22 @@ struct Plan {
   size_t total() const { return items_bytes + split_bytes + part_lse_bytes + part_o_bytes; }
 };
 
-// A work list that travels in the launch parameters.
+// Lists that travel in the launch parameters: the work items and the split sizes of the sequences.
 struct NoList {};
-struct InlineList {
-  static constexpr int MAX_ITEMS = 256;
-  WorkItem items[MAX_ITEMS];
+struct InlineItems {
+  static constexpr int MAX = 256;
+  WorkItem items[MAX];
 };
+struct InlineSplit {
+  static constexpr int MAX_BATCH = 256;
+  int32_t keys[MAX_BATCH];
+};
+struct InlineList {
+  InlineItems items;
+  InlineSplit split;
+};
+inline const InlineItems& items_of(const InlineList& l) { return l.items; }
+inline const NoList& items_of(const NoList& l) { return l; }
 
 // Host: choose the cut and size the lists; then write them.
 Plan make_plan(const efim_cache_desc* c, const efim_batch_desc* b);
