@@ -213,10 +213,9 @@ efim_status efim_append_prefill_step(const efim_cache_desc* cache, const efim_ba
  * page_size); it fixes the chunking, so no host copy of the lengths is needed.
  * ctx_len[s] == 0 gives out = 0, lse = -inf.  Query-head groups of up to 16 per kv head read
  * the K/V pages once; larger groups are cut into tiles of at most 16 heads that each read them.
- *  A device length beyond what the launch was
- * planned for (the chunks cover max_ctx_len rounded up to whole chunks, at most the block
- * table's capacity) is clamped to that and sets EFIM_DEV_BAD_POSITION; nothing outside the
- * workspace or the table is touched.
+ * A device length beyond what the launch was planned for (the chunks cover max_ctx_len rounded
+ * up to whole chunks, at most the block table's capacity) is clamped to that and sets
+ * EFIM_DEV_BAD_POSITION; nothing outside the workspace or the table is touched.
  */
 size_t efim_decode_workspace_bytes(const efim_cache_desc* cache, int32_t batch, int32_t max_ctx_len);
 /* Number of kernels the corresponding call enqueues for these arguments (the main
