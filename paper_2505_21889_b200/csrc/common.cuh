@@ -31,7 +31,7 @@ int sm_count();
 // only after it - so whatever starts early finds everything but its direct predecessor complete.
 // (Such data is read with plain loads: __ldg tells the compiler that nobody writes the data while the
 // kernel runs, and it could then be fetched before the wait.  Addresses that depend on data loaded
-// after the wait, and a plan's work list, may use it.)
+// after the wait may use it.)
 // What is saved is the launch gap and the set-up between two kernels of a call.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -486,8 +486,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
   }
 
-  // Programmatic launch: up to here a CTA has touched nothing but itself and the caller's plan;
-  // every warp that reads or writes global memory waits for the kernel before.
+  // Programmatic launch: up to here a CTA with a list of its own has touched nothing but itself; every warp that reads or writes global memory waits for the kernel before.
   if (warp < 8 && tiny) {
     pdl_wait();
     // ============================================================ softmax groups, 32-row shape
@@ -971,10 +970,12 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   if constexpr (std::is_same<List, InlineItems>::value) {
     it = list.items[blockIdx.x];
   } else {
+    // (after the wait: the kernel before may be one that leaves its list in this workspace)
+    pdl_wait();
     const uint4* src = reinterpret_cast<const uint4*>(p.items + blockIdx.x);
     uint4* dst = reinterpret_cast<uint4*>(&it);
-    dst[0] = __ldg(src);
-    dst[1] = __ldg(src + 1);
+    dst[0] = src[0];
+    dst[1] = src[1];
   }
   const int rows_here = it.new_len * p.G - it.row0;
   // the three shapes of a CTA are separate instantiations: ring size, load order and the
@@ -1002,18 +1003,18 @@ __global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p, cons
   const int lane = threadIdx.x & 31;
   const size_t th = (size_t)blockIdx.x * 4 + (threadIdx.x >> 5);
   // (everything before the attention kernel has completed, and that kernel writes partials only: the
-  // look-ups need not wait for it)
+  // look-ups need not wait for it.  Read in L2, where what has completed is visible.)
   int st = 0, nc = 0;
   if (th < (size_t)p.total_new_tokens * p.Hq) {
     const int t = (int)(th / p.Hq);
     int lo = 0, hi = p.batch;
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
-      if (p.q_indptr[mid] <= t) lo = mid; else hi = mid;
+      if (__ldcg(p.q_indptr + mid) <= t) lo = mid; else hi = mid;
     }
     if constexpr (inl) st = split.keys[lo];
-    else st = p.split_tokens[lo];
-    if (st > 0) nc = min(p.s_max, (p.cached_len[lo] + (t - p.q_indptr[lo]) + 1 + st - 1) / st);
+    else st = __ldcg(p.split_tokens + lo);
+    if (st > 0) nc = min(p.s_max, (__ldcg(p.cached_len + lo) + (t - __ldcg(p.q_indptr + lo)) + 1 + st - 1) / st);
   }
   pdl_wait();
   pdl_launch();

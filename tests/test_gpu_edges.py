@@ -462,6 +462,16 @@ def test_resident_lists_after_a_call_that_planned_for_itself(batch, new, cached,
     assert torch.equal(dw.out.view(torch.int16), want.view(torch.int16)) and torch.equal(dw.lse, want_lse)
     ref = dw.oracle_turn([0, batch - 1])
     H.assert_attn_close(H.torch_to_bits(dw.out)[ref["rows"]], ref["o"], "planned inside the call")
+    # back to back on one stream, nothing between them: the second call must not look at the lists before the
+    # first has left them (the workspace holds valid lists of the same batch, so even then it stays in bounds)
+    for _ in range(20):
+        dw.out.zero_()
+        efim.efim_append_prefill_attn(dw.cache, dw.batch, dw.q, dw.out, dw.lse, 0.0, ws, dw.status)
+        efim.efim_append_prefill_attn(dw.cache, dw.batch, dw.q, dw.out, dw.lse, 0.0, ws, dw.status, plan=plan,
+                                      lists_resident=True)
+    torch.cuda.synchronize()
+    assert int(dw.status.item()) == 0
+    assert torch.equal(dw.out.view(torch.int16), want.view(torch.int16)) and torch.equal(dw.lse, want_lse)
 
 
 def test_bounded_wait_expires_and_reports():
