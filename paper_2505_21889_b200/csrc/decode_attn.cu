@@ -475,8 +475,8 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
 // o = sum 2^(lse_c - lse) o_c.  WPR warps share one (row, head), each taking every WPR-th block of
 // four chunks; lanes over head_dim.  Latency-bound on short steps: one warp for few chunks, four
 // from 9 chunks on, where one warp's chain of dependent loads showed.  Launched programmatically, it is
-// resident when the split kernel ends: 1 row x 2.3k keys 9.0 -> 7.5 us for the step, 16 rows x 2-2.9k
-// 31.5 -> 30.8, 64 rows x 1-16k at 28/4 heads (with the append before it) 128 -> 121.
+// resident when the split kernel ends: 1 row x 2.3k keys 9.0 -> 7.3 us for the step, 16 rows x 2-2.9k
+// 31.5 -> 30.5, 64 rows x 1-16k at 28/4 heads (with the append before it) 128 -> 121.
 template <int D, int WPR>
 __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p) {
   constexpr int EPL = D / 32;
@@ -485,37 +485,48 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p)
   const int part = warp % WPR;
   const size_t row_head = (size_t)blockIdx.x * RPB + warp / WPR;
   __shared__ float s_acc[WPR > 1 ? 4 : 1][WPR > 1 ? D + 1 : 1];
+  // The row's length is an input of the step: the split kernel does not write it, and everything before
+  // that kernel has completed, so it is looked up before the wait (in L2, where what has completed is
+  // visible).  With the first partial rows fetched beside the maximum's lse values: steps of 1 to 64 rows in
+  // chunks 0.7-1.0 us shorter (1 row x 2.3k keys 7.3 -> 6.5, 16 rows x 2-2.9k 30.5 -> 29.5).
+  int nc = 0;
+  if (row_head < (size_t)p.R * p.Hq) {
+    const int len = min(__ldcg(p.row_len + row_head / p.Hq), p.key_cap);
+    nc = min((len + p.chunk_tokens - 1) / p.chunk_tokens, p.n_chunks);
+  }
   pdl_wait();
   pdl_launch();
   if (row_head >= (size_t)p.R * p.Hq) return;      // (WPR = 4: the whole CTA)
-  const int r = (int)(row_head / p.Hq);
-  const int len = min(*(p.row_len + r), p.key_cap);
-  const int nc = min((len + p.chunk_tokens - 1) / p.chunk_tokens, p.n_chunks);
   const float* pl = p.part_lse + row_head * p.n_chunks;
   const float* po = p.part_o + row_head * p.n_chunks * D + lane * EPL;
+  float L = 0.f, acc[EPL];
+#pragma unroll
+  for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+  // partial rows c0 .. c0+3 and their lse values; the first four go out together with the maximum's loads
+  float w[4];
+  __align__(16) float v[4][EPL];
+  auto fetch = [&](int c0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (c0 + i < nc) {
+        w[i] = pl[c0 + i];
+        if constexpr (EPL == 4) {
+          *reinterpret_cast<float4*>(v[i]) = *reinterpret_cast<const float4*>(po + (size_t)(c0 + i) * D);
+        } else {
+          *reinterpret_cast<float2*>(v[i]) = *reinterpret_cast<const float2*>(po + (size_t)(c0 + i) * D);
+        }
+      }
+    }
+  };
+  fetch(4 * part);
   float M = -INFINITY;
   for (int c0 = 0; c0 < nc; c0 += 32)
     if (c0 + lane < nc) M = fmaxf(M, pl[c0 + lane]);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
-  float L = 0.f, acc[EPL];
-#pragma unroll
-  for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
   if (M > -INFINITY) {                             // else a row without keys, or every chunk came back empty
     for (int c0 = 4 * part; c0 < nc; c0 += 4 * WPR) {
-      float w[4];
-      __align__(16) float v[4][EPL];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (c0 + i < nc) {
-          w[i] = pl[c0 + i];
-          if constexpr (EPL == 4) {
-            *reinterpret_cast<float4*>(v[i]) = *reinterpret_cast<const float4*>(po + (size_t)(c0 + i) * D);
-          } else {
-            *reinterpret_cast<float2*>(v[i]) = *reinterpret_cast<const float2*>(po + (size_t)(c0 + i) * D);
-          }
-        }
-      }
+      if (c0 != 4 * part) fetch(c0);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         if (c0 + i < nc) {
