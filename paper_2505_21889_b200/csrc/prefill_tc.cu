@@ -25,6 +25,7 @@
 // 1158 -> 1095 us, 64 mixed rows at 28/4 heads 342 -> 332 us.
 #include "prefill_tc.cuh"
 #include "mbar.cuh"
+#include <cfloat>
 #include <vector>
 #include <algorithm>
 #include <functional>
@@ -225,6 +226,11 @@ enum {
 // sum of one step leaves this range (2^40) takes its exact maximum as the new reference and redoes the
 // step.  P and O are floating point, so nothing is lost by a reference that is off.
 constexpr float SUM_LIMIT = 1099511627776.f;
+
+// A row's reference after its first step with largest score `mx`.  Finite also where the row saw no key
+// or infinitely low scores only: those keys' probabilities are 0 against it, and the first finite score
+// to come overflows the sum, so that the reference moves up to it.
+__device__ __forceinline__ float first_reference(float mx) { return fmaxf(mx, -FLT_MAX); }
 
 // Epilogue of the 32-row shape: the eight (max, sum, O) states of query row `lane`, left in
 // shared memory as [state][row][XROW], are merged; this thread finishes D/8 dims of the row
@@ -532,9 +538,9 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         for (int c = 0; c < KQ; ++c)
           if (kv0 + c >= vis) s[c] = 0xff800000u;           // -inf
       }
-      if (k == 0) m_ref = row_max<KQ>(s) * p.scale_log2;
+      if (k == 0) m_ref = first_reference(row_max<KQ>(s) * p.scale_log2);
       uint32_t v[KQ / 2];
-      float sum = row_exp<KQ>(s, p.scale_log2, m_ref == -INFINITY ? 0.f : -m_ref, v);
+      float sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
       if (k > 0) {
         mbar_wait(bar(BAR_PV + st), (k - 1) & 1, abort_flag, p.status, p.wait_ns);   // P of the step before is consumed
         tc_fence_after();
@@ -544,7 +550,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
           m_ref = m_new;
           l_sum *= alpha;
           rescale_o_row<D>(o_addr, alpha);
-          sum = row_exp<KQ>(s, p.scale_log2, m_ref == -INFINITY ? 0.f : -m_ref, v);
+          sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
         }
       }
       tmem_st<KQ / 2>(p_addr + KQ / 2 * w, v);
@@ -635,9 +641,9 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         warp_arrive(bar(BAR_SFREE + st), lane);             // the next step's scores may be computed
       };
       if (edge || k == 0) freed();
-      if (k == 0) m_ref = row_max<BN>(s) * p.scale_log2;
+      if (k == 0) m_ref = first_reference(row_max<BN>(s) * p.scale_log2);
       uint32_t w[BN / 2];                                   // P as bf16 pairs
-      const float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+      const float neg_m = -m_ref;
       float sum = row_exp<LA>(s, p.scale_log2, neg_m, w);
       if (!(edge || k == 0)) freed();
       sum += row_exp<BN - LA>(s + LA, p.scale_log2, neg_m, w + LA / 2);
@@ -653,7 +659,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         m_ref = m_new;
         l_sum *= alpha;
         rescale_o_row<D>(o_addr, alpha);
-        sum = row_exp<BN>(s, p.scale_log2, m_ref == -INFINITY ? 0.f : -m_ref, w);
+        sum = row_exp<BN>(s, p.scale_log2, -m_ref, w);
         tmem_st<BN / 2>(p_addr, w);
       }
       tmem_wait_st();

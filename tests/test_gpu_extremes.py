@@ -1,0 +1,74 @@
+"""GPU: infinities, NaN and values near the ends of bf16's range in the cache and in q, against the
+oracle on the same bits.  Attention is a weighted mean: a key whose score is -inf has no weight, a NaN
+that a row sees makes the row NaN, an infinite value makes its dimension infinite."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import efim_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+HQ, HKV = 8, 2
+# new tokens at 4 query heads per kv head: 32-row CTAs, one query tile, two query tiles
+SHAPES = [5, 20, 60]
+
+
+class _Rows:
+    """One sequence per entry of `cached` (`new` tokens each) over pages in order; pools and q are device tensors to be
+    edited before a call."""
+
+    def __init__(self, cached, new, D=128, seed=0):
+        import paper_2505_21889_b200 as efim
+        self.efim = efim
+        self.cached, self.new, self.D = np.array(cached, np.int32), np.full(len(cached), new, np.int32), D
+        need = -(-(self.cached + self.new) // 16)
+        g = torch.Generator(device="cuda")
+        g.manual_seed(seed)
+        shape = (int(need.sum()), HKV, 16, D)
+        self.k = torch.randn(shape, generator=g, device="cuda").bfloat16()
+        self.v = torch.randn(shape, generator=g, device="cuda").bfloat16()
+        self.q = torch.randn((int(self.new.sum()), HQ, D), generator=g, device="cuda").bfloat16()
+        first = np.concatenate([[0], np.cumsum(need)])
+        self.table = np.zeros((len(cached), int(need.max())), np.int32)
+        for s in range(len(cached)):
+            self.table[s, :need[s]] = np.arange(first[s], first[s + 1])
+        self.status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def _call(self, fn):
+        out = torch.full_like(self.q, 7.0)
+        lse = torch.full(self.q.shape[:2], 7.0, dtype=torch.float32, device="cuda")
+        fn(out, lse)
+        torch.cuda.synchronize()
+        assert int(self.status.item()) == 0
+        return out.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64)
+
+    def prefill(self):
+        efim = self.efim
+        cache, batch = efim.Cache(self.k, self.v, HQ), efim.Batch(self.cached, self.new, self.table)
+        ws = torch.empty(max(efim.efim_prefill_workspace_bytes(cache, batch), 256), dtype=torch.uint8, device="cuda")
+        return self._call(lambda out, lse: efim.efim_append_prefill_attn(cache, batch, self.q, out, lse, 0.0, ws,
+                                                                         self.status))
+
+    def _bits(self):
+        from tests.gpu_harness import torch_to_bits
+        return torch_to_bits(self.q), torch_to_bits(self.k), torch_to_bits(self.v)
+
+    def prefill_oracle(self):
+        q, k, v = self._bits()
+        with np.errstate(all="ignore"):
+            return orc.append_prefill_attention(q, k, v, self.table, self.cached, self.new, HQ)
+
+
+@pytest.mark.parametrize("new", SHAPES)
+@pytest.mark.parametrize("cached", [300, 6000])                # 6000: the key range is cut, partials are merged
+def test_prefill_first_keys_of_infinitely_low_score(cached, new):
+    """The keys of a row's first steps have the score -inf: they have no weight, and the reference comes
+    from the first finite score."""
+    r = _Rows([cached], new)
+    r.q[:, :, 0] = 1.0
+    r.k[:10] = 0.0                                             # 160 keys: two steps
+    r.k[:10, :, :, 0] = -torch.inf
+    out, lse = r.prefill()
+    o, want = r.prefill_oracle()
+    assert np.abs(out - o).max() <= 2e-2 and np.abs(lse - want).max() <= 1e-3
