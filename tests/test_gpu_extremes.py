@@ -72,3 +72,35 @@ def test_prefill_first_keys_of_infinitely_low_score(cached, new):
     out, lse = r.prefill()
     o, want = r.prefill_oracle()
     assert np.abs(out - o).max() <= 2e-2 and np.abs(lse - want).max() <= 1e-3
+
+
+@pytest.mark.parametrize("new", SHAPES)
+@pytest.mark.parametrize("cached", [300, 6000])
+def test_prefill_values_near_the_end_of_the_range(cached, new):
+    """Peaked rows over values of up to 1e36: the weighted mean of finite values is finite.  Bound: output and
+    probabilities are rounded to bf16 (2^-9 each), so the 2-norm error stays below 2 * 2^-9."""
+    r = _Rows([cached], new)
+    r.k *= 8.0
+    r.v = (r.v.float() * 2e35).bfloat16()
+    out, lse = r.prefill()
+    o, want = r.prefill_oracle()
+    assert np.isfinite(out).all()
+    assert np.linalg.norm((out - o) / 2e35) <= 2.0 ** -8 * np.linalg.norm(o / 2e35)
+    assert np.abs(lse - want).max() <= 1e-3
+
+
+@pytest.mark.parametrize("new", SHAPES)
+def test_prefill_key_far_above_the_others_is_returned_exactly(new):
+    """A key 2^30 times as heavy as any other, behind the row's first steps: its probability is 1 without
+    rounding, so the output is its value bit for bit (the others move it by 700 * 2^-30).  Against the
+    others it is 2^30.0054 = 2^30 * 1.00378, halfway between two bf16 values: rounded there, most
+    outputs would move to the neighbouring value."""
+    r = _Rows([700], new)
+    r.k.zero_()
+    r.q[:, :, 0] = 1.0
+    r.q[:, :, 1] = 1.0
+    r.k[31, :, 4, 0] = 235.0                                   # position 500; (235 + 0.3046875) log2(e) / sqrt(128)
+    r.k[31, :, 4, 1] = 0.3046875
+    out, _ = r.prefill()
+    v = r.v[31, :, 4].float().cpu().numpy()
+    assert np.array_equal(out, np.broadcast_to(np.repeat(v, HQ // HKV, axis=0), out.shape))
