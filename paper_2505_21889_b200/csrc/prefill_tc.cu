@@ -228,11 +228,24 @@ enum {
 // key far above the ones before it has the probability 1, which bf16 holds exactly: with 2^40 here the
 // outputs of peaked rows (scores of 8 sigma) were off by 2.0e-3 to 2.25e-3 (2-norm) instead of 1.7e-3.
 constexpr float SUM_LIMIT = 256.f;
+// The reference is the row's exact maximum over the first EXACT_STEPS steps of a stream, or over the first one
+// where two query tiles see more than EXACT_MAX_STEPS steps.  The key at the reference is weighted without
+// rounding and short rows live on their heaviest keys: with one step everywhere, 16 tokens over 240 at 4/4 x 64
+// were off by 2.10e-3 instead of 2.00e-3 (2-norm, scores of 1 sigma), 60 over 1,000 at 32/8 by 2.293e-3 instead
+// of 2.252e-3.  It costs a rescale of O (16 prompts of 1-3.5k tokens 1021 -> 1034 us; in every row block 1054); in long
+// rows the heaviest key is hardly ever among the first 160.
+constexpr int EXACT_STEPS = 2, EXACT_MAX_STEPS = 12;
 
-// A row's reference after its first step with largest score `mx`.  Finite also where the row saw no key
-// or infinitely low scores only: those keys' probabilities are 0 against it, and the first finite score
-// to come overflows the sum, so that the reference moves up to it.
-__device__ __forceinline__ float first_reference(float mx) { return fmaxf(mx, -FLT_MAX); }
+// Moves a row's reference `m_ref` up to the score `mx`; returns the factor that O and the row's sum take on.
+// A reference starts at -FLT_MAX and stays finite where the row has seen no key or infinitely low scores
+// only: those keys' probabilities are 0 against it, and the first finite score to come is above it or
+// overflows its step's sum.
+__device__ __forceinline__ float move_reference(float& m_ref, float mx) {
+  const float m_new = fmaxf(m_ref, mx);
+  const float alpha = m_new == m_ref ? 1.f : ex2(m_ref - m_new);
+  m_ref = m_new;
+  return alpha;
+}
 
 // Epilogue of the 32-row shape: the eight (max, sum, O) states of query row `lane`, left in
 // shared memory as [state][row][XROW], are merged; this thread finishes D/8 dims of the row
@@ -525,7 +538,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       for (int c = 0; c < BN / 2; c += 8) tmem_st<8>(p_addr + c, z);
       tmem_wait_st();
     }
-    float m_ref = -INFINITY, l_sum = 0.f;
+    float m_ref = -FLT_MAX, l_sum = 0.f;
     for (int k = 0; k < my_cnt; ++k) {
       mbar_wait(bar(BAR_S + st), k & 1, abort_flag, p.status, p.wait_ns);
       tc_fence_after();
@@ -540,19 +553,19 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         for (int c = 0; c < KQ; ++c)
           if (kv0 + c >= vis) s[c] = 0xff800000u;           // -inf
       }
-      if (k == 0) m_ref = first_reference(row_max<KQ>(s) * p.scale_log2);
+      float alpha = 1.f;                                    // what O and the sum so far are scaled by
+      if (k < EXACT_STEPS) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
       uint32_t v[KQ / 2];
       float sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
       if (k > 0) {
         mbar_wait(bar(BAR_PV + st), (k - 1) & 1, abort_flag, p.status, p.wait_ns);   // P of the step before is consumed
         tc_fence_after();
-        if (__any_sync(0xffffffffu, !(sum <= SUM_LIMIT))) {
-          const float m_new = sum <= SUM_LIMIT ? m_ref : fmaxf(m_ref, row_max<KQ>(s) * p.scale_log2);
-          const float alpha = m_new == m_ref ? 1.f : ex2(m_ref - m_new);
-          m_ref = m_new;
+        const bool redo = !(sum <= SUM_LIMIT);
+        if (__any_sync(0xffffffffu, redo || alpha != 1.f)) {
+          if (redo) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
           l_sum *= alpha;
           rescale_o_row<D>(o_addr, alpha);
-          sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
+          if (__any_sync(0xffffffffu, redo)) sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
         }
       }
       tmem_st<KQ / 2>(p_addr + KQ / 2 * w, v);
@@ -614,7 +627,8 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     const uint32_t s_addr = tmem_S + lane_addr + st * L::SP_COLS;
     const uint32_t p_addr = tmem_P + lane_addr + st * L::SP_COLS;
     const uint32_t o_addr = tmem_O + lane_addr + st * D;
-    float m_ref = -INFINITY, l_sum = 0.f;
+    const int exact = !dual || nt <= EXACT_MAX_STEPS ? EXACT_STEPS : 1;
+    float m_ref = -FLT_MAX, l_sum = 0.f;
     for (int k = 0; k < my_cnt; ++k) {
       mbar_wait(bar(BAR_S + st), k & 1, abort_flag, p.status, p.wait_ns);
       tc_fence_after();
@@ -635,34 +649,36 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         for (int c = 0; c < BN; ++c)
           if (kv0 + c >= vis) s[c] = 0xff800000u;           // -inf
       }
-      // The first step's exact maximum is the row's reference; later steps only check that their sum
-      // stays in range (SUM_LIMIT), so a step has no row maximum to take before its first exponential.
+      // The first steps' exact maximum is the row's reference; later steps only check that their sum stays
+      // in range (SUM_LIMIT), so they have no row maximum to take before their first exponential.
       auto freed = [&]() {
         tmem_wait_ld<BN - LA>(s + LA);
         tc_fence_before();
         warp_arrive(bar(BAR_SFREE + st), lane);             // the next step's scores may be computed
       };
-      if (edge || k == 0) freed();
-      if (k == 0) m_ref = first_reference(row_max<BN>(s) * p.scale_log2);
+      if (edge || k < exact) freed();
+      float alpha = 1.f;                                    // what O and the sum so far are scaled by
+      if (k < exact) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
       uint32_t w[BN / 2];                                   // P as bf16 pairs
       const float neg_m = -m_ref;
       float sum = row_exp<LA>(s, p.scale_log2, neg_m, w);
-      if (!(edge || k == 0)) freed();
+      if (!(edge || k < exact)) freed();
       sum += row_exp<BN - LA>(s + LA, p.scale_log2, neg_m, w + LA / 2);
       if (k > 0) {
         mbar_wait(bar(BAR_PV + st), (k - 1) & 1, abort_flag, p.status, p.wait_ns);   // P of the step before is consumed
         tc_fence_after();
       }
       tmem_st<BN / 2>(p_addr, w);
-      if (__any_sync(0xffffffffu, !(sum <= SUM_LIMIT)) && k > 0) {
+      const bool redo = !(sum <= SUM_LIMIT);
+      if (__any_sync(0xffffffffu, redo || alpha != 1.f) && k > 0) {
         // (O is quiet: PV(k-1) has finished and PV(k) waits for this warp)
-        const float m_new = sum <= SUM_LIMIT ? m_ref : fmaxf(m_ref, row_max<BN>(s) * p.scale_log2);
-        const float alpha = m_new == m_ref ? 1.f : ex2(m_ref - m_new);
-        m_ref = m_new;
+        if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
         l_sum *= alpha;
         rescale_o_row<D>(o_addr, alpha);
-        sum = row_exp<BN>(s, p.scale_log2, -m_ref, w);
-        tmem_st<BN / 2>(p_addr, w);
+        if (__any_sync(0xffffffffu, redo)) {
+          sum = row_exp<BN>(s, p.scale_log2, -m_ref, w);
+          tmem_st<BN / 2>(p_addr, w);
+        }
       }
       tmem_wait_st();
       tc_fence_before();

@@ -104,3 +104,21 @@ def test_prefill_key_far_above_the_others_is_returned_exactly(new):
     out, _ = r.prefill()
     v = r.v[31, :, 4].float().cpu().numpy()
     assert np.array_equal(out, np.broadcast_to(np.repeat(v, HQ // HKV, axis=0), out.shape))
+
+
+@pytest.mark.parametrize("new,pos", [(5, 200), (20, 200), (60, 100)])
+def test_prefill_heaviest_key_in_the_second_step_is_weighted_without_rounding(new, pos):
+    """A key 2^7.0055 = 128 * 1.0038 times as heavy as each of the others, in the second step of its stream, and
+    values of zero everywhere else: the output is its value times its exact weight.  Rounded to bf16 against
+    the first step's reference the weight would be off by 0.0038 and nearly every output with it."""
+    from oracle.efim_oracle import bf16_to_f64, f64_to_bf16
+    r = _Rows([300], new)
+    r.k.zero_()
+    r.v[:, :, :, :] = torch.where(torch.arange(16, device="cuda")[None, None, :, None] == pos % 16, r.v, 0)
+    r.v[:pos // 16], r.v[pos // 16 + 1:] = 0.0, 0.0
+    r.q[:, :, :2] = 1.0
+    r.k[pos // 16, :, pos % 16, 0] = 54.75                     # (54.75 + 0.1875) log2(e) / sqrt(128)
+    r.k[pos // 16, :, pos % 16, 1] = 0.1875
+    out, _ = r.prefill()
+    o, _ = r.prefill_oracle()
+    assert (out == bf16_to_f64(f64_to_bf16(o))).mean() >= 0.99
