@@ -677,6 +677,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         rescale_o_row<D>(o_addr, alpha);
         if (__any_sync(0xffffffffu, redo)) {
           sum = row_exp<BN>(s, p.scale_log2, -m_ref, w);
+          tmem_wait_st();                                   // two stores to the same columns are not ordered by themselves
           tmem_st<BN / 2>(p_addr, w);
         }
       }
