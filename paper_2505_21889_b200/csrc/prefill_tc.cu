@@ -232,7 +232,7 @@ constexpr float SUM_LIMIT = 256.f;
 // where two query tiles see more than EXACT_MAX_STEPS steps.  The key at the reference is weighted without
 // rounding and short rows live on their heaviest keys: with one step everywhere, 16 tokens over 240 at 4/4 x 64
 // were off by 2.10e-3 instead of 2.00e-3 (2-norm, scores of 1 sigma), 60 over 1,000 at 32/8 by 2.293e-3 instead
-// of 2.252e-3.  It costs a rescale of O (16 prompts of 1-3.5k tokens 1021 -> 1034 us; in every row block 1054); in long
+// of 2.252e-3.  It costs a rescale of O (16 prompts of 1-3.5k tokens 1009 -> 1015 us; in every row block 3 %); in long
 // rows the heaviest key is hardly ever among the first 160.
 constexpr int EXACT_STEPS = 2, EXACT_MAX_STEPS = 12;
 
@@ -657,8 +657,13 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         warp_arrive(bar(BAR_SFREE + st), lane);             // the next step's scores may be computed
       };
       if (edge || k < exact) freed();
-      float alpha = 1.f;                                    // what O and the sum so far are scaled by
-      if (k < exact) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
+      // alpha: what O and the sum so far are scaled by.  A moved reference lowers the limit, so that the one
+      // test below finds it (a second condition there: 8 x 128 tokens over 8k 150.0 -> 152.6 us).
+      float alpha = 1.f, limit = SUM_LIMIT;
+      if (k < exact) {
+        alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
+        if (alpha != 1.f) limit = -1.f;
+      }
       uint32_t w[BN / 2];                                   // P as bf16 pairs
       const float neg_m = -m_ref;
       float sum = row_exp<LA>(s, p.scale_log2, neg_m, w);
@@ -669,9 +674,9 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
         tc_fence_after();
       }
       tmem_st<BN / 2>(p_addr, w);
-      const bool redo = !(sum <= SUM_LIMIT);
-      if (__any_sync(0xffffffffu, redo || alpha != 1.f) && k > 0) {
+      if (__any_sync(0xffffffffu, !(sum <= limit)) && k > 0) {
         // (O is quiet: PV(k-1) has finished and PV(k) waits for this warp)
+        const bool redo = !(sum <= SUM_LIMIT);
         if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
         l_sum *= alpha;
         rescale_o_row<D>(o_addr, alpha);
