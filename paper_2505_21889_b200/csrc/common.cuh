@@ -95,6 +95,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return r;
 }
 
+// maximum that is NaN if either operand is (fmaxf drops a NaN)
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // packed pairs of fp32 (one 64-bit register): two FMAs / multiplies per instruction
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   uint64_t r;

@@ -267,7 +267,7 @@ __device__ __noinline__ void tiny_merge_store(uint16_t* out, float* lse, float* 
   for (int q = 0; q < 8; ++q) {
     const float* row = xb + (size_t)(q * 32 + lane) * L::XROW;
     const float lq = row[D + 1];
-    const float wq = lq > 0.f ? ex2(row[D] - M) : 0.f;
+    const float wq = lq == 0.f ? 0.f : ex2(row[D] - M);
     Lt = fmaf(lq, wq, Lt);
 #pragma unroll
     for (int d = 0; d < DS; d += 4) {
@@ -278,8 +278,8 @@ __device__ __noinline__ void tiny_merge_store(uint16_t* out, float* lse, float* 
       acc[d + 3] = fmaf(x.w, wq, acc[d + 3]);
     }
   }
-  const float inv = Lt > 0.f ? 1.f / Lt : 0.f;
-  const float lse2 = Lt > 0.f ? M + log2f(Lt) : -INFINITY;
+  const float inv = Lt == 0.f ? 0.f : 1.f / Lt;
+  const float lse2 = Lt == 0.f ? -INFINITY : M + log2f(Lt);
   if (!valid) return;
   if (chunk < 0) {
     uint4* dst = reinterpret_cast<uint4*>(out + row_off + sidx * DS);
@@ -582,7 +582,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     float* xb = reinterpret_cast<float*>(smem_gen + L::KV_OFF);         // [8 states][32 rows][XROW]
     const int sidx = st * 4 + w;
     float* mine = xb + (size_t)(sidx * 32 + lane) * L::XROW;
-    const bool have = my_cnt > 0 && l_sum > 0.f;
+    const bool have = my_cnt > 0 && !(l_sum == 0.f);         // (a sum of NaN is handed on, not dropped)
     if (lane < 32) {
       mine[D] = have ? m_ref : -INFINITY;
       mine[D + 1] = have ? l_sum : 0.f;
@@ -719,13 +719,13 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       if (merge) {
         const float m1 = xbuf[D], l1 = xbuf[D + 1];
         const float M = fmaxf(m_ref, m1);
-        w0 = l_sum > 0.f ? ex2(m_ref - M) : 0.f;
-        w1 = l1 > 0.f ? ex2(m1 - M) : 0.f;
+        w0 = l_sum == 0.f ? 0.f : ex2(m_ref - M);
+        w1 = l1 == 0.f ? 0.f : ex2(m1 - M);
         l_sum = l_sum * w0 + l1 * w1;
         m_ref = M;
       }
-      const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
-      const float lse2 = l_sum > 0.f ? m_ref + log2f(l_sum) : -INFINITY;
+      const float inv = l_sum == 0.f ? 0.f : 1.f / l_sum;
+      const float lse2 = l_sum == 0.f ? -INFINITY : m_ref + log2f(l_sum);
       const float a0 = w0 * inv, a1 = w1 * inv;
       const int th = valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1;
       // The rows leave through the query tile's space (its MMAs are done; a warp uses its own 32 rows
@@ -1058,11 +1058,11 @@ __global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p, cons
   const float mine = lane < nc ? pl[lane] : -INFINITY;      // at most 16 chunks
   float M = mine;
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
+  for (int d = 16; d > 0; d >>= 1) M = max_nan(M, __shfl_xor_sync(0xffffffffu, M, d));   // a NaN chunk makes the row NaN
   float Lsum = 0.f, acc[EPL];
 #pragma unroll
   for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-  if (M > -INFINITY) {
+  if (!(M == -INFINITY)) {
     const float w_mine = exp2f(mine - M);                   // 0 beyond the last chunk
     for (int c0 = 0; c0 < nc; c0 += 4) {
       __align__(16) float v[4][EPL];
@@ -1084,14 +1084,14 @@ __global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p, cons
       }
     }
   }
-  const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
+  const float inv = Lsum == 0.f ? 0.f : 1.f / Lsum;
   uint16_t* out = p.out + th * D + lane * EPL;
   if constexpr (EPL == 4) {
     *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
   } else {
     *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
   }
-  if (p.lse && lane == 0) p.lse[th] = Lsum > 0.f ? (M + log2f(Lsum)) * 0.6931471805599453f : -INFINITY;
+  if (p.lse && lane == 0) p.lse[th] = Lsum == 0.f ? -INFINITY : (M + log2f(Lsum)) * 0.6931471805599453f;
 }
 
 // ------------------------------------------------------------------ host side

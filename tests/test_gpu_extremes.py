@@ -122,3 +122,28 @@ def test_prefill_heaviest_key_in_the_second_step_is_weighted_without_rounding(ne
     out, _ = r.prefill()
     o, _ = r.prefill_oracle()
     assert (out == bf16_to_f64(f64_to_bf16(o))).mean() >= 0.99
+
+
+def _same_or_nan(out, lse, o, want):
+    """Equal within the attention tolerances, and NaN exactly where the oracle has NaN."""
+    assert np.array_equal(np.isnan(out), np.isnan(o)) and np.array_equal(np.isnan(lse), np.isnan(want))
+    ok, lok = ~np.isnan(o), ~np.isnan(want)
+    assert ok.any() and not ok.all()
+    assert np.abs(out[ok] - o[ok]).max() <= 2e-2 and np.abs(lse[lok] - want[lok]).max() <= 1e-3
+
+
+@pytest.mark.parametrize("new", SHAPES)
+@pytest.mark.parametrize("cached", [300, 6000])
+@pytest.mark.parametrize("where", ["q", "k", "many_k"])
+def test_prefill_nan_scores_make_their_rows_nan(where, cached, new):
+    """A NaN in a query row, in one cached key or in all keys of a stretch longer than any chunk: the rows
+    that see it are NaN, out and lse, and no key is silently left out; all others are untouched."""
+    r = _Rows([cached], new)
+    if where == "q":
+        r.q[1, 1, 3] = torch.nan
+    elif where == "k":
+        r.k[2, 0, 5, 7] = torch.nan                            # position 37, kv head 0
+    else:
+        r.k[:cached // 16 - 1, 0] = torch.nan
+    out, lse = r.prefill()
+    _same_or_nan(out, lse, *r.prefill_oracle())
