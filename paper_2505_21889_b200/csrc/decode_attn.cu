@@ -23,6 +23,7 @@
 #include "mbar.cuh"
 #include "prefill_tc.cuh"
 #include <algorithm>
+#include <cfloat>
 #include <atomic>
 
 namespace efim {
@@ -261,11 +262,13 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
     for (int k = 0; k < KS; ++k)
 #pragma unroll
       for (int e = 0; e < 4; ++e) o[n][k][e] = 0.f;
-  float m_ref[NT][2], l_part[NT][2];    // of heads 8 n + 2 tq + {0, 1}; the sum over this lane's tokens
+  // of heads 8 n + 2 tq + {0, 1}; the sum over this lane's tokens.  The reference is finite from the start:
+  // a key whose score is -inf then has the probability 0, also before any other key was seen.
+  float m_ref[NT][2], l_part[NT][2];
 #pragma unroll
   for (int n = 0; n < NT; ++n)
 #pragma unroll
-    for (int e = 0; e < 2; ++e) { m_ref[n][e] = -INFINITY; l_part[n][e] = 0.f; }
+    for (int e = 0; e < 2; ++e) { m_ref[n][e] = -FLT_MAX; l_part[n][e] = 0.f; }
 
   // ldmatrix row addresses of this lane inside a staged page: K (tokens along m), V (dims along m)
   const uint32_t k_lane = (uint32_t)(((lane >> 3) & 1) * (D * 16) + (lane & 7) * 128 + (((lane >> 4) ^ (lane & 7)) << 4));
@@ -363,7 +366,7 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
 #pragma unroll
             for (int off = 4; off < 32; off <<= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, off));
             const float m_new = fmaxf(m_ref[n][e], x);
-            const float alpha = m_new == -INFINITY ? 1.f : dec_ex2(m_ref[n][e] - m_new);
+            const float alpha = dec_ex2(m_ref[n][e] - m_new);
             m_ref[n][e] = m_new;
             l_part[n][e] *= alpha;
 #pragma unroll
@@ -444,19 +447,17 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
     for (int w = 1; w < DEC_WARPS; ++w) M = fmaxf(M, s_m[w][g]);
     float L = 0.f;
     float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (M > -INFINITY) {                                    // else every page of the chunk was rejected: 0, -inf
 #pragma unroll
-      for (int w = 0; w < DEC_WARPS; ++w) {
-        const float sc = exp2f(s_m[w][g] - M);
-        const float4 x = *reinterpret_cast<const float4*>(xo + (w * GP + g) * XD + d);
-        L = fmaf(s_l[w][g], sc, L);
-        O.x = fmaf(x.x, sc, O.x);
-        O.y = fmaf(x.y, sc, O.y);
-        O.z = fmaf(x.z, sc, O.z);
-        O.w = fmaf(x.w, sc, O.w);
-      }
+    for (int w = 0; w < DEC_WARPS; ++w) {
+      const float sc = exp2f(s_m[w][g] - M);
+      const float4 x = *reinterpret_cast<const float4*>(xo + (w * GP + g) * XD + d);
+      L = fmaf(s_l[w][g], sc, L);
+      O.x = fmaf(x.x, sc, O.x);
+      O.y = fmaf(x.y, sc, O.y);
+      O.z = fmaf(x.z, sc, O.z);
+      O.w = fmaf(x.w, sc, O.w);
     }
-    const float inv = L > 0.f ? 1.f / L : 0.f;
+    const float inv = L > 0.f ? 1.f / L : 0.f;              // no key of weight, or every page rejected: 0, -inf
     const float lse2 = L > 0.f ? M + log2f(L) : -INFINITY;
     const size_t row_head = (size_t)r * p.Hq + head0 + g;
     if (p.n_chunks == 1) {

@@ -50,6 +50,16 @@ class _Rows:
         return self._call(lambda out, lse: efim.efim_append_prefill_attn(cache, batch, self.q, out, lse, 0.0, ws,
                                                                          self.status))
 
+    def decode(self):
+        """One query row per sequence (new = 1) over all its keys."""
+        efim = self.efim
+        cache, total = efim.Cache(self.k, self.v, HQ), self.cached + self.new
+        ws = torch.empty(max(efim.efim_decode_workspace_bytes(cache, len(total), int(total.max())), 256),
+                         dtype=torch.uint8, device="cuda")
+        ctx, table = torch.from_numpy(total).cuda(), torch.from_numpy(self.table).cuda()
+        return self._call(lambda out, lse: efim.efim_decode_attn(cache, len(total), ctx, int(total.max()), table, self.q,
+                                                                 out, lse, 0.0, ws, self.status))
+
     def _bits(self):
         from tests.gpu_harness import torch_to_bits
         return torch_to_bits(self.q), torch_to_bits(self.k), torch_to_bits(self.v)
@@ -58,6 +68,11 @@ class _Rows:
         q, k, v = self._bits()
         with np.errstate(all="ignore"):
             return orc.append_prefill_attention(q, k, v, self.table, self.cached, self.new, HQ)
+
+    def decode_oracle(self):
+        q, k, v = self._bits()
+        with np.errstate(all="ignore"):
+            return orc.decode_attention(q, k, v, self.table, self.cached + self.new, HQ)
 
 
 @pytest.mark.parametrize("new", SHAPES)
@@ -147,3 +162,17 @@ def test_prefill_nan_scores_make_their_rows_nan(where, cached, new):
         r.k[:cached // 16 - 1, 0] = torch.nan
     out, lse = r.prefill()
     _same_or_nan(out, lse, *r.prefill_oracle())
+
+
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("total", [200, 1500])                 # 1500: several chunks, merged
+def test_decode_keys_of_infinitely_low_score(total, D):
+    """The first 160 keys (whole pages of three or four warps) and single later ones have the score -inf: no weight."""
+    r = _Rows([total - 1], 1, D=D)
+    r.q[:, :, 0] = 1.0
+    for key in list(range(160)) + [170, total - 1]:
+        r.k[key // 16, :, key % 16] = 0.0
+        r.k[key // 16, :, key % 16, 0] = -torch.inf
+    out, lse = r.decode()
+    o, want = r.decode_oracle()
+    assert np.abs(out - o).max() <= 2e-2 and np.abs(lse - want).max() <= 1e-3
