@@ -457,8 +457,8 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
       O.z = fmaf(x.z, sc, O.z);
       O.w = fmaf(x.w, sc, O.w);
     }
-    const float inv = L > 0.f ? 1.f / L : 0.f;              // no key of weight, or every page rejected: 0, -inf
-    const float lse2 = L > 0.f ? M + log2f(L) : -INFINITY;
+    const float inv = L == 0.f ? 0.f : 1.f / L;             // no key of weight, or every page rejected: 0, -inf
+    const float lse2 = L == 0.f ? -INFINITY : M + log2f(L); // (a sum of NaN stays NaN)
     const size_t row_head = (size_t)r * p.Hq + head0 + g;
     if (p.n_chunks == 1) {
       *reinterpret_cast<uint2*>(p.out + row_head * D + d) =
@@ -522,10 +522,10 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p)
   fetch(4 * part);
   float M = -INFINITY;
   for (int c0 = 0; c0 < nc; c0 += 32)
-    if (c0 + lane < nc) M = fmaxf(M, pl[c0 + lane]);
+    if (c0 + lane < nc) M = max_nan(M, pl[c0 + lane]);          // a NaN chunk makes the row NaN
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
-  if (M > -INFINITY) {                             // else a row without keys, or every chunk came back empty
+  for (int d = 16; d > 0; d >>= 1) M = max_nan(M, __shfl_xor_sync(0xffffffffu, M, d));
+  if (!(M == -INFINITY)) {                         // else a row without keys, or every chunk came back empty
     for (int c0 = 4 * part; c0 < nc; c0 += 4 * WPR) {
       if (c0 != 4 * part) fetch(c0);
 #pragma unroll
@@ -552,14 +552,14 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p)
       for (int e = 0; e < EPL; ++e) acc[e] += s_acc[w][lane * EPL + e];
     }
   }
-  const float inv = L > 0.f ? 1.f / L : 0.f;
+  const float inv = L == 0.f ? 0.f : 1.f / L;
   uint16_t* out = p.out + row_head * D + lane * EPL;
   if constexpr (EPL == 4) {
     *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
   } else {
     *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
   }
-  if (p.lse && lane == 0) p.lse[row_head] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
+  if (p.lse && lane == 0) p.lse[row_head] = L == 0.f ? -INFINITY : (M + log2f(L)) * 0.6931471805599453f;
 }
 
 DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len) {

@@ -176,3 +176,20 @@ def test_decode_keys_of_infinitely_low_score(total, D):
     out, lse = r.decode()
     o, want = r.decode_oracle()
     assert np.abs(out - o).max() <= 2e-2 and np.abs(lse - want).max() <= 1e-3
+
+
+@pytest.mark.parametrize("total", [200, 1500, 5000])           # one chunk; a few; more than eight (merge on four warps)
+@pytest.mark.parametrize("where", ["q", "k", "last_k", "many_k"])
+def test_decode_nan_scores_make_their_rows_nan(where, total):
+    """A NaN in a query row, in one key, in the last 256 keys (whole chunks) or in all but the first 16: the heads
+    that see it are NaN, out and lse; the other kv head and the other row are untouched."""
+    r = _Rows([total - 1, total // 2], 1)
+    if where == "q":
+        r.q[0, 1, 3] = torch.nan
+    elif where == "k":
+        r.k[2, 0, 5, 7] = torch.nan
+    else:
+        pages = -(-total // 16)                                # of the first row
+        r.k[pages - 16 if where == "last_k" and pages > 32 else 1:pages, 0] = torch.nan
+    out, lse = r.decode()
+    _same_or_nan(out, lse, *r.decode_oracle())
