@@ -115,6 +115,42 @@ __device__ __forceinline__ uint4 dec_rotate_vec(uint4 mine, uint4 other, const f
   return mine;
 }
 
+// Four dimensions of the weighted mean of keys [begin, end) of one (row, kv head) when some of their values
+// are infinite or NaN: every visible key has a positive weight, so a dimension is NaN if it holds a NaN or
+// infinities of both signs, else the infinity it holds.  (P enters the products as three terms, of which the
+// lower two may be 0 or negative, and 0 or a negative times infinity beside the first term's is NaN.)
+// `v_last`: the new token's values, where key `last` is one that may not be in its page yet, else null.
+// Out of line and rare: only threads whose sums came out as NaN under a sound row sum come here.
+__device__ __noinline__ float4 mean_of_unbounded(const uint16_t* v_pool, const int32_t* bt, int num_pages, int Hkv, int kvh,
+                                                 int D, int d, int begin, int end, const uint16_t* v_last, int last) {
+  uint32_t nan = 0, pos = 0, neg = 0;                        // a bit per dimension
+  for (int key = begin; key < end; ++key) {
+    const uint16_t* v;
+    if (v_last && key == last) {
+      v = v_last + d;
+    } else {
+      const int pid = *(bt + (key >> 4));
+      if (pid < 0 || pid >= num_pages) continue;             // rejected pages have no keys
+      v = v_pool + (((size_t)pid * Hkv + kvh) * 16 + (key & 15)) * D + d;
+    }
+    const uint2 w = *reinterpret_cast<const uint2*>(v);
+    const uint16_t u[4] = {(uint16_t)w.x, (uint16_t)(w.x >> 16), (uint16_t)w.y, (uint16_t)(w.y >> 16)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if ((u[i] & 0x7fff) > 0x7f80) nan |= 1u << i;
+      if (u[i] == 0x7f80) pos |= 1u << i;
+      if (u[i] == 0xff80) neg |= 1u << i;
+    }
+  }
+  float r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool p = pos >> i & 1, n = neg >> i & 1;
+    r[i] = (nan >> i & 1) || p == n ? NAN : (p ? INFINITY : -INFINITY);
+  }
+  return make_float4(r[0], r[1], r[2], r[3]);
+}
+
 // NT tiles of 8 query heads per CTA (heads beyond the group's are zero queries, dropped at the end).
 template <int D, int NT, bool FUSED>
 __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM)
@@ -459,6 +495,14 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
     }
     const float inv = L == 0.f ? 0.f : 1.f / L;             // no key of weight, or every page rejected: 0, -inf
     const float lse2 = L == 0.f ? -INFINITY : M + log2f(L); // (a sum of NaN stays NaN)
+    if (L > 0.f && (O.x != O.x || O.y != O.y || O.z != O.z || O.w != O.w)) {
+      const float4 x = mean_of_unbounded(p.v_pool, bt, p.num_pages, p.Hkv, kvh, D, d, begin, end,
+                                         FUSED && append ? p.v_new + ((size_t)r * p.Hkv + kvh) * D : nullptr, len - 1);
+      if (O.x != O.x) O.x = x.x;
+      if (O.y != O.y) O.y = x.y;
+      if (O.z != O.z) O.z = x.z;
+      if (O.w != O.w) O.w = x.w;
+    }
     const size_t row_head = (size_t)r * p.Hq + head0 + g;
     if (p.n_chunks == 1) {
       *reinterpret_cast<uint2*>(p.out + row_head * D + d) =
@@ -698,6 +742,7 @@ efim_status efim::decode_run(const efim_cache_desc* cache, int32_t batch, const 
   p.block_table = d_block_table;
   p.out = static_cast<uint16_t*>(d_out);
   p.lse = d_lse;
+  p.v_pool = static_cast<const uint16_t*>(cache->d_v_pool);
   p.part_lse = static_cast<float*>(d_workspace);
   p.part_o = need ? reinterpret_cast<float*>(static_cast<char*>(d_workspace) + pl.part_lse_bytes) : nullptr;
   p.status = d_status;

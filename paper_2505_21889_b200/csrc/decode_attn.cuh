@@ -8,6 +8,7 @@ struct DecodeParams {
   const uint16_t* q;          // [R][Hq][D] bf16
   const int32_t* row_len;     // [R] keys visible to row r: [0, row_len[r])
   const int32_t* block_table; // [R][max_pages_per_seq]
+  const uint16_t* v_pool;     // [pages][Hkv][16][D], read where values turn out not to be finite
   uint16_t* out;              // [R][Hq][D] bf16
   float* lse;                 // [R][Hq] natural log, or null
   float* part_o;              // [R][Hq][n_chunks][D]   (n_chunks > 1)

@@ -193,3 +193,39 @@ def test_decode_nan_scores_make_their_rows_nan(where, total):
         r.k[pages - 16 if where == "last_k" and pages > 32 else 1:pages, 0] = torch.nan
     out, lse = r.decode()
     _same_or_nan(out, lse, *r.decode_oracle())
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("total", [200, 1500, 5000])
+def test_decode_infinite_values(total, D, fused):
+    """Infinite values in the cache, and in the new token of a fused step: their dimensions are infinite, NaN where
+    both signs or a NaN meet, and every other dimension is what it was."""
+    r = _Rows([total - 1, total // 2], 1, D=D)
+    first = [0, 37, total // 2, total - 1]                     # keys of the first row
+    for n, key in enumerate(first):
+        r.v[key // 16, 0, key % 16, 5 + 8 * n] = torch.inf
+        r.v[key // 16, 1, key % 16, 6 + 8 * n] = -torch.inf
+    r.v[2, :, 5, 40], r.v[3, :, 7, 40] = torch.inf, -torch.inf # both signs
+    r.v[1, :, 3, 41] = torch.nan
+    if fused:
+        from paper_2505_21889_b200 import efim_decode_step, Cache, efim_decode_workspace_bytes
+        lens = r.cached + r.new
+        spot = [(int(r.table[s, (n - 1) // 16]), int(n - 1) % 16) for s, n in enumerate(lens)]
+        k_new = torch.stack([r.k[p, :, t] for p, t in spot])
+        v_new = torch.stack([r.v[p, :, t] for p, t in spot])
+        o, want = r.decode_oracle()
+        for p, t in spot:                                      # what is in the slot before is not looked at
+            r.k[p, :, t], r.v[p, :, t] = torch.nan, torch.nan
+        cache = Cache(r.k, r.v, HQ)
+        ws = torch.empty(max(efim_decode_workspace_bytes(cache, 2, total), 256), dtype=torch.uint8, device="cuda")
+        ctx, table = torch.from_numpy(lens).cuda(), torch.from_numpy(r.table).cuda()
+        out, lse = r._call(lambda out, lse: efim_decode_step(cache, 2, ctx, total, table, None, r.q, k_new, v_new, out, lse,
+                                                             0.0, ws, r.status))
+    else:
+        o, want = r.decode_oracle()
+        out, lse = r.decode()
+    assert np.array_equal(np.isnan(out), np.isnan(o)) and np.isnan(o).any()
+    assert np.array_equal(np.isposinf(out), np.isposinf(o)) and np.array_equal(np.isneginf(out), np.isneginf(o))
+    ok = np.isfinite(o)
+    assert np.abs(out[ok] - o[ok]).max() <= 2e-2 and np.abs(lse - want).max() <= 1e-3
