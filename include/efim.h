@@ -146,8 +146,9 @@ efim_status efim_kv_append(const efim_cache_desc* cache, const efim_batch_desc* 
  * sm_scale <= 0 selects 1/sqrt(head_dim).  Sequences with new_len 0 are skipped.
  * The host mirrors h_cached_len/h_new_len are read during the call to build the
  * work list, which is copied into the workspace on `stream`.
- * Workspace: at least efim_prefill_workspace_bytes() bytes, 256-byte aligned,
- * exclusively this call's until the stream has passed it.
+ * Workspace: at least efim_prefill_workspace_bytes() bytes for exactly these lengths (a smaller
+ * batch can need more: it may be cut into more key chunks), 256-byte aligned, exclusively this
+ * call's until the stream has passed it.
  */
 size_t efim_prefill_workspace_bytes(const efim_cache_desc* cache, const efim_batch_desc* batch);
 efim_status efim_append_prefill_attn(const efim_cache_desc* cache, const efim_batch_desc* batch,
@@ -216,6 +217,8 @@ efim_status efim_append_prefill_step(const efim_cache_desc* cache, const efim_ba
  * A device length beyond what the launch was planned for (the chunks cover max_ctx_len rounded
  * up to whole chunks, at most the block table's capacity) is clamped to that and sets
  * EFIM_DEV_BAD_POSITION; nothing outside the workspace or the table is touched.
+ * A workspace of efim_decode_workspace_bytes(batch, max_ctx_len) bytes also serves every call with fewer
+ * rows or a smaller max_ctx_len over a cache of the same heads and head_dim.
  */
 size_t efim_decode_workspace_bytes(const efim_cache_desc* cache, int32_t batch, int32_t max_ctx_len);
 /* Number of kernels the corresponding call enqueues for these arguments (the main

@@ -606,6 +606,10 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p)
   if (p.lse && lane == 0) p.lse[row_head] = L == 0.f ? -INFINITY : (M + log2f(L)) * 0.6931471805599453f;
 }
 
+// fp32 partials of `row_chunks` (row, chunk) pairs
+static size_t part_o_size(long long row_chunks, int Hq, int D) { return (size_t)row_chunks * Hq * D * sizeof(float); }
+static size_t part_lse_size(long long row_chunks, int Hq) { return ((size_t)row_chunks * Hq * sizeof(float) + 255) / 256 * 256; }
+
 DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len) {
   DecodePlan pl;
   const int G = Hq / Hkv;
@@ -621,23 +625,41 @@ DecodePlan plan_decode(int rows, int Hq, int Hkv, int D, int max_len) {
   // 32/8 heads in microseconds at 256 / 384 / 768 / 1024 / 2048 keys: 1 row x 2.3k keys 9.0 / 10.1 /
   // 13.1 / 15.4 / 25; 4 rows x 2-2.9k 15.8 / 15.6 / 16.5 / 17.5 / 27; 16 rows 35.3 / 35.2 / 33.7 /
   // 31.4 / 34.4; 64 rows x 4-32k - / 636 / 611 / 603 / 596.
+  // (decode_workspace_bound below follows these rules.)
   const long long slots = (long long)sm_count() * DEC_CTAS_PER_SM;
   const long long units = (long long)rows * Hkv * pl.gsplit;
   long long chunk = 2048;
   if (units * ((max_len + 2047) / 2048) < 4 * slots) {
     const long long n = std::max<long long>(1, slots / units);
     chunk = std::min<long long>(1024, std::max<long long>(256, (max_len + n - 1) / n));
-    // partials that the fixed array of efim_decode_attn_static holds, where longer chunks allow it
+    // Partials that the fixed array of efim_decode_attn_static holds, where longer chunks allow it: the two
+    // entry points give the same bits, and the array's one takes whatever fits with chunks of 2048 keys.
     const long long per_chunk = (long long)rows * Hq * (D + 1) * (long long)sizeof(float);
-    const long long n_fit = std::max<long long>(1, ((8 << 20) - 512) / per_chunk);
+    const long long n_fit = std::max<long long>(1, ((long long)DEC_STATIC_BYTES - 512) / per_chunk);
     if ((max_len + chunk - 1) / chunk > n_fit) chunk = std::min<long long>(2048, (max_len + n_fit - 1) / n_fit);
   }
   chunk = (chunk + 63) / 64 * 64;
   pl.chunk_tokens = (int)chunk;
   pl.n_chunks = (max_len + pl.chunk_tokens - 1) / pl.chunk_tokens;
-  pl.part_o_bytes = pl.n_chunks > 1 ? (size_t)rows * Hq * pl.n_chunks * D * sizeof(float) : 0;
-  pl.part_lse_bytes = pl.n_chunks > 1 ? ((size_t)rows * Hq * pl.n_chunks * sizeof(float) + 255) / 256 * 256 : 0;
+  pl.part_o_bytes = pl.n_chunks > 1 ? part_o_size((long long)rows * pl.n_chunks, Hq, D) : 0;
+  pl.part_lse_bytes = pl.n_chunks > 1 ? part_lse_size((long long)rows * pl.n_chunks, Hq) : 0;
   return pl;
+}
+
+// The most that a plan for at most `rows` rows of at most `max_len` keys needs.  The plans themselves are not
+// monotone (32/8 heads, 2,048 keys: 221 rows 7.3 MB, 256 rows none), and a serving loop that sizes its
+// workspace once has to get by as rows leave it.
+static size_t decode_workspace_bound(int rows, int Hq, int Hkv, int D, int max_len) {
+  if (max_len <= 256) return 0;                              // never cut
+  const DecodePlan pl = plan_decode(rows, Hq, Hkv, D, max_len);
+  const long long slots = (long long)sm_count() * DEC_CTAS_PER_SM, per_row = (long long)Hkv * pl.gsplit, r = rows;
+  auto chunks = [&](long long keys) { return (max_len + keys - 1) / keys; };
+  auto bytes = [&](long long row_chunks) { return part_o_size(row_chunks, Hq, D) + part_lse_size(row_chunks, Hq); };
+  // (row, chunk) pairs of less than several waves: one wave of 256 to 1024 keys each, or chunks of 1024 keys that
+  // are at most twice as many as the chunks of 2048 they replace - in either case what fits the static array
+  const long long one_wave = std::min(r * chunks(256), slots / per_row);
+  const long long of_1024 = std::min(r * chunks(1024), 2 * (4 * slots - 1) / per_row);
+  return std::max(std::min(bytes(std::max(one_wave, of_1024)), DEC_STATIC_BYTES), bytes(r * chunks(2048)));
 }
 
 // The kernel's shared-memory size has to be raised once per device.
@@ -699,9 +721,7 @@ static efim_status launch_decode(const efim_cache_desc* cache, const DecodeParam
 
 extern "C" size_t efim_decode_workspace_bytes(const efim_cache_desc* cache, int32_t batch, int32_t max_ctx_len) {
   if (efim::check_cache(cache) != EFIM_OK || batch <= 0) return 0;
-  const efim::DecodePlan pl = efim::plan_decode(batch, cache->num_q_heads, cache->num_kv_heads, cache->head_dim,
-                                                max_ctx_len);
-  return pl.part_o_bytes + pl.part_lse_bytes;
+  return efim::decode_workspace_bound(batch, cache->num_q_heads, cache->num_kv_heads, cache->head_dim, max_ctx_len);
 }
 
 extern "C" int32_t efim_decode_launch_count(const efim_cache_desc* cache, int32_t batch, int32_t max_ctx_len) {

@@ -4,6 +4,9 @@
 
 namespace efim {
 
+// bytes of the library's own array of partials (decode_static.cu)
+constexpr size_t DEC_STATIC_BYTES = 8u << 20;
+
 struct DecodeParams {
   const uint16_t* q;          // [R][Hq][D] bf16
   const int32_t* row_len;     // [R] keys visible to row r: [0, row_len[r])

@@ -13,7 +13,7 @@
 
 namespace {
 
-constexpr size_t kScratchBytes = 8u << 20;     // 8 MiB per GPU, held from library load to exit
+constexpr size_t kScratchBytes = efim::DEC_STATIC_BYTES;     // 8 MiB per GPU, held from library load to exit
 static __device__ __align__(256) unsigned char g_decode_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;

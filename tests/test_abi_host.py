@@ -157,6 +157,36 @@ def test_decode_planner_chunks():
     assert lib.efim_decode_workspace_bytes(ctypes.byref(cache), 4096, 200) == 0
 
 
+@pytest.mark.parametrize("Hq,Hkv,D", [(4, 4, 64), (32, 32, 128), (28, 4, 128), (32, 8, 128), (16, 1, 128), (64, 1, 128),
+                                      (40, 8, 128), (1, 1, 64)])
+def test_decode_workspace_also_serves_smaller_calls(Hq, Hkv, D):
+    """A workspace sized once for the largest batch and context is enough as rows leave and for shorter contexts,
+    although the chunk rule is not monotone; and what the static array takes is what the size query says."""
+    lib = efim.load_library()
+    cache = _cache_desc(D=D, Hq=Hq, Hkv=Hkv)
+    rng = np.random.default_rng([Hq, Hkv, D])
+    static = lib.efim_decode_static_scratch_bytes()
+    ref = ctypes.byref(cache)
+
+    def call(rows, ctx, workspace_bytes):
+        # a misaligned workspace is refused behind the size check: 4 if it is too small, else 1, and nothing is launched
+        return lib.efim_decode_attn(ref, rows, 0x1000, ctx, 0x1000, 1 << 14, 0x1000, 0x1000, None, 0.0, 0x1001,
+                                    int(workspace_bytes), None, None)
+    pairs = [(222, 221, 4096, 4096), (256, 221, 2048, 2048), (16, 16, 28672, 26624)]
+    for _ in range(3000):
+        big, ctx = int(2 ** rng.uniform(0, 10)), int(2 ** rng.uniform(4, 17))
+        pairs.append((big, int(rng.integers(1, big + 1)), ctx, int(rng.integers(1, ctx + 1))))
+    for big, rows, ctx, shorter in pairs:
+        size = lib.efim_decode_workspace_bytes(ref, big, ctx)
+        assert lib.efim_decode_workspace_bytes(ref, rows, shorter) <= size
+        for b, m in ((big, ctx), (rows, shorter)):
+            if lib.efim_decode_launch_count(ref, b, m) == 2:       # (else no workspace is asked for)
+                assert call(b, m, size) == 1
+                own = lib.efim_decode_workspace_bytes(ref, b, m)
+                assert (call(b, m, static) == 1) == (own <= static)
+                assert call(b, m, 256) == 4
+
+
 def test_prefill_plan_blob_sizes_and_errors():
     """efim_prefill_plan: the blob is a 256-byte head plus the work list and split sizes; a
     buffer that is too small is refused; a batch with nothing new still gets a valid (empty) plan."""
