@@ -10,8 +10,6 @@ from ctypes import c_int32, c_void_p, c_float, c_double, c_size_t, c_char_p, POI
 
 import numpy as np
 
-from torch import _C as _torch_c
-
 _LIB = None
 _HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -175,10 +173,21 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _current_stream():
+    """The raw handle of torch's current stream (building a Stream object costs 3 us more).  torch is looked up
+    on the first call: the host-only parts of the package work without it."""
+    global _current_stream
+    from torch import _C
+    raw_stream, device = _C._cuda_getCurrentRawStream, _C._cuda_getDevice
+
+    def _current_stream():
+        return raw_stream(device())
+    return _current_stream()
+
+
 def _stream_ptr(stream):
     if stream is None:
-        # the raw handle of torch's current stream (building a Stream object costs 3 us more)
-        return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -3,6 +3,8 @@ function include/efim.h declares, and rejects bad arguments before launching."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -50,6 +52,19 @@ def test_rope_table_matches_definition():
     assert abs(t[p, 4 + f] - np.sin(p * 10000.0 ** (-2 * f / 8))) < 1e-7
     with pytest.raises(efim.EfimError):
         efim.efim_rope_table_build(10000.0, 7, 4)
+
+
+def test_host_only_parts_do_not_need_torch(tmp_path):
+    """The front end and fragment tokenisation (also as a command) run where torch cannot be imported."""
+    (tmp_path / "text").write_text("def f():\n    return 1\n" * 20)
+    code = ("import sys; sys.modules['torch'] = None\n"
+            "import runpy, paper_2505_21889_b200 as efim\n"
+            "fe = efim.Frontend(1, 2, 3, 64)\n"
+            "assert fe.transform(7, [10, 11], [12])[0].tolist()\n"
+            f"sys.argv = ['fragment', {str(tmp_path / 'text')!r}, '--seed', '7']\n"
+            "runpy.run_module('paper_2505_21889_b200.fragment', run_name='__main__')\n")
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert res.returncode == 0 and res.stdout.startswith("{"), res.stderr
 
 
 def _cache_desc(D=128, P=16, Hq=8, Hkv=2, k=0x10000, v=0x20000):
