@@ -124,6 +124,42 @@ def test_bad_arguments_are_rejected_on_the_host():
     assert lib.efim_kv_append(ctypes.byref(ok), ctypes.byref(bd0), None, None, None, None, None, None) == 0
 
 
+def test_per_step_calls_take_addresses_of_what_holds_them_only():
+    """What may stand for memory in the per-step calls: tensors, integer addresses, numpy arrays and None; not numpy
+    scalars or other buffers, whose own storage would be taken for device memory.  The workspace is no
+    host array and the plan nothing but one.  (Empty batches: an accepted call returns and launches nothing.)"""
+    import torch
+    cache, empty = _cache_desc(), B._BatchDesc(0, 4, 0, None, None, None, None, None, None)
+    ca, ba = ctypes.addressof(cache), ctypes.addressof(empty)
+    t = torch.zeros(4)
+
+    def decode(q, workspace=None):
+        return B._calls.decode_attn(ca, 0, t, 16, t, 4, q, t, None, 0.0, workspace, None, 0)
+
+    def prefill(plan, workspace=None):
+        return B._calls.append_prefill_attn(ca, ba, t, t, None, 0.0, workspace, None, 0, plan, 0)
+
+    def step(plan, workspace=None):
+        return B._calls.append_prefill_step(ca, ba, None, t, t, t, t, None, 0.0, plan, 0, workspace, None, 0)
+    for q in (t, 0x1000, None, np.zeros(4), np.zeros((4, 4))[:, 1]):
+        assert decode(q) == 0
+        assert B._calls.kv_append(ca, ba, None, q, t, t, None, 0) == 0
+    for q in (np.int64(0x1000), np.array([0x1000], np.uint64)[0], b"0123456789abcdef", bytearray(16), memoryview(b"0123"), 1.0):
+        for call in (lambda: decode(q), lambda: B._calls.kv_append(ca, ba, None, q, t, t, None, 0)):
+            with pytest.raises((TypeError, AttributeError)):
+                call()
+    assert decode(t, t) == 0 and prefill(None) == 0 and step(None, t) == 0
+    for workspace in (np.zeros(256, np.uint8), 0x1000, b"0" * 256):
+        for call in (lambda: decode(t, workspace), lambda: prefill(None, workspace), lambda: step(None, workspace)):
+            with pytest.raises((TypeError, AttributeError)):
+                call()
+    assert prefill(np.zeros(256, np.uint8)) == 1 and step(np.zeros(256, np.uint8)) == 1      # read, and no plan
+    for plan in (t, 0x1000, b"0" * 256):
+        for call in (lambda: prefill(plan), lambda: step(plan)):
+            with pytest.raises((TypeError, AttributeError)):
+                call()
+
+
 def _batch_desc(cached, new, max_pages):
     c = np.asarray(cached, np.int32)
     n = np.asarray(new, np.int32)
