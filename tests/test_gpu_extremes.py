@@ -229,3 +229,27 @@ def test_decode_infinite_values(total, D, fused):
     assert np.array_equal(np.isposinf(out), np.isposinf(o)) and np.array_equal(np.isneginf(out), np.isneginf(o))
     ok = np.isfinite(o)
     assert np.abs(out[ok] - o[ok]).max() <= 2e-2 and np.abs(lse - want).max() <= 1e-3
+
+
+def test_decode_probabilities_keep_fp32_precision():
+    """46 keys of weight 1 and value 1 against 93 of weight p = 2^(-7.28125 log2(e) / sqrt(128)) = 0.5254 and value -w: the
+    mean cancels to 3e-8, so that the error of p is what is left.  Rounded to one bf16 term p is off by 2^-8.1, to
+    two by 2^-17.2.  Bound: the exponential and the two sums are good to 2^-21 of sums of weight 1."""
+    from oracle.efim_oracle import bf16_to_f64, f64_to_bf16
+    r = _Rows([138], 1)
+    r.k.zero_()
+    r.q[:, :, 0] = 1.0
+    w = 0.94140625
+    heavy = np.array([i % 3 == 0 and i < 138 for i in range(139)])
+    for i in range(139):
+        r.k[i // 16, :, i % 16, 0] = 0.0 if heavy[i] else -7.28125
+        r.v[i // 16, :, i % 16] = 1.0 if heavy[i] else -w
+    out, _ = r.decode()
+    o, _ = r.decode_oracle()
+    limit = 2.0 ** -21
+    assert np.abs(o).max() < 1e-7 and np.abs(out - o).max() <= limit
+    # the bound sees a p of one or two bf16 terms (planted here, in 64 bits)
+    p = np.exp(-7.28125 / np.sqrt(128.0))
+    high = bf16_to_f64(f64_to_bf16(p))
+    for terms in (high, high + bf16_to_f64(f64_to_bf16(p - high))):
+        assert abs((heavy.sum() - (~heavy).sum() * terms * w) / (heavy.sum() + (~heavy).sum() * p)) > 4 * limit

@@ -163,8 +163,8 @@ def test_decode_loop_small(name):
 @pytest.mark.parametrize("Hq,Hkv,D", [(5, 1, 128), (12, 2, 128), (7, 1, 64), (28, 4, 128), (8, 1, 128), (16, 1, 128),
                                         (20, 2, 64)])
 def test_decode_group_sizes_against_oracle(Hq, Hkv, D):
-    """Groups of 5 to 8 query heads per kv head run in one CTA (two passes over the page in
-    shared memory); larger groups are cut evenly.  Plain and fused steps against the oracle."""
+    """Groups of up to 16 query heads per kv head run in one CTA (8 of them, or 16, per page's matrix
+    instructions).  Plain and fused steps against the oracle."""
     H = _harness()
     import paper_2505_21889_b200 as efim
     ctx0 = [1, 15, 16, 17, 333, 1200, 2100]
@@ -229,8 +229,9 @@ def test_decode_head_tiles_and_page_edges(Hq, Hkv, D):
     assert int(dw.status.item()) == 0
     H.assert_attn_close(H.torch_to_bits(out), o, f"heads {Hq}/{Hkv} D={D}")
     H.assert_lse_close(lse_d.cpu().numpy(), lse, f"heads {Hq}/{Hkv} D={D}")
-    # mean: rounding to nearest bf16 is off by at most 2^-9 |o|, by half of it on average; probabilities
-    # of bf16 precision would add as much again
+    # mean: rounding to nearest bf16 is off by at most 2^-9 of the leading power of two, by about half of that on
+    # average; the rest covers rotated q and k (the precision of the probabilities has a test of its own,
+    # test_decode_probabilities_keep_fp32_precision)
     err = np.abs(bf16_bits_to_f32(H.torch_to_bits(out)).astype(np.float64) - o)
     assert err.mean() <= np.abs(o).mean() * 2.0 ** -9
 
