@@ -102,26 +102,6 @@ __device__ __forceinline__ float max_nan(float a, float b) {
   return r;
 }
 
-// packed pairs of fp32 (one 64-bit register): two FMAs / multiplies per instruction
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 // ---- rotary embedding, as every kernel of the library applies it: fp32 FMA from the bf16
 // inputs and the fp32 cos/sin table, one rounding to bf16.  (The same instruction sequence
 // everywhere, so a q or k rotated by one kernel equals the one rotated by another bit for bit.)

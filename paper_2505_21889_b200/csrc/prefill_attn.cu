@@ -116,7 +116,6 @@ efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch,
   p.out = static_cast<uint16_t*>(d_out);
   p.lse = d_lse;
   p.cached_len = batch->d_cached_len;
-  p.new_len = batch->d_new_len;
   p.q_indptr = batch->d_q_indptr;
   p.block_table = batch->d_block_table;
   p.items = reinterpret_cast<const pf::WorkItem*>(ws);

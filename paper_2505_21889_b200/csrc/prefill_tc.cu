@@ -170,13 +170,6 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor
-// version 1.  Offsets are in bytes and stored without their 4 low bits.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  const uint32_t lo = ((addr >> 4) & 0x3FFFu) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
-  const uint32_t hi = ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);
-  return (static_cast<uint64_t>(hi) << 32) | lo;
-}
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = n, A K-major, B K- or MN-major.
 __host__ __device__ constexpr uint32_t instr_desc(int n, int b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(b_mn_major) << 16) |
@@ -583,10 +576,8 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     const int sidx = st * 4 + w;
     float* mine = xb + (size_t)(sidx * 32 + lane) * L::XROW;
     const bool have = my_cnt > 0 && !(l_sum == 0.f);         // (a sum of NaN is handed on, not dropped)
-    if (lane < 32) {
-      mine[D] = have ? m_ref : -INFINITY;
-      mine[D + 1] = have ? l_sum : 0.f;
-    }
+    mine[D] = have ? m_ref : -INFINITY;
+    mine[D + 1] = have ? l_sum : 0.f;
 #pragma unroll
     for (int c0 = 0; c0 < D; c0 += 32) {
       uint32_t o[32];

@@ -45,7 +45,6 @@ struct Params {
   uint16_t* out;               // [T][Hq][D]
   float* lse;                  // [T][Hq] or null
   const int32_t* cached_len;
-  const int32_t* new_len;
   const int32_t* q_indptr;
   const int32_t* block_table;
   const WorkItem* items;
