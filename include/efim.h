@@ -145,7 +145,8 @@ efim_status efim_kv_append(const efim_cache_desc* cache, const efim_batch_desc* 
  * bf16 operands, fp32 accumulation and softmax, bf16 output.
  * sm_scale <= 0 selects 1/sqrt(head_dim).  Sequences with new_len 0 are skipped.
  * The host mirrors h_cached_len/h_new_len are read during the call to build the
- * work list, which is copied into the workspace on `stream`.
+ * work list, which the call leaves at the head of the workspace on `stream`: long lists are
+ * copied there, short ones travel in the launch parameters and the kernels write them out.
  * Workspace: at least efim_prefill_workspace_bytes() bytes for exactly these lengths (a smaller
  * batch can need more: it may be cut into more key chunks), 256-byte aligned, exclusively this
  * call's until the stream has passed it.
@@ -166,8 +167,9 @@ efim_status efim_append_prefill_attn(const efim_cache_desc* cache, const efim_ba
  * blob's lists are first copied to the head of the workspace on `stream`: keep the blob alive
  * and unchanged until the stream has passed the call (pinned memory makes the copy
  * asynchronous).  With lists_resident = 1 the call copies nothing and only launches: the head
- * of this workspace must still hold the lists from an earlier call with the same plan (the
- * kernels only read them; the partials live behind them) - upload once per batch, run per layer.
+ * of this workspace must still hold the lists from an earlier call with the same plan, or from a
+ * call that planned the same batch for itself (this call's kernels only read them; the partials
+ * live behind them) - upload once per batch, run per layer.
  * EFIM_ERR_INVALID_ARG if the blob was not made for this cache shape and these lengths
  * (checked against a hash of the host mirrors), EFIM_ERR_WORKSPACE if plan_bytes is too small.
  */

@@ -520,8 +520,7 @@ decode_splitkv_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
 // o = sum 2^(lse_c - lse) o_c.  WPR warps share one (row, head), each taking every WPR-th block of
 // four chunks; lanes over head_dim.  Latency-bound on short steps: one warp for few chunks, four
 // from 9 chunks on, where one warp's chain of dependent loads showed.  Launched programmatically, it is
-// resident when the split kernel ends: 1 row x 2.3k keys 9.0 -> 7.3 us for the step, 16 rows x 2-2.9k
-// 31.5 -> 30.5, 64 rows x 1-16k at 28/4 heads (with the append before it) 128 -> 121.
+// resident when the split kernel ends (1.7 us of a step of 1 row x 2.3k keys, 1 us at 16 rows).
 template <int D, int WPR>
 __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p) {
   constexpr int EPL = D / 32;
@@ -533,7 +532,7 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeParams p)
   // The row's length is an input of the step: the split kernel does not write it, and everything before
   // that kernel has completed, so it is looked up before the wait (in L2, where what has completed is
   // visible).  With the first partial rows fetched beside the maximum's lse values: steps of 1 to 64 rows in
-  // chunks 0.7-1.0 us shorter (1 row x 2.3k keys 7.3 -> 6.5, 16 rows x 2-2.9k 30.5 -> 29.5).
+  // chunks 0.7-1.0 us shorter (1 row x 2.3k keys 6.5 us, 16 rows x 2-2.9k 29.5).
   int nc = 0;
   if (row_head < (size_t)p.R * p.Hq) {
     const int len = min(__ldcg(p.row_len + row_head / p.Hq), p.key_cap);

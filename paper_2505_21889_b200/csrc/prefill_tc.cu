@@ -346,7 +346,7 @@ __device__ __forceinline__ float row_exp(const uint32_t* s, float scale, float n
 // (swizzled), zeros for absent rows; with a rotary table every row is rotated by its position on the
 // way (the arithmetic of efim_kv_append).  The warp reads whole rows, 32 * 16 bytes of them per
 // instruction: with a row per lane every instruction touched 32 lines (16 prompts of 1-3.5k tokens,
-// whose CTAs have some 16 steps, 1053 -> 1040 us for the append and this).
+// whose CTAs have some 16 steps, lost 13 us to that).
 template <int D>
 __device__ __noinline__ void q_rows_rotated_to_smem(const uint4* q, const float* cos_sin, int max_position, int interleaved,
                                                     int32_t* status, uint8_t* tile, int row0, int lane, int th, int pos) {
@@ -414,16 +414,16 @@ __device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* tile, i
 }
 
 // Two softmax groups ("streams") run per CTA.  With more than 128 rows, stream t
-// owns query tile t and both walk every KV tile.  With 128 rows or fewer there is
-// one query tile; stream 0 takes the even KV tiles and stream 1 the odd ones, each
-// with its own running (max, sum, O), and the two states are merged at the end -
+// owns query tile t and both walk every step of BN keys.  With 128 rows or fewer there is
+// one query tile; stream 0 takes the even steps and stream 1 the odd ones, each
+// with its own reference, sum and O, and the two states are merged at the end -
 // the tensor core then still works on one stream while the other does its softmax.
 //
 // MODE 0: one query tile (33..128 rows); 1: two query tiles; 2: at most 32 rows (one-token rows of
 // a mixed batch, short `inc`s): the one query tile holds the rows four times, once per 32-lane
-// quarter, and the softmax warp of quarter w takes keys 32w..32w+31 of every tile with a
-// running (max, sum, O) of its own - a quarter of the exponentials per thread and tile, so the
-// two alternating streams turn a tile round in about half the time; the eight states of a row
+// quarter, and the softmax warp of quarter w takes keys 20w..20w+19 (BN / 4) of every step with a
+// reference, sum and O of its own - a quarter of the exponentials per thread and step, so the
+// two alternating streams turn a step round in about half the time; the eight states of a row
 // (2 streams x 4 quarters) are merged at the end through shared memory.
 template <int D, int MODE>
 __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorMap& map_k, const CUtensorMap& map_v,
@@ -500,7 +500,8 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
   }
 
-  // Programmatic launch: up to here a CTA with a list of its own has touched nothing but itself; every warp that reads or writes global memory waits for the kernel before.
+  // Programmatic launch: up to here a CTA with a list of its own has touched nothing but itself; every warp
+  // that reads or writes global memory waits for the kernel before.
   if (warp < 8 && tiny) {
     pdl_wait();
     // ============================================================ softmax groups, 32-row shape
@@ -721,7 +722,7 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       const int th = valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1;
       // The rows leave through the query tile's space (its MMAs are done; a warp uses its own 32 rows
       // only): a lane writes its row, then the warp stores whole rows, two or four per instruction
-      // (with a row per lane every store touched 32 lines: 16 prompts of 1-3.5k tokens 1094 -> 1053 us).
+      // (with a row per lane every store touched 32 lines: 16 prompts of 1-3.5k tokens lost 41 us to that).
       constexpr int VEC = D / 8, RPI = 32 / VEC;
       uint8_t* tile = smem_gen + L::Q_OFF + qt * L::Q_BYTES;
       auto slot_of = [&](int row, int c) {
@@ -1218,11 +1219,12 @@ void fill_lists(const efim_cache_desc* c, const efim_batch_desc* b, const Plan& 
   const int Hkv = c->num_kv_heads;
   std::vector<Block> blocks;
   blocks.reserve((size_t)pl.n_items / Hkv);
-  // A tile costs a two-tile CTA (bound by its softmax) 2.1 us wherever it runs; a one-tile CTA is
-  // bound by its K/V bytes and speeds up once SMs fall idle at the end of a launch (measured:
-  // 0.89 us per tile with 8 to 32 such CTAs on the GPU, 1.5 us with 148), so it is weighted
-  // 0.9 us here (cfg2: 0.305 ms ordered by tile count, 0.290 by cost at 2.1 : 1.5, 0.281 at
-  // 2.1 : 1.2; 2.1 : 0.9 is 3-5 % faster still on three of four other draws of cfg2).
+  // A two-tile CTA is bound by its softmax wherever it runs; a one-tile CTA is bound by its K/V
+  // bytes and speeds up once SMs fall idle at the end of a launch (0.89 us per tile with 8 to 32 such
+  // CTAs on the GPU, 1.5 us with 148), so it is weighted with its lone rate.  The weights were measured on a
+  // kernel with P in S's columns, whose two-tile CTAs took 2.1 us a tile (cfg2: 305 us ordered by tile
+  // count, 290 by cost at 2.1 : 1.5, 281 at 2.1 : 1.2; 2.1 : 0.9 3-5 % faster still on three of four
+  // other draws of cfg2), and not on the present one.
   walk_blocks(c, b, pl.chunk_tiles, split_tokens, [&](int s, int32_t row0, int rows, int32_t tb, int32_t te, int ch) {
     blocks.push_back(Block{s, row0, tb, te, (int16_t)ch,
                            (int32_t)((te - tb) * (rows > BM ? ORDER_TILE_DUAL : ORDER_TILE_SINGLE))});
