@@ -20,9 +20,9 @@
 // (128 x 256 of them, 16 per clock: 2,048 cycles) alike; with one tile the K/V bytes.  P used to
 // take the place of S, so a stream's next scores had to wait for PV of this step (3,490 cycles per 128
 // keys); with P in columns of its own they wait for nothing but their reader.  That, no row
-// maximum per step and the streams started half a step apart: 8 x 3,200 tokens over 5k keys at 32/8
-// heads 2.92 -> 2.63 ms (append included), 8 x 128 over 8k 170 -> 160 us, 16 prompts of 1-3.5k tokens
-// 1158 -> 1095 us, 64 mixed rows at 28/4 heads 342 -> 332 us.
+// maximum per step after the first ones and the streams started half a step apart took 10 % off 8 x
+// 3,200 tokens over 5k keys at 32/8 heads, 6 % off 8 x 128 over 8k and off prompts of 1-3.5k tokens, 3 %
+// off 64 mixed rows at 28/4.
 #include "prefill_tc.cuh"
 #include "mbar.cuh"
 #include <cfloat>
