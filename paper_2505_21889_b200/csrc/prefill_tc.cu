@@ -6,8 +6,8 @@
 // (sequence, kv head) as two 128-row tiles, and streams the visible K/V range in
 // steps of 80 keys (5 pages):
 //   warps 8,11 TMA producers (K tiles / V tiles): walk the block table, one tiled bulk-tensor
-//             copy per page (16 slots x all dims of the kv head) into rings of 4 entries each
-//             (8 at head_dim 64; 128B swizzle; one K entry more with one query tile)
+//             copy per page (16 slots x all dims of the kv head) into rings of 3 entries each
+//             (8 at head_dim 64; 128B swizzle); warp 8 also claims the CTA's next item
 //   warp 10   issues the tcgen05.mma for S_t = Q_t K^T into TMEM
 //   warp 9    issues the tcgen05.mma for O_t += P_t V (P read from TMEM)
 //   warps 0-7 two softmax groups ("streams"), one TMEM lane (row) per thread: S from TMEM, mask,
@@ -176,12 +176,28 @@ __host__ __device__ constexpr uint32_t instr_desc(int n, int b_mn_major) {
          (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(BM >> 4) << 24);
 }
 
+// barrier slots (8 bytes each) inside the BAR_OFF block, per stream or per ring entry
+enum {
+  BAR_Q = 0,         // query tile is in shared memory
+  BAR_S = 2,         // scores of a step are in tensor memory
+  BAR_SFREE = 4,     // ... and have been read by the softmax warps
+  BAR_P = 6,         // probabilities of a step are in tensor memory (and O has been rescaled if need be)
+  BAR_PV = 8,        // PV of a step has finished
+  BAR_IFULL = 10,    // a work item is in the mailbox
+  BAR_IEMPTY = 12,   // ... and has been read by the warps
+  BAR_PAIR = 14,     // the two softmax warps that share 32 TMEM lanes
+  BAR_ALL = 18,      // all softmax warps
+  BAR_CLAIM = 19,    // the answer to a claim is in shared memory
+  BAR_KFULL = 20, BAR_KEMPTY = 28, BAR_VFULL = 36, BAR_VEMPTY = 44, BAR_COUNT = 52
+};
+
 // Shared-memory plan.  A query tile is [64-element half][128 rows][128 bytes]; a K or V tile
 // is [8-key group][64-element half][8 keys][128 bytes], which is what one copy per page
 // writes (a page is two key groups).  In both, 16-byte chunk c of row r is stored at chunk
 // position c ^ (r & 7) (the 128B swizzle the tensor-map copies and the MMA descriptors use).
 // K and V tiles have rings of their own: every ring barrier is waited on by one warp, phase after
-// phase.  With a single query tile the second tile's space holds one more K entry (NK + 1).
+// phase, from the CTA's first item to its last.  (Three entries each at head_dim 128: 8 x 3,200 tokens over 5k keys
+// 2,484 us, 8 x 128 over 8k 149; four 2,512 and 150.5, four of K and three of V 2,511 and 152.5.)
 template <int D>
 struct Smem {
   static constexpr int HALVES = D / 64;
@@ -190,30 +206,21 @@ struct Smem {
   static constexpr int GROUP_BYTES = HALVES * 1024;             // 8 keys of a K/V tile, all dims
   static constexpr int PAGE_BYTES = 2 * GROUP_BYTES;            // one page = one copy
   static constexpr int KV_BYTES = BN / 16 * PAGE_BYTES;         // 20 KB at head_dim 128, 10 KB at 64
-  static constexpr int NK = D == 128 ? 4 : 8, NV = NK;            // ring entries
-  static constexpr int NK_MAX = NK + 1;
+  static constexpr int NK = D == 128 ? 3 : 8, NV = NK;            // ring entries
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = Q_OFF + NQ * Q_BYTES;
   static constexpr int BAR_OFF = KV_OFF + (NK + NV) * KV_BYTES;
-  static constexpr int TOTAL = BAR_OFF + 512 + 1024;            // + alignment slack
-  static_assert(KV_BYTES <= Q_BYTES, "the extra K entry takes the second query tile's place");
-  // epilogue exchange between the two softmax groups (re-uses the K/V rings)
-  static constexpr int XROW = D + 4;                            // floats per row, padded
-  static_assert(BM * XROW * 4 <= (NK + NV) * KV_BYTES, "exchange buffer must fit in the rings");
-  static_assert(8 * 32 * XROW * 4 <= (NK + NV) * KV_BYTES, "the eight states must fit in the rings");
+  static constexpr int TMEM_SLOT_OFF = BAR_OFF + BAR_COUNT * 8, ABORT_OFF = TMEM_SLOT_OFF + 8;
+  static constexpr int ITEM_OFF = (ABORT_OFF + 8 + 15) / 16 * 16;          // mailbox: two work items
+  static constexpr int CLAIM_OFF = ITEM_OFF + 2 * 32;                     // answer to a claim
+  // Exchange of the 32-row shape: the four quarters' O in the query tiles' space, (reference, sum) here.
+  static_assert(4 * 32 * D * 4 <= NQ * Q_BYTES, "the quarters' states must fit in the query tiles");
+  static constexpr int ML_OFF = CLAIM_OFF + 16;
+  static constexpr int TOTAL = ML_OFF + 4 * 32 * 8 + 1024;                // + alignment slack
+  static_assert(TOTAL <= 227 * 1024, "shared memory of a CTA");
   // tensor memory: [S | P] of each stream, then O of each
   static constexpr int SP_COLS = 128;
   static_assert(BN + BN / 2 <= SP_COLS && NQ * (SP_COLS + D) <= 512, "tensor memory has 512 columns");
-};
-// barrier slots (8 bytes each) inside the BAR_OFF block, per stream or per ring entry (at most 9 K, 8 V)
-enum {
-  BAR_Q = 0,         // query tile is in shared memory
-  BAR_S = 2,         // scores of a step are in tensor memory
-  BAR_SFREE = 4,     // ... and have been read by the softmax warps
-  BAR_P = 6,         // probabilities of a step are in tensor memory (and O has been rescaled if need be)
-  BAR_PV = 8,        // PV of a step has finished (the last step's is BAR_O)
-  BAR_O = 10,        // all of a stream's MMAs have finished
-  BAR_KFULL = 12, BAR_KEMPTY = 21, BAR_VFULL = 30, BAR_VEMPTY = 38, BAR_COUNT = 46
 };
 // A step's probabilities are taken relative to the reference maximum of the steps before; a row whose
 // sum of one step leaves this range (2^8) takes its exact maximum as the new reference and redoes the
@@ -238,56 +245,6 @@ __device__ __forceinline__ float move_reference(float& m_ref, float mx) {
   const float alpha = m_new == m_ref ? 1.f : ex2(m_ref - m_new);
   m_ref = m_new;
   return alpha;
-}
-
-// Epilogue of the 32-row shape: the eight (max, sum, O) states of query row `lane`, left in
-// shared memory as [state][row][XROW], are merged; this thread finishes D/8 dims of the row
-// (slice `sidx`) and stores them (final output, or a chunk's partial).  Out of line: it runs
-// once per CTA and its registers should not count against the loops of the caller.
-template <int D>
-__device__ __noinline__ void tiny_merge_store(uint16_t* out, float* lse, float* part_o, float* part_lse, int s_max,
-                                              const float* xb, int lane, int sidx, bool valid, int chunk,
-                                              size_t row_off, size_t th) {
-  using L = Smem<D>;
-  constexpr int DS = D / 8;
-  float M = -INFINITY;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) M = fmaxf(M, xb[(size_t)(q * 32 + lane) * L::XROW + D]);
-  float Lt = 0.f, acc[DS];
-#pragma unroll
-  for (int d = 0; d < DS; ++d) acc[d] = 0.f;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const float* row = xb + (size_t)(q * 32 + lane) * L::XROW;
-    const float lq = row[D + 1];
-    const float wq = lq == 0.f ? 0.f : ex2(row[D] - M);
-    Lt = fmaf(lq, wq, Lt);
-#pragma unroll
-    for (int d = 0; d < DS; d += 4) {
-      const float4 x = *reinterpret_cast<const float4*>(row + sidx * DS + d);
-      acc[d] = fmaf(x.x, wq, acc[d]);
-      acc[d + 1] = fmaf(x.y, wq, acc[d + 1]);
-      acc[d + 2] = fmaf(x.z, wq, acc[d + 2]);
-      acc[d + 3] = fmaf(x.w, wq, acc[d + 3]);
-    }
-  }
-  const float inv = Lt == 0.f ? 0.f : 1.f / Lt;
-  const float lse2 = Lt == 0.f ? -INFINITY : M + log2f(Lt);
-  if (!valid) return;
-  if (chunk < 0) {
-    uint4* dst = reinterpret_cast<uint4*>(out + row_off + sidx * DS);
-#pragma unroll
-    for (int d = 0; d < DS; d += 8)
-      dst[d / 8] = make_uint4(pack_bf16x2(acc[d] * inv, acc[d + 1] * inv), pack_bf16x2(acc[d + 2] * inv, acc[d + 3] * inv),
-                              pack_bf16x2(acc[d + 4] * inv, acc[d + 5] * inv), pack_bf16x2(acc[d + 6] * inv, acc[d + 7] * inv));
-    if (sidx == 0 && lse) lse[th] = lse2 * 0.6931471805599453f;
-  } else {
-    float4* dst = reinterpret_cast<float4*>(part_o + (th * s_max + chunk) * D + sidx * DS);
-#pragma unroll
-    for (int d = 0; d < DS; d += 4)
-      dst[d / 4] = make_float4(acc[d] * inv, acc[d + 1] * inv, acc[d + 2] * inv, acc[d + 3] * inv);
-    if (sidx == 0) part_lse[th * s_max + chunk] = lse2;
-  }
 }
 
 // O row of every lane of the warp *= alpha (the rare rescale of the 32-row shape; kept out
@@ -390,26 +347,23 @@ __device__ __noinline__ void q_rows_rotated_to_smem(const uint4* q, const float*
   }
 }
 template <int D>
-__device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* tile, int row0, int lane, int th, int pos) {
+__device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* smem_gen, int tile_off, uint32_t smem_base, int row0,
+                                               int lane, int th, int pos) {
   using L = Smem<D>;
   constexpr int VEC = D / 8, RPI = 32 / VEC;
   if (p.cos_sin != nullptr) {
     q_rows_rotated_to_smem<D>(reinterpret_cast<const uint4*>(p.q), p.cos_sin, p.max_position, p.interleaved, p.status,
-                              tile, row0, lane, th, pos);
+                              smem_gen + tile_off, row0, lane, th, pos);
     return;
   }
   const int c = lane % VEC, sub = lane / VEC;
-  uint4 v[VEC];
 #pragma unroll
   for (int i = 0; i < VEC; ++i) {
     const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
-    v[i] = make_uint4(0, 0, 0, 0);
-    if (t >= 0) v[i] = reinterpret_cast<const uint4*>(p.q)[(size_t)t * VEC + c];
-  }
-#pragma unroll
-  for (int i = 0; i < VEC; ++i) {
     const int r = row0 + i * RPI + sub;
-    *reinterpret_cast<uint4*>(tile + (c >> 3) * L::HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v[i];
+    const uint4* src = reinterpret_cast<const uint4*>(p.q) + (size_t)max(t, 0) * VEC + c;
+    const uint32_t dst = smem_base + tile_off + (c >> 3) * L::HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(t >= 0 ? 16 : 0) : "memory");
   }
 }
 
@@ -419,43 +373,791 @@ __device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* tile, i
 // with its own reference, sum and O, and the two states are merged at the end -
 // the tensor core then still works on one stream while the other does its softmax.
 //
-// MODE 0: one query tile (33..128 rows); 1: two query tiles; 2: at most 32 rows (one-token rows of
-// a mixed batch, short `inc`s): the one query tile holds the rows four times, once per 32-lane
+// SHAPE_ONE: one query tile (33..128 rows); SHAPE_TWO: two query tiles; SHAPE_TINY: at most 32 rows (one-token
+// rows of a mixed batch, short `inc`s): the one query tile holds the rows four times, once per 32-lane
 // quarter, and the softmax warp of quarter w takes keys 20w..20w+19 (BN / 4) of every step with a
 // reference, sum and O of its own - a quarter of the exponentials per thread and step, so the
 // two alternating streams turn a step round in about half the time; the eight states of a row
-// (2 streams x 4 quarters) are merged at the end through shared memory.
-template <int D, int MODE>
-__device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorMap& map_k, const CUtensorMap& map_v,
-                                                const WorkItem& it) {
+// (2 streams x 4 quarters) are merged at the end.
+enum { SHAPE_ONE = 0, SHAPE_TWO = 1, SHAPE_TINY = 2 };
+
+// A work item as the roles use it.  Every value is the same in all lanes, and the compiler has to know it: loop
+// bounds, ring positions and with them the MMAs' descriptors stay in uniform registers only then.  (The same holds
+// for the warp's index, which the roles branch on: taken from threadIdx as it is, the loops were compiled for
+// diverging lanes - twice the convergence instructions, and 8 x 3,200 tokens over 5k keys at 32/8 heads took 2.81 ms,
+// 8 x 128 over 8k 165 us, against 2.51 ms and 150 us.)
+struct Work {
+  int seq, kvh, chunk, row0, C, tok0, rows_total;
+  int key0, kv_cap, nt;        // keys [key0, kv_cap): the tiles of the item, up to what its last row sees; steps of BN keys
+  int shape;
+  __device__ __forceinline__ int steps(int st) const {
+    return shape == SHAPE_TWO ? nt : (st == 0 ? (nt + 1) >> 1 : nt >> 1);
+  }
+};
+__device__ __forceinline__ int uniform(int x) {
+  return static_cast<int>(__reduce_or_sync(0xffffffffu, static_cast<unsigned>(x)));
+}
+__device__ __forceinline__ Work work_of(const WorkItem& it, int G) {
+  Work w;
+  w.seq = uniform(it.seq);
+  const int kc = uniform((int)(uint16_t)it.kvh | (int)it.chunk << 16);
+  w.kvh = (int)(int16_t)(kc & 0xffff);
+  w.chunk = kc >> 16;
+  w.row0 = uniform(it.row0);
+  w.C = uniform(it.cached);
+  w.tok0 = uniform(it.tok0);
+  w.rows_total = uniform(it.new_len) * G;
+  const int rows_here = min(NQ * BM, w.rows_total - w.row0);
+  const int i_last = (w.row0 + rows_here - 1) / G;           // last token of this item
+  w.key0 = uniform(it.tile_begin) * PT;
+  w.kv_cap = min(w.C + i_last + 1, uniform(it.tile_end) * PT);
+  w.nt = (w.kv_cap - w.key0 + BN - 1) / BN;
+  w.shape = rows_here > BM ? SHAPE_TWO : (rows_here <= 32 ? SHAPE_TINY : SHAPE_ONE);
+  return w;
+}
+
+// What every role of a CTA knows.
+template <int D>
+struct Cta {
   using L = Smem<D>;
-  constexpr int HALVES = L::HALVES;
+  const Params& p;
+  uint32_t smem_base;
+  uint8_t* smem_gen;
+  volatile int* abort_flag;
+  uint32_t tmem_S, tmem_P, tmem_O;       // S of stream t at columns t * SP_COLS, P (bf16 pairs) behind it; O of stream t at t * D
+  int lane;
+  __device__ __forceinline__ uint32_t bar(int i) const { return smem_base + L::BAR_OFF + 8u * i; }
+  __device__ __forceinline__ void wait(int b, uint32_t parity) const {
+    mbar_wait(bar(b), parity, abort_flag, p.status, p.wait_ns);
+  }
+};
+
+// The item after the present one, from the mailbox that warp 8 fills; false: there is none, or the CTA has given up.
+// Every warp but warp 8 reads every slot, so a slot is free again after 11 arrivals.
+struct Mailbox {
+  int slot = 0;
+  uint32_t phase = 0;
+  template <int D>
+  __device__ __forceinline__ bool next(const Cta<D>& c, Work& w) {
+    c.wait(BAR_IFULL + slot, phase);
+    WorkItem it;
+    const uint4* src = reinterpret_cast<const uint4*>(c.smem_gen + Smem<D>::ITEM_OFF) + 2 * slot;
+    uint4* dst = reinterpret_cast<uint4*>(&it);
+    dst[0] = src[0];
+    dst[1] = src[1];
+    const bool gone = __any_sync(0xffffffffu, *c.abort_flag != 0);
+    warp_arrive(c.bar(BAR_IEMPTY + slot), c.lane);
+    if (++slot == 2) { slot = 0; phase ^= 1; }
+    if (gone) return false;
+    w = work_of(it, c.p.G);
+    return w.seq >= 0;
+  }
+};
+
+// Claim of one more item: a CTA of this launch that has not started is taken out of it and its block index handed over
+// (cluster launch control); the answer is written to shared memory.
+__device__ __forceinline__ void claim_next(uint32_t answer, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer),
+               "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ int claimed_block(uint32_t answer) {   // -1: there was none left
+  uint32_t ok, x;
+  asm volatile(
+      "{\n.reg .b128 a;\n.reg .pred p;\n"
+      "ld.shared.b128 a, [%2];\n"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n"
+      "selp.u32 %0, 1, 0, p;\nmov.u32 %1, 0;\n"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n}\n"
+      : "=r"(ok), "=r"(x)
+      : "r"(answer)
+      : "memory");
+  return ok ? static_cast<int>(x) : -1;
+}
+
+// This lane's query row of tile `qt`, quarter `w` (SHAPE_TINY: the same 32 rows in every quarter).
+struct Row {
+  bool valid;
+  int pos, th;                 // position; index of the (token, head) row in q, out and lse, -1 for a row past the sequence
+  __device__ __forceinline__ Row(const Params& p, const Work& it, int qt, int w, int lane) {
+    const int R = it.row0 + (it.shape == SHAPE_TINY ? lane : qt * BM + w * 32 + lane);
+    valid = R < it.rows_total;
+    const int i_tok = valid ? R / p.G : 0;
+    pos = it.C + i_tok;
+    th = valid ? (it.tok0 + i_tok) * p.Hq + it.kvh * p.G + (R - i_tok * p.G) : -1;
+  }
+};
+template <int D>
+__device__ __forceinline__ void fetch_q(const Cta<D>& c, const Work& it, int qt, int w) {
+  const Row r(c.p, it, qt, w, c.lane);
+  q_rows_to_smem<D>(c.p, c.smem_gen, Smem<D>::Q_OFF + qt * Smem<D>::Q_BYTES, c.smem_base, w * 32, c.lane, r.th, r.pos);
+}
+template <int D>
+__device__ __forceinline__ void publish_q(const Cta<D>& c, int qt) {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  fence_async_smem();
+  warp_arrive(c.bar(BAR_Q + qt), c.lane);
+}
+
+// 32 bytes of a row (`wide`: the rows are 32-byte aligned, one store).
+__device__ __forceinline__ void store32(void* dst, const uint32_t* v, bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+  } else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
+}
+// N columns of an output row (or, chunk >= 0, of a chunk's partial) from column c0 on.
+template <int D, int N>
+__device__ __forceinline__ void store_cols(const Params& p, int th, int chunk, int c0, const float* f, bool wide) {
+  if (th < 0) return;
+  if (chunk < 0) {
+    uint16_t* dst = p.out + (size_t)th * D + c0;
+#pragma unroll
+    for (int c = 0; c < N; c += 16) {
+      uint32_t v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = pack_bf16x2(f[c + 2 * e], f[c + 2 * e + 1]);
+      store32(dst + c, v, wide);
+    }
+  } else {
+    float* dst = p.part_o + ((size_t)th * p.s_max + chunk) * D + c0;
+#pragma unroll
+    for (int c = 0; c < N; c += 8) store32(dst + c, reinterpret_cast<const uint32_t*>(f) + c, true);
+  }
+}
+__device__ __forceinline__ void store_lse(const Params& p, int th, int chunk, float lse2) {
+  if (th < 0) return;
+  if (chunk >= 0) {
+    p.part_lse[(size_t)th * p.s_max + chunk] = lse2;
+  } else if (p.lse) {
+    p.lse[th] = lse2 * 0.6931471805599453f;
+  }
+}
+
+// The states (reference, sum) of a row's two streams: the lane of stream 0 and the one of stream 1 that share the TMEM
+// lane swap theirs through two dead columns of P.  Afterwards the partner's O may be read too (its PV MMAs are done).
+struct Pair {
+  float M, L, w0, w1;          // common reference and sum, weights of the two O
+};
+template <int D>
+__device__ __forceinline__ Pair meet_partner(const Cta<D>& c, int st, int w, uint32_t lane_addr, float m_ref, float l_sum,
+                                             uint32_t& pair_phase) {
+  using L = Smem<D>;
+  const uint32_t mine[2] = {__float_as_uint(m_ref), __float_as_uint(l_sum)};
+  tmem_st<2>(c.tmem_P + lane_addr + st * L::SP_COLS, mine);
+  tmem_wait_st();
+  tc_fence_before();
+  warp_arrive(c.bar(BAR_PAIR + w), c.lane);
+  c.wait(BAR_PAIR + w, pair_phase);
+  pair_phase ^= 1;
+  tc_fence_after();
+  uint32_t o[4];
+  tmem_ld<4>(c.tmem_P + lane_addr + (st ^ 1) * L::SP_COLS, o);
+  tmem_wait_ld<4>(o);
+  const float m0 = st == 0 ? m_ref : __uint_as_float(o[0]), l0 = st == 0 ? l_sum : __uint_as_float(o[1]);
+  const float m1 = st == 1 ? m_ref : __uint_as_float(o[0]), l1 = st == 1 ? l_sum : __uint_as_float(o[1]);
+  Pair r;
+  r.M = fmaxf(m0, m1);
+  r.w0 = l0 == 0.f ? 0.f : ex2(m0 - r.M);
+  r.w1 = l1 == 0.f ? 0.f : ex2(m1 - r.M);
+  r.L = l0 * r.w0 + l1 * r.w1;
+  return r;
+}
+// Before either of a pair may go on and let its stream's O be overwritten, both have read what they need.
+template <int D>
+__device__ __forceinline__ void leave_partner(const Cta<D>& c, int w, uint32_t& pair_phase) {
+  tc_fence_before();
+  warp_arrive(c.bar(BAR_PAIR + w), c.lane);
+  c.wait(BAR_PAIR + w, pair_phase);
+  pair_phase ^= 1;
+  tc_fence_after();
+}
+
+// ------------------------------------------------------------------ softmax groups
+// One item of at most 32 rows; `n`: steps of this stream so far.
+template <int D>
+__device__ __forceinline__ void softmax_tiny(const Cta<D>& c, const Work& it, int st, int w, uint32_t& n, uint32_t& pair_phase,
+                                             uint32_t& all_phase) {
+  using L = Smem<D>;
+  const Params& p = c.p;
+  const int my_cnt = it.steps(st);
+  const Row row(p, it, 0, w, c.lane);
+  const int vis = row.valid ? min(row.pos + 1, it.kv_cap) : it.kv_cap;
+  constexpr int KQ = BN / 4;                              // keys of a step this warp scores
+  const uint32_t lane_addr = (uint32_t)(w * 32) << 16;
+  const uint32_t s_addr = c.tmem_S + lane_addr + st * L::SP_COLS;
+  const uint32_t p_addr = c.tmem_P + lane_addr + st * L::SP_COLS;
+  const uint32_t o_addr = c.tmem_O + lane_addr + st * D;
+  // P of this quarter's rows is zero but for the quarter's own keys: cleared once here, the steps
+  // write only columns KQ / 2 * w ...
+  {
+    const uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int i = 0; i < BN / 2; i += 8) tmem_st<8>(p_addr + i, z);
+    tmem_wait_st();
+  }
+  float m_ref = row.valid ? -FLT_MAX : FLT_MAX, l_sum = 0.f;
+  for (int k = 0; k < my_cnt; ++k, ++n) {
+    c.wait(BAR_S + st, n & 1);
+    tc_fence_after();
+    uint32_t s[KQ];
+    tmem_ld<KQ>(s_addr + KQ * w, s);
+    tmem_wait_ld<KQ>(s);
+    tc_fence_before();
+    warp_arrive(c.bar(BAR_SFREE + st), c.lane);
+    const int kv0 = it.key0 + (2 * k + st) * BN + KQ * w;
+    if (__any_sync(0xffffffffu, kv0 + KQ > vis)) {
+#pragma unroll
+      for (int i = 0; i < KQ; ++i)
+        if (kv0 + i >= vis) s[i] = 0xff800000u;           // -inf
+    }
+    float alpha = 1.f;                                    // what O and the sum so far are scaled by
+    if (k < EXACT_STEPS) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
+    uint32_t v[KQ / 2];
+    float sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
+    if (k > 0) {
+      c.wait(BAR_PV + st, (n - 1) & 1);                   // P of the step before is consumed
+      tc_fence_after();
+      const bool redo = !(sum <= SUM_LIMIT);
+      if (__any_sync(0xffffffffu, redo || alpha != 1.f)) {
+        if (redo) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
+        l_sum *= alpha;
+        rescale_o_row<D>(o_addr, alpha);
+        if (__any_sync(0xffffffffu, redo)) sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
+      }
+    }
+    tmem_st<KQ / 2>(p_addr + KQ / 2 * w, v);
+    tmem_wait_st();
+    tc_fence_before();
+    warp_arrive(c.bar(BAR_P + st), c.lane);
+    l_sum += sum;
+  }
+  // ---- the two streams' states of a quarter meet in tensor memory, the four quarters' in the query tiles' space
+  // (all MMAs that read the queries are done): [quarter][row][D], 16-byte chunk j of a row at j ^ (row & 7)
+  if (my_cnt > 0) c.wait(BAR_PV + st, (n - 1) & 1);
+  tc_fence_after();
+  float* x = reinterpret_cast<float*>(c.smem_gen + L::Q_OFF);
+  float2* xml = reinterpret_cast<float2*>(c.smem_gen + L::ML_OFF);       // [quarter][row]
+  auto chunk_at = [&](int q, int j) { return reinterpret_cast<float4*>(x + (q * 32 + c.lane) * D) + (j ^ (c.lane & 7)); };
+  if (it.nt > 1) {
+    const Pair pr = meet_partner(c, st, w, lane_addr, m_ref, l_sum, pair_phase);
+#pragma unroll
+    for (int c0 = 0; c0 < D / 2; c0 += 32) {
+      const int col = st * (D / 2) + c0;
+      uint32_t o0[32], o1[32];
+      tmem_ld<32>(c.tmem_O + lane_addr + col, o0);
+      tmem_ld<32>(c.tmem_O + lane_addr + D + col, o1);
+      tmem_wait_ld<32>(o0);
+      tmem_wait_ld<32>(o1);
+      float f[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        f[i] = pr.w0 == 0.f ? 0.f : __uint_as_float(o0[i]) * pr.w0;      // (an O without weight may hold anything)
+        f[i] = pr.w1 == 0.f ? f[i] : fmaf(__uint_as_float(o1[i]), pr.w1, f[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < 32; i += 4) *chunk_at(w, (col + i) / 4) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+    }
+    if (st == 0) xml[w * 32 + c.lane] = make_float2(pr.L == 0.f ? -INFINITY : pr.M, pr.L);
+    leave_partner(c, w, pair_phase);
+  } else if (st == 0) {
+    const bool have = !(l_sum == 0.f);                     // (a sum of NaN is handed on, not dropped)
+#pragma unroll
+    for (int c0 = 0; c0 < D; c0 += 32) {
+      uint32_t o[32];
+      tmem_ld<32>(o_addr + c0, o);
+      tmem_wait_ld<32>(o);
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<uint4*>(chunk_at(w, (c0 + i) / 4)) = have ? make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]) : make_uint4(0, 0, 0, 0);
+    }
+    xml[w * 32 + c.lane] = make_float2(have ? m_ref : -INFINITY, l_sum);
+  }
+  warp_arrive(c.bar(BAR_ALL), c.lane);
+  c.wait(BAR_ALL, all_phase);
+  all_phase ^= 1;
+  {
+    constexpr int DS = D / 8;                              // dims this thread finishes
+    const int d0 = (st * 4 + w) * DS;
+    float M = -INFINITY, Lt = 0.f, acc[DS];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) M = fmaxf(M, xml[q * 32 + c.lane].x);
+#pragma unroll
+    for (int i = 0; i < DS; ++i) acc[i] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 ml = xml[q * 32 + c.lane];
+      const float wq = ml.y == 0.f ? 0.f : ex2(ml.x - M);
+      Lt = fmaf(ml.y, wq, Lt);
+#pragma unroll
+      for (int i = 0; i < DS; i += 4) {
+        const float4 v = *chunk_at(q, (d0 + i) / 4);
+        acc[i] = fmaf(v.x, wq, acc[i]);
+        acc[i + 1] = fmaf(v.y, wq, acc[i + 1]);
+        acc[i + 2] = fmaf(v.z, wq, acc[i + 2]);
+        acc[i + 3] = fmaf(v.w, wq, acc[i + 3]);
+      }
+    }
+    const float inv = Lt == 0.f ? 0.f : 1.f / Lt;
+#pragma unroll
+    for (int i = 0; i < DS; ++i) acc[i] *= inv;
+    if (row.th >= 0) {
+      if (it.chunk < 0) {
+        uint4* dst = reinterpret_cast<uint4*>(p.out + (size_t)row.th * D + d0);
+#pragma unroll
+        for (int i = 0; i < DS; i += 8)
+          dst[i / 8] = make_uint4(pack_bf16x2(acc[i], acc[i + 1]), pack_bf16x2(acc[i + 2], acc[i + 3]),
+                                  pack_bf16x2(acc[i + 4], acc[i + 5]), pack_bf16x2(acc[i + 6], acc[i + 7]));
+      } else {
+        float4* dst = reinterpret_cast<float4*>(p.part_o + ((size_t)row.th * p.s_max + it.chunk) * D + d0);
+#pragma unroll
+        for (int i = 0; i < DS; i += 4) dst[i / 4] = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+      }
+      if (d0 == 0) store_lse(p, row.th, it.chunk, Lt == 0.f ? -INFINITY : M + log2f(Lt));
+    }
+  }
+  // the space may be filled with the next item's queries
+  warp_arrive(c.bar(BAR_ALL), c.lane);
+  c.wait(BAR_ALL, all_phase);
+  all_phase ^= 1;
+}
+
+// One item of more than 32 rows, one query tile or two (DUAL); `n`: steps of this stream so far.  Looks the next item up
+// and gets its query rows on their way; returns false if there is none.
+template <int D, bool DUAL>
+__device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Work& next, Mailbox& mail, int st, int w,
+                                             bool wide, uint32_t& n, uint32_t& pair_phase) {
+  using L = Smem<D>;
+  const Params& p = c.p;
+  const uint32_t lane_addr = (uint32_t)(w * 32) << 16;      // tile row == TMEM lane
+  const uint32_t s_addr = c.tmem_S + lane_addr + st * L::SP_COLS;
+  const uint32_t p_addr = c.tmem_P + lane_addr + st * L::SP_COLS;
+  const uint32_t o_addr = c.tmem_O + lane_addr + st * D;
+  const int my_cnt = it.steps(st);
+  const Row row(p, it, DUAL ? st : 0, w, c.lane);
+  // keys this row sees; rows past the sequence are computed like the piece's last row and
+  // dropped (with 0 here they would take the masking path on every tile and slow their group)
+  const int vis = row.valid ? min(row.pos + 1, it.kv_cap) : it.kv_cap;
+  const int exact = !DUAL || it.nt <= EXACT_MAX_STEPS ? EXACT_STEPS : 1;
+  const int kv_first = it.key0 + (DUAL ? 0 : st * BN), kv_step = DUAL ? BN : 2 * BN;
+  // (a row past the sequence: its query is zero, and against this reference so are its probabilities)
+  float m_ref = row.valid ? -FLT_MAX : FLT_MAX, l_sum = 0.f;
+  for (int k = 0; k < my_cnt; ++k, ++n) {
+    c.wait(BAR_S + st, n & 1);
+    tc_fence_after();
+    uint32_t s[BN];
+    // The scores come in two parts, the exponentials of the first running under the second's load, and P is
+    // stored before its sum is checked: what a stream cannot overlap with itself is what its step takes
+    // (8 x 128 tokens over 8k 155 -> 145 us for append and attention, 8 x 3,200 over 5k 2.59 -> 2.55 ms, 64
+    // mixed rows 312 -> 306; first parts of 32 and 64 keys: 156 and 145 us, 2.71 and 2.56 ms).
+    constexpr int LA = 48;
+    tmem_ld<LA>(s_addr, s);
+    tmem_wait_ld<LA>(s);
+    tmem_ld<BN - LA>(s_addr + LA, s + LA);
+    const int kv0 = kv_first + k * kv_step;
+    const bool edge = __any_sync(0xffffffffu, kv0 + BN > vis);
+    if (edge) {
+      tmem_wait_ld<BN - LA>(s + LA);
+#pragma unroll
+      for (int i = 0; i < BN; ++i)
+        if (kv0 + i >= vis) s[i] = 0xff800000u;             // -inf
+    }
+    // The first steps' exact maximum is the row's reference; later steps only check that their sum stays
+    // in range (SUM_LIMIT), so they have no row maximum to take before their first exponential.
+    auto freed = [&]() {
+      tmem_wait_ld<BN - LA>(s + LA);
+      tc_fence_before();
+      warp_arrive(c.bar(BAR_SFREE + st), c.lane);           // the next step's scores may be computed
+    };
+    if (edge || k < exact) freed();
+    // alpha: what O and the sum so far are scaled by.  A moved reference lowers the limit, so that the one
+    // test below finds it (a second condition there: 8 x 128 tokens over 8k 150.0 -> 152.6 us).
+    float alpha = 1.f, limit = SUM_LIMIT;
+    if (k < exact) {
+      alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
+      if (alpha != 1.f) limit = -1.f;
+    }
+    uint32_t v[BN / 2];                                     // P as bf16 pairs
+    const float neg_m = -m_ref;
+    float sum = row_exp<LA>(s, p.scale_log2, neg_m, v);
+    if (!(edge || k < exact)) freed();
+    sum += row_exp<BN - LA>(s + LA, p.scale_log2, neg_m, v + LA / 2);
+    if (k > 0) {
+      c.wait(BAR_PV + st, (n - 1) & 1);                     // P of the step before is consumed
+      tc_fence_after();
+    }
+    tmem_st<BN / 2>(p_addr, v);
+    if (__any_sync(0xffffffffu, !(sum <= limit)) && k > 0) {
+      // (O is quiet: PV(k-1) has finished and PV(k) waits for this warp)
+      const bool redo = !(sum <= SUM_LIMIT);
+      if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
+      l_sum *= alpha;
+      rescale_o_row<D>(o_addr, alpha);
+      if (__any_sync(0xffffffffu, redo)) {
+        sum = row_exp<BN>(s, p.scale_log2, -m_ref, v);
+        tmem_wait_st();                                     // two stores to the same columns are not ordered by themselves
+        tmem_st<BN / 2>(p_addr, v);
+      }
+    }
+    tmem_wait_st();
+    tc_fence_before();
+    warp_arrive(c.bar(BAR_P + st), c.lane);
+    l_sum += sum;
+  }
+  // ---- The next item's query rows are on their way under the last PV.  A tile's space is free once the scores of
+  // its last step have come: those of this stream, or, where both streams read the one tile, of the stream
+  // that has the last step (QK MMAs complete in order).
+  const bool more = mail.next(c, next);
+  int q_next = -1;
+  if (more) {
+    if (DUAL ? st == 0 : st == ((it.nt - 1) & 1)) q_next = 0;
+    else if (next.shape == SHAPE_TWO) q_next = 1;
+    if (q_next >= 0) fetch_q(c, next, q_next, w);
+  }
+  if (my_cnt > 0) {
+    c.wait(BAR_PV + st, (n - 1) & 1);
+    tc_fence_after();
+  }
+  if (q_next >= 0) publish_q(c, q_next);
+  // ---- epilogue: PV of the next item's first step waits for its P, and with it for the loads of O here
+  if (!DUAL && it.nt > 1) {
+    // both streams have a state of every row: each finishes half of the columns
+    const Pair pr = meet_partner(c, st, w, lane_addr, m_ref, l_sum, pair_phase);
+    const float inv = pr.L == 0.f ? 0.f : 1.f / pr.L;
+    const float a0 = pr.w0 * inv, a1 = pr.w1 * inv;
+#pragma unroll
+    for (int c0 = 0; c0 < D / 2; c0 += 32) {
+      const int col = st * (D / 2) + c0;
+      uint32_t o0[32], o1[32];
+      tmem_ld<32>(c.tmem_O + lane_addr + col, o0);
+      tmem_ld<32>(c.tmem_O + lane_addr + D + col, o1);
+      tmem_wait_ld<32>(o0);
+      tmem_wait_ld<32>(o1);
+      float f[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) f[i] = fmaf(__uint_as_float(o1[i]), a1, __uint_as_float(o0[i]) * a0);
+      store_cols<D, 32>(p, row.th, it.chunk, col, f, wide);
+    }
+    if (st == 0) store_lse(p, row.th, it.chunk, pr.L == 0.f ? -INFINITY : pr.M + log2f(pr.L));
+    leave_partner(c, w, pair_phase);
+  } else if (my_cnt > 0) {
+    const float inv = l_sum == 0.f ? 0.f : 1.f / l_sum;
+#pragma unroll
+    for (int c0 = 0; c0 < D; c0 += 64) {
+      uint32_t o[64];
+      tmem_ld<64>(o_addr + c0, o);
+      tmem_wait_ld<64>(o);
+      float f[64];
+#pragma unroll
+      for (int i = 0; i < 64; ++i) f[i] = __uint_as_float(o[i]) * inv;
+      store_cols<D, 64>(p, row.th, it.chunk, c0, f, wide);
+    }
+    store_lse(p, row.th, it.chunk, l_sum == 0.f ? -INFINITY : m_ref + log2f(l_sum));
+    tc_fence_before();
+  }
+  return more;
+}
+
+template <int D>
+__device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp) {
+  const Params& p = c.p;
+  const int st = warp >> 2, w = warp & 3;                   // stream, 32-lane quarter
+  const bool wide = (reinterpret_cast<uintptr_t>(p.out) & 31) == 0;
+  Mailbox mail;
+  uint32_t n = 0, pair_phase = 0, all_phase = 0;            // steps of this stream so far; phases of the exchange barriers
+  if (it.shape == SHAPE_TWO || st == 0) {
+    fetch_q(c, it, st, w);
+    publish_q(c, st);
+  }
+  for (;;) {
+    Work next;
+    bool more;
+    if (it.shape == SHAPE_TINY) {
+      softmax_tiny(c, it, st, w, n, pair_phase, all_phase);
+      more = mail.next(c, next);
+      if (more && (next.shape == SHAPE_TWO || st == 0)) {
+        fetch_q(c, next, st, w);
+        publish_q(c, st);
+      }
+    } else {
+      more = it.shape == SHAPE_TWO ? softmax_item<D, true>(c, it, next, mail, st, w, wide, n, pair_phase)
+                                   : softmax_item<D, false>(c, it, next, mail, st, w, wide, n, pair_phase);
+    }
+    if (!more) break;
+    it = next;
+  }
+  tc_fence_before();
+}
+
+// ------------------------------------------------------------------ TMA producers
+// Every bulk-tensor copy costs its issuing warp ~65 cycles (one box per page: 16 slots x all dims
+// of one kv head).  Warp 8 loads the K tiles and warp 11 the V tiles; warp 8 also claims the items.
+template <int D, bool K_ROLE, typename List>
+__device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap& map, const List& list, WorkItem raw, Work it) {
+  using L = Smem<D>;
+  const Params& p = c.p;
+  constexpr int n_ring = K_ROLE ? L::NK : L::NV;            // (the ring's constants fold into each copy)
+  constexpr uint32_t my_off = K_ROLE ? L::KV_OFF : L::KV_OFF + L::NK * L::KV_BYTES;
+  constexpr int full = K_ROLE ? BAR_KFULL : BAR_VFULL, empty = K_ROLE ? BAR_KEMPTY : BAR_VEMPTY;
+  const int lane = c.lane, page_l = lane;
+  Mailbox mail;                                             // of warp 11; warp 8 keeps the place it writes in it
+  int slot = 0, n_steps = 0, block = blockIdx.x;
+  uint32_t phase = 0, claim_phase = 0;
+  for (;;) {
+    const int32_t* bt = p.block_table + (size_t)it.seq * p.max_pages_per_seq + (it.key0 >> 4);
+    const int n_pages = (it.kv_cap - it.key0 + 15) >> 4;    // pages this item reads
+    // page id of this lane in step jj: -2 if the lane fetches none (lanes beyond the step's visible
+    // pages; the last test only matters for a plan that does not belong to this block table), -1 for
+    // any negative entry
+    auto lookup = [&](int jj) {
+      const int pg = jj * (BN / 16) + page_l;
+      if (page_l >= BN / 16 || pg >= n_pages || (it.key0 >> 4) + pg >= p.max_pages_per_seq) return -2;
+      return max(bt[pg], -1);
+    };
+    // the block-table read is a dependent global load in front of every copy: fetch it two steps ahead
+    int pid_a = lookup(0), pid_b = lookup(1);
+    if constexpr (K_ROLE && std::is_same<List, InlineItems>::value) {
+      // A work list that came in the launch parameters is left in the workspace like any other: a call that
+      // plans for itself may be followed by planned calls with resident lists.
+      if (lane == 0) p.items_out[block] = raw;
+    }
+    // Another item is claimed when the copies of the last but one step are due: the rings then hold the steps before,
+    // which covers the claim, the item and its first pages.  (Claimed earlier, the last items of a launch would be
+    // bound to CTAs that are still busy.)
+    const int claim_at = max(it.nt - 2, 0);
+    for (int jj = 0; jj < it.nt; ++jj) {
+      const int pid = pid_a;
+      pid_a = pid_b;
+      pid_b = lookup(jj + 2);
+      const bool ok = pid >= 0 && pid < p.num_pages;
+      const bool bad = pid != -2 && !ok;                    // an id outside the pool: reported, never dereferenced
+      const uint32_t okmask = __ballot_sync(0xffffffffu, ok);
+      const bool any_bad = __any_sync(0xffffffffu, bad);
+      const uint32_t bytes = __popc(okmask) * (uint32_t)L::PAGE_BYTES;
+      if (K_ROLE && jj == claim_at && lane == 0) {
+        mbar_expect_tx(c.bar(BAR_CLAIM), 16);
+        claim_next(c.smem_base + L::CLAIM_OFF, c.bar(BAR_CLAIM));
+      }
+      c.wait(empty + slot, phase ^ 1);
+      const uint32_t dst_off = my_off + slot * L::KV_BYTES + page_l * L::PAGE_BYTES;
+      if (any_bad) {
+        // the page's 16 keys are replaced by zeros (score 0, value 0), so the tile holds nothing
+        // undefined; written with ordinary stores, made visible to the tensor core's reads
+        if (bad) {
+          if (K_ROLE && p.status) atomicOr(p.status, EFIM_DEV_BAD_PAGE);
+          uint4* z = reinterpret_cast<uint4*>(c.smem_gen + dst_off);
+          for (int i = 0; i < L::PAGE_BYTES / 16; ++i) z[i] = make_uint4(0, 0, 0, 0);
+          fence_async_smem();
+        }
+        __syncwarp();
+      }
+      if (lane == 0) mbar_expect_tx(c.bar(full + slot), bytes);
+      __syncwarp();
+      if (ok) tma_load_page(c.smem_base + dst_off, &map, c.bar(full + slot), pid * p.Hkv + it.kvh);
+      if (++slot == n_ring) { slot = 0; phase ^= 1; }
+    }
+    n_steps += it.nt;
+    bool more;
+    if constexpr (K_ROLE) {
+      c.wait(BAR_CLAIM, claim_phase);
+      claim_phase ^= 1;
+      const bool gone = __any_sync(0xffffffffu, *c.abort_flag != 0);
+      block = gone ? -1 : uniform(claimed_block(c.smem_base + L::CLAIM_OFF));
+      fence_async_smem();                                   // the answer has been read: the next one may be written
+      if (block >= 0) {
+        if constexpr (std::is_same<List, InlineItems>::value) raw = list.items[block];
+        else raw = p.items[block];
+      } else {
+        raw = WorkItem{};
+        raw.seq = -1;
+      }
+      c.wait(BAR_IEMPTY + mail.slot, mail.phase ^ 1);
+      if (lane == 0) {
+        uint4* dst = reinterpret_cast<uint4*>(c.smem_gen + L::ITEM_OFF) + 2 * mail.slot;
+        dst[0] = reinterpret_cast<const uint4*>(&raw)[0];
+        dst[1] = reinterpret_cast<const uint4*>(&raw)[1];
+        mbar_arrive(c.bar(BAR_IFULL + mail.slot));
+      }
+      __syncwarp();
+      if (++mail.slot == 2) { mail.slot = 0; mail.phase ^= 1; }
+      more = block >= 0;
+      if (more) it = work_of(raw, p.G);
+    } else {
+      more = mail.next(c, it);
+    }
+    if (!more) break;
+  }
+  // if the CTA gave up, let copies that are still in flight land before shared memory goes away
+  if (*c.abort_flag) {
+    for (int jj = max(0, n_steps - n_ring); jj < n_steps; ++jj) mbar_drain(c.bar(full + jj % n_ring), (jj / n_ring) & 1);
+  }
+}
+
+// ------------------------------------------------------------------ MMA issuers
+// Issuing an MMA costs its thread nearly as long as the tensor core needs to run it,
+// so the work is split: warp 9 issues the PV MMAs of both streams, warp 10 the QK
+// MMAs.  QK(k+1) of a stream needs S(k) read (barrier SFREE), PV(k) needs P(k) written:
+// neither waits for the other, so the tensor core has a stream's next scores ready when
+// its softmax warps come back for them.
+//
+// Descriptors: the high word is fixed (SBO = distance between 8-row groups: 1024 in a
+// query tile, GROUP_BYTES in a K/V tile; version 1; 128B swizzle); the low word is
+// (address >> 4) | LBO << 16, so stepping through a tile is one add.
+template <int D>
+struct Desc {
+  static constexpr uint32_t HI_Q = (1024u >> 4) | (1u << 14) | (2u << 29);
+  static constexpr uint32_t HI_KV = ((uint32_t)Smem<D>::GROUP_BYTES >> 4) | (1u << 14) | (2u << 29);
+  static constexpr uint32_t LBO_K = 1u << 16;                                      // K-major: LBO unused
+  static constexpr uint32_t LBO_V = (1024u >> 4) << 16;                            // MN-major: next 64 dims
+  static __device__ __forceinline__ uint64_t q(uint32_t lo) { return (static_cast<uint64_t>(HI_Q) << 32) | lo; }
+  static __device__ __forceinline__ uint64_t kv(uint32_t lo) { return (static_cast<uint64_t>(HI_KV) << 32) | lo; }
+};
+
+template <int D>
+struct PvIssuer {
+  using L = Smem<D>;
+  static constexpr uint32_t V_OFF = L::KV_OFF + L::NK * L::KV_BYTES;
+  const Cta<D>& c;
+  int slot = 0;
+  uint32_t phase = 0, n[2] = {0, 0};                        // ring position; steps of each stream so far
+
+  // O_st (+)= P_st V of the step in ring entry `slot`; P from TMEM
+  __device__ __forceinline__ void issue(int st, uint32_t first) {
+    const uint32_t v_lo = (((c.smem_base + V_OFF) >> 4) | Desc<D>::LBO_V) + slot * (L::KV_BYTES >> 4);
+    constexpr uint32_t IDESC = instr_desc(D, 1);
+#pragma unroll
+    for (int k = 0; k < BN / 16; ++k)
+      umma_bf16_ts(c.tmem_O + st * D, c.tmem_P + st * L::SP_COLS + k * 8, Desc<D>::kv(v_lo + k * (L::PAGE_BYTES >> 4)), IDESC,
+                   (!first || k > 0) ? 1u : 0u);
+  }
+  // V rows past the visible range hold stale or foreign data; P is 0 there but
+  // 0 * NaN would poison O, so clear them before the step's values are used.
+  __device__ __forceinline__ void clear_tail(const Work& it, int step) {
+    const int keys = it.kv_cap - it.key0 - step * BN;
+    if (keys < BN) {
+      uint8_t* vb = c.smem_gen + V_OFF + slot * L::KV_BYTES;
+      const int first = max(keys, 0);
+      const int chunks = (BN - first) * 8;                  // 16-byte chunks to clear per 64-dim half
+#pragma unroll
+      for (int h = 0; h < L::HALVES; ++h)
+        for (int idx = c.lane; idx < chunks; idx += 32) {
+          const int key = first + (idx >> 3);
+          *reinterpret_cast<uint4*>(vb + (key >> 3) * L::GROUP_BYTES + h * 1024 + (key & 7) * 128 + ((idx & 7) << 4)) =
+              make_uint4(0, 0, 0, 0);
+        }
+      fence_async_smem();
+      __syncwarp();
+    }
+  }
+  template <bool DUAL>
+  __device__ __forceinline__ void item(const Work& it) {
+    const int cnt0 = it.steps(0), cnt1 = it.steps(1);
+    for (int k = 0; k < cnt0; ++k) {
+#pragma unroll
+      for (int st = 0; st < 2; ++st) {
+        if (k >= (st == 0 ? cnt0 : cnt1)) continue;
+        const bool last_user = !DUAL || st == 1;            // last stream to touch this V tile
+        if (!DUAL || st == 0) {
+          c.wait(BAR_VFULL + slot, phase);
+          clear_tail(it, DUAL ? k : 2 * k + st);
+        }
+        c.wait(BAR_P + st, n[st] & 1);
+        ++n[st];
+        tc_fence_after();
+        if (elect_one()) {
+          issue(st, k == 0);
+          if (last_user) tc_commit(c.bar(BAR_VEMPTY + slot));
+          tc_commit(c.bar(BAR_PV + st));
+        }
+        __syncwarp();
+        if (last_user && ++slot == L::NV) { slot = 0; phase ^= 1; }
+      }
+    }
+  }
+};
+
+template <int D>
+struct QkIssuer {
+  using L = Smem<D>;
+  const Cta<D>& c;
+  int slot = 0;
+  uint32_t phase = 0, n[2] = {0, 0}, q_phase[2] = {0, 0};
+  bool apart = false;                                       // the streams run half a step apart already
+
+  __device__ __forceinline__ void issue(int st, int tile) {
+    const uint32_t k_lo = (((c.smem_base + L::KV_OFF) >> 4) | Desc<D>::LBO_K) + slot * (L::KV_BYTES >> 4);
+    const uint32_t a_lo = (((c.smem_base + L::Q_OFF) >> 4) | Desc<D>::LBO_K) + tile * (L::Q_BYTES >> 4);
+    constexpr uint32_t IDESC = instr_desc(BN, 0);
+#pragma unroll
+    for (int k = 0; k < D / 16; ++k) {
+      const uint32_t off_q = ((k >> 2) * L::HALF_BYTES + (k & 3) * 32) >> 4;
+      const uint32_t off_k = ((k >> 2) * 1024 + (k & 3) * 32) >> 4;
+      umma_bf16(c.tmem_S + st * L::SP_COLS, Desc<D>::q(a_lo + off_q), Desc<D>::kv(k_lo + off_k), IDESC, k > 0 ? 1u : 0u);
+    }
+  }
+  template <bool DUAL>
+  __device__ __forceinline__ void item(const Work& it) {
+    const int cnt0 = it.steps(0), cnt1 = it.steps(1);
+    // The streams share the tensor core and the exponential unit, so they should run half a step
+    // apart: stream 1 starts when stream 0 has its first probabilities.  (Started together they
+    // stay together: 2,236 cycles per step against 1,796.)  From one item of two tiles to the next they stay
+    // apart by themselves; where an item's end brings them together they are set apart again.  (The first wait makes the
+    // second one's phase the next to come; it cannot move on meanwhile: stream 0's next scores are issued here.)
+    const bool set_apart = !(DUAL && apart);
+    const uint32_t p0 = n[0] & 1;
+    if (set_apart && n[0] > 0) c.wait(BAR_P + 0, p0 ^ 1);
+    for (int k = 0; k < cnt0; ++k) {
+#pragma unroll
+      for (int st = 0; st < 2; ++st) {
+        if (k >= (st == 0 ? cnt0 : cnt1)) continue;
+        const bool last_user = !DUAL || st == 1;            // last stream to touch this K tile
+        if (k == 0 && (DUAL || st == 0)) {
+          c.wait(BAR_Q + st, q_phase[st]);
+          q_phase[st] ^= 1;
+        }
+        if (!DUAL || st == 0) c.wait(BAR_KFULL + slot, phase);
+        if (n[st] > 0) c.wait(BAR_SFREE + st, (n[st] - 1) & 1);
+        if (k == 0 && st == 1 && set_apart) c.wait(BAR_P + 0, p0);
+        ++n[st];
+        tc_fence_after();
+        if (elect_one()) {
+          issue(st, DUAL ? st : 0);
+          tc_commit(c.bar(BAR_S + st));
+          if (last_user) tc_commit(c.bar(BAR_KEMPTY + slot));
+        }
+        __syncwarp();
+        if (last_user && ++slot == L::NK) { slot = 0; phase ^= 1; }
+      }
+    }
+    apart = DUAL;
+  }
+};
+
+// A CTA walks items: its own block index's first, then, one at a time, those of blocks of the launch that have not
+// started yet, until none is left - so the hardware's order and balance stay, and what a fresh CTA costs outside its
+// steps is paid once: the next item's pages are copied while the present one's last steps run, its query rows under
+// the last PV, its first scores under the epilogue.  A CTA per item spent 14,000 cycles of each outside the steps (of
+// 2,000); between two items it is 8,000.  Append and attention, one CTA per item -> this: 16 prompts of 1-3.5k tokens
+// 1,028 -> 970 us, 16 x 8-112 tokens over 1-3.4k planned in the call 69 -> 65, 64 mixed rows at 28/4 heads 320 -> 307,
+// 16 x 32-256 over 2-8k at 32/32 320 -> 308, 8 x 3,200 over 5k 2,590 -> 2,490.
+// The work list: in the workspace (List = NoList), or, a short one planned inside the call, in the launch
+// parameters (List = InlineItems) - which saves the copy between the append and this kernel.
+template <int D, typename List>
+__global__ void __launch_bounds__(THREADS, 1)
+prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                  const __grid_constant__ List list) {
+  using L = Smem<D>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t bars = smem_base + L::BAR_OFF;
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + L::BAR_OFF + BAR_COUNT * 8);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + L::BAR_OFF + BAR_COUNT * 8 + 8);
-  auto bar = [&](int i) { return bars + 8u * i; };
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int G = p.G;
-  const int C = it.cached, N = it.new_len, tok0 = it.tok0;
-  const int rows_total = N * G;
-  const int rows_here = min(NQ * BM, rows_total - it.row0);
-  constexpr bool dual = MODE == 1;                           // two query tiles (rows_here > BM)
-  constexpr bool tiny = MODE == 2;                           // at most 32 rows, held four times
-  const int i_last = (it.row0 + rows_here - 1) / G;          // last token of this CTA
-  // keys of this CTA: [key0, kv_cap) - its tiles of the work list, up to what its last row sees
-  const int key0 = it.tile_begin * PT;
-  const int kv_cap = min(C + i_last + 1, it.tile_end * PT);
-  const int nt = (kv_cap - key0 + BN - 1) / BN;              // steps of BN keys
-  const int cnt0 = dual ? nt : (nt + 1) >> 1;                // steps of stream 0 / 1
-  const int cnt1 = dual ? nt : nt >> 1;
-  // K and V rings.  With one query tile the second tile's shared memory is one more K entry.
-  constexpr int nk = dual ? L::NK : L::NK_MAX, nv = L::NV;
-  constexpr uint32_t k_off = dual ? L::KV_OFF : L::KV_OFF - L::KV_BYTES;
-  constexpr uint32_t v_off = L::KV_OFF + L::NK * L::KV_BYTES;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + L::TMEM_SLOT_OFF);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + L::ABORT_OFF);
+  auto bar = [&](int i) { return smem_base + L::BAR_OFF + 8u * i; };
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
 
   if (tid == 0) {
     for (int t = 0; t < NQ; ++t) {
@@ -464,13 +1166,15 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
       mbar_init(bar(BAR_SFREE + t), 4);
       mbar_init(bar(BAR_P + t), 4);
       mbar_init(bar(BAR_PV + t), 1);
-      mbar_init(bar(BAR_O + t), 1);
+      mbar_init(bar(BAR_IFULL + t), 1);
+      mbar_init(bar(BAR_IEMPTY + t), 11);
     }
-    for (int s = 0; s < nk; ++s) {
+    for (int s = 0; s < 4; ++s) mbar_init(bar(BAR_PAIR + s), 2);
+    mbar_init(bar(BAR_ALL), 8);
+    mbar_init(bar(BAR_CLAIM), 1);
+    for (int s = 0; s < L::NK; ++s) {
       mbar_init(bar(BAR_KFULL + s), 1);
       mbar_init(bar(BAR_KEMPTY + s), 1);
-    }
-    for (int s = 0; s < nv; ++s) {
       mbar_init(bar(BAR_VFULL + s), 1);
       mbar_init(bar(BAR_VEMPTY + s), 1);
     }
@@ -487,487 +1191,54 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t tmem_S = tmem;                         // S of stream t at columns t * SP_COLS, P (bf16 pairs) behind it
-  const uint32_t tmem_P = tmem + BN;
-  const uint32_t tmem_O = tmem + NQ * L::SP_COLS;       // O of stream t
+  const uint32_t tmem = uniform(*tmem_slot);
+  const Cta<D> c{p, smem_base, smem_gen, abort_flag, tmem, tmem + BN, tmem + NQ * L::SP_COLS, lane};
 
-  // Register split: every warp of a warpgroup runs the same setmaxnreg; the service
-  // group releases first what the two softmax groups then take.
-  if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
+  // Programmatic launch: up to here a CTA has touched nothing but itself; every warp that reads or writes global
+  // memory waits for the kernel before (which may be one that leaves its list in this workspace).
+  WorkItem raw;                                               // 32 bytes: two vector loads, no dependent load after them
+  if constexpr (std::is_same<List, InlineItems>::value) {
+    if (warp != 9 && warp != 10) pdl_wait();
+    raw = list.items[blockIdx.x];
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
+    pdl_wait();
+    const uint4* src = reinterpret_cast<const uint4*>(p.items + blockIdx.x);
+    uint4* dst = reinterpret_cast<uint4*>(&raw);
+    dst[0] = src[0];
+    dst[1] = src[1];
   }
-
-  // Programmatic launch: up to here a CTA with a list of its own has touched nothing but itself; every warp
-  // that reads or writes global memory waits for the kernel before.
-  if (warp < 8 && tiny) {
-    pdl_wait();
-    // ============================================================ softmax groups, 32-row shape
-    const int st = warp >> 2, w = warp & 3;                 // stream, 32-lane quarter
-    const int my_cnt = st == 0 ? cnt0 : cnt1;
-    const int r = w * 32 + lane;                            // tile row == TMEM lane; the query row is `lane`
-    const int R = it.row0 + lane;
-    const bool valid = R < rows_total;
-    const int i_tok = valid ? R / G : 0;
-    const int g = valid ? R - i_tok * G : 0;
-    const int vis = valid ? min(C + i_tok + 1, kv_cap) : kv_cap;
-    const size_t row_off = ((size_t)(tok0 + i_tok) * p.Hq + (size_t)it.kvh * G + g) * D;
-    if (st == 0) {
-      q_rows_to_smem<D>(p, smem_gen + L::Q_OFF, w * 32, lane, valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1, C + i_tok);
-      fence_async_smem();
-      warp_arrive(bar(BAR_Q + 0), lane);
-    }
-    constexpr int KQ = BN / 4;                              // keys of a step this warp scores
-    const uint32_t lane_addr = (uint32_t)(w * 32) << 16;
-    const uint32_t s_addr = tmem_S + lane_addr + st * L::SP_COLS;
-    const uint32_t p_addr = tmem_P + lane_addr + st * L::SP_COLS;
-    const uint32_t o_addr = tmem_O + lane_addr + st * D;
-    // P of this quarter's rows is zero but for the quarter's own keys: cleared once here, the steps
-    // write only columns KQ / 2 * w ...
-    {
-      const uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int c = 0; c < BN / 2; c += 8) tmem_st<8>(p_addr + c, z);
-      tmem_wait_st();
-    }
-    float m_ref = -FLT_MAX, l_sum = 0.f;
-    for (int k = 0; k < my_cnt; ++k) {
-      mbar_wait(bar(BAR_S + st), k & 1, abort_flag, p.status, p.wait_ns);
-      tc_fence_after();
-      uint32_t s[KQ];
-      tmem_ld<KQ>(s_addr + KQ * w, s);
-      tmem_wait_ld<KQ>(s);
+  Work it = work_of(raw, p.G);
+  // Register split: every warp of a warpgroup runs the same setmaxnreg; the service
+  // group releases first what the two softmax groups then take.  (Nothing may come between this and a role's code: past a
+  // point where the two branches meet the compiler plans with fewer registers, and the steps spilled 1.4 KB.)
+  if (warp < 8) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
+    softmax_role<D>(c, it, warp);
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
+    if (warp == 8) {
+      if (p.early_next) pdl_launch();
+      producer_role<D, true>(c, map_k, list, raw, it);
+    } else if (warp == 11) {
+      if (p.early_next) pdl_launch();
+      producer_role<D, false>(c, map_v, list, raw, it);
+    } else if (warp == 9) {
+      PvIssuer<D> pv{c};
+      Mailbox mail;
+      do {
+        if (it.shape == SHAPE_TWO) pv.template item<true>(it);
+        else pv.template item<false>(it);
+      } while (mail.next(c, it));
       tc_fence_before();
-      warp_arrive(bar(BAR_SFREE + st), lane);
-      const int kv0 = key0 + (2 * k + st) * BN + KQ * w;
-      if (__any_sync(0xffffffffu, kv0 + KQ > vis)) {
-#pragma unroll
-        for (int c = 0; c < KQ; ++c)
-          if (kv0 + c >= vis) s[c] = 0xff800000u;           // -inf
-      }
-      float alpha = 1.f;                                    // what O and the sum so far are scaled by
-      if (k < EXACT_STEPS) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
-      uint32_t v[KQ / 2];
-      float sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
-      if (k > 0) {
-        mbar_wait(bar(BAR_PV + st), (k - 1) & 1, abort_flag, p.status, p.wait_ns);   // P of the step before is consumed
-        tc_fence_after();
-        const bool redo = !(sum <= SUM_LIMIT);
-        if (__any_sync(0xffffffffu, redo || alpha != 1.f)) {
-          if (redo) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
-          l_sum *= alpha;
-          rescale_o_row<D>(o_addr, alpha);
-          if (__any_sync(0xffffffffu, redo)) sum = row_exp<KQ>(s, p.scale_log2, -m_ref, v);
-        }
-      }
-      tmem_st<KQ / 2>(p_addr + KQ / 2 * w, v);
-      tmem_wait_st();
-      tc_fence_before();
-      warp_arrive(bar(BAR_P + st), lane);
-      l_sum += sum;
-    }
-    // ---- epilogue: all MMAs of both streams done (the ring is quiet), then the eight states of
-    // every row meet in the ring's shared memory
-    mbar_wait(bar(BAR_O + 0), 0, abort_flag, p.status, p.wait_ns);
-    if (cnt1 > 0) mbar_wait(bar(BAR_O + 1), 0, abort_flag, p.status, p.wait_ns);
-    tc_fence_after();
-    float* xb = reinterpret_cast<float*>(smem_gen + L::KV_OFF);         // [8 states][32 rows][XROW]
-    const int sidx = st * 4 + w;
-    float* mine = xb + (size_t)(sidx * 32 + lane) * L::XROW;
-    const bool have = my_cnt > 0 && !(l_sum == 0.f);         // (a sum of NaN is handed on, not dropped)
-    mine[D] = have ? m_ref : -INFINITY;
-    mine[D + 1] = have ? l_sum : 0.f;
-#pragma unroll
-    for (int c0 = 0; c0 < D; c0 += 32) {
-      uint32_t o[32];
-      if (my_cnt > 0) {                                                 // warp-uniform: the load is warp-wide
-        tmem_ld<32>(o_addr + c0, o);
-        tmem_wait_ld<32>(o);
-      }
-#pragma unroll
-      for (int c = 0; c < 32; c += 4)
-        *reinterpret_cast<uint4*>(mine + c0 + c) =
-            have ? make_uint4(o[c], o[c + 1], o[c + 2], o[c + 3]) : make_uint4(0, 0, 0, 0);
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    tiny_merge_store<D>(p.out, p.lse, p.part_o, p.part_lse, p.s_max, xb, lane, sidx, valid, it.chunk, row_off,
-                        (size_t)(tok0 + i_tok) * p.Hq + (size_t)it.kvh * G + g);
-    tc_fence_before();
-  } else if (warp < 8) {
-    pdl_wait();
-    // ============================================================ softmax groups
-    const int st = warp >> 2;                               // stream
-    const int my_cnt = st == 0 ? cnt0 : cnt1;
-    const int qt = dual ? st : 0;                           // query tile of this stream
-    const int r = (warp & 3) * 32 + lane;                   // tile row == TMEM lane
-    const int R = it.row0 + qt * BM + r;                    // packed row of the (seq, kv head)
-    const bool valid = R < rows_total;
-    const int i_tok = valid ? R / G : 0;
-    const int g = valid ? R - i_tok * G : 0;
-    // keys this row sees; rows past the sequence are computed like the piece's last row and
-    // dropped (with 0 here they would take the masking path on every tile and slow their group)
-    const int vis = valid ? min(C + i_tok + 1, kv_cap) : kv_cap;
-    const size_t row_off = ((size_t)(tok0 + i_tok) * p.Hq + (size_t)it.kvh * G + g) * D;
-    if (dual || st == 0) {
-      q_rows_to_smem<D>(p, smem_gen + L::Q_OFF + qt * L::Q_BYTES, (warp & 3) * 32, lane, valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1, C + i_tok);
-      fence_async_smem();
-      warp_arrive(bar(BAR_Q + qt), lane);
-    }
-    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t s_addr = tmem_S + lane_addr + st * L::SP_COLS;
-    const uint32_t p_addr = tmem_P + lane_addr + st * L::SP_COLS;
-    const uint32_t o_addr = tmem_O + lane_addr + st * D;
-    const int exact = !dual || nt <= EXACT_MAX_STEPS ? EXACT_STEPS : 1;
-    float m_ref = -FLT_MAX, l_sum = 0.f;
-    for (int k = 0; k < my_cnt; ++k) {
-      mbar_wait(bar(BAR_S + st), k & 1, abort_flag, p.status, p.wait_ns);
-      tc_fence_after();
-      uint32_t s[BN];
-      // The scores come in two parts, the exponentials of the first running under the second's load, and P is
-      // stored before its sum is checked: what a stream cannot overlap with itself is what its step takes
-      // (8 x 128 tokens over 8k 155 -> 145 us for append and attention, 8 x 3,200 over 5k 2.59 -> 2.55 ms, 64
-      // mixed rows 312 -> 306; first parts of 32 and 64 keys: 156 and 145 us, 2.71 and 2.56 ms).
-      constexpr int LA = 48;
-      tmem_ld<LA>(s_addr, s);
-      tmem_wait_ld<LA>(s);
-      tmem_ld<BN - LA>(s_addr + LA, s + LA);
-      const int kv0 = key0 + (dual ? k : 2 * k + st) * BN;
-      const bool edge = __any_sync(0xffffffffu, kv0 + BN > vis);
-      if (edge) {
-        tmem_wait_ld<BN - LA>(s + LA);
-#pragma unroll
-        for (int c = 0; c < BN; ++c)
-          if (kv0 + c >= vis) s[c] = 0xff800000u;           // -inf
-      }
-      // The first steps' exact maximum is the row's reference; later steps only check that their sum stays
-      // in range (SUM_LIMIT), so they have no row maximum to take before their first exponential.
-      auto freed = [&]() {
-        tmem_wait_ld<BN - LA>(s + LA);
-        tc_fence_before();
-        warp_arrive(bar(BAR_SFREE + st), lane);             // the next step's scores may be computed
-      };
-      if (edge || k < exact) freed();
-      // alpha: what O and the sum so far are scaled by.  A moved reference lowers the limit, so that the one
-      // test below finds it (a second condition there: 8 x 128 tokens over 8k 150.0 -> 152.6 us).
-      float alpha = 1.f, limit = SUM_LIMIT;
-      if (k < exact) {
-        alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
-        if (alpha != 1.f) limit = -1.f;
-      }
-      uint32_t w[BN / 2];                                   // P as bf16 pairs
-      const float neg_m = -m_ref;
-      float sum = row_exp<LA>(s, p.scale_log2, neg_m, w);
-      if (!(edge || k < exact)) freed();
-      sum += row_exp<BN - LA>(s + LA, p.scale_log2, neg_m, w + LA / 2);
-      if (k > 0) {
-        mbar_wait(bar(BAR_PV + st), (k - 1) & 1, abort_flag, p.status, p.wait_ns);   // P of the step before is consumed
-        tc_fence_after();
-      }
-      tmem_st<BN / 2>(p_addr, w);
-      if (__any_sync(0xffffffffu, !(sum <= limit)) && k > 0) {
-        // (O is quiet: PV(k-1) has finished and PV(k) waits for this warp)
-        const bool redo = !(sum <= SUM_LIMIT);
-        if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
-        l_sum *= alpha;
-        rescale_o_row<D>(o_addr, alpha);
-        if (__any_sync(0xffffffffu, redo)) {
-          sum = row_exp<BN>(s, p.scale_log2, -m_ref, w);
-          tmem_wait_st();                                   // two stores to the same columns are not ordered by themselves
-          tmem_st<BN / 2>(p_addr, w);
-        }
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      warp_arrive(bar(BAR_P + st), lane);
-      l_sum += sum;
-    }
-    // ---- epilogue
-    if (my_cnt > 0) {
-      mbar_wait(bar(BAR_O + st), 0, abort_flag, p.status, p.wait_ns);
-      if (!dual && cnt1 > 0) mbar_wait(bar(BAR_O + (st ^ 1)), 0, abort_flag, p.status, p.wait_ns);   // ring is quiet
-      tc_fence_after();
-    }
-    float* xbuf = reinterpret_cast<float*>(smem_gen + L::KV_OFF) + r * L::XROW;
-    const bool merge = !dual && cnt1 > 0;
-    if (merge && st == 1) {
-      // stream 1 hands its state to stream 0 through shared memory
-      xbuf[D] = m_ref;
-      xbuf[D + 1] = l_sum;
-#pragma unroll
-      for (int c0 = 0; c0 < D; c0 += 32) {
-        uint32_t o[32];
-        tmem_ld<32>(o_addr + c0, o);
-        tmem_wait_ld<32>(o);
-#pragma unroll
-        for (int c = 0; c < 32; c += 4)
-          *reinterpret_cast<uint4*>(xbuf + c0 + c) = make_uint4(o[c], o[c + 1], o[c + 2], o[c + 3]);
-      }
-    }
-    if (merge) asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (my_cnt > 0 && (dual || st == 0)) {
-      float w0 = 1.f, w1 = 0.f;
-      if (merge) {
-        const float m1 = xbuf[D], l1 = xbuf[D + 1];
-        const float M = fmaxf(m_ref, m1);
-        w0 = l_sum == 0.f ? 0.f : ex2(m_ref - M);
-        w1 = l1 == 0.f ? 0.f : ex2(m1 - M);
-        l_sum = l_sum * w0 + l1 * w1;
-        m_ref = M;
-      }
-      const float inv = l_sum == 0.f ? 0.f : 1.f / l_sum;
-      const float lse2 = l_sum == 0.f ? -INFINITY : m_ref + log2f(l_sum);
-      const float a0 = w0 * inv, a1 = w1 * inv;
-      const int th = valid ? (tok0 + i_tok) * p.Hq + it.kvh * G + g : -1;
-      // The rows leave through the query tile's space (its MMAs are done; a warp uses its own 32 rows
-      // only): a lane writes its row, then the warp stores whole rows, two or four per instruction
-      // (with a row per lane every store touched 32 lines: 16 prompts of 1-3.5k tokens lost 41 us to that).
-      constexpr int VEC = D / 8, RPI = 32 / VEC;
-      uint8_t* tile = smem_gen + L::Q_OFF + qt * L::Q_BYTES;
-      auto slot_of = [&](int row, int c) {
-        return reinterpret_cast<uint4*>(tile + (c >> 3) * L::HALF_BYTES + row * 128 + (((c & 7) ^ (row & 7)) << 4));
-      };
-      const int cc = lane % VEC, sub = lane / VEC;
-      auto load_o = [&](int c0, float* f) {                 // 32 columns of this row, both streams' states merged
-        uint32_t o[32];
-        tmem_ld<32>(o_addr + c0, o);
-        tmem_wait_ld<32>(o);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) f[c] = __uint_as_float(o[c]) * a0;
-        if (merge) {
-#pragma unroll
-          for (int c = 0; c < 32; c += 4) {
-            const float4 x = *reinterpret_cast<const float4*>(xbuf + c0 + c);
-            f[c] = fmaf(x.x, a1, f[c]);
-            f[c + 1] = fmaf(x.y, a1, f[c + 1]);
-            f[c + 2] = fmaf(x.z, a1, f[c + 2]);
-            f[c + 3] = fmaf(x.w, a1, f[c + 3]);
-          }
-        }
-      };
-      if (it.chunk < 0) {
-#pragma unroll
-        for (int c0 = 0; c0 < D; c0 += 32) {
-          float f[32];
-          load_o(c0, f);
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            *slot_of(r, c0 / 8 + c) =
-                make_uint4(pack_bf16x2(f[c * 8], f[c * 8 + 1]), pack_bf16x2(f[c * 8 + 2], f[c * 8 + 3]),
-                           pack_bf16x2(f[c * 8 + 4], f[c * 8 + 5]), pack_bf16x2(f[c * 8 + 6], f[c * 8 + 7]));
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-          const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
-          const uint4 x = *slot_of((warp & 3) * 32 + i * RPI + sub, cc);
-          if (t >= 0) reinterpret_cast<uint4*>(p.out)[(size_t)t * VEC + cc] = x;
-        }
-      } else {
-        // a partial is fp32: half a row at a time fills the same space
-#pragma unroll
-        for (int hb = 0; hb < 2; ++hb) {
-#pragma unroll
-          for (int c0 = 0; c0 < D / 2; c0 += 32) {
-            float f[32];
-            load_o(hb * (D / 2) + c0, f);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-              *slot_of(r, c0 / 4 + c) = make_uint4(__float_as_uint(f[4 * c]), __float_as_uint(f[4 * c + 1]),
-                                                   __float_as_uint(f[4 * c + 2]), __float_as_uint(f[4 * c + 3]));
-          }
-          __syncwarp();
-#pragma unroll
-          for (int i = 0; i < VEC; ++i) {
-            const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
-            const uint4 x = *slot_of((warp & 3) * 32 + i * RPI + sub, cc);
-            if (t >= 0)
-              *reinterpret_cast<uint4*>(p.part_o + ((size_t)t * p.s_max + it.chunk) * D + hb * (D / 2) + cc * 4) = x;
-          }
-          __syncwarp();
-        }
-      }
-      if (valid) {
-        if (it.chunk < 0) {
-          if (p.lse) p.lse[th] = lse2 * 0.6931471805599453f;
-        } else {
-          p.part_lse[(size_t)th * p.s_max + it.chunk] = lse2;
-        }
-      }
-    }
-    tc_fence_before();
-  } else if (warp == 8 || warp == 11) {
-    pdl_wait();
-    if (p.early_next) pdl_launch();
-    // ============================================================ TMA producers
-    // Every bulk-tensor copy costs its issuing warp ~65 cycles (one box per page: 16 slots x all dims
-    // of one kv head).  Warp 8 loads the K tiles and warp 11 the V tiles.
-    const int page_l = lane;
-    const int32_t* bt = p.block_table + (size_t)it.seq * p.max_pages_per_seq + (key0 >> 4);
-    const int n_pages = (kv_cap - key0 + 15) >> 4;          // pages this CTA reads
-    // page id of this lane in step jj: -2 if the lane fetches none (lanes beyond the step's visible
-    // pages; the last test only matters for a plan that does not belong to this block table), -1 for
-    // any negative entry
-    auto lookup = [&](int jj) {
-      const int pg = jj * (BN / 16) + page_l;
-      if (page_l >= BN / 16 || pg >= n_pages || (key0 >> 4) + pg >= p.max_pages_per_seq) return -2;
-      return max(bt[pg], -1);
-    };
-    auto produce = [&](auto k_role) {                       // (the ring's constants fold into each copy)
-      constexpr bool is_k = decltype(k_role)::value;
-      const CUtensorMap* my_map = is_k ? &map_k : &map_v;
-      constexpr int n_ring = is_k ? nk : nv;
-      constexpr uint32_t my_off = is_k ? k_off : v_off;
-      constexpr int full = is_k ? BAR_KFULL : BAR_VFULL, empty = is_k ? BAR_KEMPTY : BAR_VEMPTY;
-      // the block-table read is a dependent global load in front of every copy: fetch it two steps ahead
-      int pid_a = lookup(0), pid_b = lookup(1);
-      int slot = 0;
-      uint32_t phase = 0;
-      for (int jj = 0; jj < nt; ++jj) {
-        const int pid = pid_a;
-        pid_a = pid_b;
-        pid_b = lookup(jj + 2);
-        const bool ok = pid >= 0 && pid < p.num_pages;
-        const bool bad = pid != -2 && !ok;                  // an id outside the pool: reported, never dereferenced
-        const uint32_t okmask = __ballot_sync(0xffffffffu, ok);
-        const bool any_bad = __any_sync(0xffffffffu, bad);
-        const uint32_t bytes = __popc(okmask) * (uint32_t)L::PAGE_BYTES;
-        mbar_wait(bar(empty + slot), phase ^ 1, abort_flag, p.status, p.wait_ns);
-        const uint32_t dst_off = my_off + slot * L::KV_BYTES + page_l * L::PAGE_BYTES;
-        if (any_bad) {
-          // the page's 16 keys are replaced by zeros (score 0, value 0), so the tile holds nothing
-          // undefined; written with ordinary stores, made visible to the tensor core's reads
-          if (bad) {
-            if (is_k && p.status) atomicOr(p.status, EFIM_DEV_BAD_PAGE);
-            uint4* z = reinterpret_cast<uint4*>(smem_gen + dst_off);
-            for (int i = 0; i < L::PAGE_BYTES / 16; ++i) z[i] = make_uint4(0, 0, 0, 0);
-            fence_async_smem();
-          }
-          __syncwarp();
-        }
-        if (lane == 0) mbar_expect_tx(bar(full + slot), bytes);
-        __syncwarp();
-        if (ok) tma_load_page(smem_base + dst_off, my_map, bar(full + slot), pid * p.Hkv + it.kvh);
-        if (++slot == n_ring) { slot = 0; phase ^= 1; }
-      }
-      // if the CTA gave up, let copies that are still in flight land before shared memory goes away
-      if (*abort_flag) {
-        for (int jj = max(0, nt - n_ring); jj < nt; ++jj) mbar_drain(bar(full + jj % n_ring), (jj / n_ring) & 1);
-      }
-    };
-    if (warp == 8) produce(std::true_type{});
-    else produce(std::false_type{});
-  } else if (warp == 9 || warp == 10) {
-    // ============================================================ MMA issuers
-    // Issuing an MMA costs its thread nearly as long as the tensor core needs to run it,
-    // so the work is split: warp 9 issues the PV MMAs of both streams, warp 10 the QK
-    // MMAs.  QK(k+1) of a stream needs S(k) read (barrier SFREE), PV(k) needs P(k) written:
-    // neither waits for the other, so the tensor core has a stream's next scores ready when
-    // its softmax warps come back for them.
-    const bool pv_role = warp == 9;
-    constexpr uint32_t IDESC_QK = instr_desc(BN, 0);
-    constexpr uint32_t IDESC_PV = instr_desc(D, 1);
-    // Descriptors: the high word is fixed (SBO = distance between 8-row groups: 1024 in a
-    // query tile, GROUP_BYTES in a K/V tile; version 1; 128B swizzle); the low word is
-    // (address >> 4) | LBO << 16, so stepping through a tile is one add.
-    constexpr uint32_t DESC_HI_Q = (1024u >> 4) | (1u << 14) | (2u << 29);
-    constexpr uint32_t DESC_HI_KV = ((uint32_t)L::GROUP_BYTES >> 4) | (1u << 14) | (2u << 29);
-    constexpr uint32_t LBO_K = 1u << 16;                                           // K-major: LBO unused
-    constexpr uint32_t LBO_V = (1024u >> 4) << 16;                                 // MN-major: next 64 dims
-    auto desc_q = [&](uint32_t lo) { return (static_cast<uint64_t>(DESC_HI_Q) << 32) | lo; };
-    auto desc = [&](uint32_t lo) { return (static_cast<uint64_t>(DESC_HI_KV) << 32) | lo; };
-    int slot = 0;
-    uint32_t phase = 0;
-    if (pv_role) {
-      const uint32_t v_lo0 = ((smem_base + v_off) >> 4) | LBO_V;
-      // O_st (+)= P_st V of the step in ring entry `slot`; P from TMEM
-      auto issue_pv = [&](int st, uint32_t first) {
-        const uint32_t v_lo = v_lo0 + slot * (L::KV_BYTES >> 4);
-#pragma unroll
-        for (int k = 0; k < BN / 16; ++k)
-          umma_bf16_ts(tmem_O + st * D, tmem_P + st * L::SP_COLS + k * 8, desc(v_lo + k * (L::PAGE_BYTES >> 4)),
-                       IDESC_PV, (!first || k > 0) ? 1u : 0u);
-      };
-      // V rows past the visible range hold stale or foreign data; P is 0 there but
-      // 0 * NaN would poison O, so clear them before the step's values are used.
-      auto clear_v_tail = [&](int n) {
-        const int keys = kv_cap - key0 - n * BN;
-        if (keys < BN) {
-          uint8_t* vb = smem_gen + v_off + slot * L::KV_BYTES;
-          const int first = max(keys, 0);
-          const int chunks = (BN - first) * 8;              // 16-byte chunks to clear per 64-dim half
-#pragma unroll
-          for (int h = 0; h < HALVES; ++h)
-            for (int idx = lane; idx < chunks; idx += 32) {
-              const int key = first + (idx >> 3);
-              *reinterpret_cast<uint4*>(vb + (key >> 3) * L::GROUP_BYTES + h * 1024 + (key & 7) * 128 +
-                                        ((idx & 7) << 4)) = make_uint4(0, 0, 0, 0);
-            }
-          fence_async_smem();
-          __syncwarp();
-        }
-      };
-      for (int k = 0; k < cnt0; ++k) {
-#pragma unroll
-        for (int st = 0; st < 2; ++st) {
-          const int my_cnt = st == 0 ? cnt0 : cnt1;
-          if (k >= my_cnt) continue;
-          const bool last_user = !dual || st == 1;          // last stream to touch this V tile
-          if (!dual || st == 0) {
-            mbar_wait(bar(BAR_VFULL + slot), phase, abort_flag, p.status, p.wait_ns);
-            clear_v_tail(dual ? k : 2 * k + st);
-          }
-          mbar_wait(bar(BAR_P + st), k & 1, abort_flag, p.status, p.wait_ns);
-          tc_fence_after();
-          if (elect_one()) {
-            issue_pv(st, k == 0);
-            if (last_user) tc_commit(bar(BAR_VEMPTY + slot));
-            tc_commit(bar(k + 1 == my_cnt ? BAR_O + st : BAR_PV + st));
-          }
-          __syncwarp();
-          if (last_user && ++slot == nv) { slot = 0; phase ^= 1; }
-        }
-      }
     } else {
-      const uint32_t k_lo0 = ((smem_base + k_off) >> 4) | LBO_K, q_lo = ((smem_base + L::Q_OFF) >> 4) | LBO_K;
-      auto issue_qk = [&](int st) {
-        const uint32_t k_lo = k_lo0 + slot * (L::KV_BYTES >> 4);
-        const uint32_t a_lo = q_lo + (dual ? st : 0) * (L::Q_BYTES >> 4);
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint32_t off_q = ((k >> 2) * L::HALF_BYTES + (k & 3) * 32) >> 4;
-          const uint32_t off_k = ((k >> 2) * 1024 + (k & 3) * 32) >> 4;
-          umma_bf16(tmem_S + st * L::SP_COLS, desc_q(a_lo + off_q), desc(k_lo + off_k), IDESC_QK, k > 0 ? 1u : 0u);
-        }
-      };
-      mbar_wait(bar(BAR_Q + 0), 0, abort_flag, p.status, p.wait_ns);
-      if (dual) mbar_wait(bar(BAR_Q + 1), 0, abort_flag, p.status, p.wait_ns);
-      for (int k = 0; k < cnt0; ++k) {
-#pragma unroll
-        for (int st = 0; st < 2; ++st) {
-          const int my_cnt = st == 0 ? cnt0 : cnt1;
-          if (k >= my_cnt) continue;
-          const bool last_user = !dual || st == 1;          // last stream to touch this K tile
-          if (!dual || st == 0) mbar_wait(bar(BAR_KFULL + slot), phase, abort_flag, p.status, p.wait_ns);
-          if (k > 0) mbar_wait(bar(BAR_SFREE + st), (k - 1) & 1, abort_flag, p.status, p.wait_ns);
-          // The streams share the tensor core and the exponential unit, so they should run half a step
-          // apart: stream 1 starts when stream 0 has its first probabilities.  (Started together they
-          // stay together: 2,236 cycles per step against 1,796.  The barrier cannot move on by another
-          // phase meanwhile: stream 0's next scores are issued by this warp.)
-          if (k == 0 && st == 1) mbar_wait(bar(BAR_P + 0), 0, abort_flag, p.status, p.wait_ns);
-          tc_fence_after();
-          if (elect_one()) {
-            issue_qk(st);
-            tc_commit(bar(BAR_S + st));
-            if (last_user) tc_commit(bar(BAR_KEMPTY + slot));
-          }
-          __syncwarp();
-          if (last_user && ++slot == nk) { slot = 0; phase ^= 1; }
-        }
-      }
+      QkIssuer<D> qk{c};
+      Mailbox mail;
+      do {
+        if (it.shape == SHAPE_TWO) qk.template item<true>(it);
+        else qk.template item<false>(it);
+      } while (mail.next(c, it));
+      tc_fence_before();
     }
-    tc_fence_before();
   }
   __syncthreads();
   if (*abort_flag) {
@@ -979,39 +1250,6 @@ __device__ __forceinline__ void prefill_tc_body(const Params& p, const CUtensorM
   if (warp == 9) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
-  }
-}
-
-// The work list: in the workspace (List = NoList), or, a short one planned inside the call, in the launch
-// parameters (List = InlineItems) - which saves the copy between the append and this kernel.
-template <int D, typename List>
-__global__ void __launch_bounds__(THREADS, 1)
-prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                  const __grid_constant__ List list) {
-  WorkItem it;                                                // 32 bytes: two vector loads, no dependent load after them
-  if constexpr (std::is_same<List, InlineItems>::value) {
-    it = list.items[blockIdx.x];
-  } else {
-    // (after the wait: the kernel before may be one that leaves its list in this workspace)
-    pdl_wait();
-    const uint4* src = reinterpret_cast<const uint4*>(p.items + blockIdx.x);
-    uint4* dst = reinterpret_cast<uint4*>(&it);
-    dst[0] = src[0];
-    dst[1] = src[1];
-  }
-  const int rows_here = it.new_len * p.G - it.row0;
-  // the three shapes of a CTA are separate instantiations: ring size, load order and the
-  // query-tile choice are compile-time constants in the issuing warps' inner loops
-  if (rows_here > BM)
-    prefill_tc_body<D, 1>(p, map_k, map_v, it);
-  else if (rows_here <= 32)
-    prefill_tc_body<D, 2>(p, map_k, map_v, it);
-  else
-    prefill_tc_body<D, 0>(p, map_k, map_v, it);
-  // A work list that came in the launch parameters is left in the workspace like any other: a call that
-  // plans for itself may be followed by planned calls with resident lists.
-  if constexpr (std::is_same<List, InlineItems>::value) {
-    if (threadIdx.x == 0) p.items_out[blockIdx.x] = list.items[blockIdx.x];
   }
 }
 
