@@ -40,6 +40,7 @@ namespace pf {
 // every wait returns at once, and the timeout is recorded in the status word.
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                           unsigned long long limit_ns) {
+  if (__builtin_expect(mbar_try(bar, parity), 1)) return;      // (what follows is laid out behind the loops)
   mbar_wait_bounded(bar, parity, limit_ns, abort_flag, status);
 }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -209,10 +210,11 @@ struct Smem {
   static constexpr int NK = D == 128 ? 3 : 8, NV = NK;            // ring entries
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = Q_OFF + NQ * Q_BYTES;
-  static constexpr int BAR_OFF = KV_OFF + (NK + NV) * KV_BYTES;
+  static constexpr int STAGE_OFF = KV_OFF + (NK + NV) * KV_BYTES;          // output rows on their way out, 4 KB per warp
+  static constexpr int BAR_OFF = STAGE_OFF + 8 * 4096;
   static constexpr int TMEM_SLOT_OFF = BAR_OFF + BAR_COUNT * 8, ABORT_OFF = TMEM_SLOT_OFF + 8;
   static constexpr int ITEM_OFF = (ABORT_OFF + 8 + 15) / 16 * 16;          // mailbox: two work items
-  static constexpr int CLAIM_OFF = ITEM_OFF + 2 * 32;                     // answer to a claim
+  static constexpr int CLAIM_OFF = ITEM_OFF + 2 * 48;                     // answer to a claim
   // Exchange of the 32-row shape: the four quarters' O in the query tiles' space, (reference, sum) here.
   static_assert(4 * 32 * D * 4 <= NQ * Q_BYTES, "the quarters' states must fit in the query tiles");
   static constexpr int ML_OFF = CLAIM_OFF + 16;
@@ -314,7 +316,7 @@ __device__ __noinline__ void q_rows_rotated_to_smem(const uint4* q, const float*
     if (status) atomicOr(status, EFIM_DEV_BAD_POSITION);
     th = -1;
   }
-#pragma unroll 4
+#pragma unroll 1
   for (int i = 0; i < VEC; ++i) {
     const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub), ps = __shfl_sync(0xffffffffu, pos, i * RPI + sub);
     const int r = row0 + i * RPI + sub;
@@ -357,7 +359,7 @@ __device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* smem_ge
     return;
   }
   const int c = lane % VEC, sub = lane / VEC;
-#pragma unroll
+#pragma unroll 1                                            // (see the note on cold code at softmax_item)
   for (int i = 0; i < VEC; ++i) {
     const int t = __shfl_sync(0xffffffffu, th, i * RPI + sub);
     const int r = row0 + i * RPI + sub;
@@ -397,7 +399,13 @@ struct Work {
 __device__ __forceinline__ int uniform(int x) {
   return static_cast<int>(__reduce_or_sync(0xffffffffu, static_cast<unsigned>(x)));
 }
-__device__ __forceinline__ Work work_of(const WorkItem& it, int G) {
+// Token of packed row R (R / G, without a division).
+__device__ __forceinline__ int token_of(const Params& p, int R) {
+  if (p.g_mul == 0) return R;
+  const int t = static_cast<int>(__umulhi(static_cast<unsigned>(R), p.g_mul));
+  return t * p.G > R ? t - 1 : t;
+}
+__device__ __forceinline__ Work work_of(const WorkItem& it, const Params& p) {
   Work w;
   w.seq = uniform(it.seq);
   const int kc = uniform((int)(uint16_t)it.kvh | (int)it.chunk << 16);
@@ -406,9 +414,9 @@ __device__ __forceinline__ Work work_of(const WorkItem& it, int G) {
   w.row0 = uniform(it.row0);
   w.C = uniform(it.cached);
   w.tok0 = uniform(it.tok0);
-  w.rows_total = uniform(it.new_len) * G;
+  w.rows_total = uniform(it.new_len) * p.G;
   const int rows_here = min(NQ * BM, w.rows_total - w.row0);
-  const int i_last = (w.row0 + rows_here - 1) / G;           // last token of this item
+  const int i_last = token_of(p, w.row0 + rows_here - 1);    // last token of this item
   w.key0 = uniform(it.tile_begin) * PT;
   w.kv_cap = min(w.C + i_last + 1, uniform(it.tile_end) * PT);
   w.nt = (w.kv_cap - w.key0 + BN - 1) / BN;
@@ -424,6 +432,7 @@ struct Cta {
   uint32_t smem_base;
   uint8_t* smem_gen;
   volatile int* abort_flag;
+  const CUtensorMap *map_q, *map_out;
   uint32_t tmem_S, tmem_P, tmem_O;       // S of stream t at columns t * SP_COLS, P (bf16 pairs) behind it; O of stream t at t * D
   int lane;
   __device__ __forceinline__ uint32_t bar(int i) const { return smem_base + L::BAR_OFF + 8u * i; }
@@ -438,19 +447,43 @@ struct Mailbox {
   int slot = 0;
   uint32_t phase = 0;
   template <int D>
+  static __device__ __forceinline__ uint4* at(const Cta<D>& c, int slot) {
+    return reinterpret_cast<uint4*>(c.smem_gen + Smem<D>::ITEM_OFF) + 3 * slot;
+  }
+  template <int D>
+  __device__ __forceinline__ void put(const Cta<D>& c, const Work& w) {    // by warp 8; seq -1: no more items
+    c.wait(BAR_IEMPTY + slot, phase ^ 1);
+    if (c.lane == 0) {
+      uint4* dst = at(c, slot);
+      dst[0] = make_uint4(w.seq, (uint32_t)(uint16_t)w.kvh | (uint32_t)w.chunk << 16, w.row0, w.C);
+      dst[1] = make_uint4(w.tok0, w.rows_total, w.key0, w.kv_cap);
+      dst[2] = make_uint4((uint32_t)w.nt << 2 | (uint32_t)w.shape, 0, 0, 0);
+      mbar_arrive(c.bar(BAR_IFULL + slot));
+    }
+    __syncwarp();
+    if (++slot == 2) { slot = 0; phase ^= 1; }
+  }
+  template <int D>
   __device__ __forceinline__ bool next(const Cta<D>& c, Work& w) {
     c.wait(BAR_IFULL + slot, phase);
-    WorkItem it;
-    const uint4* src = reinterpret_cast<const uint4*>(c.smem_gen + Smem<D>::ITEM_OFF) + 2 * slot;
-    uint4* dst = reinterpret_cast<uint4*>(&it);
-    dst[0] = src[0];
-    dst[1] = src[1];
+    const uint4* src = at(c, slot);
+    const uint4 a = src[0], b = src[1];
+    const int ns = uniform(src[2].x), seq = uniform(a.x), kc = uniform(a.y);
     const bool gone = __any_sync(0xffffffffu, *c.abort_flag != 0);
     warp_arrive(c.bar(BAR_IEMPTY + slot), c.lane);
     if (++slot == 2) { slot = 0; phase ^= 1; }
-    if (gone) return false;
-    w = work_of(it, c.p.G);
-    return w.seq >= 0;
+    w.seq = seq;
+    w.kvh = (int)(int16_t)(kc & 0xffff);
+    w.chunk = kc >> 16;
+    w.row0 = uniform(a.z);
+    w.C = uniform(a.w);
+    w.tok0 = uniform(b.x);
+    w.rows_total = uniform(b.y);
+    w.key0 = uniform(b.z);
+    w.kv_cap = uniform(b.w);
+    w.nt = ns >> 2;
+    w.shape = ns & 3;
+    return !gone && seq >= 0;
   }
 };
 
@@ -482,51 +515,102 @@ struct Row {
   __device__ __forceinline__ Row(const Params& p, const Work& it, int qt, int w, int lane) {
     const int R = it.row0 + (it.shape == SHAPE_TINY ? lane : qt * BM + w * 32 + lane);
     valid = R < it.rows_total;
-    const int i_tok = valid ? R / p.G : 0;
+    const int i_tok = valid ? token_of(p, R) : 0;
     pos = it.C + i_tok;
     th = valid ? (it.tok0 + i_tok) * p.Hq + it.kvh * p.G + (R - i_tok * p.G) : -1;
   }
 };
+// 32 rows x 64 dims between a [token][head][dim] array and shared memory (128-byte swizzle): one box is the G heads of
+// 32 / G tokens.  Coordinates (dim % 64, dim / 64, head, token); tokens past the end read as zeros.
+__device__ __forceinline__ void tma_load_rows(uint32_t dst, const CUtensorMap* map, uint32_t bar, int half, int head, int token) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+      "l"(map), "r"(bar), "r"(0), "r"(half), "r"(head), "r"(token)
+      : "memory");
+}
+__device__ __forceinline__ void tma_store_rows(uint32_t src, const CUtensorMap* map, int half, int head, int token) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%1, {%2, %3, %4, %5}], [%0];" ::"r"(src), "l"(map),
+               "r"(0), "r"(half), "r"(head), "r"(token)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// The query rows of a tile, by the four warps of a stream, each its 32-lane quarter.  Where 32 rows are whole tokens they
+// are copied as boxes: per-lane copies kept the softmax warps for 2,300 cycles per item of prompts.  (Rows past the sequence then hold what follows it; nothing of theirs is stored.)
 template <int D>
 __device__ __forceinline__ void fetch_q(const Cta<D>& c, const Work& it, int qt, int w) {
+  using L = Smem<D>;
+  if (c.p.q_tma) {
+    if (c.lane == 0) {
+      const uint32_t bar = c.bar(BAR_Q + qt), dst = c.smem_base + L::Q_OFF + qt * L::Q_BYTES + w * 4096;
+      const int token = it.tok0 + token_of(c.p, it.row0 + (it.shape == SHAPE_TINY ? 0 : qt * BM + w * 32));
+      mbar_expect_tx(bar, L::HALVES * 4096);
+#pragma unroll
+      for (int h = 0; h < L::HALVES; ++h) tma_load_rows(dst + h * L::HALF_BYTES, c.map_q, bar, h, it.kvh * c.p.G, token);
+    }
+    __syncwarp();
+    return;
+  }
   const Row r(c.p, it, qt, w, c.lane);
-  q_rows_to_smem<D>(c.p, c.smem_gen, Smem<D>::Q_OFF + qt * Smem<D>::Q_BYTES, c.smem_base, w * 32, c.lane, r.th, r.pos);
+  q_rows_to_smem<D>(c.p, c.smem_gen, L::Q_OFF + qt * L::Q_BYTES, c.smem_base, w * 32, c.lane, r.th, r.pos);
 }
 template <int D>
 __device__ __forceinline__ void publish_q(const Cta<D>& c, int qt) {
+  if (c.p.q_tma) return;                                    // (the copies complete the barrier)
   asm volatile("cp.async.wait_all;" ::: "memory");
   fence_async_smem();
   warp_arrive(c.bar(BAR_Q + qt), c.lane);
 }
 
-// 32 bytes of a row (`wide`: the rows are 32-byte aligned, one store).
-__device__ __forceinline__ void store32(void* dst, const uint32_t* v, bool wide) {
-  if (wide) {
-    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
-                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                 : "memory");
-  } else {
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
-    reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
-  }
-}
-// N columns of an output row (or, chunk >= 0, of a chunk's partial) from column c0 on.
-template <int D, int N>
-__device__ __forceinline__ void store_cols(const Params& p, int th, int chunk, int c0, const float* f, bool wide) {
-  if (th < 0) return;
-  if (chunk < 0) {
-    uint16_t* dst = p.out + (size_t)th * D + c0;
+// 64 columns (from `col` on) of this warp's 32 output rows, or of a chunk's partials; `th` as in Row, `whole`: all 32
+// rows are of the sequence, from `token` on.  The rows leave through 4 KB of shared memory, as one box, or else 128 bytes
+// of four rows per instruction.  (With a row per lane every store touched 32 lines: 4,200 cycles per item of
+// prompts.  Boxes against instructions only: 16 prompts of 1-3.5k tokens 935 and 954 us.)
+template <int D>
+__device__ __forceinline__ void store_cols(const Cta<D>& c, const Work& it, int warp, int token, int th, bool whole, int col,
+                                           const float* f) {
+  const Params& p = c.p;
+  const uint32_t off = Smem<D>::STAGE_OFF + warp * 4096;
+  auto slot_of = [&](int row, int j) {
+    return reinterpret_cast<uint4*>(c.smem_gen + off + row * 128 + ((j ^ (row & 7)) << 4));
+  };
+  const int j = c.lane & 7, sub = c.lane >> 3;
+  if (c.lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");     // (what left last has been read)
+  __syncwarp();
+  if (it.chunk < 0) {
 #pragma unroll
-    for (int c = 0; c < N; c += 16) {
-      uint32_t v[8];
+    for (int i = 0; i < 8; ++i)
+      *slot_of(c.lane, i) = make_uint4(pack_bf16x2(f[8 * i], f[8 * i + 1]), pack_bf16x2(f[8 * i + 2], f[8 * i + 3]),
+                                       pack_bf16x2(f[8 * i + 4], f[8 * i + 5]), pack_bf16x2(f[8 * i + 6], f[8 * i + 7]));
+    if (whole && p.out_tma) {
+      fence_async_smem();
+      __syncwarp();
+      if (c.lane == 0) tma_store_rows(c.smem_base + off, c.map_out, col / 64, it.kvh * p.G, token);
+    } else {
+      __syncwarp();
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = pack_bf16x2(f[c + 2 * e], f[c + 2 * e + 1]);
-      store32(dst + c, v, wide);
+      for (int i = 0; i < 8; ++i) {
+        const int t = __shfl_sync(0xffffffffu, th, i * 4 + sub);
+        const uint4 x = *slot_of(i * 4 + sub, j);
+        if (t >= 0) *reinterpret_cast<uint4*>(p.out + (size_t)t * D + col + j * 8) = x;
+      }
     }
   } else {
-    float* dst = p.part_o + ((size_t)th * p.s_max + chunk) * D + c0;
 #pragma unroll
-    for (int c = 0; c < N; c += 8) store32(dst + c, reinterpret_cast<const uint32_t*>(f) + c, true);
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *slot_of(c.lane, i) = make_uint4(__float_as_uint(f[32 * h + 4 * i]), __float_as_uint(f[32 * h + 4 * i + 1]),
+                                         __float_as_uint(f[32 * h + 4 * i + 2]), __float_as_uint(f[32 * h + 4 * i + 3]));
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int t = __shfl_sync(0xffffffffu, th, i * 4 + sub);
+        const uint4 x = *slot_of(i * 4 + sub, j);
+        if (t >= 0) *reinterpret_cast<uint4*>(p.part_o + ((size_t)t * p.s_max + it.chunk) * D + col + h * 32 + j * 4) = x;
+      }
+      __syncwarp();
+    }
   }
 }
 __device__ __forceinline__ void store_lse(const Params& p, int th, int chunk, float lse2) {
@@ -645,7 +729,7 @@ __device__ __forceinline__ void softmax_tiny(const Cta<D>& c, const Work& it, in
   auto chunk_at = [&](int q, int j) { return reinterpret_cast<float4*>(x + (q * 32 + c.lane) * D) + (j ^ (c.lane & 7)); };
   if (it.nt > 1) {
     const Pair pr = meet_partner(c, st, w, lane_addr, m_ref, l_sum, pair_phase);
-#pragma unroll
+#pragma unroll 1
     for (int c0 = 0; c0 < D / 2; c0 += 32) {
       const int col = st * (D / 2) + c0;
       uint32_t o0[32], o1[32];
@@ -666,7 +750,7 @@ __device__ __forceinline__ void softmax_tiny(const Cta<D>& c, const Work& it, in
     leave_partner(c, w, pair_phase);
   } else if (st == 0) {
     const bool have = !(l_sum == 0.f);                     // (a sum of NaN is handed on, not dropped)
-#pragma unroll
+#pragma unroll 1
     for (int c0 = 0; c0 < D; c0 += 32) {
       uint32_t o[32];
       tmem_ld<32>(o_addr + c0, o);
@@ -720,7 +804,8 @@ __device__ __forceinline__ void softmax_tiny(const Cta<D>& c, const Work& it, in
       if (d0 == 0) store_lse(p, row.th, it.chunk, Lt == 0.f ? -INFINITY : M + log2f(Lt));
     }
   }
-  // the space may be filled with the next item's queries
+  // the space may be filled with the next item's queries (by copies of the async proxy)
+  fence_async_smem();
   warp_arrive(c.bar(BAR_ALL), c.lane);
   c.wait(BAR_ALL, all_phase);
   all_phase ^= 1;
@@ -728,9 +813,13 @@ __device__ __forceinline__ void softmax_tiny(const Cta<D>& c, const Work& it, in
 
 // One item of more than 32 rows, one query tile or two (DUAL); `n`: steps of this stream so far.  Looks the next item up
 // and gets its query rows on their way; returns false if there is none.
+// A step is some 500 instructions that two warps per scheduler stream through, and a tenth of the stalls are instruction
+// fetches: code that a step rarely or never runs is kept small (rolled loops) and out of its way (__builtin_expect,
+// in the waits too).  Copy loop and epilogue rolled, then the hints: 8 x 128 tokens over 8k 154.7 -> 146.5 -> 145.6 us,
+// 8 x 3,200 over 5k 2,497 -> 2,471 -> 2,441.
 template <int D, bool DUAL>
 __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Work& next, Mailbox& mail, int st, int w,
-                                             bool wide, uint32_t& n, uint32_t& pair_phase) {
+                                             uint32_t& n, uint32_t& pair_phase) {
   using L = Smem<D>;
   const Params& p = c.p;
   const uint32_t lane_addr = (uint32_t)(w * 32) << 16;      // tile row == TMEM lane
@@ -760,7 +849,7 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
     tmem_ld<BN - LA>(s_addr + LA, s + LA);
     const int kv0 = kv_first + k * kv_step;
     const bool edge = __any_sync(0xffffffffu, kv0 + BN > vis);
-    if (edge) {
+    if (__builtin_expect(edge, 0)) {
       tmem_wait_ld<BN - LA>(s + LA);
 #pragma unroll
       for (int i = 0; i < BN; ++i)
@@ -773,25 +862,25 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
       tc_fence_before();
       warp_arrive(c.bar(BAR_SFREE + st), c.lane);           // the next step's scores may be computed
     };
-    if (edge || k < exact) freed();
+    if (__builtin_expect(edge || k < exact, 0)) freed();
     // alpha: what O and the sum so far are scaled by.  A moved reference lowers the limit, so that the one
     // test below finds it (a second condition there: 8 x 128 tokens over 8k 150.0 -> 152.6 us).
     float alpha = 1.f, limit = SUM_LIMIT;
-    if (k < exact) {
+    if (__builtin_expect(k < exact, 0)) {
       alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
       if (alpha != 1.f) limit = -1.f;
     }
     uint32_t v[BN / 2];                                     // P as bf16 pairs
     const float neg_m = -m_ref;
     float sum = row_exp<LA>(s, p.scale_log2, neg_m, v);
-    if (!(edge || k < exact)) freed();
+    if (__builtin_expect(!(edge || k < exact), 1)) freed();
     sum += row_exp<BN - LA>(s + LA, p.scale_log2, neg_m, v + LA / 2);
     if (k > 0) {
       c.wait(BAR_PV + st, (n - 1) & 1);                     // P of the step before is consumed
       tc_fence_after();
     }
     tmem_st<BN / 2>(p_addr, v);
-    if (__any_sync(0xffffffffu, !(sum <= limit)) && k > 0) {
+    if (__builtin_expect(__any_sync(0xffffffffu, !(sum <= limit)) && k > 0, 0)) {
       // (O is quiet: PV(k-1) has finished and PV(k) waits for this warp)
       const bool redo = !(sum <= SUM_LIMIT);
       if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
@@ -824,29 +913,30 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
   }
   if (q_next >= 0) publish_q(c, q_next);
   // ---- epilogue: PV of the next item's first step waits for its P, and with it for the loads of O here
+  const bool whole = __all_sync(0xffffffffu, row.valid);
+  const int token = it.tok0 + token_of(p, it.row0 + (DUAL ? st * BM : 0) + w * 32);
   if (!DUAL && it.nt > 1) {
-    // both streams have a state of every row: each finishes half of the columns
+    // both streams have a state of every row: each finishes half of the columns (at head_dim 64 stream 0 all)
     const Pair pr = meet_partner(c, st, w, lane_addr, m_ref, l_sum, pair_phase);
     const float inv = pr.L == 0.f ? 0.f : 1.f / pr.L;
     const float a0 = pr.w0 * inv, a1 = pr.w1 * inv;
+    if (D == 128 || st == 0) {
+      const int col = D == 128 ? st * 64 : 0;
+      uint32_t o0[64], o1[64];
+      tmem_ld<64>(c.tmem_O + lane_addr + col, o0);
+      tmem_ld<64>(c.tmem_O + lane_addr + D + col, o1);
+      tmem_wait_ld<64>(o0);
+      tmem_wait_ld<64>(o1);
+      float f[64];
 #pragma unroll
-    for (int c0 = 0; c0 < D / 2; c0 += 32) {
-      const int col = st * (D / 2) + c0;
-      uint32_t o0[32], o1[32];
-      tmem_ld<32>(c.tmem_O + lane_addr + col, o0);
-      tmem_ld<32>(c.tmem_O + lane_addr + D + col, o1);
-      tmem_wait_ld<32>(o0);
-      tmem_wait_ld<32>(o1);
-      float f[32];
-#pragma unroll
-      for (int i = 0; i < 32; ++i) f[i] = fmaf(__uint_as_float(o1[i]), a1, __uint_as_float(o0[i]) * a0);
-      store_cols<D, 32>(p, row.th, it.chunk, col, f, wide);
+      for (int i = 0; i < 64; ++i) f[i] = fmaf(__uint_as_float(o1[i]), a1, __uint_as_float(o0[i]) * a0);
+      store_cols<D>(c, it, st * 4 + w, token, row.th, whole, col, f);
     }
     if (st == 0) store_lse(p, row.th, it.chunk, pr.L == 0.f ? -INFINITY : pr.M + log2f(pr.L));
     leave_partner(c, w, pair_phase);
   } else if (my_cnt > 0) {
     const float inv = l_sum == 0.f ? 0.f : 1.f / l_sum;
-#pragma unroll
+#pragma unroll 1
     for (int c0 = 0; c0 < D; c0 += 64) {
       uint32_t o[64];
       tmem_ld<64>(o_addr + c0, o);
@@ -854,7 +944,7 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
       float f[64];
 #pragma unroll
       for (int i = 0; i < 64; ++i) f[i] = __uint_as_float(o[i]) * inv;
-      store_cols<D, 64>(p, row.th, it.chunk, c0, f, wide);
+      store_cols<D>(c, it, st * 4 + w, token, row.th, whole, c0, f);
     }
     store_lse(p, row.th, it.chunk, l_sum == 0.f ? -INFINITY : m_ref + log2f(l_sum));
     tc_fence_before();
@@ -864,9 +954,7 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
 
 template <int D>
 __device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp) {
-  const Params& p = c.p;
   const int st = warp >> 2, w = warp & 3;                   // stream, 32-lane quarter
-  const bool wide = (reinterpret_cast<uintptr_t>(p.out) & 31) == 0;
   Mailbox mail;
   uint32_t n = 0, pair_phase = 0, all_phase = 0;            // steps of this stream so far; phases of the exchange barriers
   if (it.shape == SHAPE_TWO || st == 0) {
@@ -884,12 +972,13 @@ __device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp)
         publish_q(c, st);
       }
     } else {
-      more = it.shape == SHAPE_TWO ? softmax_item<D, true>(c, it, next, mail, st, w, wide, n, pair_phase)
-                                   : softmax_item<D, false>(c, it, next, mail, st, w, wide, n, pair_phase);
+      more = it.shape == SHAPE_TWO ? softmax_item<D, true>(c, it, next, mail, st, w, n, pair_phase)
+                                   : softmax_item<D, false>(c, it, next, mail, st, w, n, pair_phase);
     }
     if (!more) break;
     it = next;
   }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   tc_fence_before();
 }
 
@@ -968,24 +1057,15 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
       const bool gone = __any_sync(0xffffffffu, *c.abort_flag != 0);
       block = gone ? -1 : uniform(claimed_block(c.smem_base + L::CLAIM_OFF));
       fence_async_smem();                                   // the answer has been read: the next one may be written
-      if (block >= 0) {
+      more = block >= 0;
+      if (more) {
         if constexpr (std::is_same<List, InlineItems>::value) raw = list.items[block];
         else raw = p.items[block];
+        it = work_of(raw, p);
       } else {
-        raw = WorkItem{};
-        raw.seq = -1;
+        it.seq = -1;
       }
-      c.wait(BAR_IEMPTY + mail.slot, mail.phase ^ 1);
-      if (lane == 0) {
-        uint4* dst = reinterpret_cast<uint4*>(c.smem_gen + L::ITEM_OFF) + 2 * mail.slot;
-        dst[0] = reinterpret_cast<const uint4*>(&raw)[0];
-        dst[1] = reinterpret_cast<const uint4*>(&raw)[1];
-        mbar_arrive(c.bar(BAR_IFULL + mail.slot));
-      }
-      __syncwarp();
-      if (++mail.slot == 2) { mail.slot = 0; mail.phase ^= 1; }
-      more = block >= 0;
-      if (more) it = work_of(raw, p.G);
+      mail.put(c, it);
     } else {
       more = mail.next(c, it);
     }
@@ -1149,6 +1229,7 @@ struct QkIssuer {
 template <int D, typename List>
 __global__ void __launch_bounds__(THREADS, 1)
 prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                  const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_out,
                   const __grid_constant__ List list) {
   using L = Smem<D>;
   extern __shared__ uint8_t smem_raw[];
@@ -1192,7 +1273,7 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = uniform(*tmem_slot);
-  const Cta<D> c{p, smem_base, smem_gen, abort_flag, tmem, tmem + BN, tmem + NQ * L::SP_COLS, lane};
+  const Cta<D> c{p, smem_base, smem_gen, abort_flag, &map_q, &map_out, tmem, tmem + BN, tmem + NQ * L::SP_COLS, lane};
 
   // Programmatic launch: up to here a CTA has touched nothing but itself; every warp that reads or writes global
   // memory waits for the kernel before (which may be one that leaves its list in this workspace).
@@ -1207,7 +1288,7 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
     dst[0] = src[0];
     dst[1] = src[1];
   }
-  Work it = work_of(raw, p.G);
+  Work it = work_of(raw, p);
   // Register split: every warp of a warpgroup runs the same setmaxnreg; the service
   // group releases first what the two softmax groups then take.  (Nothing may come between this and a role's code: past a
   // point where the two branches meet the compiler plans with fewer registers, and the steps spilled 1.4 KB.)
@@ -1532,6 +1613,21 @@ static bool make_pool_map(CUtensorMap* m, void* pool, int pages, int Hkv, int D)
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Rows [tokens][heads][D] bf16 as a 4-D tensor (dim % 64, dim / 64, head, token); one box = 64 dims of the G heads of 32 / G
+// tokens, 128-byte swizzled in shared memory.
+static bool make_rows_map(CUtensorMap* m, const void* rows, int tokens, int heads, int D, int G) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t row = (cuuint64_t)D * 2;
+  const cuuint64_t dims[4] = {64, (cuuint64_t)D / 64, (cuuint64_t)heads, (cuuint64_t)tokens};
+  const cuuint64_t strides[3] = {128, row, row * heads};
+  const cuuint32_t box[4] = {64, 1, (cuuint32_t)G, (cuuint32_t)(32 / G)};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(rows), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // A model calls this once per layer with the same few pools over and over: the encoded maps
 // of the pools seen last are kept per host thread (a map is a pure function of the key).
 struct PoolMapEntry {
@@ -1585,10 +1681,17 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   const CUtensorMap mk = *pk;
   const CUtensorMap* pv = pool_map(c->d_v_pool, c->num_pages, c->num_kv_heads, D);
   if (!pv) return EFIM_ERR_CUDA;
+  // Query and output rows as boxes of 32 rows, where those are whole tokens and there are as many.
+  p.g_mul = p.G == 1 ? 0u : (uint32_t)((1ull << 32) / (unsigned)p.G + 1);
+  CUtensorMap mq{}, mo{};
+  if (p.G <= 32 && 32 % p.G == 0 && (long long)p.total_new_tokens * p.G >= 32) {
+    p.q_tma = p.cos_sin == nullptr && make_rows_map(&mq, p.q, p.total_new_tokens, p.Hq, D, p.G);
+    p.out_tma = make_rows_map(&mo, p.out, p.total_new_tokens, p.Hq, D, p.G);
+  }
   using Items = std::decay_t<decltype(items_of(list))>;
   const efim_status st = raise_smem_limit<D, Items>();
   if (st != EFIM_OK) return st;
-  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, Items>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv, items_of(list)));
+  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, Items>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv, mq, mo, items_of(list)));
   if (pl.s_max > 1) {
     const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + 3) / 4);
     if constexpr (inl)

@@ -62,6 +62,8 @@ struct Params {
   const float* cos_sin;        // [max_position][D]
   int max_position, interleaved;
   int early_next;              // let the next kernel start its set-up while this one runs
+  uint32_t g_mul;              // floor(2^32 / G) + 1 (0: G = 1), see token_of
+  int q_tma, out_tma;          // 32 rows are whole tokens (G divides 32): they move as boxes of 64 dims
 };
 
 struct Plan {
