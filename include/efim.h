@@ -197,7 +197,9 @@ efim_status efim_append_prefill_attn_planned(const efim_cache_desc* cache, const
  * zero query (its output is finite and meaningless), its k/v are not appended.
  * d_k_new and d_v_new may both be NULL: the new tokens' k/v are then taken to be in the
  * pages already (an earlier efim_kv_append with d_q = NULL) and only the attention runs.
- * Two kernels are enqueued (three when the key range is split).
+ * Two kernels are enqueued (three when the key range is split); one where, without a plan, a single sequence
+ * brings at most 256 (token, head-in-group) rows and its key range is not split: the attention kernel then
+ * appends them itself.
  */
 efim_status efim_append_prefill_step(const efim_cache_desc* cache, const efim_batch_desc* batch,
                                      const efim_rope_desc* rope, const void* d_q,

@@ -2,6 +2,7 @@
 // cached `<P>prefix<S>suffix<M>` keys and over each other (EFIM Sec. 1, Sec. 2.2).
 // Host side: validates, plans the work list from the host length mirrors, copies
 // it into the workspace and launches the tensor-core kernel (prefill_tc.cu).
+#include <algorithm>
 #include <cstring>
 #include <memory>
 #include "prefill_tc.cuh"
@@ -97,11 +98,17 @@ extern "C" efim_status efim_prefill_plan(const efim_cache_desc* cache, const efi
 }
 
 namespace {
+// New tokens' k/v rows that the attention kernel itself puts into the pages.
+struct NewRows {
+  const void *k, *v;
+};
+
 // Runs a plan over validated descriptors.  `rope` with a table: the query rows are rotated as the kernel
 // loads them.  `h_lists`: the lists to copy to the head of the workspace (null: an earlier call has left
 // them there); `list`: the work list, if it travels in the launch parameters instead.
 efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
-                     const efim::pf::Plan& pl, const void* h_lists, const efim::pf::InlineList* list, const void* d_q,
+                     const efim::pf::Plan& pl, const void* h_lists, const efim::pf::InlineList* list, const NewRows* append,
+                     const void* d_q,
                      void* d_out, float* d_lse, float sm_scale, void* d_workspace, size_t workspace_bytes,
                      int32_t* d_status, void* stream) {
   using namespace efim;
@@ -140,6 +147,12 @@ efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch,
     p.max_position = rope->max_position;
     p.interleaved = rope->interleaved;
   }
+  if (append) {
+    p.k_new = static_cast<const uint16_t*>(append->k);
+    p.v_new = static_cast<const uint16_t*>(append->v);
+    p.k_pool = static_cast<uint16_t*>(cache->d_k_pool);
+    p.v_pool = static_cast<uint16_t*>(cache->d_v_pool);
+  }
   // work list + per-sequence split sizes go to the head of the workspace in one copy
   if (h_lists) EFIM_CUDA_TRY(cudaMemcpyAsync(ws, h_lists, pl.items_bytes + pl.split_bytes, cudaMemcpyHostToDevice, s));
   return pf::launch(cache, p, pl, list, s);
@@ -172,14 +185,16 @@ efim_status run_planned(const efim_cache_desc* cache, const efim_batch_desc* bat
   pl.part_lse_bytes = hd.part_lse_bytes;
   pl.part_o_bytes = hd.part_o_bytes;
   return run_plan(cache, batch, rope, pl, lists_resident ? nullptr : static_cast<const unsigned char*>(h_plan) + PLAN_HEAD_BYTES,
-                  nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
+                  nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
 }
 
 // Plans, then runs.  Lists of up to InlineItems::MAX items travel in the launch parameters: no
 // copy stands between the append and the attention kernel (append and attention of 16 tokens over 240 in
 // one call 15.2 -> 10.7 us; the kernel leaves the list in the workspace all the same).
+// `append`: rows the attention kernel is to put into the pages itself, where the plan allows it; else they are appended
+// by a kernel of their own before it.
 efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
-                         const void* d_q, void* d_out, float* d_lse, float sm_scale, void* d_workspace,
+                         const NewRows* append, const void* d_q, void* d_out, float* d_lse, float sm_scale, void* d_workspace,
                          size_t workspace_bytes, int32_t* d_status, void* stream) {
   using namespace efim;
   efim_status st = check_cache(cache);
@@ -189,17 +204,37 @@ efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* ba
   if (!batch_has_work(batch)) return EFIM_OK;
   const pf::Plan pl = pf::make_plan(cache, batch);
   if (pl.n_items == 0) return EFIM_OK;
+  if (append && (pl.s_max > 1 || (reinterpret_cast<uintptr_t>(append->k) | reinterpret_cast<uintptr_t>(append->v)) & 15)) {
+    st = efim_kv_append(cache, batch, rope, nullptr, append->k, append->v, d_status, stream);
+    if (st != EFIM_OK) return st;
+    append = nullptr;
+  }
   if (pl.n_items <= pf::InlineItems::MAX && batch->batch <= pf::InlineSplit::MAX_BATCH) {
     pf::InlineList list;
     pf::fill_lists(cache, batch, pl, list.items.items, list.split.keys);
-    return run_plan(cache, batch, rope, pl, nullptr, &list, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
+    return run_plan(cache, batch, rope, pl, nullptr, &list, append, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
                     d_status, stream);
   }
   const std::unique_ptr<unsigned char[]> lists(new unsigned char[pl.items_bytes + pl.split_bytes]);
   pf::fill_lists(cache, batch, pl, reinterpret_cast<pf::WorkItem*>(lists.get()),
                  reinterpret_cast<int32_t*>(lists.get() + pl.items_bytes));
-  return run_plan(cache, batch, rope, pl, lists.get(), nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
+  return run_plan(cache, batch, rope, pl, lists.get(), nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
                   d_status, stream);
+}
+
+// Whether a step's new rows may be appended by the attention kernel: one sequence brings all of them (another one might
+// count them among its cached tokens, in pages that both share), as one block of rows per kv head (so nobody else reads what
+// a block appends), with at most a CTA per SM.
+bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* batch) {
+  if (efim::check_cache(cache) != EFIM_OK || efim::check_batch(cache, batch, true) != EFIM_OK) return false;
+  const long long G = cache->num_q_heads / cache->num_kv_heads;
+  int with_work = 0;
+  for (int s = 0; s < batch->batch; ++s) {
+    if (batch->h_new_len[s] * G > efim::pf::NQ * efim::pf::BM) return false;
+    with_work += batch->h_new_len[s] > 0;
+  }
+  return with_work == 1 && cache->num_kv_heads <= std::min(efim::sm_count(), (int)efim::pf::InlineItems::MAX) &&
+         batch->batch <= efim::pf::InlineSplit::MAX_BATCH;
 }
 }  // namespace
 
@@ -217,7 +252,7 @@ extern "C" efim_status efim_append_prefill_attn(const efim_cache_desc* cache, co
                                                 const void* d_q, void* d_out, float* d_lse, float sm_scale,
                                                 void* d_workspace, size_t workspace_bytes, int32_t* d_status,
                                                 void* stream) {
-  return plan_and_run(cache, batch, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status,
+  return plan_and_run(cache, batch, nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status,
                       stream);
 }
 
@@ -230,6 +265,9 @@ extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, co
                                                 void* d_workspace, size_t workspace_bytes, int32_t* d_status,
                                                 void* stream) {
   if ((d_k_new == nullptr) != (d_v_new == nullptr)) return EFIM_ERR_INVALID_ARG;
+  const NewRows rows{d_k_new, d_v_new};
+  if (d_k_new && !h_plan && appends_in_attention(cache, batch))
+    return plan_and_run(cache, batch, rope, &rows, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
   if (d_k_new) {
     const efim_status st = efim_kv_append(cache, batch, rope, nullptr, d_k_new, d_v_new, d_status, stream);
     if (st != EFIM_OK) return st;
@@ -237,5 +275,5 @@ extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, co
   if (h_plan)
     return run_planned(cache, batch, rope, h_plan, plan_bytes, lists_resident, d_q, d_out, d_lse, sm_scale,
                        d_workspace, workspace_bytes, d_status, stream);
-  return plan_and_run(cache, batch, rope, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
+  return plan_and_run(cache, batch, rope, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
 }

@@ -189,7 +189,9 @@ enum {
   BAR_PAIR = 14,     // the two softmax warps that share 32 TMEM lanes
   BAR_ALL = 18,      // all softmax warps
   BAR_CLAIM = 19,    // the answer to a claim is in shared memory
-  BAR_KFULL = 20, BAR_KEMPTY = 28, BAR_VFULL = 36, BAR_VEMPTY = 44, BAR_COUNT = 52
+  BAR_KFULL = 20, BAR_KEMPTY = 28, BAR_VFULL = 36, BAR_VEMPTY = 44,
+  BAR_NEW = 52,      // the item's new k/v are in their pages
+  BAR_COUNT = 53
 };
 
 // Shared-memory plan.  A query tile is [64-element half][128 rows][128 bytes]; a K or V tile
@@ -367,6 +369,56 @@ __device__ __forceinline__ void q_rows_to_smem(const Params& p, uint8_t* smem_ge
     const uint32_t dst = smem_base + tile_off + (c >> 3) * L::HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(t >= 0 ? 16 : 0) : "memory");
   }
+}
+
+// The N new k (rotated) and v rows of one (sequence, kv head) into their page slots, by 128 threads: the arithmetic and
+// the checks of efim_kv_append.  Afterwards they may be read by bulk-tensor copies.
+template <int D>
+__device__ __noinline__ void append_rows(const uint4* k_new, const uint4* v_new, uint4* k_pool, uint4* v_pool, const int32_t* bt,
+                                         const float* cos_sin, int max_position, int interleaved, int32_t* status, int max_pages,
+                                         int num_pages, int Hkv, int kvh, int C, int N, int tok0, int t) {
+  constexpr int VEC = D / 8;
+  for (int u = t; u < N * VEC; u += 128) {
+    const int i = u / VEC, j = u % VEC, pos = C + i;
+    int err = 0, page = -1;
+    if ((pos >> 4) >= max_pages || (cos_sin && pos >= max_position)) {
+      err = EFIM_DEV_BAD_POSITION;
+    } else {
+      page = bt[pos >> 4];
+      if (page < 0 || page >= num_pages) err = EFIM_DEV_BAD_PAGE;
+    }
+    if (err) {
+      if (j == 0 && status) atomicOr(status, err);
+      continue;
+    }
+    const size_t src = ((size_t)(tok0 + i) * Hkv + kvh) * VEC;
+    uint4 k = k_new[src + j];
+    const uint4 v = v_new[src + j];
+    if (cos_sin) {
+      const float* cs = cos_sin + (size_t)pos * D;
+      if (!interleaved) {
+        uint4 o = k_new[src + (j ^ (VEC / 2))];
+        const float* cp = cs + (j % (VEC / 2)) * 8;
+        float cf[8], sf[8];
+        *reinterpret_cast<float4*>(cf) = *reinterpret_cast<const float4*>(cp);
+        *reinterpret_cast<float4*>(cf + 4) = *reinterpret_cast<const float4*>(cp + 4);
+        *reinterpret_cast<float4*>(sf) = *reinterpret_cast<const float4*>(cp + D / 2);
+        *reinterpret_cast<float4*>(sf + 4) = *reinterpret_cast<const float4*>(cp + D / 2 + 4);
+        if (j < VEC / 2) rotate8(k, o, cf, sf);
+        else rotate8(o, k, cf, sf);
+      } else {
+        float cf[4], sf[4];
+        *reinterpret_cast<float4*>(cf) = *reinterpret_cast<const float4*>(cs + j * 4);
+        *reinterpret_cast<float4*>(sf) = *reinterpret_cast<const float4*>(cs + D / 2 + j * 4);
+        rotate4_interleaved(k, cf, sf);
+      }
+    }
+    const size_t dst = (((size_t)page * Hkv + kvh) * 16 + (pos & 15)) * VEC + j;
+    k_pool[dst] = k;
+    v_pool[dst] = v;
+  }
+  __threadfence();
+  asm volatile("fence.proxy.async;" ::: "memory");           // the copies read what ordinary stores wrote
 }
 
 // Two softmax groups ("streams") run per CTA.  With more than 128 rows, stream t
@@ -952,7 +1004,7 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
   return more;
 }
 
-template <int D>
+template <int D, bool APPEND>
 __device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp) {
   const int st = warp >> 2, w = warp & 3;                   // stream, 32-lane quarter
   Mailbox mail;
@@ -962,6 +1014,14 @@ __device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp)
     publish_q(c, st);
   }
   for (;;) {
+    if (APPEND && st == 1) {
+      const Params& p = c.p;
+      append_rows<D>(reinterpret_cast<const uint4*>(p.k_new), reinterpret_cast<const uint4*>(p.v_new),
+                     reinterpret_cast<uint4*>(p.k_pool), reinterpret_cast<uint4*>(p.v_pool),
+                     p.block_table + (size_t)it.seq * p.max_pages_per_seq, p.cos_sin, p.max_position, p.interleaved, p.status,
+                     p.max_pages_per_seq, p.num_pages, p.Hkv, it.kvh, it.C, token_of(p, it.rows_total), it.tok0, w * 32 + c.lane);
+      warp_arrive(c.bar(BAR_NEW), c.lane);
+    }
     Work next;
     bool more;
     if (it.shape == SHAPE_TINY) {
@@ -985,7 +1045,7 @@ __device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp)
 // ------------------------------------------------------------------ TMA producers
 // Every bulk-tensor copy costs its issuing warp ~65 cycles (one box per page: 16 slots x all dims
 // of one kv head).  Warp 8 loads the K tiles and warp 11 the V tiles; warp 8 also claims the items.
-template <int D, bool K_ROLE, typename List>
+template <int D, bool K_ROLE, bool APPEND, typename List>
 __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap& map, const List& list, WorkItem raw, Work it) {
   using L = Smem<D>;
   const Params& p = c.p;
@@ -995,7 +1055,7 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
   const int lane = c.lane, page_l = lane;
   Mailbox mail;                                             // of warp 11; warp 8 keeps the place it writes in it
   int slot = 0, n_steps = 0, block = blockIdx.x;
-  uint32_t phase = 0, claim_phase = 0;
+  uint32_t phase = 0, claim_phase = 0, new_phase = 0;
   for (;;) {
     const int32_t* bt = p.block_table + (size_t)it.seq * p.max_pages_per_seq + (it.key0 >> 4);
     const int n_pages = (it.kv_cap - it.key0 + 15) >> 4;    // pages this item reads
@@ -1018,6 +1078,7 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
     // which covers the claim, the item and its first pages.  (Claimed earlier, the last items of a launch would be
     // bound to CTAs that are still busy.)
     const int claim_at = max(it.nt - 2, 0);
+    const int first_new = APPEND ? (it.C - it.key0) / BN : -1;   // step that holds the first key this kernel appends
     for (int jj = 0; jj < it.nt; ++jj) {
       const int pid = pid_a;
       pid_a = pid_b;
@@ -1032,6 +1093,11 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
         claim_next(c.smem_base + L::CLAIM_OFF, c.bar(BAR_CLAIM));
       }
       c.wait(empty + slot, phase ^ 1);
+      if (APPEND && jj == first_new) {
+        c.wait(BAR_NEW, new_phase);
+        new_phase ^= 1;
+        asm volatile("fence.proxy.async;" ::: "memory");
+      }
       const uint32_t dst_off = my_off + slot * L::KV_BYTES + page_l * L::PAGE_BYTES;
       if (any_bad) {
         // the page's 16 keys are replaced by zeros (score 0, value 0), so the tile holds nothing
@@ -1226,7 +1292,10 @@ struct QkIssuer {
 // 16 x 32-256 over 2-8k at 32/32 320 -> 308, 8 x 3,200 over 5k 2,590 -> 2,490.
 // The work list: in the workspace (List = NoList), or, a short one planned inside the call, in the launch
 // parameters (List = InlineItems) - which saves the copy between the append and this kernel.
-template <int D, typename List>
+// APPEND: the softmax warps of stream 1 first put the item's new k/v rows into their pages, and the copies of those pages
+// wait for them: a step of a few short rows is one launch instead of two (16 tokens over 240 at 4/4 heads x 64 9.85 ->
+// 7.35 us).  A kernel of its own: in the others' place it cost their steps 5 %.
+template <int D, typename List, bool APPEND>
 __global__ void __launch_bounds__(THREADS, 1)
 prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                   const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_out,
@@ -1253,6 +1322,7 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
     for (int s = 0; s < 4; ++s) mbar_init(bar(BAR_PAIR + s), 2);
     mbar_init(bar(BAR_ALL), 8);
     mbar_init(bar(BAR_CLAIM), 1);
+    mbar_init(bar(BAR_NEW), 4);
     for (int s = 0; s < L::NK; ++s) {
       mbar_init(bar(BAR_KFULL + s), 1);
       mbar_init(bar(BAR_KEMPTY + s), 1);
@@ -1294,15 +1364,15 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   // point where the two branches meet the compiler plans with fewer registers, and the steps spilled 1.4 KB.)
   if (warp < 8) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
-    softmax_role<D>(c, it, warp);
+    softmax_role<D, APPEND>(c, it, warp);
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
     if (warp == 8) {
       if (p.early_next) pdl_launch();
-      producer_role<D, true>(c, map_k, list, raw, it);
+      producer_role<D, true, APPEND>(c, map_k, list, raw, it);
     } else if (warp == 11) {
       if (p.early_next) pdl_launch();
-      producer_role<D, false>(c, map_v, list, raw, it);
+      producer_role<D, false, APPEND>(c, map_v, list, raw, it);
     } else if (warp == 9) {
       PvIssuer<D> pv{c};
       Mailbox mail;
@@ -1654,14 +1724,14 @@ const CUtensorMap* pool_map(void* pool, int pages, int Hkv, int D) {
 }
 
 // The kernel's shared-memory size has to be raised once per device.
-template <int D, typename List>
+template <int D, typename List, bool APPEND>
 static efim_status raise_smem_limit() {
   constexpr int kMaxDevices = 64;
   static std::atomic<bool> done[kMaxDevices];
   int dev = 0;
   EFIM_CUDA_TRY(cudaGetDevice(&dev));
   if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return EFIM_OK;
-  EFIM_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<D, List>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  EFIM_CUDA_TRY(cudaFuncSetAttribute(prefill_tc_kernel<D, List, APPEND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      Smem<D>::TOTAL));
   if (dev >= 0 && dev < kMaxDevices) done[dev].store(true, std::memory_order_release);
   return EFIM_OK;
@@ -1689,9 +1759,18 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
     p.out_tma = make_rows_map(&mo, p.out, p.total_new_tokens, p.Hq, D, p.G);
   }
   using Items = std::decay_t<decltype(items_of(list))>;
-  const efim_status st = raise_smem_limit<D, Items>();
+  auto start = [&](auto append) -> efim_status {
+    constexpr bool APPEND = decltype(append)::value;
+    const efim_status st = raise_smem_limit<D, Items, APPEND>();
+    if (st != EFIM_OK) return st;
+    EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, Items, APPEND>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv,
+                             mq, mo, items_of(list)));
+    return EFIM_OK;
+  };
+  efim_status st;
+  if constexpr (inl) st = p.k_new ? start(std::true_type{}) : start(std::false_type{});
+  else st = start(std::false_type{});
   if (st != EFIM_OK) return st;
-  EFIM_CUDA_TRY(launch_pdl(prefill_tc_kernel<D, Items>, dim3(pl.n_items), dim3(THREADS), Smem<D>::TOTAL, s, p, mk, *pv, mq, mo, items_of(list)));
   if (pl.s_max > 1) {
     const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + 3) / 4);
     if constexpr (inl)

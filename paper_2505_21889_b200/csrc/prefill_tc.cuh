@@ -59,9 +59,13 @@ struct Params {
   float scale_log2;
   unsigned long long wait_ns;  // limit of every device-side wait
   // rotation of the query rows as they are loaded (null: q is already rotated)
-  const float* cos_sin;        // [max_position][D]
+  const float* cos_sin;        // [max_position][D] (and of the new k)
   int max_position, interleaved;
   int early_next;              // let the next kernel start its set-up while this one runs
+  // the new tokens' k/v, put into their page slots by this kernel (null: they are there already); every item is all
+  // the rows of its (sequence, kv head) then, and of one sequence
+  const uint16_t *k_new, *v_new;   // [T][Hkv][D]
+  uint16_t *k_pool, *v_pool;   // [pages][Hkv][16][D]
   uint32_t g_mul;              // floor(2^32 / G) + 1 (0: G = 1), see token_of
   int q_tma, out_tma;          // 32 rows are whole tokens (G divides 32): they move as boxes of 64 dims
 };

@@ -19,3 +19,36 @@ def test_items_of_every_shape_in_turn(Hq, Hkv, D):
     new = np.maximum(1, rng.permutation(np.tile(rows, 12))[:160] // G).astype(np.int32)
     cached = rng.choice([0, 1, 15, 16, 79, 80, 81, 160, 200, 239], 160).astype(np.int32)
     _check_turn(_custom(Hq, Hkv, D, cached, new, seed=Hq + D), use_rope=False)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new,interleaved,max_position,bad_page", [
+    (4, 4, 64, [240], [16], False, None, False),
+    (32, 8, 128, [0], [64], False, None, False),               # 256 rows, nothing cached
+    (28, 4, 128, [79, 300], [36, 0], True, None, False),       # the last key of a step is new; an idle sequence beside it
+    (8, 8, 128, [0, 80], [0, 256], False, None, False),        # the first key of a step is new
+    (16, 1, 128, [81], [1], True, None, False),
+    (24, 8, 64, [1000], [33], False, 1010, False),             # positions beyond the rotary table
+    (8, 2, 128, [250], [40], False, None, True),               # a new token's page id outside the pool
+])
+def test_rows_appended_by_the_attention_kernel(Hq, Hkv, D, cached, new, interleaved, max_position, bad_page):
+    """A step of one sequence of at most 256 rows (one launch) against efim_kv_append without q and the attention-only
+    step: out, lse, pools and status bit for bit."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, D, cached, new, seed=3 * D + Hq)
+    if bad_page:
+        w.block_table[0, cached[0] // 16 + 1] = w.num_pages + 5
+    a, b = H.DeviceWorkload(w, interleaved=interleaved), H.DeviceWorkload(w, interleaved=interleaved)
+    rope = efim.Rope(w.rope_base, D, max_position or int((w.cached_len + w.new_len).max()), interleaved)
+    ws = torch.empty(max(efim.efim_prefill_workspace_bytes(a.cache, a.batch), 256), dtype=torch.uint8, device="cuda")
+    efim.efim_kv_append(a.cache, a.batch, rope, None, a.k_new, a.v_new, a.status)
+    efim.efim_append_prefill_step(a.cache, a.batch, rope, a.q, None, None, a.out, a.lse, 0.0, ws, a.status)
+    for _ in range(2):                                         # (again over pages that hold the tokens already)
+        efim.efim_append_prefill_step(b.cache, b.batch, rope, b.q, b.k_new, b.v_new, b.out, b.lse, 0.0, ws, b.status)
+    torch.cuda.synchronize()
+    assert int(a.status.item()) == int(b.status.item()) == (2 if max_position else 1 if bad_page else 0)
+    assert torch.equal(a.out.view(torch.int16), b.out.view(torch.int16)) and torch.equal(a.lse, b.lse)
+    assert torch.equal(a.k_pool.view(torch.int16), b.k_pool.view(torch.int16))
+    assert torch.equal(a.v_pool.view(torch.int16), b.v_pool.view(torch.int16))
