@@ -1477,11 +1477,13 @@ __global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p, cons
 
 // ------------------------------------------------------------------ host side
 namespace {
-// Cost of a CTA in tenths of a microsecond, as measured on B200 with a wave or less of them: a 128-key
-// tile with two query tiles is bound by the softmax / tensor pipeline, with one by its K/V bytes; every
-// CTA pays for its set-up, query load, pipeline fill and epilogue; a split adds the partials' round
-// trip and the merge.
-constexpr long long COST_TILE_DUAL = 18, COST_TILE_SINGLE = 12, COST_CTA = 95, COST_PARTIAL = 8, COST_MERGE = 40;
+// Cost of a work item in tenths of a microsecond: a 128-key tile with two query tiles is bound by the softmax / tensor
+// pipeline, with one by its K/V bytes; every item pays for what lies between it and the one before on its CTA (what a
+// CTA pays before its first one is the same for every cut); a split adds the partials' round trip and the merge.  Of 16
+// batches, with the costs of a kernel of one item per CTA (18, 12, 95 instead of 16, 10, 40) -> with these: two of 13 drawn ones
+// 125 -> 119 and 62.4 -> 60.3 us, 64 mixed rows 303.9 -> 302.3, 16 x 32-256 over 2-8k at 32/32 heads 306.9 -> 305.7, the
+// others the same.  (18, 12, 40: 16 x 8-112 tokens over 1-3.4k are cut too fine, 65 -> 92 us.)
+constexpr long long COST_TILE_DUAL = 16, COST_TILE_SINGLE = 10, COST_CTA = 40, COST_PARTIAL = 8, COST_MERGE = 40;
 // Weights of a tile in the launch order of a few waves (see fill_lists).
 constexpr long long ORDER_TILE_DUAL = 21, ORDER_TILE_SINGLE = 9;
 
