@@ -2,8 +2,8 @@
 // `inc` queries attend causally over the cached `<P>prefix<S>suffix<M>` keys and
 // over each other).
 //
-// One CTA owns up to 256 packed query rows (row = token * G + head-in-group) of one
-// (sequence, kv head) as two 128-row tiles, and streams the visible K/V range in
+// A work item is up to 256 packed query rows (row = token * G + head-in-group) of one
+// (sequence, kv head) as two 128-row tiles; a CTA walks items and streams each one's visible K/V range in
 // steps of 80 keys (5 pages):
 //   warps 8,11 TMA producers (K tiles / V tiles): walk the block table, one tiled bulk-tensor
 //             copy per page (16 slots x all dims of the kv head) into rings of 3 entries each
@@ -885,7 +885,7 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
   const int vis = row.valid ? min(row.pos + 1, it.kv_cap) : it.kv_cap;
   const int exact = !DUAL || it.nt <= EXACT_MAX_STEPS ? EXACT_STEPS : 1;
   const int kv_first = it.key0 + (DUAL ? 0 : st * BN), kv_step = DUAL ? BN : 2 * BN;
-  // (a row past the sequence: its query is zero, and against this reference so are its probabilities)
+  // (a row past the sequence holds zeros or what follows the sequence: against this reference its probabilities are zero)
   float m_ref = row.valid ? -FLT_MAX : FLT_MAX, l_sum = 0.f;
   for (int k = 0; k < my_cnt; ++k, ++n) {
     c.wait(BAR_S + st, n & 1);

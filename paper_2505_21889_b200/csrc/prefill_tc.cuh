@@ -25,7 +25,7 @@ constexpr int THREADS = 384;   // 2 softmax warpgroups + 1 service warpgroup (2 
 constexpr int REGS_SOFTMAX = 216;
 constexpr int REGS_SERVICE = 72;
 
-// One CTA's work: packed rows [row0, row0 + 256) of (seq, kv head) against the keys of the
+// One work item: packed rows [row0, row0 + 256) of (seq, kv head) against the keys of the
 // 128-key tiles [tile_begin, tile_end).  Packed row R = token * G + head-in-group.  The sequence's
 // lengths and first query row ride along (the planner has them from the host mirrors),
 // so that a CTA's first dependent chain is "item -> block table / query rows" instead of
