@@ -222,11 +222,22 @@ efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* ba
                   d_status, stream);
 }
 
+bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return a && b && x < y + b_bytes && y < x + a_bytes;
+}
+
 // Whether a step's new rows may be appended by the attention kernel: one sequence brings all of them (another one might
 // count them among its cached tokens, in pages that both share), as one block of rows per kv head (so nobody else reads what
-// a block appends), with at most a CTA per SM.
-bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* batch) {
+// a block appends), with at most a CTA per SM; and what the kernel writes does not lie on the rows (a CTA may store its output
+// before another one has read its k and v, which an append of its own has all read by then).
+bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* batch, const NewRows& rows, const void* d_out,
+                          const float* d_lse) {
   if (efim::check_cache(cache) != EFIM_OK || efim::check_batch(cache, batch, true) != EFIM_OK) return false;
+  const size_t tokens = (size_t)batch->total_new_tokens, row_bytes = tokens * cache->num_kv_heads * cache->head_dim * 2;
+  const size_t out_bytes = tokens * cache->num_q_heads * cache->head_dim * 2, lse_bytes = tokens * cache->num_q_heads * sizeof(float);
+  for (const void* r : {rows.k, rows.v})
+    if (overlap(r, row_bytes, d_out, out_bytes) || overlap(r, row_bytes, d_lse, lse_bytes)) return false;
   const long long G = cache->num_q_heads / cache->num_kv_heads;
   int with_work = 0;
   for (int s = 0; s < batch->batch; ++s) {
@@ -266,7 +277,7 @@ extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, co
                                                 void* stream) {
   if ((d_k_new == nullptr) != (d_v_new == nullptr)) return EFIM_ERR_INVALID_ARG;
   const NewRows rows{d_k_new, d_v_new};
-  if (d_k_new && !h_plan && appends_in_attention(cache, batch))
+  if (d_k_new && !h_plan && appends_in_attention(cache, batch, rows, d_out, d_lse))
     return plan_and_run(cache, batch, rope, &rows, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
   if (d_k_new) {
     const efim_status st = efim_kv_append(cache, batch, rope, nullptr, d_k_new, d_v_new, d_status, stream);

@@ -52,3 +52,69 @@ def test_rows_appended_by_the_attention_kernel(Hq, Hkv, D, cached, new, interlea
     assert torch.equal(a.out.view(torch.int16), b.out.view(torch.int16)) and torch.equal(a.lse, b.lse)
     assert torch.equal(a.k_pool.view(torch.int16), b.k_pool.view(torch.int16))
     assert torch.equal(a.v_pool.view(torch.int16), b.v_pool.view(torch.int16))
+
+
+def _kernels_of(call):
+    """Number of kernels a call enqueues: the nodes of a graph it is captured into (these calls copy nothing)."""
+    import ctypes
+    import torch
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    n = ctypes.c_size_t()
+    assert ctypes.CDLL("libcudart.so.12").cudaGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
+
+
+class _OneSequenceStep:
+    """The same step twice over: as one call (`b`), and as efim_kv_append without q followed by the attention only (`a`)."""
+
+    def __init__(self, w, interleaved=False, max_position=None):
+        import torch
+        import paper_2505_21889_b200 as efim
+        import tests.gpu_harness as H
+        self.efim, self.torch = efim, torch
+        self.a, self.b = H.DeviceWorkload(w, interleaved=interleaved), H.DeviceWorkload(w, interleaved=interleaved)
+        self.rope = efim.Rope(w.rope_base, w.head_dim, max_position or int((w.cached_len + w.new_len).max()), interleaved)
+        self.ws = torch.empty(max(efim.efim_prefill_workspace_bytes(self.a.cache, self.a.batch), 256), dtype=torch.uint8,
+                              device="cuda")
+        assert efim.efim_prefill_launch_count(self.a.cache, self.a.batch) == 1       # not cut
+
+    def two_calls(self, sm_scale=0.0, lse=True):
+        a = self.a
+        self.efim.efim_kv_append(a.cache, a.batch, self.rope, None, a.k_new, a.v_new, a.status)
+        self.efim.efim_append_prefill_step(a.cache, a.batch, self.rope, a.q, None, None, a.out, a.lse if lse else None, sm_scale,
+                                           self.ws, a.status)
+
+    def one_call(self, sm_scale=0.0, lse=True, out=None, out_lse=None):
+        b = self.b
+        out_lse = (b.lse if out_lse is None else out_lse) if lse else None
+        self.efim.efim_append_prefill_step(b.cache, b.batch, self.rope, b.q, b.k_new, b.v_new, b.out if out is None else out,
+                                           out_lse, sm_scale, self.ws, b.status)
+
+    def same(self, out=None, out_lse=None):
+        a, b, i16, equal = self.a, self.b, self.torch.int16, self.torch.equal
+        self.torch.cuda.synchronize()
+        return (equal(a.out.view(i16), (b.out if out is None else out).view(i16))
+                and equal(a.lse, b.lse if out_lse is None else out_lse)
+                and equal(a.k_pool.view(i16), b.k_pool.view(i16)) and equal(a.v_pool.view(i16), b.v_pool.view(i16)))
+
+
+@pytest.mark.parametrize("what", ["nothing", "out on k", "out on v", "lse on k", "lse on v"])
+def test_outputs_may_overlap_the_new_rows(what):
+    """A step whose output or lse lies on its new k or v rows equals append, then attention; it takes two kernels then, as the
+    append has to have read all rows before the first output is stored."""
+    import torch
+    from tests.test_gpu_parity import _custom
+    s = _OneSequenceStep(_custom(8, 8, 128, [100], [20], seed=11))
+    s.two_calls()
+    args = {}
+    rows = s.b.k_new if what.endswith("k") else s.b.v_new
+    if what.startswith("out"):
+        args["out"] = rows
+    if what.startswith("lse"):
+        args["out_lse"] = rows.view(torch.uint8).flatten()[256:256 + 20 * 8 * 4].view(torch.float32).view(20, 8)
+    s.one_call(**args)
+    assert s.same(**args) and int(s.b.status.item()) == 0
+    assert _kernels_of(lambda: s.one_call(**args)) == (1 if what == "nothing" else 2)
