@@ -1078,7 +1078,14 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
     // which covers the claim, the item and its first pages.  (Claimed earlier, the last items of a launch would be
     // bound to CTAs that are still busy.)
     const int claim_at = max(it.nt - 2, 0);
-    const int first_new = APPEND ? (it.C - it.key0) / BN : -1;   // step that holds the first key this kernel appends
+    // APPEND: step that holds the first key this kernel appends, and the pages it appends to, one per lane from lane 8 on
+    // (256 new tokens lie in 17 pages at most).
+    const int first_new = APPEND ? (it.C - it.key0) / BN : -1;
+    int new_page = -1;
+    if constexpr (APPEND) {
+      const int pg = (it.C >> 4) + lane - 8;
+      if (lane >= 8 && pg * 16 < it.kv_cap && pg < p.max_pages_per_seq) new_page = p.block_table[(size_t)it.seq * p.max_pages_per_seq + pg];
+    }
     for (int jj = 0; jj < it.nt; ++jj) {
       const int pid = pid_a;
       pid_a = pid_b;
@@ -1093,10 +1100,14 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
         claim_next(c.smem_base + L::CLAIM_OFF, c.bar(BAR_CLAIM));
       }
       c.wait(empty + slot, phase ^ 1);
-      if (APPEND && jj == first_new) {
-        c.wait(BAR_NEW, new_phase);
-        new_phase ^= 1;
-        asm volatile("fence.proxy.async;" ::: "memory");
+      if constexpr (APPEND) {
+        // (A table may name a page twice: one of the cached keys' pages is then among those appended to.)
+        const int key = lane < 8 ? pid : new_page;
+        const uint32_t twins = __match_any_sync(0xffffffffu, key >= 0 ? key : -3 - lane) >> 8;
+        if (jj >= first_new || __any_sync(0xffffffffu, lane < 8 && twins != 0)) {
+          c.wait(BAR_NEW, new_phase);
+          asm volatile("fence.proxy.async;" ::: "memory");
+        }
       }
       const uint32_t dst_off = my_off + slot * L::KV_BYTES + page_l * L::PAGE_BYTES;
       if (any_bad) {
@@ -1116,6 +1127,7 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
       if (++slot == n_ring) { slot = 0; phase ^= 1; }
     }
     n_steps += it.nt;
+    if (APPEND) new_phase ^= 1;                             // (the last step holds new keys: it has been waited for)
     bool more;
     if constexpr (K_ROLE) {
       c.wait(BAR_CLAIM, claim_phase);

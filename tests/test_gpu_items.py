@@ -118,3 +118,27 @@ def test_outputs_may_overlap_the_new_rows(what):
     s.one_call(**args)
     assert s.same(**args) and int(s.b.status.item()) == 0
     assert _kernels_of(lambda: s.one_call(**args)) == (1 if what == "nothing" else 2)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new,old,renewed", [
+    (32, 8, 128, 300, 16, 1, 19),          # a page of the first step is the one that the new tokens fill
+    (8, 8, 64, 330, 40, 7, 21),            # ... of a later step, and the second of three pages
+    (4, 4, 64, 17, 16, 0, 2),              # within the first step
+])
+def test_a_page_named_twice(Hq, Hkv, D, cached, new, old, renewed):
+    """A table that names one page for cached keys and again for new ones: the cached keys are what the step writes there, as
+    they are behind an append of its own.  (New k and v each time: a copy made too early would bring the old ones.)"""
+    import torch
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, D, [cached], [new], seed=5)
+    w.block_table[0, old] = w.block_table[0, renewed]
+    s = _OneSequenceStep(w)
+    assert _kernels_of(s.one_call) == 1
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    for _ in range(20):
+        for x, y in ((s.a.k_new, s.b.k_new), (s.a.v_new, s.b.v_new)):
+            x.copy_(torch.randn(x.shape, device="cuda", generator=gen))
+            y.copy_(x)
+        s.two_calls()
+        s.one_call()
+        assert s.same()
