@@ -198,7 +198,7 @@ efim_status efim_append_prefill_attn_planned(const efim_cache_desc* cache, const
  * d_k_new and d_v_new may both be NULL: the new tokens' k/v are then taken to be in the
  * pages already (an earlier efim_kv_append with d_q = NULL) and only the attention runs.
  * Two kernels are enqueued (three when the key range is split); one where, without a plan, a single sequence
- * brings at most 256 (token, head-in-group) rows and its key range is not split: the attention kernel then
+ * brings at most 128 (token, head-in-group) rows and its key range is not split: the attention kernel then
  * appends them itself (not where d_out or d_lse overlaps d_k_new or d_v_new, which stays allowed).
  */
 efim_status efim_append_prefill_step(const efim_cache_desc* cache, const efim_batch_desc* batch,

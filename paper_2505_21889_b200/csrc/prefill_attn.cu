@@ -228,9 +228,12 @@ bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
 }
 
 // Whether a step's new rows may be appended by the attention kernel: one sequence brings all of them (another one might
-// count them among its cached tokens, in pages that both share), as one block of rows per kv head (so nobody else reads what
-// a block appends), with at most a CTA per SM; and what the kernel writes does not lie on the rows (a CTA may store its output
-// before another one has read its k and v, which an append of its own has all read by then).
+// count them among its cached tokens, in pages that both share), as one query tile per kv head (so nobody else reads what
+// a CTA appends), with at most a CTA per SM; and what the kernel writes does not lie on the rows (a CTA may store its output
+// before another one has read its k and v, which an append of its own has all read by then).  One tile: its second stream has no
+// query rows to fetch and appends meanwhile.  With two tiles, or more than 128 tokens, two kernels are faster - one kernel against
+// two, tokens over 0 at 4/4 heads x 64: 16 6.3 and 9.3 us, 128 11.5 and 13.5, 192 18.7 and 14.1, 256 22.7 and 15.9; at 8/8 x 128:
+// 128 17.1 and 18.7, 256 34.7 and 20.8; at 32/8 x 128: 32 10.7 and 16.3, 64 18.6 and 16.1.
 bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* batch, const NewRows& rows, const void* d_out,
                           const float* d_lse) {
   if (efim::check_cache(cache) != EFIM_OK || efim::check_batch(cache, batch, true) != EFIM_OK) return false;
@@ -241,7 +244,7 @@ bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* b
   const long long G = cache->num_q_heads / cache->num_kv_heads;
   int with_work = 0;
   for (int s = 0; s < batch->batch; ++s) {
-    if (batch->h_new_len[s] * G > efim::pf::NQ * efim::pf::BM) return false;
+    if (batch->h_new_len[s] * G > efim::pf::BM) return false;
     with_work += batch->h_new_len[s] > 0;
   }
   return with_work == 1 && cache->num_kv_heads <= std::min(efim::sm_count(), (int)efim::pf::InlineItems::MAX) &&

@@ -1079,7 +1079,7 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
     // bound to CTAs that are still busy.)
     const int claim_at = max(it.nt - 2, 0);
     // APPEND: step that holds the first key this kernel appends, and the pages it appends to, one per lane from lane 8 on
-    // (256 new tokens lie in 17 pages at most).
+    // (128 new tokens lie in 9 pages at most).
     const int first_new = APPEND ? (it.C - it.key0) / BN : -1;
     int new_page = -1;
     if constexpr (APPEND) {

@@ -142,3 +142,15 @@ def test_a_page_named_twice(Hq, Hkv, D, cached, new, old, renewed):
         s.two_calls()
         s.one_call()
         assert s.same()
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,new,kernels", [(4, 4, 64, 128, 1), (4, 4, 64, 129, 2), (32, 8, 128, 32, 1), (32, 8, 128, 33, 2),
+                                                  (16, 1, 128, 8, 1), (16, 1, 128, 16, 2), (8, 8, 128, 256, 2)])
+def test_one_kernel_up_to_one_query_tile(Hq, Hkv, D, new, kernels):
+    """A step of one sequence is one kernel up to 128 rows, where that is the faster form, and two beyond; the same bits."""
+    from tests.test_gpu_parity import _custom
+    s = _OneSequenceStep(_custom(Hq, Hkv, D, [0], [new], seed=new))
+    s.two_calls()
+    assert _kernels_of(s.one_call) == kernels
+    s.one_call()
+    assert s.same()
