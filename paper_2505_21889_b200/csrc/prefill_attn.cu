@@ -2,7 +2,6 @@
 // cached `<P>prefix<S>suffix<M>` keys and over each other (EFIM Sec. 1, Sec. 2.2).
 // Host side: validates, plans the work list from the host length mirrors, copies
 // it into the workspace and launches the tensor-core kernel (prefill_tc.cu).
-#include <algorithm>
 #include <cstring>
 #include <memory>
 #include "prefill_tc.cuh"
@@ -204,12 +203,14 @@ efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* ba
   if (!batch_has_work(batch)) return EFIM_OK;
   const pf::Plan pl = pf::make_plan(cache, batch);
   if (pl.n_items == 0) return EFIM_OK;
-  if (append && (pl.s_max > 1 || (reinterpret_cast<uintptr_t>(append->k) | reinterpret_cast<uintptr_t>(append->v)) & 15)) {
+  const bool in_params = pl.n_items <= pf::InlineItems::MAX && batch->batch <= pf::InlineSplit::MAX_BATCH;
+  const bool aligned = !append || ((reinterpret_cast<uintptr_t>(append->k) | reinterpret_cast<uintptr_t>(append->v)) & 15) == 0;
+  if (append && !(in_params && pl.s_max == 1 && aligned)) {  // (the kernel that appends is one of those with the list in its parameters)
     st = efim_kv_append(cache, batch, rope, nullptr, append->k, append->v, d_status, stream);
     if (st != EFIM_OK) return st;
     append = nullptr;
   }
-  if (pl.n_items <= pf::InlineItems::MAX && batch->batch <= pf::InlineSplit::MAX_BATCH) {
+  if (in_params) {
     pf::InlineList list;
     pf::fill_lists(cache, batch, pl, list.items.items, list.split.keys);
     return run_plan(cache, batch, rope, pl, nullptr, &list, append, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
@@ -247,8 +248,7 @@ bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* b
     if (batch->h_new_len[s] * G > efim::pf::BM) return false;
     with_work += batch->h_new_len[s] > 0;
   }
-  return with_work == 1 && cache->num_kv_heads <= std::min(efim::sm_count(), (int)efim::pf::InlineItems::MAX) &&
-         batch->batch <= efim::pf::InlineSplit::MAX_BATCH;
+  return with_work == 1 && cache->num_kv_heads <= efim::sm_count();
 }
 }  // namespace
 

@@ -154,3 +154,15 @@ def test_one_kernel_up_to_one_query_tile(Hq, Hkv, D, new, kernels):
     assert _kernels_of(s.one_call) == kernels
     s.one_call()
     assert s.same()
+
+
+def test_one_sequence_step_whose_list_is_copied():
+    """One sequence brings new tokens, in a batch too long for lists in the launch parameters: its rows are appended by a kernel
+    of their own, as only kernels with the list in the parameters can."""
+    from tests.test_gpu_parity import _custom
+    new = np.zeros(257, np.int32)
+    new[100] = 20
+    s = _OneSequenceStep(_custom(8, 8, 128, np.full(257, 40, np.int32), new, seed=4))
+    s.two_calls()
+    s.one_call()
+    assert s.same() and int(s.b.status.item()) == 0
