@@ -166,3 +166,34 @@ def test_one_sequence_step_whose_list_is_copied():
     s.two_calls()
     s.one_call()
     assert s.same() and int(s.b.status.item()) == 0
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,new", [(32, 8, 128, 36), (8, 8, 64, 100), (32, 8, 128, 5), (32, 8, 128, 40)])
+def test_nan_queries_of_one_sequence_do_not_slow_another(Hq, Hkv, D, new):
+    """The rows past a sequence in a block of 32 may hold the next sequence's queries; NaN there must not change what the
+    sequence gets, nor make its warps redo their steps (which took 1.25 times as long and more)."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    dw = H.DeviceWorkload(_custom(Hq, Hkv, D, [16384, 0], [new, 8], seed=8), use_rope=False)
+    ws = torch.empty(efim.efim_prefill_workspace_bytes(dw.cache, dw.batch), dtype=torch.uint8, device="cuda")
+    clean = dw.q.clone()
+    poisoned = dw.q.clone()
+    poisoned[new:] = float("nan")
+    out = {}
+    times = {"clean": [], "poisoned": []}
+    for _ in range(15):
+        for what, q in (("clean", clean), ("poisoned", poisoned)):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            for _ in range(10):
+                efim.efim_append_prefill_attn(dw.cache, dw.batch, q, dw.out, dw.lse, 0.0, ws, dw.status)
+            end.record()
+            torch.cuda.synchronize()
+            times[what].append(start.elapsed_time(end))
+            out[what] = dw.out[:new].clone()
+    assert torch.equal(out["clean"].view(torch.int16), out["poisoned"].view(torch.int16))
+    assert dw.out[new:].isnan().all()
+    ratio = np.median(times["poisoned"]) / np.median(times["clean"])
+    assert ratio < 1.1, f"{ratio:.3f} times as long behind NaN queries"
