@@ -122,6 +122,19 @@ __device__ __forceinline__ void rotate8(uint4& va, uint4& vb, const float* c, co
   }
 }
 
+// One half of rotate8: `v` alone, 8 values of either half of a row, with their partners `o`; `flip` turns the sign of the sines
+// (0x80000000 for the first half, which takes a c - b s, else 0).  The same products and roundings, so the same bits: one piece of
+// code for both halves where a warp's lanes hold vectors of either.
+__device__ __forceinline__ void rotate_half(uint4& v, const uint4& o, const float* c, const float* s, uint32_t flip) {
+  uint32_t* a = reinterpret_cast<uint32_t*>(&v);
+  const uint32_t* b = reinterpret_cast<const uint32_t*>(&o);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float s0 = __uint_as_float(__float_as_uint(s[2 * i]) ^ flip), s1 = __uint_as_float(__float_as_uint(s[2 * i + 1]) ^ flip);
+    a[i] = pack_bf16x2(fmaf(bf16lo(a[i]), c[2 * i], bf16lo(b[i]) * s0), fmaf(bf16hi(a[i]), c[2 * i + 1], bf16hi(b[i]) * s1));
+  }
+}
+
 // Interleaved pairing: one 16-byte vector holds 4 pairs (2f, 2f+1).
 __device__ __forceinline__ void rotate4_interleaved(uint4& v, const float* c, const float* s) {
   uint32_t* w = reinterpret_cast<uint32_t*>(&v);
