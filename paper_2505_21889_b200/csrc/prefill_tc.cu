@@ -1060,7 +1060,7 @@ __device__ __forceinline__ void softmax_role(const Cta<D>& c, Work it, int warp)
 // Every bulk-tensor copy costs its issuing warp ~65 cycles (one box per page: 16 slots x all dims
 // of one kv head).  Warp 8 loads the K tiles and warp 11 the V tiles; warp 8 also claims the items.
 template <int D, bool K_ROLE, bool APPEND, typename List>
-__device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap& map, const List& list, WorkItem raw, Work it) {
+__device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap& map, const List& list, Work it) {
   using L = Smem<D>;
   const Params& p = c.p;
   constexpr int n_ring = K_ROLE ? L::NK : L::NV;            // (the ring's constants fold into each copy)
@@ -1068,7 +1068,7 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
   constexpr int full = K_ROLE ? BAR_KFULL : BAR_VFULL, empty = K_ROLE ? BAR_KEMPTY : BAR_VEMPTY;
   const int lane = c.lane, page_l = lane;
   Mailbox mail;                                             // of warp 11; warp 8 keeps the place it writes in it
-  int slot = 0, n_steps = 0, block = blockIdx.x;
+  int slot = 0, n_steps = 0;
   uint32_t phase = 0, claim_phase = 0, new_phase = 0;
   for (;;) {
     const int32_t* bt = p.block_table + (size_t)it.seq * p.max_pages_per_seq + (it.key0 >> 4);
@@ -1083,11 +1083,6 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
     };
     // the block-table read is a dependent global load in front of every copy: fetch it two steps ahead
     int pid_a = lookup(0), pid_b = lookup(1);
-    if constexpr (K_ROLE && std::is_same<List, InlineItems>::value) {
-      // A work list that came in the launch parameters is left in the workspace like any other: a call that
-      // plans for itself may be followed by planned calls with resident lists.
-      if (lane == 0) p.items_out[block] = raw;
-    }
     // Another item is claimed when the copies of the last but one step are due: the rings then hold the steps before,
     // which covers the claim, the item and its first pages.  (Claimed earlier, the last items of a launch would be
     // bound to CTAs that are still busy.)
@@ -1147,13 +1142,12 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
       c.wait(BAR_CLAIM, claim_phase);
       claim_phase ^= 1;
       const bool gone = __any_sync(0xffffffffu, *c.abort_flag != 0);
-      block = gone ? -1 : uniform(claimed_block(c.smem_base + L::CLAIM_OFF));
+      const int block = gone ? -1 : uniform(claimed_block(c.smem_base + L::CLAIM_OFF));
       fence_async_smem();                                   // the answer has been read: the next one may be written
       more = block >= 0;
       if (more) {
-        if constexpr (std::is_same<List, InlineItems>::value) raw = list.items[block];
-        else raw = p.items[block];
-        it = work_of(raw, p);
+        if constexpr (std::is_same<List, InlineItems>::value) it = work_of(list.items[block], p);
+        else it = work_of(p.items[block], p);
       } else {
         it.seq = -1;
       }
@@ -1375,7 +1369,15 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   // memory waits for the kernel before (which may be one that leaves its list in this workspace).
   WorkItem raw;                                               // 32 bytes: two vector loads, no dependent load after them
   if constexpr (std::is_same<List, InlineItems>::value) {
-    if (warp != 9 && warp != 10) pdl_wait();
+    if ((warp != 9 && warp != 10) || blockIdx.x == 0) pdl_wait();
+    // A work list that came in the launch parameters is left in the workspace like any other (a call that plans for itself may
+    // be followed by planned calls with resident lists): by block 0, which always runs, all at once.  (Written by warp 8 of every
+    // CTA, an item at a time, the steps of two-tile items took 6 % longer than those of the kernel without this: 8 x
+    // 128 tokens over 8k planned in the call 131 us, now 124, and 122 with resident lists.)
+    if (blockIdx.x == 0) {
+      const uint4* src = reinterpret_cast<const uint4*>(list.items);
+      for (int i = tid; i < 2 * (int)gridDim.x; i += THREADS) reinterpret_cast<uint4*>(p.items_out)[i] = src[i];
+    }
     raw = list.items[blockIdx.x];
   } else {
     pdl_wait();
@@ -1395,10 +1397,10 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
     if (warp == 8) {
       if (p.early_next) pdl_launch();
-      producer_role<D, true, APPEND>(c, map_k, list, raw, it);
+      producer_role<D, true, APPEND>(c, map_k, list, it);
     } else if (warp == 11) {
       if (p.early_next) pdl_launch();
-      producer_role<D, false, APPEND>(c, map_v, list, raw, it);
+      producer_role<D, false, APPEND>(c, map_v, list, it);
     } else if (warp == 9) {
       PvIssuer<D> pv{c};
       Mailbox mail;
