@@ -13,12 +13,62 @@ def test_items_of_every_shape_in_turn(Hq, Hkv, D):
     that the oracle's queries and keys are the kernel's bit for bit: in a row of one key a single bf16 tie that rounds the
     other way moves the lse by up to 2.7e-3.)"""
     from tests.test_gpu_parity import _check_turn, _custom
+    _check_turn(_custom(Hq, Hkv, D, *_lengths_of_every_shape(Hq, Hkv, D), seed=Hq + D), use_rope=False)
+
+
+def _lengths_of_every_shape(Hq, Hkv, D):
+    """Cached and new tokens of 160 sequences."""
     G = Hq // Hkv
     rng = np.random.default_rng([Hq, Hkv, D])
     rows = np.array([G, 20, 31, 32, 33, 64, 100, 128, 129, 200, 256, 257, 300, 520])
     new = np.maximum(1, rng.permutation(np.tile(rows, 12))[:160] // G).astype(np.int32)
-    cached = rng.choice([0, 1, 15, 16, 79, 80, 81, 160, 200, 239], 160).astype(np.int32)
-    _check_turn(_custom(Hq, Hkv, D, cached, new, seed=Hq + D), use_rope=False)
+    return rng.choice([0, 1, 15, 16, 79, 80, 81, 160, 200, 239], 160).astype(np.int32), new
+
+
+def _items(dw):
+    """Number of work items in the plan of a workload's batch (the seventh word of the plan)."""
+    import paper_2505_21889_b200 as efim
+    plan = efim.efim_prefill_plan(dw.cache, dw.batch)
+    return int(np.frombuffer(bytes(bytearray(np.asarray(plan)[:32].view(np.uint8))), np.int32)[6])
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,D", [(32, 8, 128), (24, 8, 128), (8, 8, 64), (24, 8, 64)])
+def test_items_of_every_shape_rotated_on_load(Hq, Hkv, D, interleaved):
+    """The same batches as one-call steps, whose CTAs rotate the queries of their second and later items as they load them:
+    the bits of efim_kv_append, which rotates them in memory, followed by the attention."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, D, *_lengths_of_every_shape(Hq, Hkv, D), seed=Hq + D)
+    a, b = H.DeviceWorkload(w, interleaved=interleaved), H.DeviceWorkload(w, interleaved=interleaved)
+    assert _items(a) >= 3 * torch.cuda.get_device_properties(0).multi_processor_count
+    a.gpu_kv_append()
+    a.gpu_prefill()
+    ws = torch.empty(efim.efim_prefill_workspace_bytes(b.cache, b.batch), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        b.out.fill_(float("nan"))
+        efim.efim_append_prefill_step(b.cache, b.batch, b.rope, b.q, b.k_new, b.v_new, b.out, b.lse, 0.0, ws, b.status)
+        torch.cuda.synchronize()
+        assert int(a.status.item()) == int(b.status.item()) == 0
+        assert torch.equal(a.out.view(torch.int16), b.out.view(torch.int16)) and torch.equal(a.lse, b.lse)
+        assert torch.equal(a.k_pool.view(torch.int16), b.k_pool.view(torch.int16))
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new", [
+    (32, 8, 64, [849, 472, 698, 78, 63, 600, 43, 820, 527, 225, 117, 432], [1, 8, 1, 35, 32, 32, 8, 50, 64, 1, 8, 32]),
+    (24, 8, 128, [647, 606, 35, 261, 177, 737, 776, 180, 115, 612, 541, 163, 67], [1, 6, 1, 66, 6, 46, 6, 66, 1, 46, 11, 6, 33]),
+])
+def test_items_of_cut_key_ranges_in_turn(Hq, Hkv, D, cached, new):
+    """More items than SMs, of all three shapes and of sequences cut into key chunks: partials leave through the staged stores
+    of a CTA's second item too."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    from tests.test_gpu_parity import _check_turn, _custom
+    dw, _ = _check_turn(_custom(Hq, Hkv, D, cached, new, seed=D), use_rope=False)
+    assert _items(dw) > torch.cuda.get_device_properties(0).multi_processor_count
+    assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 2
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,cached,new,interleaved,max_position,bad_page", [
@@ -197,3 +247,32 @@ def test_nan_queries_of_one_sequence_do_not_slow_another(Hq, Hkv, D, new):
     assert dw.out[new:].isnan().all()
     ratio = np.median(times["poisoned"]) / np.median(times["clean"])
     assert ratio < 1.1, f"{ratio:.3f} times as long behind NaN queries"
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new,interleaved,max_position,sm_scale,lse", [
+    (8, 8, 128, [0, 80], [0, 128], False, None, 0.0, True),     # 128 rows; the first key of a step is new; an idle sequence
+    (32, 8, 128, [79], [32], True, None, 0.3, True),            # the last key of a step is new
+    (24, 8, 64, [200], [33], False, 210, 0.0, True),            # positions beyond the rotary table
+    (24, 8, 64, [200], [33], True, 210, 0.0, True),
+    (64, 2, 128, [100], [4], False, None, 0.05, False),         # 32 heads a group; no lse
+    (16, 1, 128, [0], [8], False, None, 0.0, False),
+])
+def test_rows_appended_by_the_only_kernel(Hq, Hkv, D, cached, new, interleaved, max_position, sm_scale, lse):
+    """Steps that are one kernel, against efim_kv_append without q and the attention-only step, bit for bit."""
+    from tests.test_gpu_parity import _custom
+    s = _OneSequenceStep(_custom(Hq, Hkv, D, cached, new, seed=D + Hq), interleaved, max_position)
+    for d in (s.a, s.b):
+        d.lse.fill_(7.0)
+    s.two_calls(sm_scale, lse)
+    s.one_call(sm_scale, lse)
+    assert s.same()
+    assert int(s.a.status.item()) == int(s.b.status.item()) == (2 if max_position else 0)
+    assert bool((s.b.lse == 7.0).all()) == (not lse)
+    assert _kernels_of(lambda: s.one_call(sm_scale, lse)) == 1
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(64, 2, 128), (32, 1, 64), (32, 2, 64)])
+def test_rows_of_wide_groups_as_boxes(Hq, Hkv, D):
+    """32 and 16 query heads to a kv head: a box of 32 rows is one token's, or two tokens'."""
+    from tests.test_gpu_parity import _check_turn, _custom
+    _check_turn(_custom(Hq, Hkv, D, [70, 0, 200, 31], [1, 9, 8, 17], seed=Hq), use_rope=False)
