@@ -1110,10 +1110,13 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
       }
       c.wait(empty + slot, phase ^ 1);
       if constexpr (APPEND) {
-        // (A table may name a page twice: one of the cached keys' pages is then among those appended to.)
-        const int key = lane < 8 ? pid : new_page;
-        const uint32_t twins = __match_any_sync(0xffffffffu, key >= 0 ? key : -3 - lane) >> 8;
-        if (jj >= first_new || __any_sync(0xffffffffu, lane < 8 && twins != 0)) {
+        bool held = jj >= first_new;
+        if (!held) {                                        // (a table may name a page twice: for cached keys and for new ones)
+          const int key = lane < 8 ? pid : new_page;
+          const uint32_t twins = __match_any_sync(0xffffffffu, key >= 0 ? key : -3 - lane) >> 8;
+          held = __any_sync(0xffffffffu, lane < 8 && twins != 0);
+        }
+        if (held) {
           c.wait(BAR_NEW, new_phase);
           asm volatile("fence.proxy.async;" ::: "memory");
         }
