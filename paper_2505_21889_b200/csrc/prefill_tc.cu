@@ -232,11 +232,6 @@ struct Smem {
 // key far above the ones before it has the probability 1, which bf16 holds exactly: with 2^40 here the
 // outputs of peaked rows (scores of 8 sigma) were off by 2.0e-3 to 2.25e-3 (2-norm) instead of 1.7e-3.
 constexpr float SUM_LIMIT = 256.f;
-// The test is made on the bits: a sum is +0 or above, or NaN (0x7fffffff as arithmetic gives it), so they order as the values
-// do, NaN above all.  A row past the sequence holds whatever follows the sequence and must not make its warp redo
-// steps: nothing reaches its limit, NaN neither.  (With its sums tested like the others', NaN in the queries behind a sequence of 36
-// tokens over 16k at 32/8 heads made its attention 41.5 us instead of 30.3.)
-constexpr uint32_t SUM_REDO = 0x43800001u, SUM_NEVER = 0xffffffffu;      // bits above SUM_LIMIT's
 // The reference is the row's exact maximum over the first EXACT_STEPS steps of a stream, or over the first one
 // where two query tiles see more than EXACT_MAX_STEPS steps.  The key at the reference is weighted without
 // rounding and short rows live on their heaviest keys: with one step everywhere, 16 tokens over 240 at 4/4 x 64
@@ -770,7 +765,7 @@ __device__ __forceinline__ void softmax_tiny(const Cta<D>& c, const Work& it, in
     if (k > 0) {
       c.wait(BAR_PV + st, (n - 1) & 1);                   // P of the step before is consumed
       tc_fence_after();
-      const bool redo = row.valid && !(sum <= SUM_LIMIT);   // (a row past the sequence asks for nothing: see SUM_REDO)
+      const bool redo = row.valid && !(sum <= SUM_LIMIT);   // (a row past the sequence asks for nothing: see softmax_item)
       if (__any_sync(0xffffffffu, redo || (row.valid && alpha != 1.f))) {
         if (redo) alpha = move_reference(m_ref, row_max<KQ>(s) * p.scale_log2);
         l_sum *= alpha;
@@ -899,7 +894,6 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
   const int kv_first = it.key0 + (DUAL ? 0 : st * BN), kv_step = DUAL ? BN : 2 * BN;
   // (a row past the sequence holds zeros or what follows the sequence: against this reference its probabilities are zero)
   float m_ref = row.valid ? -FLT_MAX : FLT_MAX, l_sum = 0.f;
-  const uint32_t sum_redo = row.valid ? SUM_REDO : SUM_NEVER;
   for (int k = 0; k < my_cnt; ++k, ++n) {
     c.wait(BAR_S + st, n & 1);
     tc_fence_after();
@@ -930,11 +924,10 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
     if (__builtin_expect(edge || k < exact, 0)) freed();
     // alpha: what O and the sum so far are scaled by.  A moved reference lowers the limit, so that the one
     // test below finds it (a second condition there: 8 x 128 tokens over 8k 150.0 -> 152.6 us).
-    float alpha = 1.f;
-    uint32_t limit = sum_redo;
+    float alpha = 1.f, limit = SUM_LIMIT;
     if (__builtin_expect(k < exact, 0)) {
       alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
-      if (row.valid && alpha != 1.f) limit = 0u;
+      if (alpha != 1.f) limit = -1.f;
     }
     uint32_t v[BN / 2];                                     // P as bf16 pairs
     const float neg_m = -m_ref;
@@ -946,16 +939,21 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
       tc_fence_after();
     }
     tmem_st<BN / 2>(p_addr, v);
-    if (__builtin_expect(__any_sync(0xffffffffu, __float_as_uint(sum) >= limit) && k > 0, 0)) {
+    if (__builtin_expect(__any_sync(0xffffffffu, !(sum <= limit)) && k > 0, 0)) {
       // (O is quiet: PV(k-1) has finished and PV(k) waits for this warp)
-      const bool redo = __float_as_uint(sum) >= sum_redo;
-      if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
-      l_sum *= alpha;
-      rescale_o_row<D>(o_addr, alpha);
-      if (__any_sync(0xffffffffu, redo)) {
-        sum = row_exp<BN>(s, p.scale_log2, -m_ref, v);
-        tmem_wait_st();                                     // two stores to the same columns are not ordered by themselves
-        tmem_st<BN / 2>(p_addr, v);
+      // A row past the sequence holds whatever follows it and asks for nothing.  (With its sums heard like the others', NaN in the
+      // queries behind a sequence of 36 tokens over 16k at 32/8 heads made its attention 41.5 us instead of 30.3; now 30.6.
+      // A limit of its own for every lane instead, in the test above: prompts of 1-3.5k tokens 0.7 % slower.)
+      const bool redo = row.valid && !(sum <= SUM_LIMIT);
+      if (__any_sync(0xffffffffu, row.valid && !(sum <= limit))) {
+        if (redo) alpha = move_reference(m_ref, row_max<BN>(s) * p.scale_log2);
+        l_sum *= alpha;
+        rescale_o_row<D>(o_addr, alpha);
+        if (__any_sync(0xffffffffu, redo)) {
+          sum = row_exp<BN>(s, p.scale_log2, -m_ref, v);
+          tmem_wait_st();                                   // two stores to the same columns are not ordered by themselves
+          tmem_st<BN / 2>(p_addr, v);
+        }
       }
     }
     tmem_wait_st();
