@@ -321,38 +321,47 @@ __device__ __noinline__ void q_rows_rotated_to_smem(const uint4* q, const float*
   // The loads of two instructions' rows are on their way together (a store between them would keep the second's back), and both
   // halves of a row go through the same code: the warp's lanes hold vectors of either.  One at a time, a branch per half: 16
   // prompts of 1-3.5k tokens 1,022 us for append and attention, 53 x 1-406 over 100-549 at 24/8 heads 119, 16 over 240 at
-  // 4/4 x 64 7.8; this: 920, 96.5, 7.6; with a branch per half 945, 101, 8.0, and four at a time 995, 95, -.
+  // 4/4 x 64 7.8; this: 920, 97, 7.5; with a branch per half 945, 101, 8.0, and four at a time 995, 95, -.  (20 x 1 over 0 at 32/32:
+  // 33.9; 36 with groups without rows rotated too; 32.)
   constexpr int AT_ONCE = 2;
   const int cs_off = interleaved ? c * 4 : (c % (VEC / 2)) * 8;
   const uint32_t flip = c < VEC / 2 ? 0x80000000u : 0u;
+  uint32_t have = __ballot_sync(0xffffffffu, th >= 0);
 #pragma unroll 1
-  for (int i0 = 0; i0 < VEC; i0 += AT_ONCE) {
+  for (int i0 = 0; i0 < VEC; i0 += AT_ONCE, have >>= AT_ONCE * RPI) {
     uint4 v[AT_ONCE], o[AT_ONCE];
-    float4 cf[AT_ONCE][2], sf[AT_ONCE][2];
 #pragma unroll
-    for (int b = 0; b < AT_ONCE; ++b) {
-      const int t = __shfl_sync(0xffffffffu, th, (i0 + b) * RPI + sub), ps = __shfl_sync(0xffffffffu, pos, (i0 + b) * RPI + sub);
-      v[b] = o[b] = make_uint4(0, 0, 0, 0);
-      cf[b][0] = cf[b][1] = sf[b][0] = sf[b][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (t >= 0) {
-        const uint4* src = q + (size_t)t * VEC;
-        const float4* cs = reinterpret_cast<const float4*>(cos_sin + (size_t)ps * D + cs_off);
-        v[b] = src[c];
-        cf[b][0] = cs[0];
-        sf[b][0] = cs[D / 8];
-        if (!interleaved) {
-          o[b] = src[c ^ (VEC / 2)];
-          cf[b][1] = cs[1];
-          sf[b][1] = cs[D / 8 + 1];
+    for (int b = 0; b < AT_ONCE; ++b) v[b] = make_uint4(0, 0, 0, 0);
+    if (have & ((1u << AT_ONCE * RPI) - 1)) {               // (none in most of a block of one token's rows)
+      float4 cf[AT_ONCE][2], sf[AT_ONCE][2];
+#pragma unroll
+      for (int b = 0; b < AT_ONCE; ++b) {
+        const int t = __shfl_sync(0xffffffffu, th, (i0 + b) * RPI + sub), ps = __shfl_sync(0xffffffffu, pos, (i0 + b) * RPI + sub);
+        o[b] = v[b];
+        cf[b][0] = cf[b][1] = sf[b][0] = sf[b][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t >= 0) {
+          const uint4* src = q + (size_t)t * VEC;
+          const float4* cs = reinterpret_cast<const float4*>(cos_sin + (size_t)ps * D + cs_off);
+          v[b] = src[c];
+          cf[b][0] = cs[0];
+          sf[b][0] = cs[D / 8];
+          if (!interleaved) {
+            o[b] = src[c ^ (VEC / 2)];
+            cf[b][1] = cs[1];
+            sf[b][1] = cs[D / 8 + 1];
+          }
         }
+      }
+#pragma unroll
+      for (int b = 0; b < AT_ONCE; ++b) {
+        const float *cp = reinterpret_cast<const float*>(cf[b]), *sp = reinterpret_cast<const float*>(sf[b]);
+        if (interleaved) rotate4_interleaved(v[b], cp, sp);
+        else rotate_half(v[b], o[b], cp, sp, flip);
       }
     }
 #pragma unroll
     for (int b = 0; b < AT_ONCE; ++b) {
       const int r = row0 + (i0 + b) * RPI + sub;
-      const float *cp = reinterpret_cast<const float*>(cf[b]), *sp = reinterpret_cast<const float*>(sf[b]);
-      if (interleaved) rotate4_interleaved(v[b], cp, sp);
-      else rotate_half(v[b], o[b], cp, sp, flip);
       *reinterpret_cast<uint4*>(tile + (c >> 3) * L::HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v[b];
     }
   }
