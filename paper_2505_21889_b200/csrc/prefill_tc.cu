@@ -1077,6 +1077,14 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
   Mailbox mail;                                             // of warp 11; warp 8 keeps the place it writes in it
   int slot = 0, n_steps = 0;
   uint32_t phase = 0, claim_phase = 0, new_phase = 0;
+  // A work list that came in the launch parameters is left in the workspace like any other: a call that plans for itself may be
+  // followed by planned calls with resident lists.  A CTA's first item is written here, a claimed one by warp 8 as it
+  // claims it.  (By warp 8 at the head of each item's copies, the steps of two-tile items took 6 % longer than in the kernel for
+  // resident lists: 8 x 128 tokens over 8k planned in the call 130 us against 121, now 121.  All by block 0: 121 too, but 14
+  // x 8-14 over 0 at 32/8 x 64 7.8 us instead of 6.8.)
+  if constexpr (!K_ROLE && std::is_same<List, InlineItems>::value) {
+    if (lane == 0) p.items_out[blockIdx.x] = list.items[blockIdx.x];
+  }
   for (;;) {
     const int32_t* bt = p.block_table + (size_t)it.seq * p.max_pages_per_seq + (it.key0 >> 4);
     const int n_pages = (it.kv_cap - it.key0 + 15) >> 4;    // pages this item reads
@@ -1156,8 +1164,13 @@ __device__ __forceinline__ void producer_role(const Cta<D>& c, const CUtensorMap
       fence_async_smem();                                   // the answer has been read: the next one may be written
       more = block >= 0;
       if (more) {
-        if constexpr (std::is_same<List, InlineItems>::value) it = work_of(list.items[block], p);
-        else it = work_of(p.items[block], p);
+        if constexpr (std::is_same<List, InlineItems>::value) {
+          const WorkItem w = list.items[block];
+          if (lane == 0) p.items_out[block] = w;
+          it = work_of(w, p);
+        } else {
+          it = work_of(p.items[block], p);
+        }
       } else {
         it.seq = -1;
       }
@@ -1379,15 +1392,7 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   // memory waits for the kernel before (which may be one that leaves its list in this workspace).
   WorkItem raw;                                               // 32 bytes: two vector loads, no dependent load after them
   if constexpr (std::is_same<List, InlineItems>::value) {
-    if ((warp != 9 && warp != 10) || blockIdx.x == 0) pdl_wait();
-    // A work list that came in the launch parameters is left in the workspace like any other (a call that plans for itself may
-    // be followed by planned calls with resident lists): by block 0, which always runs, all at once.  (Written by warp 8 of every
-    // CTA, an item at a time, the steps of two-tile items took 6 % longer than those of the kernel without this: 8 x
-    // 128 tokens over 8k planned in the call 131 us, now 124, and 122 with resident lists.)
-    if (blockIdx.x == 0) {
-      const uint4* src = reinterpret_cast<const uint4*>(list.items);
-      for (int i = tid; i < 2 * (int)gridDim.x; i += THREADS) reinterpret_cast<uint4*>(p.items_out)[i] = src[i];
-    }
+    if (warp != 9 && warp != 10) pdl_wait();
     raw = list.items[blockIdx.x];
   } else {
     pdl_wait();

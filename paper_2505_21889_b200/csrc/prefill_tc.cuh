@@ -84,7 +84,7 @@ struct Plan {
 // items) hides the copy, while room for 640 items costs every call 0.7 us more on the host.  A sequence with
 // work has at least one item, so both lists get the same size.
 struct NoList {};
-struct alignas(16) InlineItems {          // read as 16-byte vectors
+struct InlineItems {
   static constexpr int MAX = 256;
   WorkItem items[MAX];
 };
