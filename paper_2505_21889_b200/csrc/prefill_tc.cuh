@@ -18,12 +18,13 @@ constexpr int NQ = 2;          // query tiles per CTA sharing one K/V stream
 constexpr int BN = 80;
 constexpr int THREADS = 384;   // 2 softmax warpgroups + 1 service warpgroup (2 TMA warps, 2 MMA warps)
 // Register split (setmaxnreg): the block launches with 168 registers per thread
-// (65536 / 384, rounded to 8) = 64512 in total; 2 x 128 x 216 + 128 x 72 = 64512 uses them all
-// (the sum must not exceed the launch total: an increase beyond it would wait forever).  208 / 88: the softmax warps
-// spill seven words a step (16 prompts of 1-3.5k tokens 975 -> 1,012 us, 8 x 3,200 tokens over 5k 2.51 -> 2.55 ms);
-// 224 / 56: the service warps spill (1,027 us, 2.72 ms).
-constexpr int REGS_SOFTMAX = 216;
-constexpr int REGS_SERVICE = 72;
+// (65536 / 384, rounded to 8) = 64512 in total; 2 x 128 x 216 + 128 x 72 and 2 x 128 x 208 + 128 x 88 use them all
+// (the sum must not exceed the launch total: an increase beyond it would wait forever).  At head_dim 128 with 208 / 88 the
+// softmax warps spill seven words a step (16 prompts of 1-3.5k tokens 975 -> 1,012 us, 8 x 3,200 tokens over 5k 2.51 -> 2.55 ms);
+// 224 / 56: the service warps spill (1,027 us, 2.72 ms).  At head_dim 64 216 / 72 and 208 / 88 need the same spills, and 37 x 128
+// tokens over 4,000 keys at 4/4 heads take 40.6 and 39.2 us, 26 x 1-132 over 6-15k at 32/8 297.6 and 295.3.
+template <int D> constexpr int REGS_SOFTMAX = D == 128 ? 216 : 208;
+template <int D> constexpr int REGS_SERVICE = D == 128 ? 72 : 88;
 
 // One work item: packed rows [row0, row0 + 256) of (seq, kv head) against the keys of the
 // 128-key tiles [tile_begin, tile_end).  Packed row R = token * G + head-in-group.  The sequence's
