@@ -199,8 +199,9 @@ enum {
 // writes (a page is two key groups).  In both, 16-byte chunk c of row r is stored at chunk
 // position c ^ (r & 7) (the 128B swizzle the tensor-map copies and the MMA descriptors use).
 // K and V tiles have rings of their own: every ring barrier is waited on by one warp, phase after
-// phase, from the CTA's first item to its last.  (Three entries each at head_dim 128: 8 x 3,200 tokens over 5k keys
-// 2,484 us, 8 x 128 over 8k 149; four 2,512 and 150.5, four of K and three of V 2,511 and 152.5.)
+// phase, from the CTA's first item to its last.  Three entries each at head_dim 128: more do not fit beside the output rows
+// (and without those four each, or four of K, were no faster: 8 x 3,200 tokens over 5k keys 2,512 and 2,511 us against
+// 2,484, 8 x 128 over 8k 150.5 and 152.5 against 149).
 template <int D>
 struct Smem {
   static constexpr int HALVES = D / 64;
@@ -607,7 +608,8 @@ __device__ __forceinline__ void tma_store_rows(uint32_t src, const CUtensorMap* 
 }
 
 // The query rows of a tile, by the four warps of a stream, each its 32-lane quarter.  Where 32 rows are whole tokens they
-// are copied as boxes: per-lane copies kept the softmax warps for 2,300 cycles per item of prompts.  (Rows past the sequence then hold what follows it; nothing of theirs is stored.)
+// are copied as boxes: per-lane copies kept the softmax warps for 2,300 cycles per item of prompts.  (Rows past the sequence then
+// hold what follows it; nothing of theirs is stored, nor heard by the steps.)
 template <int D>
 __device__ __forceinline__ void fetch_q(const Cta<D>& c, const Work& it, int qt, int w) {
   using L = Smem<D>;
@@ -899,8 +901,8 @@ __device__ __forceinline__ bool softmax_item(const Cta<D>& c, const Work& it, Wo
   const uint32_t o_addr = c.tmem_O + lane_addr + st * D;
   const int my_cnt = it.steps(st);
   const Row row(p, it, DUAL ? st : 0, w, c.lane);
-  // keys this row sees; rows past the sequence are computed like the piece's last row and
-  // dropped (with 0 here they would take the masking path on every tile and slow their group)
+  // keys this row sees; a row past the sequence is shown all of the item's, each with probability 0 (with 0 keys it would
+  // take the masking path on every step and slow its group)
   const int vis = row.valid ? min(row.pos + 1, it.kv_cap) : it.kv_cap;
   const int exact = !DUAL || it.nt <= EXACT_MAX_STEPS ? EXACT_STEPS : 1;
   const int kv_first = it.key0 + (DUAL ? 0 : st * BN), kv_step = DUAL ? BN : 2 * BN;
@@ -1333,14 +1335,16 @@ struct QkIssuer {
 // started yet, until none is left - so the hardware's order and balance stay, and what a fresh CTA costs outside its
 // steps is paid once: the next item's pages are copied while the present one's last steps run, its query rows under
 // the last PV, its first scores under the epilogue.  A CTA per item spent 14,000 cycles of each outside the steps (of
-// 2,000); between two items it is 8,000.  Append and attention, one CTA per item -> this: 16 prompts of 1-3.5k tokens
-// 1,028 -> 970 us, 16 x 8-112 tokens over 1-3.4k planned in the call 69 -> 65, 64 mixed rows at 28/4 heads 320 -> 307,
-// 16 x 32-256 over 2-8k at 32/32 320 -> 308, 8 x 3,200 over 5k 2,590 -> 2,490.
+// 2,000): launch gap, set-up, query rows and first pages in front, the last PV, the output and the exit behind.  From one item
+// to the next it is 4,300 to 4,600 (prompts: look-up 400, query boxes 470 and 210, last PV 250, output 2,560, wait for the
+// first scores 640), 8,800 where the query rows come per lane and 16,300 where they are rotated as they come.  Append and attention,
+// one CTA per item -> now: 16 prompts of 1-3.5k tokens 1,017 -> 898 us, 16 x 8-112 tokens over 1-3.4k planned in the call 69 -> 64,
+// 64 mixed rows at 28/4 heads 316 -> 302, 16 x 32-256 over 2-8k at 32/32 317 -> 308, 8 x 3,200 over 5k 2,555 -> 2,450.
 // The work list: in the workspace (List = NoList), or, a short one planned inside the call, in the launch
 // parameters (List = InlineItems) - which saves the copy between the append and this kernel.
 // APPEND: the softmax warps of stream 1 first put the item's new k/v rows into their pages, and the copies of those pages
 // wait for them: a step of a few short rows is one launch instead of two (16 tokens over 240 at 4/4 heads x 64 9.85 ->
-// 7.35 us).  A kernel of its own: in the others' place it cost their steps 5 %.
+// 7.35 us, now 7.5 with the rows' pages compared).  A kernel of its own: in the others' place it cost their steps 5 %.
 template <int D, typename List, bool APPEND>
 __global__ void __launch_bounds__(THREADS, 1)
 prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -1799,7 +1803,8 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   const CUtensorMap mk = *pk;
   const CUtensorMap* pv = pool_map(c->d_v_pool, c->num_pages, c->num_kv_heads, D);
   if (!pv) return EFIM_ERR_CUDA;
-  // Query and output rows as boxes of 32 rows, where those are whole tokens and there are as many.
+  // Query and output rows as boxes of 32 rows, where those are whole tokens and there are as many.  (Encoding a map takes the
+  // host 0.09 us; they are of this call's buffers and not kept.)
   p.g_mul = p.G == 1 ? 0u : (uint32_t)((1ull << 32) / (unsigned)p.G + 1);
   CUtensorMap mq{}, mo{};
   if (p.G <= 32 && 32 % p.G == 0 && (long long)p.total_new_tokens * p.G >= 32) {
