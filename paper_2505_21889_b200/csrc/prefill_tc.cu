@@ -1454,75 +1454,119 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   }
 }
 
-// Merge the KV-chunk partials of split sequences: one warp per (token, head), four partial rows in flight.
-// `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the launch
-// parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
+// Merge the KV-chunk partials of split sequences.  A warp takes up to MERGE_ROWS consecutive heads of one token, their partial
+// rows of two chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the
+// launch parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
+//
+// Bound: the partials' bytes, which the kernel before has left in L2, behind a chain of dependent look-ups.  The lanes look
+// a token's sequence up together, 32 candidates a trip, and bring its lengths along in the last one; with a warp per row
+// that bisected q_indptr and then read one value after the other, a chain of ten trips in each of 8 waves of CTAs,
+// the merge of 960 tokens at 32/8 heads took 25 us and that of 2,800 tokens at 28/4 97 us.
+constexpr int MERGE_WARPS = 8, MERGE_ROWS = 4;
+__host__ __device__ constexpr int merge_rows(int Hq) { return Hq % 4 == 0 ? 4 : (Hq % 2 == 0 ? 2 : 1); }
 template <int D, typename Split>
-__global__ void __launch_bounds__(128) prefill_merge_kernel(const Params p, const __grid_constant__ Split split) {
-  constexpr int EPL = D / 32;
+__global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const Params p, const __grid_constant__ Split split) {
+  constexpr int EPL = D / 32;                               // dims of a lane
+  constexpr int AT_ONCE = 2;                                // chunks whose rows are in flight together
   constexpr bool inl = std::is_same<Split, InlineSplit>::value;
   const int lane = threadIdx.x & 31;
-  const size_t th = (size_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int nr = merge_rows(p.Hq);                          // rows of this warp: heads of one token
+  const size_t th = ((size_t)blockIdx.x * MERGE_WARPS + (threadIdx.x >> 5)) * nr;
   // (everything before the attention kernel has completed, and that kernel writes partials only: the
   // look-ups need not wait for it.  Read in L2, where what has completed is visible.)
   int st = 0, nc = 0;
   if (th < (size_t)p.total_new_tokens * p.Hq) {
     const int t = (int)(th / p.Hq);
-    int lo = 0, hi = p.batch;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (__ldcg(p.q_indptr + mid) <= t) lo = mid; else hi = mid;
+    int lo = 0, n = p.batch;                                // the last sequence that starts at or before t is one of [lo, lo + n)
+    while (n > 32) {
+      const int step = (n + 31) / 32, probe = lo + lane * step;
+      const bool le = lane * step < n && __ldcg(p.q_indptr + probe) <= t;
+      const int i = 31 - __clz((int)(__ballot_sync(0xffffffffu, le) | 1u));
+      n = min(step, n - i * step);
+      lo += i * step;
     }
-    if constexpr (inl) st = split.keys[lo];
-    else st = __ldcg(p.split_tokens + lo);
-    if (st > 0) nc = min(p.s_max, (__ldcg(p.cached_len + lo) + (t - __ldcg(p.q_indptr + lo)) + 1 + st - 1) / st);
+    int first = 0x7fffffff, cached = 0, keys = 0;
+    if (lane < n) {
+      first = __ldcg(p.q_indptr + lo + lane);
+      cached = __ldcg(p.cached_len + lo + lane);
+      if constexpr (inl) keys = split.keys[lo + lane];
+      else keys = __ldcg(p.split_tokens + lo + lane);
+    }
+    const int i = 31 - __clz((int)(__ballot_sync(0xffffffffu, first <= t) | 1u));
+    st = __shfl_sync(0xffffffffu, keys, i);
+    const int pos = __shfl_sync(0xffffffffu, cached, i) + t - __shfl_sync(0xffffffffu, first, i);
+    if (st > 0) nc = min(p.s_max, (pos + 1 + st - 1) / st);
   }
   pdl_wait();
   pdl_launch();
   if constexpr (inl) {
     if (blockIdx.x == 0)
-      for (int i = threadIdx.x; i < p.batch; i += 128) p.split_out[i] = split.keys[i];
+      for (int i = threadIdx.x; i < p.batch; i += 32 * MERGE_WARPS) p.split_out[i] = split.keys[i];
   }
   if (nc == 0) return;                                      // written directly by the main kernel
-  const float* pl = p.part_lse + th * p.s_max;
+  // rows r of chunks c .. c + AT_ONCE - 1 (rows and chunks past the last: read again, without weight)
   const float* po = p.part_o + th * p.s_max * D + lane * EPL;
-  const float mine = lane < nc ? pl[lane] : -INFINITY;      // at most 16 chunks
-  float M = mine;
+  __align__(16) float v[AT_ONCE][MERGE_ROWS][EPL];
+  auto fetch = [&](int c0) {
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) M = max_nan(M, __shfl_xor_sync(0xffffffffu, M, d));   // a NaN chunk makes the row NaN
-  float Lsum = 0.f, acc[EPL];
+    for (int c = 0; c < AT_ONCE; ++c)
 #pragma unroll
-  for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-  if (!(M == -INFINITY)) {
-    const float w_mine = exp2f(mine - M);                   // 0 beyond the last chunk
-    for (int c0 = 0; c0 < nc; c0 += 4) {
-      __align__(16) float v[4][EPL];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float* src = po + (size_t)min(c0 + i, nc - 1) * D;
+      for (int r = 0; r < MERGE_ROWS; ++r) {
+        const float* src = po + ((size_t)min(r, nr - 1) * p.s_max + min(c0 + c, nc - 1)) * D;
         if constexpr (EPL == 4) {
-          *reinterpret_cast<float4*>(v[i]) = *reinterpret_cast<const float4*>(src);
+          *reinterpret_cast<float4*>(v[c][r]) = __ldcg(reinterpret_cast<const float4*>(src));
         } else {
-          *reinterpret_cast<float2*>(v[i]) = *reinterpret_cast<const float2*>(src);
+          *reinterpret_cast<float2*>(v[c][r]) = __ldcg(reinterpret_cast<const float2*>(src));
         }
       }
+  };
+  // lane 16 h + c: the lse of chunk c (at most 16) of rows h and h + 2
+  const int my_c = lane & 15, my_r = lane >> 4;
+  float lse[2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float w = __shfl_sync(0xffffffffu, w_mine, c0 + i);
-        Lsum += w;
+  for (int j = 0; j < 2; ++j)
+    lse[j] = my_c < nc && my_r + 2 * j < nr ? __ldcg(p.part_lse + (th + my_r + 2 * j) * p.s_max + my_c) : -INFINITY;
+  fetch(0);
+  float M[2], L[2], w[2];
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[e] = fmaf(w, v[i][e], acc[e]);
+  for (int j = 0; j < 2; ++j) {
+    M[j] = lse[j];
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) M[j] = max_nan(M[j], __shfl_xor_sync(0xffffffffu, M[j], d));   // a NaN chunk makes the row NaN
+    w[j] = M[j] == -INFINITY ? 0.f : exp2f(lse[j] - M[j]);                                       // 0 beyond the last chunk
+    L[j] = w[j];
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) L[j] += __shfl_xor_sync(0xffffffffu, L[j], d);
+  }
+  float acc[MERGE_ROWS][EPL];
+#pragma unroll
+  for (int r = 0; r < MERGE_ROWS; ++r)
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) acc[r][e] = 0.f;
+  for (int c0 = 0; c0 < nc; c0 += AT_ONCE) {
+    if (c0 > 0) fetch(c0);
+#pragma unroll
+    for (int c = 0; c < AT_ONCE; ++c)
+#pragma unroll
+      for (int r = 0; r < MERGE_ROWS; ++r) {
+        const float wc = __shfl_sync(0xffffffffu, w[r >> 1], (r & 1) * 16 + ((c0 + c) & 15));
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[r][e] = c0 + c < nc ? fmaf(wc, v[c][r][e], acc[r][e]) : acc[r][e];
       }
+  }
+#pragma unroll
+  for (int r = 0; r < MERGE_ROWS; ++r) {
+    const float Lr = __shfl_sync(0xffffffffu, L[r >> 1], (r & 1) * 16), Mr = __shfl_sync(0xffffffffu, M[r >> 1], (r & 1) * 16);
+    if (r >= nr) break;
+    const float inv = Lr == 0.f ? 0.f : 1.f / Lr;
+    uint16_t* out = p.out + (th + r) * D + lane * EPL;
+    if constexpr (EPL == 4) {
+      *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[r][0] * inv, acc[r][1] * inv), pack_bf16x2(acc[r][2] * inv, acc[r][3] * inv));
+    } else {
+      *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[r][0] * inv, acc[r][1] * inv);
     }
+    if (p.lse && lane == 0) p.lse[th + r] = Lr == 0.f ? -INFINITY : (Mr + log2f(Lr)) * 0.6931471805599453f;
   }
-  const float inv = Lsum == 0.f ? 0.f : 1.f / Lsum;
-  uint16_t* out = p.out + th * D + lane * EPL;
-  if constexpr (EPL == 4) {
-    *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
-  } else {
-    *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
-  }
-  if (p.lse && lane == 0) p.lse[th] = Lsum == 0.f ? -INFINITY : (M + log2f(Lsum)) * 0.6931471805599453f;
 }
 
 // ------------------------------------------------------------------ host side
@@ -1825,11 +1869,12 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   else st = start(std::false_type{});
   if (st != EFIM_OK) return st;
   if (pl.s_max > 1) {
-    const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + 3) / 4);
+    const size_t per_block = MERGE_WARPS * merge_rows(p.Hq);
+    const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + per_block - 1) / per_block);
     if constexpr (inl)
-      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, InlineSplit>, dim3(blocks), dim3(128), 0, s, p, list.split));
+      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, InlineSplit>, dim3(blocks), dim3(32 * MERGE_WARPS), 0, s, p, list.split));
     else
-      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, NoList>, dim3(blocks), dim3(128), 0, s, p, NoList{}));
+      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, NoList>, dim3(blocks), dim3(32 * MERGE_WARPS), 0, s, p, NoList{}));
   }
   return EFIM_OK;
 }
