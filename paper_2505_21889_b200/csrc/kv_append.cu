@@ -30,117 +30,121 @@ struct KvAppendParams {
 // in flight per lane; v is copied straight into the page slot.  Many tokens: one warp per
 // token keeps every SM full of independent streams.  Few tokens (a decode step): eight
 // warps per token, because then the time is one token's latency.
+//
+// Bound: HBM with many tokens, else a chain of dependent loads.  A token's rows do not depend on where it goes, so the first
+// of them (all, with few tokens) are on their way before its sequence is looked up; the warp's lanes look that up together,
+// 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.
 constexpr int KV_APPEND_THREADS = 256;
 
 template <int D, int WPT>
-__global__ void __launch_bounds__(KV_APPEND_THREADS) kv_append_kernel(const KvAppendParams p) {
+__global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const KvAppendParams p) {
   constexpr int VEC = D / 8;            // 16-byte vectors per head row
   constexpr int HALF = VEC / 2;
   constexpr int LANES = 32 * WPT;       // lanes working on one token
-  const int lane = threadIdx.x % LANES;
+  constexpr int COPIES = WPT == 1 ? 4 : 2;   // vectors of a straight copy in flight per lane
+  constexpr bool AHEAD = WPT > 1;       // first rows fetched before the look-up
+  const int lane = threadIdx.x % LANES, wl = threadIdx.x & 31;
   const int t = blockIdx.x * (KV_APPEND_THREADS / LANES) + threadIdx.x / LANES;
   pdl_wait();
   if (p.early_next) pdl_launch();
   if (t >= p.total_new_tokens) return;
-  // sequence of this token: last s with q_indptr[s] <= t.  Up to 32 sequences are probed by the
-  // warp's lanes at once (one round trip instead of a chain of five); more by bisection.
-  int s;
-  if (p.batch <= 32) {
-    const int wl = threadIdx.x & 31;
-    const bool le = wl < p.batch && *(p.q_indptr + wl) <= t;
-    s = 31 - __clz((int)(__ballot_sync(0xffffffffu, le) | 1u));
-  } else {
-    int lo = 0, hi = p.batch;
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (*(p.q_indptr + mid) <= t) lo = mid; else hi = mid;
-    }
-    s = lo;
-  }
-  const int pos = *(p.cached_len + s) + (t - *(p.q_indptr + s));
-  const int page_idx = pos >> 4;
-  int err = 0;
-  int page = -1;
-  if (pos < 0 || page_idx >= p.max_pages_per_seq || (p.cos_sin && pos >= p.max_position)) {
-    err = EFIM_DEV_BAD_POSITION;
-  } else {
-    page = *(p.block_table + (size_t)s * p.max_pages_per_seq + page_idx);
-    if (page < 0 || page >= p.num_pages) err = EFIM_DEV_BAD_PAGE;
-  }
-  if (err) {
-    if (lane == 0 && p.status) atomicOr(p.status, err);
-    return;
-  }
-  const int slot = pos & 15;
-  const size_t pool_tok = ((size_t)page * p.Hkv) * 16 * D + (size_t)slot * D;   // + h * 16 * D
   const uint4* kin = reinterpret_cast<const uint4*>(p.k_new + (size_t)t * p.Hkv * D);
   const uint4* vin = reinterpret_cast<const uint4*>(p.v_new + (size_t)t * p.Hkv * D);
   uint4* qio = p.q ? reinterpret_cast<uint4*>(p.q + (size_t)t * p.Hq * D) : nullptr;
-  const int nq = p.q ? p.Hq : 0;
-  // straight copy of a [Hkv][D] row into the page slot, four vectors in flight per lane
+  const int nq = p.q ? p.Hq : 0, nh = nq + p.Hkv, n_vec = p.Hkv * VEC;
+  // rotated heads: this lane's position j and first head, heads that the token's lanes cover at once
+  const bool halves = !p.interleaved;
+  const int per_head = halves ? HALF : VEC, HP = LANES / per_head;
+  const int j = lane % per_head, h0 = lane / per_head;
+  auto row_of = [&](int h) -> const uint4* { return h < nq ? qio + h * VEC : kin + (h - nq) * VEC; };
+  uint4 v[COPIES], a[2], b[2];
+  auto fetch_copy = [&](const uint4* src, int u0) {
+#pragma unroll
+    for (int i = 0; i < COPIES; ++i)
+      if (u0 + LANES * i < n_vec) v[i] = ldg_stream(src + u0 + LANES * i);
+  };
+  auto fetch_heads = [&](int h) {       // vectors of heads h and h + HP
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (h + i * HP < nh) {
+        a[i] = ldg_stream(row_of(h + i * HP) + j);
+        if (halves) b[i] = ldg_stream(row_of(h + i * HP) + j + HALF);
+      }
+  };
+  if constexpr (AHEAD) {
+    if (p.cos_sin) fetch_heads(h0);
+    fetch_copy(vin, lane);
+  }
+  // sequence of this token: the last one that starts at or before t, one of [lo, lo + n)
+  int lo = 0, n = p.batch;
+  while (n > 32) {
+    const int step = (n + 31) / 32;
+    const bool le = wl * step < n && *(p.q_indptr + lo + wl * step) <= t;
+    const int i = 31 - __clz((int)(__ballot_sync(0xffffffffu, le) | 1u));
+    n = min(step, n - i * step);
+    lo += i * step;
+  }
+  int first = 0, cached = 0;
+  if (wl < n) {
+    first = *(p.q_indptr + lo + wl);
+    cached = *(p.cached_len + lo + wl);
+  }
+  const int i_seq = 31 - __clz((int)(__ballot_sync(0xffffffffu, wl < n && first <= t) | 1u));
+  const int pos = __shfl_sync(0xffffffffu, cached, i_seq) + t - __shfl_sync(0xffffffffu, first, i_seq);
+  const int page_idx = pos >> 4;
+  if (pos < 0 || page_idx >= p.max_pages_per_seq || (p.cos_sin && pos >= p.max_position)) {
+    if (lane == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_POSITION);
+    return;
+  }
+  const int page = *(p.block_table + (size_t)(lo + i_seq) * p.max_pages_per_seq + page_idx);
+  // rotary values: position j of the row's halves (8 of either), or the 4 pairs of vector j
+  float c[8], sn[8];
+  if (p.cos_sin) {
+    const float* cs = p.cos_sin + (size_t)pos * D + j * (halves ? 8 : 4);      // cos[0..D/2) then sin[0..D/2)
+    *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(cs));
+    *reinterpret_cast<float4*>(sn) = __ldg(reinterpret_cast<const float4*>(cs + D / 2));
+    if (halves) {
+      *reinterpret_cast<float4*>(c + 4) = __ldg(reinterpret_cast<const float4*>(cs + 4));
+      *reinterpret_cast<float4*>(sn + 4) = __ldg(reinterpret_cast<const float4*>(cs + D / 2 + 4));
+    }
+  }
+  if (page < 0 || page >= p.num_pages) {
+    if (lane == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_PAGE);
+    return;
+  }
+  const size_t pool_tok = ((size_t)page * p.Hkv) * 16 * D + (size_t)(pos & 15) * D;   // + h * 16 * D
+  // straight copy of a [Hkv][D] row into the page slot; its first vectors have been fetched
   auto copy_row = [&](const uint4* src, uint16_t* pool) {
-    const int n = p.Hkv * VEC;
-    for (int u0 = lane; u0 < n; u0 += 4 * LANES) {
-      uint4 v[4];
+    for (int u0 = lane; u0 < n_vec; u0 += COPIES * LANES) {
+      if (!AHEAD || u0 != lane) fetch_copy(src, u0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (u0 + LANES * i < n) v[i] = ldg_stream(src + u0 + LANES * i);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < COPIES; ++i) {
         const int u = u0 + LANES * i;
-        if (u < n) *reinterpret_cast<uint4*>(pool + pool_tok + (size_t)(u / VEC) * 16 * D + (u % VEC) * 8) = v[i];
+        if (u < n_vec) *reinterpret_cast<uint4*>(pool + pool_tok + (size_t)(u / VEC) * 16 * D + (u % VEC) * 8) = v[i];
       }
     }
   };
   copy_row(vin, p.v_pool);
   if (!p.cos_sin) {
+    if constexpr (AHEAD) fetch_copy(kin, lane);
     copy_row(kin, p.k_pool);
     return;
   }
-  const float* cs = p.cos_sin + (size_t)pos * D;     // cos[0..D/2) then sin[0..D/2)
-  const int nh = nq + p.Hkv;
-  // where vector `vec` of head h is read from / written to
-  auto src_of = [&](int h, int vec) { return h < nq ? qio + h * VEC + vec : kin + (h - nq) * VEC + vec; };
-  auto dst_of = [&](int h, int vec) {
-    return h < nq ? qio + h * VEC + vec
-                  : reinterpret_cast<uint4*>(p.k_pool + pool_tok + (size_t)(h - nq) * 16 * D + vec * 8);
-  };
-  if (!p.interleaved) {
-    constexpr int HP = LANES / HALF;                 // heads the token's lanes cover at once
-    const int j = lane % HALF, h0 = lane / HALF;
-    float c[8], sn[8];
-    *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(cs + j * 8));
-    *reinterpret_cast<float4*>(c + 4) = __ldg(reinterpret_cast<const float4*>(cs + j * 8 + 4));
-    *reinterpret_cast<float4*>(sn) = __ldg(reinterpret_cast<const float4*>(cs + D / 2 + j * 8));
-    *reinterpret_cast<float4*>(sn + 4) = __ldg(reinterpret_cast<const float4*>(cs + D / 2 + j * 8 + 4));
-    for (int h = h0; h < nh; h += 2 * HP) {
-      const int h2 = h + HP;
-      uint4 a = *src_of(h, j), b = *src_of(h, j + HALF), a2, b2;
-      if (h2 < nh) { a2 = *src_of(h2, j); b2 = *src_of(h2, j + HALF); }
-      rotate8(a, b, c, sn);
-      *dst_of(h, j) = a;
-      *dst_of(h, j + HALF) = b;
-      if (h2 < nh) {
-        rotate8(a2, b2, c, sn);
-        *dst_of(h2, j) = a2;
-        *dst_of(h2, j + HALF) = b2;
-      }
-    }
-  } else {
-    constexpr int HP = LANES / VEC;
-    const int j = lane % VEC, h0 = lane / VEC;
-    float c[4], sn[4];
-    *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(cs + j * 4));
-    *reinterpret_cast<float4*>(sn) = __ldg(reinterpret_cast<const float4*>(cs + D / 2 + j * 4));
-    for (int h = h0; h < nh; h += 2 * HP) {
-      const int h2 = h + HP;
-      uint4 a = *src_of(h, j), a2;
-      if (h2 < nh) a2 = *src_of(h2, j);
-      rotate4_interleaved(a, c, sn);
-      *dst_of(h, j) = a;
-      if (h2 < nh) {
-        rotate4_interleaved(a2, c, sn);
-        *dst_of(h2, j) = a2;
+  for (int h = h0; h < nh; h += 2 * HP) {
+    if (!AHEAD || h != h0) fetch_heads(h);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int hh = h + i * HP;
+      if (hh < nh) {
+        uint4* dst = hh < nq ? qio + hh * VEC : reinterpret_cast<uint4*>(p.k_pool + pool_tok + (size_t)(hh - nq) * 16 * D);
+        if (halves) {
+          rotate8(a[i], b[i], c, sn);
+          dst[j] = a[i];
+          dst[j + HALF] = b[i];
+        } else {
+          rotate4_interleaved(a[i], c, sn);
+          dst[j] = a[i];
+        }
       }
     }
   }
@@ -196,9 +200,14 @@ extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_b
   p.Hq = cache->num_q_heads;
   p.Hkv = cache->num_kv_heads;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // warps per token: 1 when there are enough tokens to fill the GPU with independent warps, up to 8 for a handful
-  const int T = batch->total_new_tokens;
-  const int wpt = T >= 16384 ? 1 : T >= 4096 ? 2 : T >= 1024 ? 4 : 8;
+  // Warps per token: 8, and 4, while every token's CTA is resident at once (a token's latency is the time); beyond that as many as
+  // its rows keep busy for a few vectors each.  Microseconds with 1 / 2 / 4 / 8 (in brackets as it was: 8 below 1,024 tokens, 4 below
+  // 4,096, 2 below 16,384, look-ups before the rows): 256 tokens at 32/8 heads x 128 5.6 / 4.1 / 3.3 / 3.0 [3.9], 960 5.4 / 4.5 /
+  // 4.7 / 5.1 [5.6], 2,336 7.2 / 7.1 / 8.0 / 9.8 [8.2], 25,600 99.4 / 97.6 / 98.7 / 118 [99.4]; 2,336 at 4/4 x 64 2.8 / 2.7 / 4.3 /
+  // 7.0 [4.5], 8,192 5.5 / 7.1 / 11.5 / 20.5 [7.6]; 4,096 at 32/32 x 128 34.4 / 32.4 / 31.8 / 31.5 [33.2], 25,600 201 / 200 / 196 / 201 [201].
+  const int T = batch->total_new_tokens, resident = 4 * efim::sm_count();
+  const int vectors = (p.Hq + 2 * p.Hkv) * (cache->head_dim / 8);            // of a token's q, k and v
+  const int wpt = T <= resident ? 8 : T <= 2 * resident || vectors >= 1024 ? 4 : vectors >= 384 || T <= 4 * resident ? 2 : 1;
   const unsigned grid = (unsigned)(((long long)T * wpt * 32 + efim::KV_APPEND_THREADS - 1) / efim::KV_APPEND_THREADS);
   // With at most a CTA per SM the next kernel may start early (a step of 64 rows with its decode
   // attention 128 -> 121 us).  Beside more CTAs the attention kernel's, which take an SM each, are dealt
