@@ -1454,23 +1454,26 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   }
 }
 
-// Merge the KV-chunk partials of split sequences.  A warp takes up to MERGE_ROWS consecutive heads of one token, their partial
-// rows of two chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the
+// Merge the KV-chunk partials of split sequences.  A warp takes up to ROWS consecutive heads of one token, with the partial
+// rows of 8 / ROWS chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the
 // launch parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
 //
 // Bound: the partials' bytes, which the kernel before has left in L2, behind a chain of dependent look-ups.  The lanes look
 // a token's sequence up together, 32 candidates a trip, and bring its lengths along in the last one; with a warp per row
 // that bisected q_indptr and then read one value after the other, a chain of ten trips in each of 8 waves of CTAs,
-// the merge of 960 tokens at 32/8 heads took 25 us and that of 2,800 tokens at 28/4 97 us.
-constexpr int MERGE_WARPS = 8, MERGE_ROWS = 4;
-__host__ __device__ constexpr int merge_rows(int Hq) { return Hq % 4 == 0 ? 4 : (Hq % 2 == 0 ? 2 : 1); }
-template <int D, typename Split>
+// the merge of 960 tokens at 32/8 heads in two chunks took 25 us; now 6.2, and 64 mixed rows at 28/4 cut into 516 items 300 us
+// instead of 355 for the layer.  A row a warp while there are few, else four.  Attention and merge with one / four [a warp per
+// row, bisecting]: 2 x 1-2 tokens over 8-10k at 4/4 heads x 64 10.7 / 14.2 [12.0] us, 111 tokens over 3-14k at 32/8 (3,552 rows)
+// 45.8 / 48.9 [46.2], 150 over 3-5k at 32/32 (4,800) 35.5 / 35.6 [35.6], 380 over 4-8k at 24/8 (9,120) 53.5 / 49.5 [51.9].
+constexpr int MERGE_WARPS = 8;
+__host__ __device__ constexpr int merge_rows(int Hq, int at_most) { return at_most >= 4 && Hq % 4 == 0 ? 4 : (at_most >= 2 && Hq % 2 == 0 ? 2 : 1); }
+template <int D, int MERGE_ROWS, typename Split>
 __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const Params p, const __grid_constant__ Split split) {
   constexpr int EPL = D / 32;                               // dims of a lane
-  constexpr int AT_ONCE = 2;                                // chunks whose rows are in flight together
+  constexpr int AT_ONCE = 8 / MERGE_ROWS;                   // chunks whose rows are in flight together
   constexpr bool inl = std::is_same<Split, InlineSplit>::value;
   const int lane = threadIdx.x & 31;
-  const int nr = merge_rows(p.Hq);                          // rows of this warp: heads of one token
+  const int nr = merge_rows(p.Hq, MERGE_ROWS);              // rows of this warp: heads of one token
   const size_t th = ((size_t)blockIdx.x * MERGE_WARPS + (threadIdx.x >> 5)) * nr;
   // (everything before the attention kernel has completed, and that kernel writes partials only: the
   // look-ups need not wait for it.  Read in L2, where what has completed is visible.)
@@ -1504,7 +1507,7 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
       for (int i = threadIdx.x; i < p.batch; i += 32 * MERGE_WARPS) p.split_out[i] = split.keys[i];
   }
   if (nc == 0) return;                                      // written directly by the main kernel
-  // rows r of chunks c .. c + AT_ONCE - 1 (rows and chunks past the last: read again, without weight)
+  // rows r of chunks c0 .. c0 + AT_ONCE - 1 (rows past the last: read again, not used)
   const float* po = p.part_o + th * p.s_max * D + lane * EPL;
   __align__(16) float v[AT_ONCE][MERGE_ROWS][EPL];
   auto fetch = [&](int c0) {
@@ -1512,7 +1515,8 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
     for (int c = 0; c < AT_ONCE; ++c)
 #pragma unroll
       for (int r = 0; r < MERGE_ROWS; ++r) {
-        const float* src = po + ((size_t)min(r, nr - 1) * p.s_max + min(c0 + c, nc - 1)) * D;
+        if (c0 + c >= nc) continue;
+        const float* src = po + ((size_t)min(r, nr - 1) * p.s_max + c0 + c) * D;
         if constexpr (EPL == 4) {
           *reinterpret_cast<float4*>(v[c][r]) = __ldcg(reinterpret_cast<const float4*>(src));
         } else {
@@ -1869,12 +1873,18 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   else st = start(std::false_type{});
   if (st != EFIM_OK) return st;
   if (pl.s_max > 1) {
-    const size_t per_block = MERGE_WARPS * merge_rows(p.Hq);
-    const unsigned blocks = (unsigned)(((size_t)p.total_new_tokens * p.Hq + per_block - 1) / per_block);
-    if constexpr (inl)
-      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, InlineSplit>, dim3(blocks), dim3(32 * MERGE_WARPS), 0, s, p, list.split));
-    else
-      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, NoList>, dim3(blocks), dim3(32 * MERGE_WARPS), 0, s, p, NoList{}));
+    const size_t rows = (size_t)p.total_new_tokens * p.Hq;
+    auto merge = [&](auto kernel, int at_most, const auto& split) -> efim_status {
+      const size_t per_block = (size_t)MERGE_WARPS * merge_rows(p.Hq, at_most);
+      EFIM_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)((rows + per_block - 1) / per_block)), dim3(32 * MERGE_WARPS), 0, s, p, split));
+      return EFIM_OK;
+    };
+    using Split = std::conditional_t<inl, InlineSplit, NoList>;
+    const Split* split;
+    NoList none;
+    if constexpr (inl) split = &list.split;
+    else split = &none;
+    return rows <= (size_t)32 * sm_count() ? merge(prefill_merge_kernel<D, 1, Split>, 1, *split) : merge(prefill_merge_kernel<D, 4, Split>, 4, *split);
   }
   return EFIM_OK;
 }
