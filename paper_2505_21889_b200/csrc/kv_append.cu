@@ -2,13 +2,14 @@
 // of k/v into the paged cache (EFIM Sec. 1: only the `inc` tokens are new and
 // they follow `<P>prefix<S>suffix<M>`, so token i of sequence s has position
 // cached_len[s] + i).  Pure streaming: every byte is read once and written once.
-#include "common.cuh"
+#include "kv_append.cuh"
 #include <math.h>
 
 namespace efim {
 
 struct KvAppendParams {
-  uint16_t* q;              // [T][Hq][D] in/out, may be null
+  const uint16_t* q;        // [T][Hq][D], may be null
+  uint16_t* q_out;          // where the rotated rows go: q, or an array of its own
   const uint16_t* k_new;    // [T][Hkv][D]
   const uint16_t* v_new;
   uint16_t* k_pool;         // [pages][Hkv][P][D]
@@ -36,7 +37,9 @@ struct KvAppendParams {
 // 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.
 constexpr int KV_APPEND_THREADS = 256;
 
-template <int D, int WPT>
+// ASIDE: the rotated queries go to an array of their own, where rows whose keys have no place are written all the same, zeros where
+// the table has no row.
+template <int D, int WPT, bool ASIDE>
 __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const KvAppendParams p) {
   constexpr int VEC = D / 8;            // 16-byte vectors per head row
   constexpr int HALF = VEC / 2;
@@ -50,13 +53,13 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
   if (t >= p.total_new_tokens) return;
   const uint4* kin = reinterpret_cast<const uint4*>(p.k_new + (size_t)t * p.Hkv * D);
   const uint4* vin = reinterpret_cast<const uint4*>(p.v_new + (size_t)t * p.Hkv * D);
-  uint4* qio = p.q ? reinterpret_cast<uint4*>(p.q + (size_t)t * p.Hq * D) : nullptr;
+  const uint4* qin = p.q ? reinterpret_cast<const uint4*>(p.q + (size_t)t * p.Hq * D) : nullptr;
   const int nq = p.q ? p.Hq : 0, nh = nq + p.Hkv, n_vec = p.Hkv * VEC;
   // rotated heads: this lane's position j and first head, heads that the token's lanes cover at once
   const bool halves = !p.interleaved;
   const int per_head = halves ? HALF : VEC, HP = LANES / per_head;
   const int j = lane % per_head, h0 = lane / per_head;
-  auto row_of = [&](int h) -> const uint4* { return h < nq ? qio + h * VEC : kin + (h - nq) * VEC; };
+  auto row_of = [&](int h) -> const uint4* { return h < nq ? qin + h * VEC : kin + (h - nq) * VEC; };
   uint4 v[COPIES], a[2], b[2];
   auto fetch_copy = [&](const uint4* src, int u0) {
 #pragma unroll
@@ -92,14 +95,18 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
   const int i_seq = 31 - __clz((int)(__ballot_sync(0xffffffffu, wl < n && first <= t) | 1u));
   const int pos = __shfl_sync(0xffffffffu, cached, i_seq) + t - __shfl_sync(0xffffffffu, first, i_seq);
   const int page_idx = pos >> 4;
-  if (pos < 0 || page_idx >= p.max_pages_per_seq || (p.cos_sin && pos >= p.max_position)) {
+  const bool in_table = !p.cos_sin || (pos >= 0 && pos < p.max_position);
+  int err = 0, page = 0;
+  if (pos < 0 || page_idx >= p.max_pages_per_seq || !in_table) {
     if (lane == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_POSITION);
-    return;
+    if (!ASIDE) return;
+    err = EFIM_DEV_BAD_POSITION;
+  } else {
+    page = *(p.block_table + (size_t)(lo + i_seq) * p.max_pages_per_seq + page_idx);
   }
-  const int page = *(p.block_table + (size_t)(lo + i_seq) * p.max_pages_per_seq + page_idx);
   // rotary values: position j of the row's halves (8 of either), or the 4 pairs of vector j
   float c[8], sn[8];
-  if (p.cos_sin) {
+  if (p.cos_sin && (!ASIDE || in_table)) {
     const float* cs = p.cos_sin + (size_t)pos * D + j * (halves ? 8 : 4);      // cos[0..D/2) then sin[0..D/2)
     *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(cs));
     *reinterpret_cast<float4*>(sn) = __ldg(reinterpret_cast<const float4*>(cs + D / 2));
@@ -110,9 +117,11 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
   }
   if (page < 0 || page >= p.num_pages) {
     if (lane == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_PAGE);
-    return;
+    if (!ASIDE) return;
+    err = EFIM_DEV_BAD_PAGE;
   }
   const size_t pool_tok = ((size_t)page * p.Hkv) * 16 * D + (size_t)(pos & 15) * D;   // + h * 16 * D
+  uint4* q_out = reinterpret_cast<uint4*>(const_cast<uint16_t*>(ASIDE ? p.q_out : p.q) + (size_t)t * p.Hq * D);
   // straight copy of a [Hkv][D] row into the page slot; its first vectors have been fetched
   auto copy_row = [&](const uint4* src, uint16_t* pool) {
     for (int u0 = lane; u0 < n_vec; u0 += COPIES * LANES) {
@@ -124,7 +133,7 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
       }
     }
   };
-  copy_row(vin, p.v_pool);
+  if (!ASIDE || !err) copy_row(vin, p.v_pool);
   if (!p.cos_sin) {
     if constexpr (AHEAD) fetch_copy(kin, lane);
     copy_row(kin, p.k_pool);
@@ -135,9 +144,12 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int hh = h + i * HP;
-      if (hh < nh) {
-        uint4* dst = hh < nq ? qio + hh * VEC : reinterpret_cast<uint4*>(p.k_pool + pool_tok + (size_t)(hh - nq) * 16 * D);
-        if (halves) {
+      if (hh < nh && (!ASIDE || hh < nq || !err)) {
+        uint4* dst = hh < nq ? q_out + hh * VEC : reinterpret_cast<uint4*>(p.k_pool + pool_tok + (size_t)(hh - nq) * 16 * D);
+        if (ASIDE && !in_table) {
+          dst[j] = make_uint4(0, 0, 0, 0);
+          if (halves) dst[j + HALF] = make_uint4(0, 0, 0, 0);
+        } else if (halves) {
           rotate8(a[i], b[i], c, sn);
           dst[j] = a[i];
           dst[j + HALF] = b[i];
@@ -168,6 +180,12 @@ extern "C" efim_status efim_rope_table_build(double base, int32_t head_dim, int3
 extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_batch_desc* batch,
                                       const efim_rope_desc* rope, void* d_q, const void* d_k_new,
                                       const void* d_v_new, int32_t* d_status, void* stream) {
+  return efim::append_run(cache, batch, rope, d_q, d_q, d_k_new, d_v_new, d_status, stream);
+}
+
+efim_status efim::append_run(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
+                             const void* d_q, void* d_q_out, const void* d_k_new, const void* d_v_new, int32_t* d_status,
+                             void* stream) {
   efim_status st = efim::check_cache(cache);
   if (st != EFIM_OK) return st;
   st = efim::check_batch(cache, batch, false);
@@ -177,7 +195,8 @@ extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_b
   if ((reinterpret_cast<uintptr_t>(d_k_new) | reinterpret_cast<uintptr_t>(d_v_new) |
        reinterpret_cast<uintptr_t>(d_q)) & 15) return EFIM_ERR_INVALID_ARG;
   efim::KvAppendParams p{};
-  p.q = static_cast<uint16_t*>(d_q);
+  p.q = static_cast<const uint16_t*>(d_q);
+  p.q_out = static_cast<uint16_t*>(d_q_out);
   p.k_new = static_cast<const uint16_t*>(d_k_new);
   p.v_new = static_cast<const uint16_t*>(d_v_new);
   p.k_pool = static_cast<uint16_t*>(cache->d_k_pool);
@@ -214,19 +233,24 @@ extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_b
   // out to whichever SMs run dry first, and the launch lost more than the set-up it hid (append +
   // attention of 64 mixed rows 349 -> 391 us, 16 rows at 32/32 heads 336 -> 351).
   p.early_next = grid <= (unsigned)efim::sm_count();
-#define EFIM_KV_APPEND_LAUNCH(D_, W_) \
-  EFIM_CUDA_TRY(efim::launch_pdl(efim::kv_append_kernel<D_, W_>, dim3(grid), dim3(efim::KV_APPEND_THREADS), 0, s, p))
+#define EFIM_KV_APPEND_LAUNCH(D_, W_, A_) \
+  EFIM_CUDA_TRY(efim::launch_pdl(efim::kv_append_kernel<D_, W_, A_>, dim3(grid), dim3(efim::KV_APPEND_THREADS), 0, s, p))
+#define EFIM_KV_APPEND_WARPS(D_, A_)                  \
+  do {                                                \
+    if (wpt == 1) EFIM_KV_APPEND_LAUNCH(D_, 1, A_);      \
+    else if (wpt == 2) EFIM_KV_APPEND_LAUNCH(D_, 2, A_); \
+    else if (wpt == 4) EFIM_KV_APPEND_LAUNCH(D_, 4, A_); \
+    else EFIM_KV_APPEND_LAUNCH(D_, 8, A_);               \
+  } while (0)
+  const bool aside = d_q_out != d_q;
   if (cache->head_dim == 128) {
-    if (wpt == 1) EFIM_KV_APPEND_LAUNCH(128, 1);
-    else if (wpt == 2) EFIM_KV_APPEND_LAUNCH(128, 2);
-    else if (wpt == 4) EFIM_KV_APPEND_LAUNCH(128, 4);
-    else EFIM_KV_APPEND_LAUNCH(128, 8);
+    if (aside) EFIM_KV_APPEND_WARPS(128, true);
+    else EFIM_KV_APPEND_WARPS(128, false);
   } else {
-    if (wpt == 1) EFIM_KV_APPEND_LAUNCH(64, 1);
-    else if (wpt == 2) EFIM_KV_APPEND_LAUNCH(64, 2);
-    else if (wpt == 4) EFIM_KV_APPEND_LAUNCH(64, 4);
-    else EFIM_KV_APPEND_LAUNCH(64, 8);
+    if (aside) EFIM_KV_APPEND_WARPS(64, true);
+    else EFIM_KV_APPEND_WARPS(64, false);
   }
+#undef EFIM_KV_APPEND_WARPS
 #undef EFIM_KV_APPEND_LAUNCH
   return EFIM_OK;
 }

@@ -4,6 +4,7 @@
 // it into the workspace and launches the tensor-core kernel (prefill_tc.cu).
 #include <cstring>
 #include <memory>
+#include "kv_append.cuh"
 #include "prefill_tc.cuh"
 #include "mbar.cuh"
 
@@ -250,6 +251,22 @@ bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* b
   }
   return with_work == 1 && cache->num_kv_heads <= efim::sm_count();
 }
+// Whether the append kernel rotates a step's query rows, and leaves them where their outputs go: a work item has its rows in shared
+// memory before it writes them, and no other one reads them (the chunks of a cut key range write partials, and the merge comes
+// after all of them).  Not where the output lies on the rows that the append reads, beyond row for row on q itself.  The
+// attention kernel can rotate rows as it loads them, but its CTAs' warps wait for that, 12,300 cycles per item.  One-call steps with it
+// and with the append: 16 prompts of 1-3.5k tokens 869 and 827 us, 53 x 1-406 over 100-549 at 24/8 100 and 75, 40 x 10-22 over
+// 24-125 at 40/8 39 and 30, 39 x 1-5 over 0 at 16/1 12.3 and 9.2, 9 x 1 over 193-632 at 32/8 x 64 10.9 and 10.7.
+bool rotates_into_out(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope, const NewRows& rows,
+                      const void* d_q, const void* d_out) {
+  if (!rope || !rope->d_cos_sin || !d_q || !d_out || efim::check_cache(cache) != EFIM_OK) return false;
+  if (efim::check_batch(cache, batch, false) != EFIM_OK) return false;
+  if ((reinterpret_cast<uintptr_t>(d_q) | reinterpret_cast<uintptr_t>(d_out)) & 15) return false;
+  const size_t row = (size_t)cache->head_dim * 2, tokens = (size_t)batch->total_new_tokens;
+  const size_t q_bytes = tokens * cache->num_q_heads * row, kv_bytes = tokens * cache->num_kv_heads * row;
+  return !overlap(rows.k, kv_bytes, d_out, q_bytes) && !overlap(rows.v, kv_bytes, d_out, q_bytes) &&
+         (d_q == d_out || !overlap(d_q, q_bytes, d_out, q_bytes));
+}
 }  // namespace
 
 extern "C" efim_status efim_append_prefill_attn_planned(const efim_cache_desc* cache, const efim_batch_desc* batch,
@@ -283,8 +300,14 @@ extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, co
   if (d_k_new && !h_plan && appends_in_attention(cache, batch, rows, d_out, d_lse))
     return plan_and_run(cache, batch, rope, &rows, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
   if (d_k_new) {
-    const efim_status st = efim_kv_append(cache, batch, rope, nullptr, d_k_new, d_v_new, d_status, stream);
+    const bool by_append = rotates_into_out(cache, batch, rope, rows, d_q, d_out);
+    const efim_status st = efim::append_run(cache, batch, rope, by_append ? d_q : nullptr, by_append ? d_out : nullptr, d_k_new,
+                                            d_v_new, d_status, stream);
     if (st != EFIM_OK) return st;
+    if (by_append) {
+      d_q = d_out;
+      rope = nullptr;
+    }
   }
   if (h_plan)
     return run_planned(cache, batch, rope, h_plan, plan_bytes, lists_resident, d_q, d_out, d_lse, sm_scale,

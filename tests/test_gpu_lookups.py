@@ -1,9 +1,11 @@
 """Kernels whose warps look a token's sequence up 32 candidates at a time: batches of more than one and of more than two such
-trips, with sequences that bring nothing among them; and every number of warps per token of the append."""
+trips, with sequences that bring nothing among them; every number of warps per token of the append; and one-call steps, whose
+append rotates the queries too."""
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
+BAD_PAGE, BAD_POSITION = 1, 2            # EFIM_DEV_*
 
 
 def _new_lengths(batch, tokens, seed):
@@ -56,3 +58,63 @@ def test_merge_of_cut_sequences_among_many(Hq, Hkv, D, batch, tokens):
     cached = np.where(new > 0, 3000 + 7 * np.arange(batch), 5).astype(np.int32)
     dw, _ = _check_turn(_custom(Hq, Hkv, D, cached, new, seed=batch), use_rope=False)
     assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 2
+
+
+def _step(dw, rope, q, k, v, out, ws, plan=None):
+    import paper_2505_21889_b200 as efim
+    efim.efim_append_prefill_step(dw.cache, dw.batch, rope, q, k, v, out, dw.lse, 0.0, ws, dw.status, plan=plan)
+
+
+@pytest.mark.parametrize("where", ["beside", "on q", "on k", "on v"])
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new", [
+    (32, 8, 128, [6000, 5, 700], [20, 70, 3]),          # cut key ranges: several work items read the rows
+    (7, 1, 64, [0, 33, 100, 16], [300, 1, 40, 5]),      # row blocks that end inside a token
+])
+def test_step_with_its_output_on_other_rows(Hq, Hkv, D, cached, new, where):
+    """The one-call step leaves the rotated queries where the outputs go, if nothing that the append reads lies there: the bits of
+    the two calls wherever the output is."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, D, cached, new, seed=Hq)
+    a, b = H.DeviceWorkload(w), H.DeviceWorkload(w)
+    a.gpu_kv_append()
+    a.gpu_prefill()
+    n_q, n_k, odd = b.q.numel(), b.k_new.numel(), 8 * D
+    mem = torch.zeros(3 * n_q + 2 * n_k + odd, dtype=torch.bfloat16, device="cuda")
+    q, k, v = mem[:n_q], mem[2 * n_q: 2 * n_q + n_k], mem[2 * n_q + n_k: 2 * n_q + 2 * n_k]
+    for dst, src in ((q, b.q), (k, b.k_new), (v, b.v_new)):
+        dst.copy_(src.flatten())
+    start = {"beside": n_q, "on q": 0, "on k": n_q + odd, "on v": 2 * n_q + n_k}[where]
+    out = mem[start: start + n_q]
+    ws = torch.empty(efim.efim_prefill_workspace_bytes(b.cache, b.batch), dtype=torch.uint8, device="cuda")
+    _step(b, b.rope, q.view_as(b.q), k.view_as(b.k_new), v.view_as(b.v_new), out.view_as(b.q), ws)
+    torch.cuda.synchronize()
+    assert int(a.status.item()) == int(b.status.item()) == 0
+    assert torch.equal(a.out.view(torch.int16), out.view_as(b.q).view(torch.int16)) and torch.equal(a.lse, b.lse)
+    assert torch.equal(a.k_pool.view(torch.int16), b.k_pool.view(torch.int16))
+    assert torch.equal(a.v_pool.view(torch.int16), b.v_pool.view(torch.int16))
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+def test_step_rotates_queries_whose_keys_have_no_page(interleaved):
+    """A rejected page drops its keys and nothing else: the token's query attends over the others, as it does when the attention
+    kernel rotates the rows (the form of the call without k and v, here over the pages of the first one)."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    w = _custom(8, 2, 128, [60, 200], [40, 9], seed=5)
+    w.block_table[0, 5] = w.num_pages + 3               # keys 80 .. 95 of the first sequence, new ones
+    dw = H.DeviceWorkload(w, interleaved=interleaved)
+    ws = torch.empty(efim.efim_prefill_workspace_bytes(dw.cache, dw.batch), dtype=torch.uint8, device="cuda")
+    short = efim.Rope(w.rope_base, w.head_dim, 205, interleaved)        # and the last positions of the second have no table row
+    outs = []
+    for k, v in ((dw.k_new, dw.v_new), (None, None)):
+        out = torch.full_like(dw.q, float("nan"))
+        _step(dw, short, dw.q, k, v, out, ws)
+        torch.cuda.synchronize()
+        outs.append(out.view(torch.int16).clone())
+        assert int(dw.status.item()) == BAD_PAGE | BAD_POSITION
+    assert torch.equal(*outs) and torch.isfinite(out.float()).all()
