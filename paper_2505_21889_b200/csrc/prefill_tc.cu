@@ -1624,7 +1624,8 @@ int walk_blocks(const efim_cache_desc* c, const efim_batch_desc* b, long long ch
 }
 
 // Finish time of the launch with that cut: the hardware hands CTAs, longest first, to whichever SM is
-// free.  `best`: the earliest finish known; a cut whose lower bound is no better is not simulated.
+// free.  `best`: the earliest finish known; a cut whose lower bound is no better is not simulated, and a simulation
+// ends where it is no better any more.
 long long estimate_makespan(const efim_cache_desc* c, const efim_batch_desc* b, long long chunk_tiles, int n_sm,
                             long long best, std::vector<int32_t>& cost, std::vector<int32_t>& sm) {
   cost.clear();
@@ -1640,12 +1641,22 @@ long long estimate_makespan(const efim_cache_desc* c, const efim_batch_desc* b, 
   const long long bound = std::max(longest, (total * Hkv + n_sm - 1) / n_sm) + merge;
   if (bound >= best || (long long)cost.size() * Hkv <= n_sm) return bound;
   std::sort(cost.begin(), cost.end(), std::greater<int32_t>());
-  sm.assign((size_t)n_sm, 0);                                // min-heap of SM finish times
-  long long end = 0;
-  for (int32_t x : cost)
-    for (long long h = 0; h < Hkv; ++h) {
-      const int32_t v = sm[0] + x;                           // the earliest SM takes the item: sift it down
-      end = std::max<long long>(end, v);
+  // The first items go to one SM each: their finish times, the last of them first, are a min-heap as they stand.
+  sm.resize((size_t)n_sm);
+  size_t i0 = 0;
+  long long h0 = 0;
+  for (int k = n_sm; k-- > 0;) {
+    sm[(size_t)k] = cost[i0];
+    if (++h0 == Hkv) { h0 = 0; ++i0; }
+  }
+  long long end = sm[(size_t)n_sm - 1];
+  for (; i0 < cost.size(); ++i0, h0 = 0)
+    for (; h0 < Hkv; ++h0) {
+      const int32_t v = sm[0] + cost[i0];                    // the earliest SM takes the item: sift it down
+      if (v > end) {
+        end = v;
+        if (end + merge >= best) return end + merge;         // (no better than the best, whatever follows)
+      }
       size_t i = 0;
       for (size_t k = 1; k < sm.size(); k = 2 * i + 1) {
         if (k + 1 < sm.size() && sm[k + 1] < sm[k]) ++k;
