@@ -201,6 +201,8 @@ efim_status efim_append_prefill_attn_planned(const efim_cache_desc* cache, const
  * Two kernels are enqueued (three when the key range is split); one where, without a plan, a single sequence
  * brings at most 128 (token, head-in-group) rows and its key range is not split: the attention kernel then
  * appends them itself (not where d_out or d_lse overlaps d_k_new or d_v_new, which stays allowed).
+ * A call that is refused (EFIM_ERR_INVALID_ARG, _UNSUPPORTED, _OUT_OF_RANGE, _WORKSPACE) has enqueued nothing: d_q, d_out and
+ * the pages are as they were, and it may be repeated.
  */
 efim_status efim_append_prefill_step(const efim_cache_desc* cache, const efim_batch_desc* batch,
                                      const efim_rope_desc* rope, const void* d_q,

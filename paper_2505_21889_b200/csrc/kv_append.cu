@@ -180,36 +180,43 @@ extern "C" efim_status efim_rope_table_build(double base, int32_t head_dim, int3
 extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_batch_desc* batch,
                                       const efim_rope_desc* rope, void* d_q, const void* d_k_new,
                                       const void* d_v_new, int32_t* d_status, void* stream) {
-  return efim::append_run(cache, batch, rope, d_q, d_q, d_k_new, d_v_new, d_status, stream);
+  const efim::Append a{rope, d_q, d_q, d_k_new, d_v_new};
+  const efim_status st = efim::append_check(cache, batch, a);
+  return st != EFIM_OK ? st : efim::append_launch(cache, batch, a, d_status, stream);
 }
 
-efim_status efim::append_run(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
-                             const void* d_q, void* d_q_out, const void* d_k_new, const void* d_v_new, int32_t* d_status,
-                             void* stream) {
+efim_status efim::append_check(const efim_cache_desc* cache, const efim_batch_desc* batch, const Append& a) {
   efim_status st = efim::check_cache(cache);
   if (st != EFIM_OK) return st;
   st = efim::check_batch(cache, batch, false);
   if (st != EFIM_OK) return st;
   if (batch->batch == 0 || batch->total_new_tokens == 0) return EFIM_OK;
-  if (!d_k_new || !d_v_new) return EFIM_ERR_INVALID_ARG;
-  if ((reinterpret_cast<uintptr_t>(d_k_new) | reinterpret_cast<uintptr_t>(d_v_new) |
-       reinterpret_cast<uintptr_t>(d_q)) & 15) return EFIM_ERR_INVALID_ARG;
+  if (!a.k_new || !a.v_new) return EFIM_ERR_INVALID_ARG;
+  if ((reinterpret_cast<uintptr_t>(a.k_new) | reinterpret_cast<uintptr_t>(a.v_new) | reinterpret_cast<uintptr_t>(a.q)) & 15)
+    return EFIM_ERR_INVALID_ARG;
+  if (a.rope && a.rope->d_cos_sin && (a.rope->max_position <= 0 || (reinterpret_cast<uintptr_t>(a.rope->d_cos_sin) & 15)))
+    return EFIM_ERR_INVALID_ARG;
+  return EFIM_OK;
+}
+
+efim_status efim::append_launch(const efim_cache_desc* cache, const efim_batch_desc* batch, const Append& a, int32_t* d_status,
+                                void* stream) {
+  if (batch->batch == 0 || batch->total_new_tokens == 0) return EFIM_OK;
   efim::KvAppendParams p{};
-  p.q = static_cast<const uint16_t*>(d_q);
-  p.q_out = static_cast<uint16_t*>(d_q_out);
-  p.k_new = static_cast<const uint16_t*>(d_k_new);
-  p.v_new = static_cast<const uint16_t*>(d_v_new);
+  p.q = static_cast<const uint16_t*>(a.q);
+  p.q_out = static_cast<uint16_t*>(a.q_out);
+  p.k_new = static_cast<const uint16_t*>(a.k_new);
+  p.v_new = static_cast<const uint16_t*>(a.v_new);
   p.k_pool = static_cast<uint16_t*>(cache->d_k_pool);
   p.v_pool = static_cast<uint16_t*>(cache->d_v_pool);
   p.cached_len = batch->d_cached_len;
   p.q_indptr = batch->d_q_indptr;
   p.block_table = batch->d_block_table;
   p.cos_sin = nullptr;
-  if (rope && rope->d_cos_sin) {
-    if (rope->max_position <= 0 || (reinterpret_cast<uintptr_t>(rope->d_cos_sin) & 15)) return EFIM_ERR_INVALID_ARG;
-    p.cos_sin = rope->d_cos_sin;
-    p.max_position = rope->max_position;
-    p.interleaved = rope->interleaved;
+  if (a.rope && a.rope->d_cos_sin) {
+    p.cos_sin = a.rope->d_cos_sin;
+    p.max_position = a.rope->max_position;
+    p.interleaved = a.rope->interleaved;
   }
   p.status = d_status;
   p.batch = batch->batch;
@@ -242,7 +249,7 @@ efim_status efim::append_run(const efim_cache_desc* cache, const efim_batch_desc
     else if (wpt == 4) EFIM_KV_APPEND_LAUNCH(D_, 4, A_); \
     else EFIM_KV_APPEND_LAUNCH(D_, 8, A_);               \
   } while (0)
-  const bool aside = d_q_out != d_q;
+  const bool aside = a.q_out != a.q;
   if (cache->head_dim == 128) {
     if (aside) EFIM_KV_APPEND_WARPS(128, true);
     else EFIM_KV_APPEND_WARPS(128, false);

@@ -4,9 +4,18 @@
 
 namespace efim {
 
-// efim_kv_append, with the rotated query rows going to `d_q_out`: `d_q` itself, or an array of its own (16-byte aligned).  There
-// every row is written, also of tokens whose keys are reported and dropped: rotated, or zero where the rotary table has no row.
-efim_status append_run(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope, const void* d_q,
-                       void* d_q_out, const void* d_k_new, const void* d_v_new, int32_t* d_status, void* stream);
+// Arguments of an append: efim_kv_append's, with the rotated query rows going to `q_out`: `q` itself, or an array of its own (16-byte
+// aligned).  There every row is written, also of tokens whose keys are reported and dropped: rotated, or zero where the rotary table
+// has no row.
+struct Append {
+  const efim_rope_desc* rope;
+  const void* q;
+  void* q_out;
+  const void *k_new, *v_new;
+};
+// Host checks of the arguments; and the launch, of arguments that have passed them.
+efim_status append_check(const efim_cache_desc* cache, const efim_batch_desc* batch, const Append& a);
+efim_status append_launch(const efim_cache_desc* cache, const efim_batch_desc* batch, const Append& a, int32_t* d_status,
+                          void* stream);
 
 }  // namespace efim

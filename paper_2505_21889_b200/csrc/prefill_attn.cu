@@ -103,19 +103,27 @@ struct NewRows {
   const void *k, *v;
 };
 
-// Runs a plan over validated descriptors.  `rope` with a table: the query rows are rotated as the kernel
-// loads them.  `h_lists`: the lists to copy to the head of the workspace (null: an earlier call has left
-// them there); `list`: the work list, if it travels in the launch parameters instead.
-efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
-                     const efim::pf::Plan& pl, const void* h_lists, const efim::pf::InlineList* list, const NewRows* append,
-                     const void* d_q,
-                     void* d_out, float* d_lse, float sm_scale, void* d_workspace, size_t workspace_bytes,
-                     int32_t* d_status, void* stream) {
-  using namespace efim;
+// The host checks of what a plan is run on.  They come before a call's first launch: a call that is refused has enqueued
+// nothing, so it may be repeated, also where its append would have rotated the queries in place.
+efim_status check_run(const efim_rope_desc* rope, const efim::pf::Plan& pl, const void* d_q, const void* d_out,
+                      const void* d_workspace, size_t workspace_bytes) {
   if (!d_q || !d_out) return EFIM_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(d_q) | reinterpret_cast<uintptr_t>(d_out)) & 15) return EFIM_ERR_INVALID_ARG;
   if (!d_workspace || workspace_bytes < pl.total()) return EFIM_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(d_workspace) & 255) return EFIM_ERR_INVALID_ARG;
+  if (rope && rope->d_cos_sin && (rope->max_position <= 0 || (reinterpret_cast<uintptr_t>(rope->d_cos_sin) & 15)))
+    return EFIM_ERR_INVALID_ARG;
+  return EFIM_OK;
+}
+
+// Runs a plan on what check_run has passed.  `rope` with a table: the query rows are rotated as the kernel
+// loads them.  `h_lists`: the lists to copy to the head of the workspace (null: an earlier call has left
+// them there); `list`: the work list, if it travels in the launch parameters instead.
+efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
+                     const efim::pf::Plan& pl, const void* h_lists, const efim::pf::InlineList* list, const NewRows* append,
+                     const void* d_q, void* d_out, float* d_lse, float sm_scale, void* d_workspace, int32_t* d_status,
+                     void* stream) {
+  using namespace efim;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(d_workspace);
   pf::Params p{};
@@ -142,7 +150,6 @@ efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch,
   p.scale_log2 = scale * 1.4426950408889634f;
   p.wait_ns = WAIT_LIMIT_NS;
   if (rope && rope->d_cos_sin) {
-    if (rope->max_position <= 0 || (reinterpret_cast<uintptr_t>(rope->d_cos_sin) & 15)) return EFIM_ERR_INVALID_ARG;
     p.cos_sin = rope->d_cos_sin;
     p.max_position = rope->max_position;
     p.interleaved = rope->interleaved;
@@ -158,11 +165,11 @@ efim_status run_plan(const efim_cache_desc* cache, const efim_batch_desc* batch,
   return pf::launch(cache, p, pl, list, s);
 }
 
-// Runs the plan in a blob of efim_prefill_plan().
+// Runs the plan in a blob of efim_prefill_plan().  `before`: an append, checked, that goes before the attention.
 efim_status run_planned(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
-                        const void* h_plan, size_t plan_bytes, int32_t lists_resident, const void* d_q, void* d_out,
-                        float* d_lse, float sm_scale, void* d_workspace, size_t workspace_bytes, int32_t* d_status,
-                        void* stream) {
+                        const efim::Append* before, const void* h_plan, size_t plan_bytes, int32_t lists_resident,
+                        const void* d_q, void* d_out, float* d_lse, float sm_scale, void* d_workspace, size_t workspace_bytes,
+                        int32_t* d_status, void* stream) {
   using namespace efim;
   efim_status st = check_cache(cache);
   if (st != EFIM_OK) return st;
@@ -184,18 +191,22 @@ efim_status run_planned(const efim_cache_desc* cache, const efim_batch_desc* bat
   pl.split_bytes = hd.split_bytes;
   pl.part_lse_bytes = hd.part_lse_bytes;
   pl.part_o_bytes = hd.part_o_bytes;
+  st = check_run(rope, pl, d_q, d_out, d_workspace, workspace_bytes);
+  if (st != EFIM_OK) return st;
+  if (before && (st = append_launch(cache, batch, *before, d_status, stream)) != EFIM_OK) return st;
   return run_plan(cache, batch, rope, pl, lists_resident ? nullptr : static_cast<const unsigned char*>(h_plan) + PLAN_HEAD_BYTES,
-                  nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
+                  nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, d_status, stream);
 }
 
 // Plans, then runs.  Lists of up to InlineItems::MAX items travel in the launch parameters: no
 // copy stands between the append and the attention kernel (append and attention of 16 tokens over 240 in
 // one call 15.2 -> 10.7 us; the kernel leaves the list in the workspace all the same).
-// `append`: rows the attention kernel is to put into the pages itself, where the plan allows it; else they are appended
-// by a kernel of their own before it.
+// `before`: an append, checked, that goes before the attention; it is launched between the plan, which says how large the
+// workspace has to be, and the lists, which are written meanwhile.  `append`: rows the attention kernel is to put into the
+// pages itself, where the plan allows it; else they are appended by a kernel of their own before it.
 efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* batch, const efim_rope_desc* rope,
-                         const NewRows* append, const void* d_q, void* d_out, float* d_lse, float sm_scale, void* d_workspace,
-                         size_t workspace_bytes, int32_t* d_status, void* stream) {
+                         const efim::Append* before, const NewRows* append, const void* d_q, void* d_out, float* d_lse,
+                         float sm_scale, void* d_workspace, size_t workspace_bytes, int32_t* d_status, void* stream) {
   using namespace efim;
   efim_status st = check_cache(cache);
   if (st != EFIM_OK) return st;
@@ -206,22 +217,28 @@ efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* ba
   if (pl.n_items == 0) return EFIM_OK;
   const bool in_params = pl.n_items <= pf::InlineItems::MAX && batch->batch <= pf::InlineSplit::MAX_BATCH;
   const bool aligned = !append || ((reinterpret_cast<uintptr_t>(append->k) | reinterpret_cast<uintptr_t>(append->v)) & 15) == 0;
+  Append own;
   if (append && !(in_params && pl.s_max == 1 && aligned)) {  // (the kernel that appends is one of those with the list in its parameters)
-    st = efim_kv_append(cache, batch, rope, nullptr, append->k, append->v, d_status, stream);
+    own = Append{rope, nullptr, nullptr, append->k, append->v};
+    st = append_check(cache, batch, own);
     if (st != EFIM_OK) return st;
+    before = &own;
     append = nullptr;
   }
+  st = check_run(rope, pl, d_q, d_out, d_workspace, workspace_bytes);
+  if (st != EFIM_OK) return st;
+  if (before && (st = append_launch(cache, batch, *before, d_status, stream)) != EFIM_OK) return st;
   if (in_params) {
     pf::InlineList list;
     pf::fill_lists(cache, batch, pl, list.items.items, list.split.keys);
-    return run_plan(cache, batch, rope, pl, nullptr, &list, append, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
-                    d_status, stream);
+    return run_plan(cache, batch, rope, pl, nullptr, &list, append, d_q, d_out, d_lse, sm_scale, d_workspace, d_status,
+                    stream);
   }
   const std::unique_ptr<unsigned char[]> lists(new unsigned char[pl.items_bytes + pl.split_bytes]);
   pf::fill_lists(cache, batch, pl, reinterpret_cast<pf::WorkItem*>(lists.get()),
                  reinterpret_cast<int32_t*>(lists.get() + pl.items_bytes));
-  return run_plan(cache, batch, rope, pl, lists.get(), nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
-                  d_status, stream);
+  return run_plan(cache, batch, rope, pl, lists.get(), nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, d_status,
+                  stream);
 }
 
 bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
@@ -274,7 +291,7 @@ extern "C" efim_status efim_append_prefill_attn_planned(const efim_cache_desc* c
                                                         int32_t lists_resident, const void* d_q, void* d_out,
                                                         float* d_lse, float sm_scale, void* d_workspace,
                                                         size_t workspace_bytes, int32_t* d_status, void* stream) {
-  return run_planned(cache, batch, nullptr, h_plan, plan_bytes, lists_resident, d_q, d_out, d_lse, sm_scale,
+  return run_planned(cache, batch, nullptr, nullptr, h_plan, plan_bytes, lists_resident, d_q, d_out, d_lse, sm_scale,
                      d_workspace, workspace_bytes, d_status, stream);
 }
 
@@ -283,8 +300,8 @@ extern "C" efim_status efim_append_prefill_attn(const efim_cache_desc* cache, co
                                                 const void* d_q, void* d_out, float* d_lse, float sm_scale,
                                                 void* d_workspace, size_t workspace_bytes, int32_t* d_status,
                                                 void* stream) {
-  return plan_and_run(cache, batch, nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status,
-                      stream);
+  return plan_and_run(cache, batch, nullptr, nullptr, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes,
+                      d_status, stream);
 }
 
 // Steps 1 and 2 of a turn: the new tokens' k/v go into the pages (k rotated), then the new
@@ -298,19 +315,23 @@ extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, co
   if ((d_k_new == nullptr) != (d_v_new == nullptr)) return EFIM_ERR_INVALID_ARG;
   const NewRows rows{d_k_new, d_v_new};
   if (d_k_new && !h_plan && appends_in_attention(cache, batch, rows, d_out, d_lse))
-    return plan_and_run(cache, batch, rope, &rows, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
+    return plan_and_run(cache, batch, rope, nullptr, &rows, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status,
+                        stream);
+  efim::Append rows_first{rope, nullptr, nullptr, d_k_new, d_v_new};
   if (d_k_new) {
-    const bool by_append = rotates_into_out(cache, batch, rope, rows, d_q, d_out);
-    const efim_status st = efim::append_run(cache, batch, rope, by_append ? d_q : nullptr, by_append ? d_out : nullptr, d_k_new,
-                                            d_v_new, d_status, stream);
-    if (st != EFIM_OK) return st;
-    if (by_append) {
+    if (rotates_into_out(cache, batch, rope, rows, d_q, d_out)) {
+      rows_first.q = d_q;
+      rows_first.q_out = d_out;
       d_q = d_out;
       rope = nullptr;
     }
+    const efim_status st = efim::append_check(cache, batch, rows_first);
+    if (st != EFIM_OK) return st;
   }
+  const efim::Append* before = d_k_new ? &rows_first : nullptr;
   if (h_plan)
-    return run_planned(cache, batch, rope, h_plan, plan_bytes, lists_resident, d_q, d_out, d_lse, sm_scale,
+    return run_planned(cache, batch, rope, before, h_plan, plan_bytes, lists_resident, d_q, d_out, d_lse, sm_scale,
                        d_workspace, workspace_bytes, d_status, stream);
-  return plan_and_run(cache, batch, rope, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status, stream);
+  return plan_and_run(cache, batch, rope, before, nullptr, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status,
+                      stream);
 }
