@@ -9,7 +9,7 @@ namespace efim {
 
 struct KvAppendParams {
   const uint16_t* q;        // [T][Hq][D], may be null
-  uint16_t* q_out;          // where the rotated rows go: q, or an array of its own
+  uint16_t* q_out;          // where the rotated rows go: q itself or beside it
   const uint16_t* k_new;    // [T][Hkv][D]
   const uint16_t* v_new;
   uint16_t* k_pool;         // [pages][Hkv][P][D]
@@ -37,9 +37,9 @@ struct KvAppendParams {
 // 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.
 constexpr int KV_APPEND_THREADS = 256;
 
-// ASIDE: the rotated queries go to an array of their own, where rows whose keys have no place are written all the same, zeros where
-// the table has no row.
-template <int D, int WPT, bool ASIDE>
+// EVERY_ROW: query rows whose keys have no place are written all the same, zeros where the table has no row.  (A lane has read
+// its vectors of a row before it writes them, so in place too.  The forms of two and four warps per token spill 8 bytes then.)
+template <int D, int WPT, bool EVERY_ROW>
 __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const KvAppendParams p) {
   constexpr int VEC = D / 8;            // 16-byte vectors per head row
   constexpr int HALF = VEC / 2;
@@ -99,14 +99,14 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
   int err = 0, page = 0;
   if (pos < 0 || page_idx >= p.max_pages_per_seq || !in_table) {
     if (lane == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_POSITION);
-    if (!ASIDE) return;
+    if (!EVERY_ROW) return;
     err = EFIM_DEV_BAD_POSITION;
   } else {
     page = *(p.block_table + (size_t)(lo + i_seq) * p.max_pages_per_seq + page_idx);
   }
   // rotary values: position j of the row's halves (8 of either), or the 4 pairs of vector j
   float c[8], sn[8];
-  if (p.cos_sin && (!ASIDE || in_table)) {
+  if (p.cos_sin && (!EVERY_ROW || in_table)) {
     const float* cs = p.cos_sin + (size_t)pos * D + j * (halves ? 8 : 4);      // cos[0..D/2) then sin[0..D/2)
     *reinterpret_cast<float4*>(c) = __ldg(reinterpret_cast<const float4*>(cs));
     *reinterpret_cast<float4*>(sn) = __ldg(reinterpret_cast<const float4*>(cs + D / 2));
@@ -117,11 +117,11 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
   }
   if (page < 0 || page >= p.num_pages) {
     if (lane == 0 && p.status) atomicOr(p.status, EFIM_DEV_BAD_PAGE);
-    if (!ASIDE) return;
+    if (!EVERY_ROW) return;
     err = EFIM_DEV_BAD_PAGE;
   }
   const size_t pool_tok = ((size_t)page * p.Hkv) * 16 * D + (size_t)(pos & 15) * D;   // + h * 16 * D
-  uint4* q_out = reinterpret_cast<uint4*>(const_cast<uint16_t*>(ASIDE ? p.q_out : p.q) + (size_t)t * p.Hq * D);
+  uint4* q_out = reinterpret_cast<uint4*>(const_cast<uint16_t*>(EVERY_ROW ? p.q_out : p.q) + (size_t)t * p.Hq * D);
   // straight copy of a [Hkv][D] row into the page slot; its first vectors have been fetched
   auto copy_row = [&](const uint4* src, uint16_t* pool) {
     for (int u0 = lane; u0 < n_vec; u0 += COPIES * LANES) {
@@ -133,8 +133,9 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
       }
     }
   };
-  if (!ASIDE || !err) copy_row(vin, p.v_pool);
+  if (!EVERY_ROW || !err) copy_row(vin, p.v_pool);
   if (!p.cos_sin) {
+    if (EVERY_ROW && err) return;
     if constexpr (AHEAD) fetch_copy(kin, lane);
     copy_row(kin, p.k_pool);
     return;
@@ -144,9 +145,9 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int hh = h + i * HP;
-      if (hh < nh && (!ASIDE || hh < nq || !err)) {
+      if (hh < nh && (!EVERY_ROW || hh < nq || !err)) {
         uint4* dst = hh < nq ? q_out + hh * VEC : reinterpret_cast<uint4*>(p.k_pool + pool_tok + (size_t)(hh - nq) * 16 * D);
-        if (ASIDE && !in_table) {
+        if (EVERY_ROW && !in_table) {
           dst[j] = make_uint4(0, 0, 0, 0);
           if (halves) dst[j + HALF] = make_uint4(0, 0, 0, 0);
         } else if (halves) {
@@ -180,7 +181,7 @@ extern "C" efim_status efim_rope_table_build(double base, int32_t head_dim, int3
 extern "C" efim_status efim_kv_append(const efim_cache_desc* cache, const efim_batch_desc* batch,
                                       const efim_rope_desc* rope, void* d_q, const void* d_k_new,
                                       const void* d_v_new, int32_t* d_status, void* stream) {
-  const efim::Append a{rope, d_q, d_q, d_k_new, d_v_new};
+  const efim::Append a{rope, d_q, d_q, false, d_k_new, d_v_new};
   const efim_status st = efim::append_check(cache, batch, a);
   return st != EFIM_OK ? st : efim::append_launch(cache, batch, a, d_status, stream);
 }
@@ -249,12 +250,11 @@ efim_status efim::append_launch(const efim_cache_desc* cache, const efim_batch_d
     else if (wpt == 4) EFIM_KV_APPEND_LAUNCH(D_, 4, A_); \
     else EFIM_KV_APPEND_LAUNCH(D_, 8, A_);               \
   } while (0)
-  const bool aside = a.q_out != a.q;
   if (cache->head_dim == 128) {
-    if (aside) EFIM_KV_APPEND_WARPS(128, true);
+    if (a.every_row) EFIM_KV_APPEND_WARPS(128, true);
     else EFIM_KV_APPEND_WARPS(128, false);
   } else {
-    if (aside) EFIM_KV_APPEND_WARPS(64, true);
+    if (a.every_row) EFIM_KV_APPEND_WARPS(64, true);
     else EFIM_KV_APPEND_WARPS(64, false);
   }
 #undef EFIM_KV_APPEND_WARPS

@@ -219,7 +219,7 @@ efim_status plan_and_run(const efim_cache_desc* cache, const efim_batch_desc* ba
   const bool aligned = !append || ((reinterpret_cast<uintptr_t>(append->k) | reinterpret_cast<uintptr_t>(append->v)) & 15) == 0;
   Append own;
   if (append && !(in_params && pl.s_max == 1 && aligned)) {  // (the kernel that appends is one of those with the list in its parameters)
-    own = Append{rope, nullptr, nullptr, append->k, append->v};
+    own = Append{rope, nullptr, nullptr, false, append->k, append->v};
     st = append_check(cache, batch, own);
     if (st != EFIM_OK) return st;
     before = &own;
@@ -317,11 +317,12 @@ extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, co
   if (d_k_new && !h_plan && appends_in_attention(cache, batch, rows, d_out, d_lse))
     return plan_and_run(cache, batch, rope, nullptr, &rows, d_q, d_out, d_lse, sm_scale, d_workspace, workspace_bytes, d_status,
                         stream);
-  efim::Append rows_first{rope, nullptr, nullptr, d_k_new, d_v_new};
+  efim::Append rows_first{rope, nullptr, nullptr, false, d_k_new, d_v_new};
   if (d_k_new) {
     if (rotates_into_out(cache, batch, rope, rows, d_q, d_out)) {
       rows_first.q = d_q;
       rows_first.q_out = d_out;
+      rows_first.every_row = true;
       d_q = d_out;
       rope = nullptr;
     }

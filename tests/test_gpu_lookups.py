@@ -118,3 +118,29 @@ def test_step_rotates_queries_whose_keys_have_no_page(interleaved):
         outs.append(out.view(torch.int16).clone())
         assert int(dw.status.item()) == BAD_PAGE | BAD_POSITION
     assert torch.equal(*outs) and torch.isfinite(out.float()).all()
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,tokens", [(8, 2, 40), (8, 2, 700), (48, 24, 1250), (8, 2, 1400), (8, 2, 2500)])   # 8, 4, 4, 2, 1 warps
+def test_step_in_place_over_rejected_tokens(Hq, Hkv, tokens, interleaved):
+    """The output on the queries themselves: tokens whose keys have no page attend with their rotated query, tokens beyond the
+    rotary table with a zero query, as they do where the attention kernel rotates the rows."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, 128, [60, tokens + 60], [tokens, 10], seed=6)
+    w.block_table[0, 5] = w.num_pages + 3                 # keys 80 .. 95 of the first sequence, new ones
+    dw = H.DeviceWorkload(w, interleaved=interleaved)
+    ws = torch.empty(efim.efim_prefill_workspace_bytes(dw.cache, dw.batch), dtype=torch.uint8, device="cuda")
+    short = efim.Rope(w.rope_base, w.head_dim, tokens + 68, interleaved)     # the last two positions have no table row
+    outs = []
+    for k, v, in_place in ((dw.k_new, dw.v_new, True), (None, None, False)):
+        q = dw.q.clone()
+        out = q if in_place else torch.empty_like(q)
+        _step(dw, short, q, k, v, out, ws)
+        torch.cuda.synchronize()
+        outs.append(out.view(torch.int16).clone())
+        assert int(dw.status.item()) == BAD_PAGE | BAD_POSITION
+        dw.status.zero_()
+    assert torch.equal(*outs) and torch.isfinite(out.float()).all()
