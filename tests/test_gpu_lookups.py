@@ -144,3 +144,30 @@ def test_step_in_place_over_rejected_tokens(Hq, Hkv, tokens, interleaved):
         assert int(dw.status.item()) == BAD_PAGE | BAD_POSITION
         dw.status.zero_()
     assert torch.equal(*outs) and torch.isfinite(out.float()).all()
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,D", [(32, 8, 128), (24, 8, 128), (8, 8, 64), (24, 8, 64)])
+def test_attention_of_many_items_rotates_on_load(Hq, Hkv, D, interleaved):
+    """The attention-only form of the step, whose CTAs rotate the queries of their second and later items as they load
+    them: the bits of efim_kv_append, which rotates them in memory, followed by the attention; the queries stay."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_items import _items, _lengths_of_every_shape
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, D, *_lengths_of_every_shape(Hq, Hkv, D), seed=Hq + D)
+    a = H.DeviceWorkload(w, interleaved=interleaved)
+    assert _items(a) >= 3 * torch.cuda.get_device_properties(0).multi_processor_count
+    q = a.q.clone()
+    a.gpu_kv_append()
+    a.gpu_prefill()
+    ws = torch.empty(efim.efim_prefill_workspace_bytes(a.cache, a.batch), dtype=torch.uint8, device="cuda")
+    out, lse = torch.empty_like(q), torch.empty_like(a.lse)
+    for _ in range(2):
+        out.fill_(float("nan"))
+        efim.efim_append_prefill_step(a.cache, a.batch, a.rope, q, None, None, out, lse, 0.0, ws, a.status)
+        torch.cuda.synchronize()
+        assert int(a.status.item()) == 0
+        assert torch.equal(a.out.view(torch.int16), out.view(torch.int16)) and torch.equal(a.lse, lse)
+        assert torch.equal(q.view(torch.int16), H.bits_to_torch(a.q_bits).view(torch.int16))
