@@ -232,8 +232,9 @@ efim_status efim::append_launch(const efim_cache_desc* cache, const efim_batch_d
   // 4,096, 2 below 16,384, look-ups before the rows): 256 tokens at 32/8 heads x 128 5.6 / 4.1 / 3.3 / 3.0 [3.9], 960 5.4 / 4.5 /
   // 4.7 / 5.1 [5.6], 2,336 7.2 / 7.1 / 8.0 / 9.8 [8.2], 25,600 99.4 / 97.6 / 98.7 / 118 [99.4]; 2,336 at 4/4 x 64 2.8 / 2.7 / 4.3 /
   // 7.0 [4.5], 8,192 5.5 / 7.1 / 11.5 / 20.5 [7.6]; 4,096 at 32/32 x 128 34.4 / 32.4 / 31.8 / 31.5 [33.2], 25,600 201 / 200 / 196 / 201 [201].
+  // Rows of q count where there are any: k and v alone of 16,384 tokens at 28/4 took 13.8 us with q's counted, 11.3 without.
   const int T = batch->total_new_tokens, resident = 4 * efim::sm_count();
-  const int vectors = (p.Hq + 2 * p.Hkv) * (cache->head_dim / 8);            // of a token's q, k and v
+  const int vectors = ((p.q ? p.Hq : 0) + 2 * p.Hkv) * (cache->head_dim / 8);   // of the rows that a token moves
   const int wpt = T <= resident ? 8 : T <= 2 * resident || vectors >= 1024 ? 4 : vectors >= 384 || T <= 4 * resident ? 2 : 1;
   const unsigned grid = (unsigned)(((long long)T * wpt * 32 + efim::KV_APPEND_THREADS - 1) / efim::KV_APPEND_THREADS);
   // With at most a CTA per SM the next kernel may start early (a step of 64 rows with its decode

@@ -1,6 +1,8 @@
 """Kernels whose warps look a token's sequence up 32 candidates at a time: batches of more than one and of more than two such
 trips, with sequences that bring nothing among them; every number of warps per token of the append; and one-call steps, whose
 append rotates the queries too."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -171,3 +173,40 @@ def test_attention_of_many_items_rotates_on_load(Hq, Hkv, D, interleaved):
         assert int(a.status.item()) == 0
         assert torch.equal(a.out.view(torch.int16), out.view(torch.int16)) and torch.equal(a.lse, lse)
         assert torch.equal(q.view(torch.int16), H.bits_to_torch(a.q_bits).view(torch.int16))
+
+
+class _KernelNodeParams(ctypes.Structure):       # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def _blocks_of(call):
+    """Blocks of the one kernel that a call enqueues, read off a graph it is captured into."""
+    import torch
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    cu, handle = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph())
+    nodes, n, p = (ctypes.c_void_p * 2)(), ctypes.c_size_t(2), _KernelNodeParams()
+    assert cu.cuGraphGetNodes(handle, nodes, ctypes.byref(n)) == 0 and n.value == 1
+    assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(nodes[0]), ctypes.byref(p)) == 0
+    return p.grid[0]
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,tokens,with_q,without", [
+    (28, 4, 128, 3000, 2, 1),              # warps per token
+    (48, 8, 64, 2400, 2, 1),
+    (32, 32, 128, 1200, 4, 4),             # k and v alone are as many rows
+    (4, 4, 64, 3000, 1, 1),
+])
+def test_append_without_queries_has_the_warps_that_its_rows_keep_busy(Hq, Hkv, D, tokens, with_q, without):
+    """Beyond what is resident at once, a token has as many warps as the rows that are moved keep busy: without q those of k
+    and v."""
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    dw = H.DeviceWorkload(_custom(Hq, Hkv, D, [5, 40], [tokens - 10, 10], seed=1))
+    for q, warps in ((dw.q, with_q), (None, without)):
+        blocks = _blocks_of(lambda: efim.efim_kv_append(dw.cache, dw.batch, dw.rope, q, dw.k_new, dw.v_new, dw.status))
+        assert blocks == -(-tokens * warps * 32 // 256)
