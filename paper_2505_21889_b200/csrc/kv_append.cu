@@ -34,11 +34,14 @@ struct KvAppendParams {
 //
 // Bound: HBM with many tokens, else a chain of dependent loads.  A token's rows do not depend on where it goes, so the first
 // of them (all, with few tokens) are on their way before its sequence is looked up; the warp's lanes look that up together,
-// 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.
+// 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.  The rotated
+// rows come by ordinary loads: kept out of L1 as v's are, 2,336 tokens at 32/32 heads take 13.4 us instead of 12.6 (k and v alone 10.2
+// and 8.8), 16,384 at 4/4 x 64 10.0 and 9.0, 25,600 at 32/32 195.8 and 193.3 (the other way round where q, k, v and pages are just as much
+// as L2 holds: 8,192 at 32/8 31.1 and 32.3).
 constexpr int KV_APPEND_THREADS = 256;
 
 // EVERY_ROW: query rows whose keys have no place are written all the same, zeros where the table has no row.  (A lane has read
-// its vectors of a row before it writes them, so in place too.  The forms of two and four warps per token spill 8 bytes then.)
+// its vectors of a row before it writes them, so in place too.)
 template <int D, int WPT, bool EVERY_ROW>
 __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const KvAppendParams p) {
   constexpr int VEC = D / 8;            // 16-byte vectors per head row
@@ -70,8 +73,8 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
 #pragma unroll
     for (int i = 0; i < 2; ++i)
       if (h + i * HP < nh) {
-        a[i] = ldg_stream(row_of(h + i * HP) + j);
-        if (halves) b[i] = ldg_stream(row_of(h + i * HP) + j + HALF);
+        a[i] = row_of(h + i * HP)[j];
+        if (halves) b[i] = row_of(h + i * HP)[j + HALF];
       }
   };
   if constexpr (AHEAD) {
@@ -228,11 +231,11 @@ efim_status efim::append_launch(const efim_cache_desc* cache, const efim_batch_d
   p.Hkv = cache->num_kv_heads;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // Warps per token: 8, and 4, while every token's CTA is resident at once (a token's latency is the time); beyond that as many as
-  // its rows keep busy for a few vectors each.  Microseconds with 1 / 2 / 4 / 8 (in brackets as it was: 8 below 1,024 tokens, 4 below
-  // 4,096, 2 below 16,384, look-ups before the rows): 256 tokens at 32/8 heads x 128 5.6 / 4.1 / 3.3 / 3.0 [3.9], 960 5.4 / 4.5 /
-  // 4.7 / 5.1 [5.6], 2,336 7.2 / 7.1 / 8.0 / 9.8 [8.2], 25,600 99.4 / 97.6 / 98.7 / 118 [99.4]; 2,336 at 4/4 x 64 2.8 / 2.7 / 4.3 /
-  // 7.0 [4.5], 8,192 5.5 / 7.1 / 11.5 / 20.5 [7.6]; 4,096 at 32/32 x 128 34.4 / 32.4 / 31.8 / 31.5 [33.2], 25,600 201 / 200 / 196 / 201 [201].
-  // Rows of q count where there are any: k and v alone of 16,384 tokens at 28/4 took 13.8 us with q's counted, 11.3 without.
+  // its rows - q's where there are any - keep busy for a few vectors each.  Microseconds with 1 / 2 / 4 / 8 (in brackets with 8 below
+  // 1,024 tokens, 4 below 4,096, 2 below 16,384 and look-ups before the rows): 256 tokens at 32/8 heads x 128 4.9 / 3.5 / 3.5 / 3.6
+  // [3.4], 960 5.1 / 4.3 / 4.4 / 4.6 [5.6], 2,336 7.1 / 6.9 / 7.4 / 9.1 [8.4], 25,600 99.1 / 97.5 / 98.8 / 110 [99.3]; 2,336 at 4/4 x 64
+  // 3.6 / 3.5 / 4.1 / 6.4 [4.4], 8,192 5.4 / 6.8 / 11.2 / 18.9 [7.5]; 4,096 at 32/32 x 128 34.6 / 33.1 / 32.5 / 32.5 [33.4], 25,600
+  // 199 / 197 / 193 / 193 [201]; k and v alone of 16,384 at 28/4 9.9 / 13.2 / 22.2 / 38.5 [10.5].
   const int T = batch->total_new_tokens, resident = 4 * efim::sm_count();
   const int vectors = ((p.q ? p.Hq : 0) + 2 * p.Hkv) * (cache->head_dim / 8);   // of the rows that a token moves
   const int wpt = T <= resident ? 8 : T <= 2 * resident || vectors >= 1024 ? 4 : vectors >= 384 || T <= 4 * resident ? 2 : 1;
