@@ -1563,6 +1563,10 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
     const float Lr = __shfl_sync(0xffffffffu, L[r >> 1], (r & 1) * 16), Mr = __shfl_sync(0xffffffffu, M[r >> 1], (r & 1) * 16);
     if (r >= nr) break;
     const float inv = Lr == 0.f ? 0.f : 1.f / Lr;
+    if (Lr == 0.f) {                                        // (no chunk has a weight: what their partials hold is not looked at)
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) acc[r][e] = 0.f;
+    }
     uint16_t* out = p.out + (th + r) * D + lane * EPL;
     if constexpr (EPL == 4) {
       *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16x2(acc[r][0] * inv, acc[r][1] * inv), pack_bf16x2(acc[r][2] * inv, acc[r][3] * inv));

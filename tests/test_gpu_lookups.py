@@ -210,3 +210,23 @@ def test_append_without_queries_has_the_warps_that_its_rows_keep_busy(Hq, Hkv, D
     for q, warps in ((dw.q, with_q), (None, without)):
         blocks = _blocks_of(lambda: efim.efim_kv_append(dw.cache, dw.batch, dw.rope, q, dw.k_new, dw.v_new, dw.status))
         assert blocks == -(-tokens * warps * 32 // 256)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(32, 8, 128), (6, 2, 64), (3, 1, 128)])
+def test_merge_of_rows_without_a_finite_score(Hq, Hkv, D):
+    """All scores of a row that is cut into key chunks are minus infinity (their keys are -3e38, the queries 3e38): output 0 and
+    lse -inf, whatever its values hold - a partial without weight is not looked at."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    import tests.gpu_harness as H
+    from tests.test_gpu_parity import _custom
+    w = _custom(Hq, Hkv, D, [9000, 40], [20, 3], seed=D + Hq)      # (more than 32 rows to a kv head)
+    dw = H.DeviceWorkload(w, use_rope=False)
+    assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 2
+    dw.k_pool.fill_(-3e38)
+    dw.v_pool.fill_(float("inf"))
+    dw.q[:20].fill_(3e38)
+    dw.gpu_prefill()
+    torch.cuda.synchronize()
+    assert int(dw.status.item()) == 0
+    assert bool((dw.out[:20].float() == 0).all()) and bool((dw.lse[:20] == float("-inf")).all())
