@@ -1454,8 +1454,8 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
   }
 }
 
-// Merge the KV-chunk partials of split sequences.  A warp takes up to ROWS consecutive heads of one token, with the partial
-// rows of 8 / ROWS chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the
+// Merge the KV-chunk partials of split sequences.  A warp takes MERGE_ROWS consecutive heads of one token (a divisor of all), with
+// the partial rows of AT_ONCE chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the
 // launch parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
 //
 // Bound: the partials' bytes, which the kernel before has left in L2, behind a chain of dependent look-ups.  The lanes look
@@ -1465,16 +1465,18 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
 // instead of 355 for the layer.  A row a warp while there are few, else four.  Attention and merge with one / four [a warp per
 // row, bisecting]: 2 x 1-2 tokens over 8-10k at 4/4 heads x 64 10.7 / 14.2 [12.0] us, 111 tokens over 3-14k at 32/8 (3,552 rows)
 // 45.8 / 48.9 [46.2], 150 over 3-5k at 32/32 (4,800) 35.5 / 35.6 [35.6], 380 over 4-8k at 24/8 (9,120) 53.5 / 49.5 [51.9].
+//
+// Many rows of heads that are no multiple of four: two rows a warp, or one, with four chunks in flight (eight: 4 x 500-620 tokens over
+// 3-4k at 5/1 36.9 us instead of 35.3, 4 x 100-300 over 5-9k at 9/3 45.5 and 42.2).  With the form for four fetching its last row
+// again, in brackets a warp per row: these 40.8 [35.4] and 49.0 [42.5], 8 x 900-1,000 over 6-9k at 5/1 177.8 [178.2] and now 161.5,
+// 3 x 400-700 over 3-6k at 6/2 40.3 [36.2] and 35.6, 3 x 90-200 at 14/2 31.1 [28.8] and 30.0.
 constexpr int MERGE_WARPS = 8;
-__host__ __device__ constexpr int merge_rows(int Hq, int at_most) { return at_most >= 4 && Hq % 4 == 0 ? 4 : (at_most >= 2 && Hq % 2 == 0 ? 2 : 1); }
-template <int D, int MERGE_ROWS, typename Split>
+template <int D, int MERGE_ROWS, int AT_ONCE, typename Split>
 __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const Params p, const __grid_constant__ Split split) {
   constexpr int EPL = D / 32;                               // dims of a lane
-  constexpr int AT_ONCE = 8 / MERGE_ROWS;                   // chunks whose rows are in flight together
   constexpr bool inl = std::is_same<Split, InlineSplit>::value;
   const int lane = threadIdx.x & 31;
-  const int nr = merge_rows(p.Hq, MERGE_ROWS);              // rows of this warp: heads of one token
-  const size_t th = ((size_t)blockIdx.x * MERGE_WARPS + (threadIdx.x >> 5)) * nr;
+  const size_t th = ((size_t)blockIdx.x * MERGE_WARPS + (threadIdx.x >> 5)) * MERGE_ROWS;    // this warp's rows: heads of one token
   // (everything before the attention kernel has completed, and that kernel writes partials only: the
   // look-ups need not wait for it.  Read in L2, where what has completed is visible.)
   int st = 0, nc = 0;
@@ -1507,7 +1509,7 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
       for (int i = threadIdx.x; i < p.batch; i += 32 * MERGE_WARPS) p.split_out[i] = split.keys[i];
   }
   if (nc == 0) return;                                      // written directly by the main kernel
-  // rows r of chunks c0 .. c0 + AT_ONCE - 1 (rows past the last: read again, not used)
+  // rows r of chunks c0 .. c0 + AT_ONCE - 1
   const float* po = p.part_o + th * p.s_max * D + lane * EPL;
   __align__(16) float v[AT_ONCE][MERGE_ROWS][EPL];
   auto fetch = [&](int c0) {
@@ -1516,7 +1518,7 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
 #pragma unroll
       for (int r = 0; r < MERGE_ROWS; ++r) {
         if (c0 + c >= nc) continue;
-        const float* src = po + ((size_t)min(r, nr - 1) * p.s_max + c0 + c) * D;
+        const float* src = po + ((size_t)r * p.s_max + c0 + c) * D;
         if constexpr (EPL == 4) {
           *reinterpret_cast<float4*>(v[c][r]) = __ldcg(reinterpret_cast<const float4*>(src));
         } else {
@@ -1529,7 +1531,7 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
   float lse[2];
 #pragma unroll
   for (int j = 0; j < 2; ++j)
-    lse[j] = my_c < nc && my_r + 2 * j < nr ? __ldcg(p.part_lse + (th + my_r + 2 * j) * p.s_max + my_c) : -INFINITY;
+    lse[j] = my_c < nc && my_r + 2 * j < MERGE_ROWS ? __ldcg(p.part_lse + (th + my_r + 2 * j) * p.s_max + my_c) : -INFINITY;
   fetch(0);
   float M[2], L[2], w[2];
 #pragma unroll
@@ -1561,7 +1563,6 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const P
 #pragma unroll
   for (int r = 0; r < MERGE_ROWS; ++r) {
     const float Lr = __shfl_sync(0xffffffffu, L[r >> 1], (r & 1) * 16), Mr = __shfl_sync(0xffffffffu, M[r >> 1], (r & 1) * 16);
-    if (r >= nr) break;
     const float inv = Lr == 0.f ? 0.f : 1.f / Lr;
     if (Lr == 0.f) {                                        // (no chunk has a weight: what their partials hold is not looked at)
 #pragma unroll
@@ -1891,17 +1892,22 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
   if (st != EFIM_OK) return st;
   if (pl.s_max > 1) {
     const size_t rows = (size_t)p.total_new_tokens * p.Hq;
-    auto merge = [&](auto kernel, int at_most, const auto& split) -> efim_status {
-      const size_t per_block = (size_t)MERGE_WARPS * merge_rows(p.Hq, at_most);
-      EFIM_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)((rows + per_block - 1) / per_block)), dim3(32 * MERGE_WARPS), 0, s, p, split));
-      return EFIM_OK;
-    };
     using Split = std::conditional_t<inl, InlineSplit, NoList>;
     const Split* split;
     NoList none;
     if constexpr (inl) split = &list.split;
     else split = &none;
-    return rows <= (size_t)32 * sm_count() ? merge(prefill_merge_kernel<D, 1, Split>, 1, *split) : merge(prefill_merge_kernel<D, 4, Split>, 4, *split);
+    auto merge = [&](auto per_warp, auto at_once) -> efim_status {
+      constexpr int ROWS = decltype(per_warp)::value, per_block = MERGE_WARPS * ROWS;
+      EFIM_CUDA_TRY(launch_pdl(prefill_merge_kernel<D, ROWS, decltype(at_once)::value, Split>,
+                               dim3((unsigned)((rows + per_block - 1) / per_block)), dim3(32 * MERGE_WARPS), 0, s, p, *split));
+      return EFIM_OK;
+    };
+    using One = std::integral_constant<int, 1>;
+    using Two = std::integral_constant<int, 2>;
+    using Four = std::integral_constant<int, 4>;
+    if (rows <= (size_t)32 * sm_count()) return merge(One{}, std::integral_constant<int, 8>{});
+    return p.Hq % 4 == 0 ? merge(Four{}, Two{}) : p.Hq % 2 == 0 ? merge(Two{}, Four{}) : merge(One{}, Four{});
   }
   return EFIM_OK;
 }

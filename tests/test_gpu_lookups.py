@@ -230,3 +230,17 @@ def test_merge_of_rows_without_a_finite_score(Hq, Hkv, D):
     torch.cuda.synchronize()
     assert int(dw.status.item()) == 0
     assert bool((dw.out[:20].float() == 0).all()) and bool((dw.lse[:20] == float("-inf")).all())
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new", [
+    (6, 2, 64, [4000, 10, 5000, 4500], [300, 5, 330, 280]),        # two rows a warp
+    (5, 1, 128, [3000, 0, 4000], [500, 7, 620]),                   # one
+])
+def test_merge_of_many_rows_at_other_head_counts(Hq, Hkv, D, cached, new):
+    """Cut key ranges and more rows than a row a warp is for, where four heads are not a divisor of all."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    from tests.test_gpu_parity import _check_turn, _custom
+    assert sum(new) * Hq > 32 * torch.cuda.get_device_properties(0).multi_processor_count
+    dw, _ = _check_turn(_custom(Hq, Hkv, D, cached, new, seed=Hq), use_rope=False)
+    assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 2
