@@ -189,8 +189,8 @@ efim_status efim_append_prefill_attn_planned(const efim_cache_desc* cache, const
  * - out, lse and the pools bit for bit - but d_q is READ ONLY (unless d_out is d_q): the append leaves each query
  * row, rotated by its position cached_len[s] + i (the same fp32 arithmetic and single bf16 rounding), in d_out,
  * where the attention takes it from and then writes the row's output.  Where d_out overlaps d_k_new, d_v_new or
- * another part of d_q, without k/v (below) and in one-kernel steps, the attention kernel rotates the rows of d_q
- * as it loads them instead.
+ * another part of d_q, without k/v (below) and, without a plan, where a single sequence brings new tokens, at most 128
+ * (token, head-in-group) rows, the attention kernel rotates the rows of d_q as it loads them instead.
  * h_plan = NULL: the work list is planned inside the call (as efim_append_prefill_attn does);
  * otherwise h_plan / plan_bytes / lists_resident are those of
  * efim_append_prefill_attn_planned.  `rope` may be NULL or hold a NULL table (no rotation).

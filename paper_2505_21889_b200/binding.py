@@ -280,8 +280,9 @@ def efim_append_prefill_attn(cache: Cache, batch: Batch, q, out, lse=None, sm_sc
 
 def efim_append_prefill_step(cache: Cache, batch: Batch, rope, q, k_new, v_new, out, lse=None, sm_scale=0.0,
                              workspace=None, status=None, stream=None, plan=None, lists_resident=False):
-    """kv_append of the new tokens' k/v and append-prefill attention with q rotated on load
-    (q is not modified)."""
+    """kv_append of the new tokens' k/v, then append-prefill attention of q rotated by its positions.  q is not modified, unless
+    out is q (which is allowed): the append may leave the rotated queries in out, where their outputs go afterwards.  A call that
+    is refused has changed nothing."""
     st = _calls.append_prefill_step(_addr(cache.desc), _addr(batch.desc), _addr(rope.desc) if rope is not None else None,
                                     q, k_new, v_new, out, lse, sm_scale, plan, 1 if lists_resident else 0, workspace,
                                     status, _stream_ptr(stream))

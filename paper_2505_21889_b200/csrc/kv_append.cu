@@ -28,9 +28,9 @@ struct KvAppendParams {
 // dimension (vector j, and for the rotate-half pairing its partner j + D/16), so its
 // cos/sin values are loaded once, and walks the heads - q heads (rotated in place), then
 // k heads (rotated into the page slot) - two at a time so that several 16-byte loads are
-// in flight per lane; v is copied straight into the page slot.  Many tokens: one warp per
-// token keeps every SM full of independent streams.  Few tokens (a decode step): eight
-// warps per token, because then the time is one token's latency.
+// in flight per lane; v is copied straight into the page slot.  Few tokens (a decode step): eight
+// warps per token, because then the time is one token's latency.  Many: as few as its rows keep busy,
+// from one to four (append_launch), so that every SM is full of independent streams.
 //
 // Bound: HBM with many tokens, else a chain of dependent loads.  A token's rows do not depend on where it goes, so the first
 // of them (all, with few tokens) are on their way before its sequence is looked up; the warp's lanes look that up together,

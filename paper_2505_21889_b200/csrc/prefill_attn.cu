@@ -269,8 +269,9 @@ bool appends_in_attention(const efim_cache_desc* cache, const efim_batch_desc* b
   return with_work == 1 && cache->num_kv_heads <= efim::sm_count();
 }
 // Whether the append kernel rotates a step's query rows, and leaves them where their outputs go: a work item has its rows in shared
-// memory before it writes them, and no other one reads them (the chunks of a cut key range write partials, and the merge comes
-// after all of them).  Not where the output lies on the rows that the append reads, beyond row for row on q itself.  The
+// memory before it writes them, and no other one computes with them (the chunks of a cut key range write partials, and the merge
+// comes after all of them).  Copies of 32 rows that reach past an item's last one may read rows that another CTA is writing: nothing
+// of theirs is stored, nor does it steer a step.  Not where the output lies on the rows that the append reads, beyond row for row on q itself.  The
 // attention kernel can rotate rows as it loads them, but its CTAs' warps wait for that, 12,300 cycles per item.  One-call steps with it
 // and with the append: 16 prompts of 1-3.5k tokens 869 and 827 us, 53 x 1-406 over 100-549 at 24/8 100 and 75, 40 x 10-22 over
 // 24-125 at 40/8 39 and 30, 39 x 1-5 over 0 at 16/1 12.3 and 9.2, 9 x 1 over 193-632 at 32/8 x 64 10.9 and 10.7.
@@ -304,8 +305,9 @@ extern "C" efim_status efim_append_prefill_attn(const efim_cache_desc* cache, co
                       d_status, stream);
 }
 
-// Steps 1 and 2 of a turn: the new tokens' k/v go into the pages (k rotated), then the new
-// queries, rotated as they are loaded, attend over everything before them.
+// Steps 1 and 2 of a turn: the new tokens' k/v go into the pages (k rotated), then the new queries - rotated by the append
+// into d_out, or by the attention kernel as it loads them (rotates_into_out, appends_in_attention) - attend over everything before
+// them.
 extern "C" efim_status efim_append_prefill_step(const efim_cache_desc* cache, const efim_batch_desc* batch,
                                                 const efim_rope_desc* rope, const void* d_q, const void* d_k_new,
                                                 const void* d_v_new, void* d_out, float* d_lse, float sm_scale,

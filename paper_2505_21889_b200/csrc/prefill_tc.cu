@@ -1455,16 +1455,17 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
 }
 
 // Merge the KV-chunk partials of split sequences.  A warp takes MERGE_ROWS consecutive heads of one token (a divisor of all), with
-// the partial rows of AT_ONCE chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList) or in the
-// launch parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
+// the partial rows of AT_ONCE chunks in flight.  `split`: keys per chunk of every sequence, 0 = not split - in the workspace (NoList)
+// or in the launch parameters (InlineSplit), in which case the kernel leaves it in the workspace too.
 //
 // Bound: the partials' bytes, which the kernel before has left in L2, behind a chain of dependent look-ups.  The lanes look
 // a token's sequence up together, 32 candidates a trip, and bring its lengths along in the last one; with a warp per row
 // that bisected q_indptr and then read one value after the other, a chain of ten trips in each of 8 waves of CTAs,
-// the merge of 960 tokens at 32/8 heads in two chunks took 25 us; now 6.2, and 64 mixed rows at 28/4 cut into 516 items 300 us
-// instead of 355 for the layer.  A row a warp while there are few, else four.  Attention and merge with one / four [a warp per
-// row, bisecting]: 2 x 1-2 tokens over 8-10k at 4/4 heads x 64 10.7 / 14.2 [12.0] us, 111 tokens over 3-14k at 32/8 (3,552 rows)
-// 45.8 / 48.9 [46.2], 150 over 3-5k at 32/32 (4,800) 35.5 / 35.6 [35.6], 380 over 4-8k at 24/8 (9,120) 53.5 / 49.5 [51.9].
+// the merge of 960 tokens at 32/8 heads in two chunks took 25 us; now 6.2, and 64 mixed rows at 28/4, cut into 516 items on trial
+// (the planner leaves 500; 304 us), 307 us instead of 355 for the layer.  A row a warp while there are few, else four.  Attention and
+// merge with one / four [a warp per row, bisecting]: 2 x 1-2 tokens over 8-10k at 4/4 heads x 64 10.7 / 14.2 [12.0] us, 111 tokens
+// over 3-14k at 32/8 (3,552 rows) 45.8 / 48.9 [46.2], 150 over 3-5k at 32/32 (4,800) 35.5 / 35.6 [35.6], 380 over 4-8k at 24/8
+// (9,120) 53.5 / 49.5 [51.9].
 //
 // Many rows of heads that are no multiple of four: two rows a warp, or one, with four chunks in flight (eight: 4 x 500-620 tokens over
 // 3-4k at 5/1 36.9 us instead of 35.3, 4 x 100-300 over 5-9k at 9/3 45.5 and 42.2).  With the form for four fetching its last row
