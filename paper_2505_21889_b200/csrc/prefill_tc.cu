@@ -1462,15 +1462,16 @@ prefill_tc_kernel(const Params p, const __grid_constant__ CUtensorMap map_k, con
 // a token's sequence up together, 32 candidates a trip, and bring its lengths along in the last one; with a warp per row
 // that bisected q_indptr and then read one value after the other, a chain of ten trips in each of 8 waves of CTAs,
 // the merge of 960 tokens at 32/8 heads in two chunks took 25 us; now 6.2, and 64 mixed rows at 28/4, cut into 516 items on trial
-// (the planner leaves 500; 304 us), 307 us instead of 355 for the layer.  A row a warp while there are few, else four.  Attention and
-// merge with one / four [a warp per row, bisecting]: 2 x 1-2 tokens over 8-10k at 4/4 heads x 64 10.7 / 14.2 [12.0] us, 111 tokens
-// over 3-14k at 32/8 (3,552 rows) 45.8 / 48.9 [46.2], 150 over 3-5k at 32/32 (4,800) 35.5 / 35.6 [35.6], 380 over 4-8k at 24/8
-// (9,120) 53.5 / 49.5 [51.9].
+// (the planner leaves 500; 304 us), 307 us instead of 355 for the layer.
 //
-// Many rows of heads that are no multiple of four: two rows a warp, or one, with four chunks in flight (eight: 4 x 500-620 tokens over
-// 3-4k at 5/1 36.9 us instead of 35.3, 4 x 100-300 over 5-9k at 9/3 45.5 and 42.2).  With the form for four fetching its last row
-// again, in brackets a warp per row: these 40.8 [35.4] and 49.0 [42.5], 8 x 900-1,000 over 6-9k at 5/1 177.8 [178.2] and now 161.5,
-// 3 x 400-700 over 3-6k at 6/2 40.3 [36.2] and 35.6, 3 x 90-200 at 14/2 31.1 [28.8] and 30.0.
+// Rows of a warp and chunks in flight.  Up to 32 rows an SM there are warps enough resident for a row each, with eight chunks in flight
+// (2 x 1-2 tokens over 8-10k at 4/4 heads x 64 attention and merge 10.7 us, four rows a warp 14.2 [a warp per row, bisecting, 12.0]); up
+// to 80 a row each, with four, which leaves room for more warps; beyond that looking up is what there is to save: four heads, or two.
+// Append, attention and merge with 1 x 4 / 2 x 4 / 4 x 2 [as in the brackets above]: 2 x 150-160 over 9-12k at 16/1 (4,900 rows)
+// 38.0 / 38.9 / 40.3 [37.9], 6 x 20-30 over 3-8k at 32/8 x 64 (4,900) 27.5 / 28.0 / 28.8 [28.3], 12 x 10-60 over 0.5-4k at 16/1 (7,600)
+// 26.0 / 26.6 / 27.9 [29.6], 4 x 60-110 over 5-9k at 32/8 (10,100) 73.3 / 74.2 / 75.3 [73.2], 10 x 20-60 over 0.8-3k at 28/4 (11,700)
+// 36.0 / 33.0 / 32.1 [39.6], 12 x 10-60 over 0.5-4k at 32/8 (15,100) 58.5 / 57.9 / 57.3 [64.4].  An odd number of heads: one row, four
+// chunks at any size (eight: 4 x 500-620 tokens over 3-4k at 5/1 36.9 us instead of 35.3, 4 x 100-300 over 5-9k at 9/3 45.5 and 42.2).
 constexpr int MERGE_WARPS = 8;
 template <int D, int MERGE_ROWS, int AT_ONCE, typename Split>
 __global__ void __launch_bounds__(32 * MERGE_WARPS) prefill_merge_kernel(const Params p, const __grid_constant__ Split split) {
@@ -1908,7 +1909,8 @@ static efim_status launch_d(const efim_cache_desc* c, const Params& args, const 
     using Two = std::integral_constant<int, 2>;
     using Four = std::integral_constant<int, 4>;
     if (rows <= (size_t)32 * sm_count()) return merge(One{}, std::integral_constant<int, 8>{});
-    return p.Hq % 4 == 0 ? merge(Four{}, Two{}) : p.Hq % 2 == 0 ? merge(Two{}, Four{}) : merge(One{}, Four{});
+    if (rows <= (size_t)80 * sm_count() || p.Hq % 2 != 0) return merge(One{}, Four{});
+    return p.Hq % 4 == 0 ? merge(Four{}, Two{}) : merge(Two{}, Four{});
   }
   return EFIM_OK;
 }

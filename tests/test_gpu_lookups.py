@@ -233,14 +233,32 @@ def test_merge_of_rows_without_a_finite_score(Hq, Hkv, D):
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,cached,new", [
-    (6, 2, 64, [4000, 10, 5000, 4500], [300, 5, 330, 280]),        # two rows a warp
-    (5, 1, 128, [3000, 0, 4000], [500, 7, 620]),                   # one
+    (6, 2, 64, [4000, 10, 5000, 4500], [300, 5, 330, 280]),
+    (5, 1, 128, [3000, 0, 4000], [500, 7, 620]),
 ])
 def test_merge_of_many_rows_at_other_head_counts(Hq, Hkv, D, cached, new):
-    """Cut key ranges and more rows than a row a warp is for, where four heads are not a divisor of all."""
+    """Cut key ranges and more rows than eight chunks in flight are for, where four heads are not a divisor of all."""
     import torch
     import paper_2505_21889_b200 as efim
     from tests.test_gpu_parity import _check_turn, _custom
     assert sum(new) * Hq > 32 * torch.cuda.get_device_properties(0).multi_processor_count
+    dw, _ = _check_turn(_custom(Hq, Hkv, D, cached, new, seed=Hq), use_rope=False)
+    assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 2
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,cached,new,rows_per_sm", [
+    (16, 1, 128, [2000, 900, 7], [200, 150, 4], 32),       # one row a warp, four chunks in flight
+    (32, 8, 128, [1500, 900, 7], [300, 90, 4], 80),        # four rows a warp
+    (28, 4, 64, [2000, 900, 7], [300, 150, 4], 80),
+    (6, 2, 64, [3000, 10], [2000, 5], 80),                 # two
+    (14, 2, 128, [3000, 2000], [600, 300], 80),
+])
+def test_merge_forms_of_many_rows(Hq, Hkv, D, cached, new, rows_per_sm):
+    """Cut key ranges on either side of where a warp takes more than one row."""
+    import torch
+    import paper_2505_21889_b200 as efim
+    from tests.test_gpu_parity import _check_turn, _custom
+    rows = sum(new) * Hq / torch.cuda.get_device_properties(0).multi_processor_count
+    assert rows > 80 if rows_per_sm == 80 else 32 < rows <= 80
     dw, _ = _check_turn(_custom(Hq, Hkv, D, cached, new, seed=Hq), use_rope=False)
     assert efim.efim_prefill_launch_count(dw.cache, dw.batch) == 2
