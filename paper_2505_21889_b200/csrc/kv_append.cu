@@ -34,10 +34,11 @@ struct KvAppendParams {
 //
 // Bound: HBM with many tokens, else a chain of dependent loads.  A token's rows do not depend on where it goes, so the first
 // of them (all, with few tokens) are on their way before its sequence is looked up; the warp's lanes look that up together,
-// 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.  The rotated
-// rows come by ordinary loads: kept out of L1 as v's are, 2,336 tokens at 32/32 heads take 13.4 us instead of 12.6 (k and v alone 10.2
-// and 8.8), 16,384 at 4/4 x 64 10.0 and 9.0, 25,600 at 32/32 195.8 and 193.3 (the other way round where q, k, v and pages are just as much
-// as L2 holds: 8,192 at 32/8 31.1 and 32.3).
+// 32 candidates a trip, and bring the lengths along in the last one; page id and rotary row are fetched side by side.
+// Rotated rows come past L1, as v's do, where they are fetched ahead with q among them, else by ordinary loads.  Past L1 everywhere:
+// k and v alone of 2,336 tokens at 32/32 heads 10.1 us instead of 8.9, of 25,600 at 32/32 132.6 and 130.6, and with a warp a token
+// 16,384 at 4/4 x 64 9.5 and 8.7.  Ordinary loads everywhere: some appends alone are shorter (2,336 at 32/32 13.5 -> 12.6), but one-call
+// steps of 9 x 500-900 tokens at 28/4 are 82.9 us instead of 79.3, of 9 x 200-400 at 32/32 64.1 and 59.5.
 constexpr int KV_APPEND_THREADS = 256;
 
 // EVERY_ROW: query rows whose keys have no place are written all the same, zeros where the table has no row.  (A lane has read
@@ -73,8 +74,14 @@ __global__ void __launch_bounds__(KV_APPEND_THREADS, 4) kv_append_kernel(const K
 #pragma unroll
     for (int i = 0; i < 2; ++i)
       if (h + i * HP < nh) {
-        a[i] = row_of(h + i * HP)[j];
-        if (halves) b[i] = row_of(h + i * HP)[j + HALF];
+        const uint4* row = row_of(h + i * HP) + j;
+        if (AHEAD && p.q) {
+          a[i] = ldg_stream(row);
+          if (halves) b[i] = ldg_stream(row + HALF);
+        } else {
+          a[i] = *row;
+          if (halves) b[i] = row[HALF];
+        }
       }
   };
   if constexpr (AHEAD) {
@@ -232,10 +239,10 @@ efim_status efim::append_launch(const efim_cache_desc* cache, const efim_batch_d
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // Warps per token: 8, and 4, while every token's CTA is resident at once (a token's latency is the time); beyond that as many as
   // its rows - q's where there are any - keep busy for a few vectors each.  Microseconds with 1 / 2 / 4 / 8 (in brackets with 8 below
-  // 1,024 tokens, 4 below 4,096, 2 below 16,384 and look-ups before the rows): 256 tokens at 32/8 heads x 128 4.9 / 3.5 / 3.5 / 3.6
-  // [3.4], 960 5.1 / 4.3 / 4.4 / 4.6 [5.6], 2,336 7.1 / 6.9 / 7.4 / 9.1 [8.4], 25,600 99.1 / 97.5 / 98.8 / 110 [99.3]; 2,336 at 4/4 x 64
-  // 3.6 / 3.5 / 4.1 / 6.4 [4.4], 8,192 5.4 / 6.8 / 11.2 / 18.9 [7.5]; 4,096 at 32/32 x 128 34.6 / 33.1 / 32.5 / 32.5 [33.4], 25,600
-  // 199 / 197 / 193 / 193 [201]; k and v alone of 16,384 at 28/4 9.9 / 13.2 / 22.2 / 38.5 [10.5].
+  // 1,024 tokens, 4 below 4,096, 2 below 16,384 and look-ups before the rows): 64 tokens at 32/8 heads x 128 4.9 / 3.5 / 3.2 / 3.2 [3.2],
+  // 960 5.0 / 4.3 / 4.4 / 4.7 [5.4], 2,336 6.8 / 7.1 / 7.9 / 9.4 [8.0], 25,600 99.0 / 97.7 / 99.1 / 110 [99.5]; 2,336 at 4/4 x 64 3.3 / 3.3 /
+  // 4.2 / 6.6 [4.4], 8,192 4.9 / 7.0 / 11.7 / 19.6 [7.5]; 4,096 at 32/32 x 128 34.9 / 32.2 / 31.9 / 31.7 [34.0], 25,600 199 / 199 / 195 / 194
+  // [201]; k and v alone of 16,384 at 28/4 10.0 / 13.4 / 22.3 / 38.5 [10.5].
   const int T = batch->total_new_tokens, resident = 4 * efim::sm_count();
   const int vectors = ((p.q ? p.Hq : 0) + 2 * p.Hkv) * (cache->head_dim / 8);   // of the rows that a token moves
   const int wpt = T <= resident ? 8 : T <= 2 * resident || vectors >= 1024 ? 4 : vectors >= 384 || T <= 4 * resident ? 2 : 1;
